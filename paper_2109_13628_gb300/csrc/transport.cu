@@ -34,15 +34,17 @@ static constexpr double kStabC = 1.620, kStabR = 0.314;
 __constant__ int t_dir_i[4] = {1, -1, 0, 0};
 __constant__ int t_dir_j[4] = {0, 0, 1, -1};
 
+// Fields of one evaluation in the caller's layout (NY rows of NX), read at fluid nodes only; the
+// extensions at the A- nodes are kept per A- index, so no field is copied or rewritten.
 struct TrView {
     int NX, NY, nx;
-    double h;
+    double h, rh;            // cell size and 1 / h
+    int h_pow2;              // 1 / h is exact
     const uint8_t* cls;      // padded
     const int* minus_map;    // padded -> A- index
-    const double* w;         // padded vorticity (fluid values)
-    const double* ux;        // padded velocity with A- ghosts
-    const double* uy;
-    const double* g4;        // per A- node: fourth-order extension with omega_b
+    const double *w, *ux, *uy;
+    const double *gux, *guy; // per A- node: third-order velocity extension with u_b
+    const double* g4;        //              fourth-order vorticity extension with omega_b
     const double* g3;        //              third-order with omega_b
     const double* g3n;       //              third-order without boundary condition
     double Ux, Uy;
@@ -50,22 +52,27 @@ struct TrView {
 
 __device__ __forceinline__ bool t_inside(const TrView& v, int i, int j) { return i >= 0 && i < v.NX && j >= 0 && j < v.NY; }
 __device__ __forceinline__ long t_pidx(const TrView& v, int i, int j) { return (long)j * v.nx + 1 + i; }
+__device__ __forceinline__ long t_uidx(const TrView& v, int i, int j) { return (long)j * v.NX + i; }
 __device__ __forceinline__ bool t_solid(const TrView& v, int i, int j) {
     return t_inside(v, i, j) && v.cls[t_pidx(v, i, j)] >= CLS_MINUS;
 }
 __device__ __forceinline__ double t_vel(const TrView& v, int comp, int i, int j) {
     if (!t_inside(v, i, j)) return comp ? v.Uy : v.Ux;
-    return (comp ? v.uy : v.ux)[t_pidx(v, i, j)];
+    const long p = t_pidx(v, i, j);
+    const uint8_t c = v.cls[p];
+    if (c <= CLS_PLUS) return (comp ? v.uy : v.ux)[t_uidx(v, i, j)];
+    return c == CLS_MINUS ? (comp ? v.guy : v.gux)[v.minus_map[p]] : 0.0;
 }
 // kind 0: fourth-order extension with omega_b, 1: third-order with omega_b, 2: third-order without
 __device__ __forceinline__ double t_omega(const TrView& v, int kind, int i, int j) {
     if (!t_inside(v, i, j)) {
-        if (i >= v.NX && j >= 0 && j < v.NY) return v.w[t_pidx(v, v.NX - 1, j)];
-        return 0.0;
+        if (!(i >= v.NX && j >= 0 && j < v.NY)) return 0.0;
+        i = v.NX - 1;
+        return v.cls[t_pidx(v, i, j)] <= CLS_PLUS ? v.w[t_uidx(v, i, j)] : 0.0;
     }
     const long p = t_pidx(v, i, j);
     const uint8_t c = v.cls[p];
-    if (c <= CLS_PLUS) return v.w[p];
+    if (c <= CLS_PLUS) return v.w[t_uidx(v, i, j)];
     if (c == CLS_MINUS) {
         const int m = v.minus_map[p];
         return kind == 0 ? v.g4[m] : (kind == 1 ? v.g3[m] : v.g3n[m]);
@@ -73,116 +80,128 @@ __device__ __forceinline__ double t_omega(const TrView& v, int kind, int i, int 
     return 0.0;
 }
 
-// Flux f + q on the face between interior nodes a = (ai, aj) and a + e_axis.
-__device__ double t_face_flux(const TrView& v, double nu, int axis, int ai, int aj) {
+// f + q on a face from the point fluxes p of the upwind-biased stencil in order along the axis
+// (pos: nodes a - e, a, b; else a, b, b + e) and the vorticity of the face's two nodes (diffusion);
+// c = nu / h.
+__device__ __forceinline__ double t_flux(bool pos, double p0, double p1, double p2, double wa, double wb, double c) {
+    const double k0 = pos ? -1.0 / 6.0 : 1.0 / 3.0, k2 = pos ? 1.0 / 3.0 : -1.0 / 6.0;
+    return fma(k0, p0, fma(5.0 / 6.0, p1, k2 * p2)) - c * (wb - wa);
+}
+
+// Flux f + q on the face between interior nodes a = (ai, aj) and a + e_axis: the general form, any
+// of the stencil's nodes in a solid or beyond the box.
+__device__ __noinline__ double t_face_flux(const TrView& v, double c, int axis, int ai, int aj) {
     const int di = axis == 0 ? 1 : 0, dj = axis == 0 ? 0 : 1;
     const int bi = ai + di, bj = aj + dj;
-    const double ua = t_vel(v, axis, ai, aj), ub = t_vel(v, axis, bi, bj);
-    const double uf = 0.5 * (ua + ub);
-    bool pos = uf >= 0.0;
+    bool pos = t_vel(v, axis, ai, aj) + t_vel(v, axis, bi, bj) >= 0.0;
+    const bool up_left = pos;
     const bool sa = t_solid(v, ai, aj), sb = t_solid(v, bi, bj);
     if (sa != sb) {
         const bool inflow = (sb && !pos) || (sa && pos);
         if (inflow) pos = !pos;   // downwind stencil at inflow boundary faces
     }
-    const bool up_left = uf >= 0.0;
-    int ni[3], nj[3];
-    double wt[3];
-    bool left[3];
-    if (pos) {
-        ni[0] = ai - di; nj[0] = aj - dj; ni[1] = ai; nj[1] = aj; ni[2] = bi; nj[2] = bj;
-        wt[0] = -1.0 / 6.0; wt[1] = 5.0 / 6.0; wt[2] = 1.0 / 3.0;
-        left[0] = true; left[1] = true; left[2] = false;
-    } else {
-        ni[0] = ai; nj[0] = aj; ni[1] = bi; nj[1] = bj; ni[2] = bi + di; nj[2] = bj + dj;
-        wt[0] = 1.0 / 3.0; wt[1] = 5.0 / 6.0; wt[2] = -1.0 / 6.0;
-        left[0] = true; left[1] = false; left[2] = false;
-    }
-    double f = 0.0;
+    double p[3];
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const int kind = t_solid(v, ni[k], nj[k]) ? ((left[k] == up_left) ? 1 : 2) : 1;
-        f += wt[k] * t_vel(v, axis, ni[k], nj[k]) * t_omega(v, kind, ni[k], nj[k]);
+        const int o = pos ? k - 1 : k;            // node a + o e_axis
+        const int ni = ai + o * di, nj = aj + o * dj;
+        const int kind = t_solid(v, ni, nj) ? (((o <= 0) == up_left) ? 1 : 2) : 1;
+        p[k] = t_vel(v, axis, ni, nj) * t_omega(v, kind, ni, nj);
     }
-    const double q = -nu * (t_omega(v, 0, bi, bj) - t_omega(v, 0, ai, aj)) / v.h;
-    return f + q;
+    return t_flux(pos, p[0], p[1], p[2], t_omega(v, 0, ai, aj), t_omega(v, 0, bi, bj), c);
 }
 
-// user layout (NX stride) -> padded, fluid values only
-__global__ void k_pack(int NX, int NY, const double* __restrict__ src, const uint8_t* __restrict__ cls, double* __restrict__ dst) {
-    const int nx = NX + 1;   // a power of two
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nx * NY) return;
-    const int j = k >> (__ffs(nx) - 1), i = (k & (nx - 1)) - 1;
-    dst[k] = (i >= 0 && cls[k] <= CLS_PLUS) ? src[(long)j * NX + i] : 0.0;
+// a / h: a product when 1 / h is exact, else the product corrected by one residual step (Markstein).
+__device__ __forceinline__ double t_div_h(const TrView& v, double a) {
+    const double q = a * v.rh;
+    return v.h_pow2 ? q : fma(fma(-q, v.h, a), v.rh, q);
 }
 
-// Third-order velocity extension with u_b at every A- node (both components).
-__global__ void k_ext_velocity(int nm, int nx, const int* __restrict__ minus_node, const int* __restrict__ minus_cp,
+// Sums over the four lanes of one A- node in direction order (the lanes of a warp are nodes x
+// directions), as a loop over the directions would add them.
+__device__ __forceinline__ double sum_dirs(double x) {
+    const int base = (threadIdx.x & 31) & ~3;
+    double s = __shfl_sync(0xffffffffu, x, base);
+#pragma unroll
+    for (int d = 1; d < 4; ++d) s += __shfl_sync(0xffffffffu, x, base + d);
+    return s;
+}
+
+// Third-order velocity extension with u_b at every A- node (both components); four lanes per node,
+// one per direction: the kernel is a chain of dependent loads and divisions, so its time is that of
+// one direction.
+__global__ void k_ext_velocity(int nm, TrView v, const int* __restrict__ minus_node, const int* __restrict__ minus_cp,
                                const uint8_t* __restrict__ minus_mask, const double* __restrict__ cp_t,
-                               const double* __restrict__ ubx, const double* __restrict__ uby, double* __restrict__ ux,
-                               double* __restrict__ uy) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= nm) return;
-    const long p = minus_node[m];
-    const uint8_t mask = minus_mask[m];
+                               const double* __restrict__ ubx, const double* __restrict__ uby, double* __restrict__ gux,
+                               double* __restrict__ guy) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3;
+    const int m = min(t >> 2, nm - 1);   // the last warp stays whole for the shuffles
+    const int mask = minus_mask[m] >> 4;
     double sx = 0.0, sy = 0.0;
-    int cnt = 0;
-    for (int d = 0; d < 4; ++d) {
-        if (!(mask & (16 << d))) continue;
+    if (mask & (1 << d)) {
+        const int p = minus_node[m], j = p / v.nx, i = p - j * v.nx - 1;
         const int c = minus_cp[4 * m + d];
         const double a = 1.0 - cp_t[c];
         // Lagrange weights at 0 of the quadratic through a (boundary), 2, 3
         const double w0 = 6.0 / ((a - 2.0) * (a - 3.0));
         const double w2 = -3.0 * a / (2.0 - a);
         const double w3 = 2.0 * a / (3.0 - a);
-        const long step = (long)t_dir_j[d] * nx + t_dir_i[d];
-        sx += w0 * ubx[c] + w2 * ux[p + 2 * step] + w3 * ux[p + 3 * step];
-        sy += w0 * uby[c] + w2 * uy[p + 2 * step] + w3 * uy[p + 3 * step];
-        ++cnt;
+        const long q = t_uidx(v, i, j), step = (long)t_dir_j[d] * v.NX + t_dir_i[d];
+        sx = w0 * ubx[c] + w2 * v.ux[q + 2 * step] + w3 * v.ux[q + 3 * step];
+        sy = w0 * uby[c] + w2 * v.uy[q + 2 * step] + w3 * v.uy[q + 3 * step];
     }
-    ux[p] = cnt ? sx / cnt : 0.0;
-    uy[p] = cnt ? sy / cnt : 0.0;
+    sx = sum_dirs(sx);
+    sy = sum_dirs(sy);
+    if (d == 0 && (t >> 2) < nm) {
+        const int cnt = __popc(mask & 15);
+        gux[m] = cnt ? sx / cnt : 0.0;
+        guy[m] = cnt ? sy / cnt : 0.0;
+    }
 }
 
-// The three vorticity extensions at every A- node.
-__global__ void k_ext_vorticity(int nm, int nx, const int* __restrict__ minus_node, const int* __restrict__ minus_cp,
+// The three vorticity extensions at every A- node (four lanes per node, as k_ext_velocity).
+__global__ void k_ext_vorticity(int nm, TrView v, const int* __restrict__ minus_node, const int* __restrict__ minus_cp,
                                 const uint8_t* __restrict__ minus_mask, const double* __restrict__ cp_t,
-                                const double* __restrict__ wb, const double* __restrict__ w, double* __restrict__ g4,
-                                double* __restrict__ g3, double* __restrict__ g3n) {
-    const int m = blockIdx.x * blockDim.x + threadIdx.x;
-    if (m >= nm) return;
-    const long p = minus_node[m];
-    const uint8_t mask = minus_mask[m];
+                                const double* __restrict__ wb, double* __restrict__ g4, double* __restrict__ g3,
+                                double* __restrict__ g3n) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3;
+    const int m = min(t >> 2, nm - 1);
+    int mask = minus_mask[m];
     double s4 = 0.0, s3 = 0.0, s3n = 0.0;
-    int c4 = 0, c3 = 0;
-    for (int d = 0; d < 4; ++d) {
-        const int c = minus_cp[4 * m + d];
-        if (c < 0) continue;
-        const long step = (long)t_dir_j[d] * nx + t_dir_i[d];
+    const int c = minus_cp[4 * m + d];
+    if (c >= 0 && (mask & (17 << d))) {
+        const int p = minus_node[m], j = p / v.nx, i = p - j * v.nx - 1;
+        const long q = t_uidx(v, i, j), step = (long)t_dir_j[d] * v.NX + t_dir_i[d];
         const double a = 1.0 - cp_t[c];
+        const double x2 = v.w[q + 2 * step], x3 = v.w[q + 3 * step];
         if (mask & (1 << d)) {
             // cubic through a (boundary), 2, 3, 4
             const double w0 = -24.0 / ((a - 2.0) * (a - 3.0) * (a - 4.0));
             const double w2 = -6.0 * a / (2.0 - a);
             const double w3 = 8.0 * a / (3.0 - a);
             const double w4 = -3.0 * a / (4.0 - a);
-            s4 += w0 * wb[c] + w2 * w[p + 2 * step] + w3 * w[p + 3 * step] + w4 * w[p + 4 * step];
-            ++c4;
+            s4 = w0 * wb[c] + w2 * x2 + w3 * x3 + w4 * v.w[q + 4 * step];
         }
         if (mask & (16 << d)) {
             const double w0 = 6.0 / ((a - 2.0) * (a - 3.0));
             const double w2 = -3.0 * a / (2.0 - a);
             const double w3 = 2.0 * a / (3.0 - a);
-            s3 += w0 * wb[c] + w2 * w[p + 2 * step] + w3 * w[p + 3 * step];
+            s3 = w0 * wb[c] + w2 * x2 + w3 * x3;
             // quadratic through the fluid nodes 1, 2, 3 (no boundary condition)
-            s3n += 3.0 * w[p + step] - 3.0 * w[p + 2 * step] + w[p + 3 * step];
-            ++c3;
+            s3n = 3.0 * v.w[q + step] - 3.0 * x2 + x3;
         }
     }
-    g4[m] = c4 ? s4 / c4 : 0.0;
-    g3[m] = c3 ? s3 / c3 : 0.0;
-    g3n[m] = c3 ? s3n / c3 : 0.0;
+    s4 = sum_dirs(s4);
+    s3 = sum_dirs(s3);
+    s3n = sum_dirs(s3n);
+    // directions without a control point have no bit in the counts
+    const unsigned has = __ballot_sync(0xffffffffu, c >= 0) >> ((threadIdx.x & 31) & ~3);
+    if (d == 0 && (t >> 2) < nm) {
+        const int c4 = __popc(mask & 15 & has), c3 = __popc((mask >> 4) & 15 & has);
+        g4[m] = c4 ? s4 / c4 : 0.0;
+        g3[m] = c3 ? s3 / c3 : 0.0;
+        g3n[m] = c3 ? s3n / c3 : 0.0;
+    }
 }
 
 // omega_b = curl of the extended velocity at each control point (Sec. 5.3, reading above).
@@ -348,39 +367,24 @@ __global__ void k_wall_values(int ncp, TrView v, const int* __restrict__ cp_axis
     out[c] = r;
 }
 
-// Transport right-hand side at fluid nodes.  mode 0: out_user = rhs (caller layout);
-// mode 1: dw = a * dw + dt * rhs (padded).
-__global__ void k_transport_rhs(TrView v, double nu, int mode, double a, double dt, double* __restrict__ out_user,
-                                double* __restrict__ dw) {
-    const long n = (long)v.NX * v.NY;
-    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    const int i = (int)(k % v.NX), j = (int)(k / v.NX);
-    const long p = t_pidx(v, i, j);
-    double r = 0.0;
-    if (v.cls[p] <= CLS_PLUS) {
-        const double fr = t_face_flux(v, nu, 0, i, j), fl = t_face_flux(v, nu, 0, i - 1, j);
-        const double gt = t_face_flux(v, nu, 1, i, j), gb = t_face_flux(v, nu, 1, i, j - 1);
-        r = -((fr - fl) + (gt - gb)) / v.h;
-    }
-    if (mode == 0) out_user[k] = r;
-    else dw[p] = a * dw[p] + dt * r;
-}
-
-// Kelvin ODE per body: dGdt[k] = -h sum_{dR_k}(f+q).n; with rk != 0 also the Williamson update
+// Kelvin ODE of body k: dGdt[k] = -h sum_{dR_k}(f+q).n; with rk != 0 also the Williamson update
 // dG = a dG + dt dGdt, Gamma += b dG (every body; fixed-psibar bodies do not read Gamma).
+struct KelvinArgs {
+    const iim_region* R;
+    double* dgdt;
+    int rk;
+    double b;
+    double *dG, *gamma;
+};
 template <int BLOCK>
-__global__ void k_kelvin(TrView v, double nu, const iim_region* __restrict__ R, const int* __restrict__ body_circ,
-                         double* __restrict__ dgdt, int rk, double a, double b, double dt, double* __restrict__ dG,
-                         double* __restrict__ gamma) {
-    const int k = blockIdx.x;
-    const iim_region r = R[k];
+__device__ __forceinline__ void kelvin_body(const TrView& v, double c, int k, const KelvinArgs& g, double a, double dt) {
+    const iim_region r = g.R[k];
     double s = 0.0;
     // interior coordinates = global - 1
     for (int jj = r.ly + threadIdx.x; jj <= r.ry; jj += BLOCK)
-        s += t_face_flux(v, nu, 0, r.rx - 1, jj - 1) - t_face_flux(v, nu, 0, r.lx - 2, jj - 1);
+        s += t_face_flux(v, c, 0, r.rx - 1, jj - 1) - t_face_flux(v, c, 0, r.lx - 2, jj - 1);
     for (int ii = r.lx + threadIdx.x; ii <= r.rx; ii += BLOCK)
-        s += t_face_flux(v, nu, 1, ii - 1, r.ry - 1) - t_face_flux(v, nu, 1, ii - 1, r.ly - 2);
+        s += t_face_flux(v, c, 1, ii - 1, r.ry - 1) - t_face_flux(v, c, 1, ii - 1, r.ly - 2);
     __shared__ double red[BLOCK / 32];
     for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
@@ -389,11 +393,165 @@ __global__ void k_kelvin(TrView v, double nu, const iim_region* __restrict__ R, 
         double tot = 0.0;
         for (int w = 0; w < BLOCK / 32; ++w) tot += red[w];
         const double rate = -v.h * tot;
-        if (dgdt) dgdt[k] = rate;
-        if (rk) {
-            dG[k] = a * dG[k] + dt * rate;
-            gamma[k] += b * dG[k];
+        if (g.dgdt) g.dgdt[k] = rate;
+        if (g.rk) {
+            g.dG[k] = a * g.dG[k] + dt * rate;
+            g.gamma[k] += g.b * g.dG[k];
         }
+    }
+}
+
+// Transport right-hand side at fluid nodes.  mode 0: out = rhs; mode 1: dw = a * dw + dt * rhs (a = 0
+// does not read dw).  Both in the caller's layout.
+//
+// The FP64 pipe bounds it (two lanes per clock and SM: 1.7 us per instruction and million nodes), so
+// every face is evaluated once: a block stages its nodes (and two beyond each side) in shared memory
+// with the point fluxes u w formed once per node, evaluates its faces into shared memory, and
+// differences them -- about 20 FP64 instructions per node instead of 88 (four faces per node with a
+// division each).  Faces whose stencil meets a solid node (found per block, then per face) take the
+// general form, from the tile and the extensions, so a face has one value whichever block evaluates
+// it.  The first nk blocks integrate
+// one body's Kelvin ODE each (a chain of latencies: started first).  1024 x 512, one cylinder:
+// 98 -> 30 us (the whole right-hand side 177 -> 65 us).
+constexpr int TR_X = 32, TR_Y = 16, TR_THREADS = 256, TR_W = TR_X + 4, TR_H = TR_Y + 4;
+__global__ void __launch_bounds__(TR_THREADS)
+k_transport_rhs(TrView v, double c, int mode, double a, double dt, double* __restrict__ out, int tx, int nk,
+                KelvinArgs kv) {
+    if ((int)blockIdx.x < nk) {
+        kelvin_body<TR_THREADS>(v, c, blockIdx.x, kv, a, dt);
+        return;
+    }
+    __shared__ double sw[TR_H][TR_W], sux[TR_H][TR_W], suy[TR_H][TR_W], spx[TR_H][TR_W], spy[TR_H][TR_W];
+    __shared__ uint8_t ss[TR_H][TR_W];
+    // the faces, once every node has been read, take the place of the point fluxes (29 KB: seven
+    // blocks on an SM)
+    double(*fx)[TR_X + 1] = reinterpret_cast<double(*)[TR_X + 1]>(&spx[0][0]);
+    double(*fy)[TR_X] = reinterpret_cast<double(*)[TR_X]>(&spy[0][0]);
+    const int tile = blockIdx.x - nk, by = tile / tx, i0 = (tile - by * tx) * TR_X, j0 = by * TR_Y;
+    // nodes: flag 0 fluid or beyond the box, 1 A- node (velocity: its extension), 2 deeper in a solid
+    constexpr int NN = TR_H * TR_W, PN = (NN + TR_THREADS - 1) / TR_THREADS;
+    int flag[PN];
+    double w[PN], ux[PN], uy[PN];
+#pragma unroll
+    for (int b = 0; b < PN; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS, r = t / TR_W, q = t - r * TR_W, i = i0 - 2 + q, j = j0 - 2 + r;
+        flag[b] = -1;
+        w[b] = ux[b] = uy[b] = 0.0;
+        if (t < NN && j >= 0 && j < v.NY && i >= 0) {
+            const int ic = min(i, v.NX - 1);     // the right edge copies the last column's vorticity
+            const long k = t_uidx(v, ic, j);
+            flag[b] = v.cls[t_pidx(v, ic, j)];
+            w[b] = v.w[k];
+            ux[b] = v.ux[k];
+            uy[b] = v.uy[k];
+        }
+    }
+    int solid_any = 0;
+#pragma unroll
+    for (int b = 0; b < PN; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS, r = t / TR_W, q = t - r * TR_W, i = i0 - 2 + q, j = j0 - 2 + r;
+        if (t >= NN) continue;
+        int sol = 0;
+        if (flag[b] >= (int)CLS_MINUS) {
+            sol = flag[b] == (int)CLS_MINUS ? 1 : 2;
+            w[b] = ux[b] = uy[b] = 0.0;
+            if (sol == 1 && i < v.NX) {
+                const int m = v.minus_map[t_pidx(v, i, j)];
+                ux[b] = v.gux[m];
+                uy[b] = v.guy[m];
+            }
+        }
+        if (flag[b] < 0 || i >= v.NX) {
+            ux[b] = v.Ux;
+            uy[b] = v.Uy;
+            sol = 0;
+        }
+        solid_any |= sol;
+        sw[r][q] = w[b];
+        sux[r][q] = ux[b];
+        suy[r][q] = uy[b];
+        spx[r][q] = ux[b] * w[b];
+        spy[r][q] = uy[b] * w[b];
+        ss[r][q] = (uint8_t)sol;
+    }
+    solid_any = __syncthreads_or(solid_any);
+    // a face next to a solid, from the tile: t_face_flux's form with the A- vorticities from the extensions
+    auto solid_face = [&](const double (*su)[TR_W], int y, int x, int dy, int dx) -> double {
+        const int fa = ss[y][x], fb = ss[y + dy][x + dx];
+        if (fa && fb) return 0.0;   // no fluid node reads it
+        bool pos = su[y][x] + su[y + dy][x + dx] >= 0.0;
+        const bool up_left = pos;
+        if ((fa != 0) != (fb != 0) && ((fb && !pos) || (fa && pos))) pos = !pos;
+        auto om = [&](int kind, int o) -> double {
+            const int yy = y + o * dy, xx = x + o * dx, fl = ss[yy][xx];
+            if (fl == 0) return sw[yy][xx];
+            if (fl == 2) return 0.0;
+            const int m = v.minus_map[t_pidx(v, i0 - 2 + xx, j0 - 2 + yy)];
+            return kind == 0 ? v.g4[m] : kind == 1 ? v.g3[m] : v.g3n[m];
+        };
+        double p[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const int o = pos ? k - 1 : k;
+            p[k] = su[y + o * dy][x + o * dx] * om(((o <= 0) == up_left) ? 1 : 2, o);
+        }
+        return t_flux(pos, p[0], p[1], p[2], om(0, 0), om(0, 1), c);
+    };
+    constexpr int NFX = TR_Y * (TR_X + 1), NFY = (TR_Y + 1) * TR_X;
+    constexpr int PX = (NFX + TR_THREADS - 1) / TR_THREADS, PY = (NFY + TR_THREADS - 1) / TR_THREADS;
+    double vx[PX], vy[PY];
+    // x faces: face (r, q) between nodes q - 1 and q of row r (tile nodes offset by 2)
+#pragma unroll
+    for (int b = 0; b < PX; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS;
+        vx[b] = 0.0;
+        if (t < NFX) {
+            const int r = t / (TR_X + 1), q = t - r * (TR_X + 1), y = r + 2, x = q + 1;   // nodes x, x + 1
+            if (solid_any && (ss[y][x - 1] | ss[y][x] | ss[y][x + 1] | ss[y][x + 2])) {
+                vx[b] = solid_face(sux, y, x, 0, 1);
+            } else {
+                const bool pos = sux[y][x] + sux[y][x + 1] >= 0.0;
+                const double* p = &spx[y][pos ? x - 1 : x];
+                vx[b] = t_flux(pos, p[0], p[1], p[2], sw[y][x], sw[y][x + 1], c);
+            }
+        }
+    }
+#pragma unroll
+    for (int b = 0; b < PY; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS;
+        vy[b] = 0.0;
+        if (t < NFY) {
+            const int r = t / TR_X, q = t - r * TR_X, y = r + 1, x = q + 2;               // nodes y, y + 1
+            if (solid_any && (ss[y - 1][x] | ss[y][x] | ss[y + 1][x] | ss[y + 2][x])) {
+                vy[b] = solid_face(suy, y, x, 1, 0);
+            } else {
+                const bool pos = suy[y][x] + suy[y + 1][x] >= 0.0;
+                const double* p = &spy[pos ? y - 1 : y][x];
+                vy[b] = t_flux(pos, p[0], p[TR_W], p[2 * TR_W], sw[y][x], sw[y + 1][x], c);
+            }
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int b = 0; b < PX; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS;
+        if (t < NFX) (&fx[0][0])[t] = vx[b];
+    }
+#pragma unroll
+    for (int b = 0; b < PY; ++b) {
+        const int t = threadIdx.x + b * TR_THREADS;
+        if (t < NFY) (&fy[0][0])[t] = vy[b];
+    }
+    __syncthreads();
+    for (int t = threadIdx.x; t < TR_Y * TR_X; t += TR_THREADS) {
+        const int r = t / TR_X, q = t - r * TR_X;
+        if (i0 + q >= v.NX || j0 + r >= v.NY) continue;
+        double rate = 0.0;
+        if (!ss[r + 2][q + 2])
+            rate = -t_div_h(v, (fx[r][q + 1] - fx[r][q]) + (fy[r + 1][q] - fy[r][q]));
+        const long k = t_uidx(v, i0 + q, j0 + r);
+        if (mode == 0) out[k] = rate;
+        else out[k] = a != 0.0 ? a * out[k] + dt * rate : dt * rate;
     }
 }
 
@@ -404,7 +562,7 @@ __global__ void k_rk_omega(int NX, int NY, double b, const double* __restrict__ 
     if (k >= n) return;
     const int j = k / NX, i = k - j * NX;
     const int p = j * (NX + 1) + 1 + i;
-    omega[k] = cls[p] <= CLS_PLUS ? omega[k] + b * dw[p] : 0.0;
+    omega[k] = cls[p] <= CLS_PLUS ? omega[k] + b * dw[k] : 0.0;
 }
 
 template <int BLOCK>
@@ -425,22 +583,20 @@ __global__ void k_speed_max(long n, const double* __restrict__ ux, const double*
 
 // Transport workspace inside g->tr_buf (doubles).
 struct TrWork {
-    double *w, *ux, *uy, *dw, *g4, *g3, *g3n, *wb, *dG, *part, *psi, *vx, *vy, *zeros, *dgdt, *ub_stage;
+    double *dw, *gux, *guy, *g4, *g3, *g3n, *wb, *dG, *part, *psi, *vx, *vy, *zeros, *ub_stage;
 };
 
 static iim_status tr_work(iim_geometry g, TrWork* W) {
-    const size_t npad = (size_t)g->nx * g->NY, n = (size_t)g->NX * g->NY, nm = (size_t)std::max(g->nminus, 1),
-                 ncp = (size_t)std::max(g->ncp, 1);
-    const size_t total = 4 * npad + 3 * nm + ncp + 64 + 1024 + 3 * n + ncp + 64 + 2 * ncp;
+    const size_t n = (size_t)g->NX * g->NY, nm = (size_t)std::max(g->nminus, 1), ncp = (size_t)std::max(g->ncp, 1);
+    const size_t total = 4 * n + 5 * nm + ncp + 64 + 1024 + ncp + 2 * ncp;
     if (!g->tr_buf) {
         IIM_TRY(cudaMalloc(&g->tr_buf, total * sizeof(double)));
         IIM_TRY(cudaMemset(g->tr_buf, 0, total * sizeof(double)));
     }
     double* p = g->tr_buf;
-    W->w = p; p += npad;
-    W->ux = p; p += npad;
-    W->uy = p; p += npad;
-    W->dw = p; p += npad;
+    W->dw = p; p += n;
+    W->gux = p; p += nm;
+    W->guy = p; p += nm;
     W->g4 = p; p += nm;
     W->g3 = p; p += nm;
     W->g3n = p; p += nm;
@@ -451,45 +607,57 @@ static iim_status tr_work(iim_geometry g, TrWork* W) {
     W->vx = p; p += n;
     W->vy = p; p += n;
     W->zeros = p; p += ncp;
-    W->dgdt = p; p += 64;
     W->ub_stage = p; p += 2 * ncp;
     return IIM_OK;
 }
 
-static TrView make_view(iim_geometry g, const TrWork& W, const double Uinf[2]) {
+static TrView make_view(iim_geometry g, const TrWork& W, const double Uinf[2], const double* omega, const double* ux,
+                        const double* uy) {
     TrView v;
     v.NX = g->NX; v.NY = g->NY; v.nx = g->nx; v.h = g->h;
+    v.rh = 1.0 / g->h;
+    int e = 0;
+    v.h_pow2 = std::frexp(g->h, &e) == 0.5;
     v.cls = g->node_class; v.minus_map = g->minus_map;
-    v.w = W.w; v.ux = W.ux; v.uy = W.uy; v.g4 = W.g4; v.g3 = W.g3; v.g3n = W.g3n;
+    v.w = omega; v.ux = ux; v.uy = uy;
+    v.gux = W.gux; v.guy = W.guy; v.g4 = W.g4; v.g3 = W.g3; v.g3n = W.g3n;
     v.Ux = Uinf ? Uinf[0] : 0.0;
     v.Uy = Uinf ? Uinf[1] : 0.0;
     return v;
 }
 
-// Velocity (caller layout) -> padded + extension; vorticity BC; vorticity -> padded + extensions.
-static iim_status prepare_stage(iim_geometry g, const TrWork& W, const TrView& v, const double* omega, const double* ux,
-                                const double* uy, const double* u_b, const double* wb_in, double* wb_out, cudaStream_t s) {
-    const long npad = (long)g->nx * g->NY;
-    const unsigned gp = (unsigned)((npad + 255) / 256);
+// Velocity extension; vorticity BC; vorticity extensions (v holds the fields).
+static iim_status prepare_stage(iim_geometry g, const TrWork& W, const TrView& v, const double* u_b,
+                                const double* wb_in, double* wb_out, cudaStream_t s) {
     const double* ubx = u_b ? u_b : W.zeros;
     const double* uby = u_b ? u_b + g->ncp : W.zeros;
-    launch("tr_pack", 0.0, 0.0, k_pack, gp, 256, 0, s, g->NX, g->NY, ux, g->node_class, W.ux);
-    launch("tr_pack", 0.0, 0.0, k_pack, gp, 256, 0, s, g->NX, g->NY, uy, g->node_class, W.uy);
-    launch("tr_pack", 0.0, 0.0, k_pack, gp, 256, 0, s, g->NX, g->NY, omega, g->node_class, W.w);
+    const unsigned eb = (unsigned)((4 * g->nminus + 127) / 128);   // four lanes per A- node
     if (g->nminus > 0)
-        launch("tr_ext_velocity", 0.0, 0.0, k_ext_velocity, (g->nminus + 127) / 128, 128, 0, s, g->nminus, g->nx,
-               g->minus_node, g->minus_cp, g->minus_mask, g->cp_t, ubx, uby, W.ux, W.uy);
+        launch("tr_ext_velocity", 0.0, 0.0, k_ext_velocity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
+               g->minus_mask, g->cp_t, ubx, uby, W.gux, W.guy);
     if (g->ncp > 0 && wb_in) {
         IIM_TRY(cudaMemcpyAsync(W.wb, wb_in, g->ncp * sizeof(double), cudaMemcpyDeviceToDevice, s));
     } else if (g->ncp > 0)
-        launch("tr_vorticity_bc", 0.0, 0.0, k_vorticity_bc, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->nx, g->ny,
+        launch("tr_vorticity_bc", 0.0, 0.0, k_vorticity_bc, (g->ncp + 63) / 64, 64, 0, s, g->ncp, v, g->nx, g->ny,
                g->cp_axis, g->cp_ei, g->cp_ej, g->cp_t, ubx, uby, W.wb);
     if (g->nminus > 0)
-        launch("tr_ext_vorticity", 0.0, 0.0, k_ext_vorticity, (g->nminus + 127) / 128, 128, 0, s, g->nminus, g->nx,
-               g->minus_node, g->minus_cp, g->minus_mask, g->cp_t, W.wb, W.w, W.g4, W.g3, W.g3n);
+        launch("tr_ext_vorticity", 0.0, 0.0, k_ext_vorticity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
+               g->minus_mask, g->cp_t, W.wb, W.g4, W.g3, W.g3n);
     IIM_LAUNCHED();
     if (wb_out && g->ncp > 0)
         IIM_TRY(cudaMemcpyAsync(wb_out, W.wb, g->ncp * sizeof(double), cudaMemcpyDeviceToDevice, s));
+    return IIM_OK;
+}
+
+// The right-hand side (out: rhs, or with rk the Williamson increment dw) and, with bodies and kv.R,
+// the Kelvin ODE, in one launch.
+static iim_status transport_rhs(iim_geometry g, const TrView& v, double nu, int mode, double a, double dt, double* out,
+                                const KelvinArgs& kv, cudaStream_t s) {
+    const int tx = (g->NX + TR_X - 1) / TR_X, ty = (g->NY + TR_Y - 1) / TR_Y;
+    const int nk = kv.R ? g->nb : 0;
+    launch("tr_rhs", 40.0 * (double)g->NX * g->NY, 0.0, k_transport_rhs, tx * ty + nk, TR_THREADS, 0, s, v, nu / g->h, mode,
+           a, dt, out, tx, nk, kv);
+    IIM_LAUNCHED();
     return IIM_OK;
 }
 
@@ -504,16 +672,10 @@ extern "C" iim_status iim_transport_rhs(iim_geometry g, const double* omega, con
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
-    const TrView v = make_view(g, W, Uinf);
-    IIM_CHECK(prepare_stage(g, W, v, omega, ux, uy, u_b, omega_b_in, omega_b_out, s));
-    const long n = (long)g->NX * g->NY;
-    launch("tr_rhs", 40.0 * (double)n, 0.0, k_transport_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, nu, 0, 0.0, 1.0,
-           rhs_out, W.dw);
-    if (g->nb > 0 && dgamma_out)
-        launch("tr_kelvin", 0.0, 0.0, k_kelvin<256>, g->nb, 256, 0, s, v, nu, g->d_regions, g->body_circ, dgamma_out, 0,
-               0.0, 0.0, 0.0, W.dG, (double*)nullptr);
-    IIM_LAUNCHED();
-    return IIM_OK;
+    const TrView v = make_view(g, W, Uinf, omega, ux, uy);
+    IIM_CHECK(prepare_stage(g, W, v, u_b, omega_b_in, omega_b_out, s));
+    const KelvinArgs kv{dgamma_out ? g->d_regions : nullptr, dgamma_out, 0, 0.0, nullptr, nullptr};
+    return transport_rhs(g, v, nu, 0, 0.0, 1.0, rhs_out, kv, s);
 }
 
 extern "C" iim_status iim_total_pressure_problem(iim_geometry g, const double* omega, const double* ux,
@@ -524,8 +686,8 @@ extern "C" iim_status iim_total_pressure_problem(iim_geometry g, const double* o
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
-    const TrView v = make_view(g, W, Uinf);
-    IIM_CHECK(prepare_stage(g, W, v, omega, ux, uy, u_b, omega_b_in, omega_b_out, s));
+    const TrView v = make_view(g, W, Uinf, omega, ux, uy);
+    IIM_CHECK(prepare_stage(g, W, v, u_b, omega_b_in, omega_b_out, s));
     const long n = (long)g->NX * g->NY;
     launch("pressure_rhs", 48.0 * (double)n, 0.0, k_pressure_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, f_out);
     if (g->ncp > 0)
@@ -541,7 +703,7 @@ extern "C" iim_status iim_wall_values(iim_geometry g, const double* field, doubl
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
-    const TrView v = make_view(g, W, nullptr);
+    const TrView v = make_view(g, W, nullptr, nullptr, nullptr, nullptr);
     launch("wall_values", 0.0, 0.0, k_wall_values, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->cp_axis, g->cp_ei,
            g->cp_ej, g->cp_t, field, out);
     IIM_LAUNCHED();
@@ -586,9 +748,8 @@ static iim_status rk3_step(iim_geometry g, double* omega, double* gamma, double*
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
-    const TrView v = make_view(g, W, Uinf);
-    const long n = (long)g->NX * g->NY, npad = (long)g->nx * g->NY;
-    IIM_TRY(cudaMemsetAsync(W.dw, 0, npad * sizeof(double), s));
+    const TrView v = make_view(g, W, Uinf, omega, W.vx, W.vy);
+    const long n = (long)g->NX * g->NY;
     IIM_TRY(cudaMemsetAsync(W.dG, 0, 64 * sizeof(double), s));
     double dt = *dt_inout;
     for (int st = 0; st < 3; ++st) {
@@ -617,12 +778,9 @@ static iim_status rk3_step(iim_geometry g, double* omega, double* gamma, double*
                        kRK3C[st] * dt, W.ub_stage);
             ub = W.ub_stage;
         }
-        IIM_CHECK(prepare_stage(g, W, v, omega, W.vx, W.vy, ub, nullptr, nullptr, s));
-        launch("tr_rhs", 40.0 * (double)n, 0.0, k_transport_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, nu, 1,
-               kRK3A[st], dt, (double*)nullptr, W.dw);
-        if (g->nb > 0)
-            launch("tr_kelvin", 0.0, 0.0, k_kelvin<256>, g->nb, 256, 0, s, v, nu, g->d_regions, g->body_circ,
-                   (double*)nullptr, 1, kRK3A[st], kRK3B[st], dt, W.dG, gamma);
+        IIM_CHECK(prepare_stage(g, W, v, ub, nullptr, nullptr, s));
+        const KelvinArgs kv{g->d_regions, nullptr, 1, kRK3B[st], W.dG, gamma};
+        IIM_CHECK(transport_rhs(g, v, nu, 1, kRK3A[st], dt, W.dw, kv, s));
         launch("tr_rk_omega", 24.0 * (double)n, 0.0, k_rk_omega, (unsigned)((n + 255) / 256), 256, 0, s, g->NX, g->NY,
                kRK3B[st], (const double*)W.dw, g->node_class, omega);
         IIM_LAUNCHED();
