@@ -64,6 +64,9 @@ const cpx<float>* twiddles32();
 // device, built by ensure_twiddles for every n = 16..4096.
 template <typename T>
 const cpx<T>* twiddle_region(int n, int fp);
+// Table of the row transforms (sine.cuh) for lines of n = 16..2048 points, same lifetime.
+template <typename T>
+const cpx<T>* sine_table(int n);
 
 // ------------------------------------------------------------------------- node classes
 enum : uint8_t { CLS_FLUID = 0, CLS_PLUS = 1, CLS_MINUS = 2, CLS_SOLID = 3 };

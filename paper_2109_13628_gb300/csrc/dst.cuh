@@ -619,29 +619,6 @@ __device__ __forceinline__ void store_row_vec(T* __restrict__ g, const T* line, 
     for (int q = lane; q < nv; q += TN) dst[q] = line_get16<T, PADL>(line, q);
 }
 
-// Loads a padded FP64 row (16-byte aligned, nx values) into a line buffer of T.
-template <typename T, int TN = 32, bool PADL = false>
-__device__ __forceinline__ void load_row_f64(T* line, const double* __restrict__ g, int nx, int lane) {
-    const double2* src = reinterpret_cast<const double2*>(g);
-    const int nv = nx / 2;
-    for (int q0 = lane; q0 < nv; q0 += 8 * TN) {
-        double2 v[8];
-#pragma unroll
-        for (int b = 0; b < 8; ++b)
-            if (q0 + TN * b < nv) v[b] = src[q0 + TN * b];
-#pragma unroll
-        for (int b = 0; b < 8; ++b) {
-            const int q = q0 + TN * b;
-            if (q < nv) {
-                vec2_t<T> w;
-                w.x = (T)v[b].x;
-                w.y = (T)v[b].y;
-                *reinterpret_cast<vec2_t<T>*>(line + lp<PADL>(2 * q)) = w;
-            }
-        }
-    }
-}
-
 // Krylov-vector argument: base + (jidx ? *jidx + joff : 0) * stride
 struct VecArg {
     const double* base;
@@ -677,40 +654,28 @@ __host__ __device__ constexpr size_t twiddle_smem(int n, int fp) {
 // Per-line scratch for the 64-thread path's prefix sum (16 values per line).
 constexpr int kLineScratch = 16;
 
-// Forward row transforms.  Row r (interior row index) of the input is
-//   dense[r*dld + doff + i] (FP64, optional) + box terms / h^2 (optional ring)
-//   + gsign * gamma at the affected points of the row (optional)
-// and the transformed row is written to out (padded layout).  `stop` (optional): a set flag
-// makes the launch a no-op.  Each line is handled by line_threads(FP) threads.
+// Row transforms of the FP32 box solve for callers (the solves' own row passes are in sine.cuh).
+// Forward: row r (interior row index) of the input is the caller's dense[r NX + i] (FP64) + box
+// terms / h^2 (optional ring); the transformed row is written to out (padded layout).  One warp per
+// line.
 template <typename T, int WARPS, int FP>
-__device__ __forceinline__ void
-rows_fwd_body(int NX, int NY, int n, int logn, int row0, int nrows, const double* __restrict__ dense, int dld, int doff,
-              const double* __restrict__ ring, double ih2, const int* __restrict__ aff_row_ptr,
-              const int* __restrict__ aff_node, VecArg gam, double gsign, const cpx<T>* __restrict__ g_tw,
-              T* __restrict__ out) {
-    constexpr int TN = line_threads(FP), LPB = WARPS * 32 / TN;
+__global__ void __launch_bounds__(WARPS * 32)
+k_rows_fwd(int NX, int NY, int n, int logn, const double* __restrict__ dense, const double* __restrict__ ring,
+           double ih2, const cpx<T>* __restrict__ g_tw, T* __restrict__ out) {
     constexpr bool PADL = padded_lines(FP);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const cpx<T>* s_tw = block_twiddles<FP, T>(smem_raw, g_tw, n);
-    const int grp = threadIdx.x / TN, tid = threadIdx.x - grp * TN;
+    const int grp = threadIdx.x >> 5, tid = threadIdx.x & 31;
     const int LN = line_len(n, FP);
-    T* lines = reinterpret_cast<T*>(smem_raw + twiddle_smem<T>(n, FP));
-    T* b0 = lines + (size_t)grp * (2 * LN);
+    T* b0 = reinterpret_cast<T*>(smem_raw + twiddle_smem<T>(n, FP)) + (size_t)grp * (2 * LN);
     T* b1 = b0 + LN;
-    T* tot = lines + (size_t)LPB * 2 * LN + grp * kLineScratch;
     if (FP == 0) __syncthreads();
-    const int r = row0 + blockIdx.x * LPB + grp;
-    if (r >= row0 + nrows || r >= NY) return;   // uniform over the line's threads
-    if (dense && dld == n && doff == 1) {
-        load_row_f64<T, TN, PADL>(b0, dense + (size_t)r * n, n, tid);   // padded row: slot 0 is a pad
-    } else if (dense) {
-        const double* src = dense + (size_t)r * dld + doff;
+    const int r = blockIdx.x * WARPS + grp;
+    if (r >= NY) return;   // uniform over the warp
+    const double* src = dense + (size_t)r * NX;
 #pragma unroll 8
-        for (int i = tid; i < NX; i += TN) b0[lp<PADL>(i + 1)] = (T)src[i];
-    } else {
-        for (int i = tid; i < NX; i += TN) b0[lp<PADL>(i + 1)] = T(0);
-    }
-    line_sync<TN>(grp);
+    for (int i = tid; i < NX; i += 32) b0[lp<PADL>(i + 1)] = (T)src[i];
+    __syncwarp();
     if (ring) {
         // ring: bottom row (nx+1), top row (nx+1), left column (ny-1), right column (ny-1)
         const int nxp1 = NX + 2;
@@ -718,36 +683,17 @@ rows_fwd_body(int NX, int NY, int n, int logn, int row0, int nrows, const double
             b0[lp<PADL>(1)] += (T)(ring[2 * nxp1 + r] * ih2);
             b0[lp<PADL>(NX)] += (T)(ring[2 * nxp1 + NY + r] * ih2);
         }
-        line_sync<TN>(grp);
+        __syncwarp();
         if (r == 0)
-            for (int i = tid; i < NX; i += TN) b0[lp<PADL>(i + 1)] += (T)(ring[i + 1] * ih2);
+            for (int i = tid; i < NX; i += 32) b0[lp<PADL>(i + 1)] += (T)(ring[i + 1] * ih2);
         if (r == NY - 1)
-            for (int i = tid; i < NX; i += TN) b0[lp<PADL>(i + 1)] += (T)(ring[nxp1 + i + 1] * ih2);
-        line_sync<TN>(grp);
+            for (int i = tid; i < NX; i += 32) b0[lp<PADL>(i + 1)] += (T)(ring[nxp1 + i + 1] * ih2);
+        __syncwarp();
     }
-    if (gam.base) {
-        const double* gv = gam.get();
-        const int a0 = aff_row_ptr[r], a1 = aff_row_ptr[r + 1];
-        for (int a = a0 + tid; a < a1; a += TN) b0[lp<PADL>(aff_node[a] - r * n)] += (T)(gsign * gv[a]);
-        line_sync<TN>(grp);
-    }
-    T* res = dst_line<T, FP, PADL>(b0, b1, s_tw, n, logn, tid, grp, tot);
+    T* res = dst_line<T, FP, PADL>(b0, b1, s_tw, n, logn, tid, grp, nullptr);
     if (tid == 0) res[0] = T(0);
-    line_sync<TN>(grp);
-    store_row_vec<T, TN, PADL>(out + (size_t)r * n, res, n, tid);
-}
-
-// blockIdx.y selects one of several fields: dense input dfs and output ofs elements apart.
-template <typename T, int WARPS, int FP>
-__global__ void __launch_bounds__(WARPS * 32)
-k_rows_fwd(int NX, int NY, int n, int logn, int row0, int nrows, const double* __restrict__ dense, int dld, int doff,
-           const double* __restrict__ ring, double ih2, const int* __restrict__ aff_row_ptr,
-           const int* __restrict__ aff_node, VecArg gam, double gsign, const cpx<T>* __restrict__ g_tw,
-           T* __restrict__ out, const int* __restrict__ stop, long dfs, long ofs) {
-    if (stop && *stop) return;
-    rows_fwd_body<T, WARPS, FP>(NX, NY, n, logn, row0, nrows, dense ? dense + (long)blockIdx.y * dfs : nullptr, dld,
-                                doff, ring, ih2, aff_row_ptr, aff_node, gam, gsign, g_tw,
-                                out + (long)blockIdx.y * ofs);
+    __syncwarp();
+    store_row_vec<T, 32, PADL>(out + (size_t)r * n, res, n, tid);
 }
 
 // Column pass on padded columns p = 1..NX (p = 0 is the pad): forward y transform, division
@@ -849,91 +795,34 @@ k_cols(int NX, int NY, int n, int logn, int in0, int in1, int out0, int out1, T*
                         g_tw);
 }
 
-enum RowsInvMode { INV_STORE_T = 0, INV_STORE_F64 = 1, INV_ACCUM_FLUID = 2, INV_ACCUM_T = 3 };
+// Inverse: transforms of the padded rows, written to the caller's dense FP64 rows.
+template <typename T, int WARPS, int FP>
+__global__ void __launch_bounds__(WARPS * 32)
+k_rows_inv(int NX, int NY, int n, int logn, const T* __restrict__ in, double* __restrict__ out,
+           const cpx<T>* __restrict__ g_tw) {
+    constexpr bool PADL = padded_lines(FP);
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const cpx<T>* s_tw = block_twiddles<FP, T>(smem_raw, g_tw, n);
+    const int grp = threadIdx.x >> 5, tid = threadIdx.x & 31;
+    const int LN = line_len(n, FP);
+    T* b0 = reinterpret_cast<T*>(smem_raw + twiddle_smem<T>(n, FP)) + (size_t)grp * (2 * LN);
+    T* b1 = b0 + LN;
+    if (FP == 0) __syncthreads();
+    const int r = blockIdx.x * WARPS + grp;
+    if (r >= NY) return;   // uniform over the warp
+    load_row_vec<T, 32, PADL>(b0, in + (size_t)r * n, n, tid);
+    __syncwarp();
+    T* res = dst_line<T, FP, PADL>(b0, b1, s_tw, n, logn, tid, grp, nullptr);
+    double* dst = out + (size_t)r * NX;
+#pragma unroll 4
+    for (int i = tid; i < NX; i += 32) dst[i] = (double)res[lp<PADL>(i + 1)];
+}
 
-// Inverse row transforms of rows [row0, row0 + nrows) of a padded buffer.
+// What the inverse row transforms of a solve do with their rows (sine.cuh):
 //   INV_STORE_T     outT (padded) = transform
 //   INV_STORE_F64   out64[r*old + ooff + i] = transform
 //   INV_ACCUM_FLUID out64 (padded) += transform at fluid nodes (class FLUID / PLUS) only
 //   INV_ACCUM_T     outT (padded) += transform
-// blockIdx.y selects one of several fields fstride elements apart (in and outT).
-template <typename T, int WARPS, int MODE, int FP>
-__device__ __forceinline__ void
-rows_inv_body(int NX, int NY, int n, int logn, int row0, int nrows, const T* __restrict__ in, T* __restrict__ outT,
-              double* __restrict__ out64, int old, int ooff, const uint8_t* __restrict__ cls,
-              const cpx<T>* __restrict__ g_tw) {
-    constexpr int TN = line_threads(FP), LPB = WARPS * 32 / TN;
-    constexpr bool PADL = padded_lines(FP);
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const cpx<T>* s_tw = block_twiddles<FP, T>(smem_raw, g_tw, n);
-    const int grp = threadIdx.x / TN, tid = threadIdx.x - grp * TN;
-    const int LN = line_len(n, FP);
-    T* lines = reinterpret_cast<T*>(smem_raw + twiddle_smem<T>(n, FP));
-    T* b0 = lines + (size_t)grp * (2 * LN);
-    T* b1 = b0 + LN;
-    T* tot = lines + (size_t)LPB * 2 * LN + grp * kLineScratch;
-    if (FP == 0) __syncthreads();
-    const int r = row0 + blockIdx.x * LPB + grp;
-    if (r >= row0 + nrows || r >= NY) return;   // uniform over the line's threads
-    load_row_vec<T, TN, PADL>(b0, in + (size_t)r * n, n, tid);
-    line_sync<TN>(grp);
-    T* res = dst_line<T, FP, PADL>(b0, b1, s_tw, n, logn, tid, grp, tot);
-    if (MODE == INV_STORE_T) {
-        if (tid == 0) res[0] = T(0);
-        line_sync<TN>(grp);
-        store_row_vec<T, TN, PADL>(outT + (size_t)r * n, res, n, tid);
-    } else if (MODE == INV_STORE_F64) {
-        double* dst = out64 + (size_t)r * old + ooff;
-#pragma unroll 4
-        for (int i = tid; i < NX; i += TN) dst[i] = (double)res[lp<PADL>(i + 1)];
-    } else if (MODE == INV_ACCUM_T) {
-        T* dst = outT + (size_t)r * n + 1;
-#pragma unroll 4
-        for (int i = tid; i < NX; i += TN) dst[i] += res[lp<PADL>(i + 1)];
-    } else {
-        // padded positions p = 1..NX of the row: p = 1 alone, then the pairs (p, p + 1) for even
-        // p, each one 16-byte FP64 read-modify-write (rows start on even indices) with a 2-byte
-        // class load; each lane issues all its loads before its first add
-        const size_t base = (size_t)r * n;
-        if (tid == 0 && cls[base + 1] <= CLS_PLUS) out64[base + 1] += (double)res[lp<PADL>(1)];
-        const int npair = (NX - 1) / 2;
-        double2* o2 = reinterpret_cast<double2*>(out64 + base + 2);
-        const uchar2* c2 = reinterpret_cast<const uchar2*>(cls + base + 2);
-        constexpr int B = 8;
-        for (int q0 = tid; q0 < npair; q0 += B * TN) {
-            double2 o[B];
-            uchar2 c[B];
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int q = q0 + b * TN;
-                if (q < npair) {
-                    c[b] = c2[q];
-                    o[b] = o2[q];
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < B; ++b) {
-                const int q = q0 + b * TN;
-                if (q < npair) {
-                    const int pp = 2 + 2 * q;   // even: lp keeps (pp, pp + 1) adjacent
-                    const vec2_t<T> v = *reinterpret_cast<const vec2_t<T>*>(res + lp<PADL>(pp));
-                    if (c[b].x <= CLS_PLUS) o[b].x += (double)v.x;
-                    if (c[b].y <= CLS_PLUS) o[b].y += (double)v.y;
-                    o2[q] = o[b];
-                }
-            }
-        }
-    }
-}
-
-template <typename T, int WARPS, int MODE, int FP>
-__global__ void __launch_bounds__(WARPS * 32)
-k_rows_inv(int NX, int NY, int n, int logn, int row0, int nrows, const T* __restrict__ in, T* __restrict__ outT,
-           double* __restrict__ out64, int old, int ooff, const uint8_t* __restrict__ cls,
-           const cpx<T>* __restrict__ g_tw, const int* __restrict__ stop, long fstride) {
-    if (stop && *stop) return;
-    rows_inv_body<T, WARPS, MODE, FP>(NX, NY, n, logn, row0, nrows, in + (long)blockIdx.y * fstride,
-                                      outT ? outT + (long)blockIdx.y * fstride : nullptr, out64, old, ooff, cls, g_tw);
-}
+enum RowsInvMode { INV_STORE_T = 0, INV_STORE_F64 = 1, INV_ACCUM_FLUID = 2, INV_ACCUM_T = 3 };
 
 }  // namespace iim

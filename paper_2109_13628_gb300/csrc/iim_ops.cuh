@@ -48,8 +48,6 @@ inline size_t cols_smem(int n, int C = cols_per_block<T>(), bool wide = false) {
     return twiddle_smem<T>(n, fp) + (size_t)n * sizeof(T) +
            (size_t)C * (2 * line_len(n, fp) + pad + kLineScratch) * sizeof(T);
 }
-// Rows per block of the row passes for lines of n points.
-inline int rows_per_block(int n, bool wide) { return kRowWarps * 32 / line_threads(fft_path(n, wide)); }
 
 // Tile widths the column pass supports: FP32 4 or 8 columns, FP64 2 or 4 (16-byte row segments).
 template <typename T>

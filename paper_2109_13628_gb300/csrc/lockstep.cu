@@ -29,6 +29,7 @@
 #include "common.cuh"
 #include "dst.cuh"
 #include "iim_ops.cuh"
+#include "sine.cuh"
 
 namespace iim {
 
@@ -92,19 +93,17 @@ __device__ __forceinline__ VecArg ls_vec(const LsProb& p, int mode) {
     return VecArg{nullptr, nullptr, 0, 0};
 }
 
-template <typename T, int WARPS, int FP>
-__global__ void __launch_bounds__(WARPS * 32)
-kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, const cpx<T>* __restrict__ tw) {
+template <typename T, int N, int L>
+__global__ void __launch_bounds__((Sine<N, L>::kBlock))
+kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, const cpx<T>* __restrict__ tab) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
-    constexpr int LPB = WARPS * 32 / line_threads(FP);
     const bool dense = mode == M_RHS || mode == M_RECOVER;
     const int row0 = dense ? 0 : p.ja0, nrows = dense ? p.NY : p.ja1 - p.ja0 + 1;
-    if ((int)blockIdx.x * LPB >= nrows) return;   // uniform over the block
-    rows_fwd_body<T, WARPS, FP>(p.NX, p.NY, p.nx, __ffs(p.nx) - 1, row0, nrows, dense ? p.res : nullptr, p.nx, 1,
-                                nullptr, 0.0, mode == M_RHS ? nullptr : p.aff_row_ptr,
-                                mode == M_RHS ? nullptr : p.aff_node, ls_vec(p, mode), mode == M_RECOVER ? -1.0 : 1.0,
-                                tw, (T*)p.tbuf);
+    if ((int)blockIdx.x * L >= nrows) return;   // uniform over the block
+    sine_rows_fwd_body<T, N, L>(p.NX, p.NY, p.nx, row0, nrows, dense ? p.res : nullptr, p.nx, 1, nullptr, 0.0,
+                             mode == M_RHS ? nullptr : p.aff_row_ptr, mode == M_RHS ? nullptr : p.aff_node,
+                             ls_vec(p, mode), mode == M_RECOVER ? -1.0 : 1.0, tab, (T*)p.tbuf);
 }
 
 template <typename T, int C, int FP>
@@ -135,17 +134,16 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4) kb_cols_scan(const LsP
     cols_scan_body<T, CW, NT>(p.NX, p.NY, p.nx, in0, in1, out0, out1, (T*)p.tbuf, ls_scan<T>(p));
 }
 
-template <typename T, int WARPS, int MODE, int FP>
-__global__ void __launch_bounds__(WARPS * 32)
-kb_rows_inv(const LsProb* __restrict__ P, int gate, const cpx<T>* __restrict__ tw) {
+template <typename T, int MODE, int N, int L>
+__global__ void __launch_bounds__((Sine<N, L>::kBlock))
+kb_rows_inv(const LsProb* __restrict__ P, int gate, const cpx<T>* __restrict__ tab) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (MODE == INV_STORE_T && p.na == 0)) return;
-    constexpr int LPB = WARPS * 32 / line_threads(FP);
     const int row0 = MODE == INV_STORE_T ? p.jo0 : 0, nrows = MODE == INV_STORE_T ? p.jo1 - p.jo0 + 1 : p.NY;
-    if ((int)blockIdx.x * LPB >= nrows) return;
-    rows_inv_body<T, WARPS, MODE, FP>(p.NX, p.NY, p.nx, __ffs(p.nx) - 1, row0, nrows, (const T*)p.tbuf,
-                                      MODE == INV_STORE_T ? (T*)p.psiT : nullptr,
-                                      MODE == INV_STORE_T ? nullptr : p.psi_ext, 0, 0, p.cls, tw);
+    if ((int)blockIdx.x * L >= nrows) return;
+    sine_rows_inv_body<T, MODE, N, L>(p.NX, p.NY, p.nx, row0, nrows, (const T*)p.tbuf,
+                                   MODE == INV_STORE_T ? (T*)p.psiT : nullptr,
+                                   MODE == INV_STORE_T ? nullptr : p.psi_ext, 0, 0, p.cls, tab);
 }
 
 // gamma-space gathers: the right-hand side b (no input vector, grid = gather blocks only) or
@@ -580,23 +578,19 @@ struct LsEmit {
 
     template <typename T>
     iim_status rows_fwd(int mode, int gate) {
-        const size_t sm = rows_smem<T>(G->nx);
-        const int rpb = rows_per_block(G->nx, G->wide);
         const bool dense = mode == M_RHS || mode == M_RECOVER;
         const int rows = dense ? G->NY : G->max_ja_rows;
         const double bytes = sum_rows(dense ? 0 : 1, G->NX * ((dense ? 8.0 : 0.0) + sizeof(T)));
-        auto go = [&](auto kern) -> iim_status {
+        const int lpb = sine_lines(G->nx, (long)rows * G->n());
+        IIM_CHECK(sine_dispatch(G->nx, lpb, [&](auto N, auto L) -> iim_status {
+            auto kern = kb_rows_fwd<T, N.value, L.value>;
+            const size_t sm = sine_smem<T>(G->nx, lpb);
             IIM_CHECK(allow_smem(kern, sm));
             launch(sizeof(T) == 8 ? "ls_rows_fwd_f64" : "ls_rows_fwd_f32", bytes, 0.0, kern,
-                   grid((rows + rpb - 1) / rpb), kRowWarps * 32, sm, s, (const LsProb*)G->d_probs, mode, gate,
-                   twiddle_region<T>(G->nx, fft_path(G->nx, G->wide)));
+                   grid((rows + lpb - 1) / lpb), (Sine<N.value, L.value>::kBlock), sm, s, (const LsProb*)G->d_probs, mode,
+                   gate, sine_table<T>(G->nx));
             return IIM_OK;
-        };
-        const int fp = fft_path(G->nx, G->wide);
-        if (fp == 64) IIM_CHECK(go(kb_rows_fwd<T, kRowWarps, 64>));
-        else if (fp == 16) IIM_CHECK(go(kb_rows_fwd<T, kRowWarps, 16>));
-        else if (fp == 8) IIM_CHECK(go(kb_rows_fwd<T, kRowWarps, 8>));
-        else IIM_CHECK(go(kb_rows_fwd<T, kRowWarps, 0>));
+        }));
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -662,22 +656,18 @@ struct LsEmit {
 
     template <typename T, int MODE>
     iim_status rows_inv(int gate) {
-        const size_t sm = rows_smem<T>(G->nx);
-        const int rpb = rows_per_block(G->nx, G->wide);
         const int rows = MODE == INV_STORE_T ? G->max_jo_rows : G->NY;
         const double bytes = sum_rows(MODE == INV_STORE_T ? 2 : 0, G->NX * (sizeof(T) + (MODE == INV_STORE_T ? sizeof(T) : 17.0)));
-        auto go = [&](auto kern) -> iim_status {
+        const int lpb = sine_lines(G->nx, (long)rows * G->n());
+        IIM_CHECK(sine_dispatch(G->nx, lpb, [&](auto N, auto L) -> iim_status {
+            auto kern = kb_rows_inv<T, MODE, N.value, L.value>;
+            const size_t sm = sine_smem<T>(G->nx, lpb);
             IIM_CHECK(allow_smem(kern, sm));
             launch(sizeof(T) == 8 ? "ls_rows_inv_f64" : "ls_rows_inv_f32", bytes, 0.0, kern,
-                   grid((rows + rpb - 1) / rpb), kRowWarps * 32, sm, s, (const LsProb*)G->d_probs, gate,
-                   twiddle_region<T>(G->nx, fft_path(G->nx, G->wide)));
+                   grid((rows + lpb - 1) / lpb), (Sine<N.value, L.value>::kBlock), sm, s, (const LsProb*)G->d_probs, gate,
+                   sine_table<T>(G->nx));
             return IIM_OK;
-        };
-        const int fp = fft_path(G->nx, G->wide);
-        if (fp == 64) IIM_CHECK(go(kb_rows_inv<T, kRowWarps, MODE, 64>));
-        else if (fp == 16) IIM_CHECK(go(kb_rows_inv<T, kRowWarps, MODE, 16>));
-        else if (fp == 8) IIM_CHECK(go(kb_rows_inv<T, kRowWarps, MODE, 8>));
-        else IIM_CHECK(go(kb_rows_inv<T, kRowWarps, MODE, 0>));
+        }));
         IIM_LAUNCHED();
         return IIM_OK;
     }

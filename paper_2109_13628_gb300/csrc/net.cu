@@ -277,7 +277,7 @@ inline size_t wgrad_smem(int nog, int ncg, int d) {
 __global__ void __launch_bounds__(WG_THREADS, 2)
 k_conv_wgrad(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ gate,
              float* __restrict__ part, int Ci, int Co, int H, int W, int d, int strips) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
+    extern __shared__ __align__(128) unsigned char smem_raw[];
     const int nog = wg_groups(Co, 8), ncg = wg_groups(Ci, 4);
     const int GP = wg_stride(8 * nog), XP = wg_stride(4 * ncg);
     float* gs = reinterpret_cast<float*>(smem_raw);

@@ -27,6 +27,7 @@
 #include "common.cuh"
 #include "dst.cuh"
 #include "iim_ops.cuh"
+#include "sine.cuh"
 
 namespace iim {
 
@@ -55,6 +56,16 @@ constexpr long twr_total() {
 __device__ cpx<double> g_twr64[twr_total()];
 __device__ cpx<float> g_twr32[twr_total()];
 
+// Tables of the row transforms (sine.cuh), one per line length n = 2^4..2^11.
+constexpr int kSineLog0 = 4, kSineLog1 = 11;
+constexpr long sine_total() {
+    long t = 0;
+    for (int l = kSineLog0; l <= kSineLog1; ++l) t += sine_region(1 << l);
+    return t;
+}
+__device__ cpx<double> g_sine64[sine_total()];
+__device__ cpx<float> g_sine32[sine_total()];
+
 template <typename T, int FP>
 __global__ void k_twiddle_region(const cpx<T>* __restrict__ g_tw, int n, int logn, cpx<T>* __restrict__ out) {
     load_twiddles<FP>(out, g_tw, n, logn);
@@ -66,6 +77,19 @@ static const cpx<double>* g_tw64_addr[64];
 static const cpx<float>* g_tw32_addr[64];
 static const cpx<double>* g_twr64_addr[64][kTwrSlots];
 static const cpx<float>* g_twr32_addr[64][kTwrSlots];
+static const cpx<double>* g_sine64_addr[64][kSineLog1 + 1];
+static const cpx<float>* g_sine32_addr[64][kSineLog1 + 1];
+
+template <typename T>
+static iim_status fill_sine(const cpx<T>* base, cpx<T>* regions, const cpx<T>** addr) {
+    for (int l = kSineLog0; l <= kSineLog1; ++l) {
+        k_sine_region<T><<<1, 256>>>(base, 1 << l, l, regions);
+        IIM_TRY(cudaGetLastError());
+        addr[l] = regions;
+        regions += sine_region(1 << l);
+    }
+    return IIM_OK;
+}
 
 template <typename T>
 static iim_status fill_regions(const cpx<T>* base, cpx<T>* regions, const cpx<T>** addr) {
@@ -113,6 +137,12 @@ iim_status ensure_twiddles() {
     IIM_TRY(cudaGetSymbolAddress(&r32, g_twr32));
     IIM_CHECK(fill_regions<double>(g_tw64_addr[dev], (cpx<double>*)r64, g_twr64_addr[dev]));
     IIM_CHECK(fill_regions<float>(g_tw32_addr[dev], (cpx<float>*)r32, g_twr32_addr[dev]));
+    void* s64 = nullptr;
+    void* s32 = nullptr;
+    IIM_TRY(cudaGetSymbolAddress(&s64, g_sine64));
+    IIM_TRY(cudaGetSymbolAddress(&s32, g_sine32));
+    IIM_CHECK(fill_sine<double>(g_tw64_addr[dev], (cpx<double>*)s64, g_sine64_addr[dev]));
+    IIM_CHECK(fill_sine<float>(g_tw32_addr[dev], (cpx<float>*)s32, g_sine32_addr[dev]));
     IIM_TRY(cudaDeviceSynchronize());
     g_tw_ready[dev] = true;
     return IIM_OK;
@@ -129,6 +159,19 @@ const cpx<float>* twiddle_region<float>(int n, int fp) {
     int dev = 0;
     cudaGetDevice(&dev);
     return g_twr32_addr[dev][twr_slot(ilog2(n), fp == 64)];
+}
+
+template <>
+const cpx<double>* sine_table<double>(int n) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return g_sine64_addr[dev][ilog2(n)];
+}
+template <>
+const cpx<float>* sine_table<float>(int n) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return g_sine32_addr[dev][ilog2(n)];
 }
 
 const cpx<double>* twiddles64() {
@@ -151,23 +194,53 @@ static iim_status rows_fwd(const Plan<T>& p, int row0, int nrows, const double* 
                            double gsign, T* out, const int* stop, cudaStream_t s, int batch = 1, long dfs = 0,
                            long ofs = 0) {
     if (nrows <= 0) return IIM_OK;
-    const size_t sm = rows_smem<T>(p.nx);
-    auto go = [&](auto kern) -> iim_status {
+    const int lpb = sine_lines(p.nx, (long)nrows * batch);
+    const size_t sm = sine_smem<T>(p.nx, lpb);
+    IIM_CHECK(sine_dispatch(p.nx, lpb, [&](auto N, auto L) -> iim_status {
+        auto kern = k_sine_rows_fwd<T, N.value, L.value>;
         IIM_CHECK(allow_smem(kern, sm));
         launch(sizeof(T) == 8 ? "dst_rows_fwd_f64" : "dst_rows_fwd_f32",
                (double)batch * nrows * p.NX * ((dense ? 8.0 : 0.0) + sizeof(T)), (double)batch * nrows * dst_flops(p.nx),
-               kern,
-               dim3((nrows + rows_per_block(p.nx, p.wide) - 1) / rows_per_block(p.nx, p.wide), batch), kRowWarps * 32,
-               sm, s, p.NX, p.NY, p.nx,
-               p.lognx, row0, nrows, dense, dld, doff, ring, ih2, row_ptr, aff_node, gam, gsign,
-               twiddle_region<T>(p.nx, fft_path(p.nx, p.wide)), out, stop, dfs, ofs);
+               kern, dim3((nrows + lpb - 1) / lpb, batch), (Sine<N.value, L.value>::kBlock), sm, s, p.NX, p.NY, p.nx, row0, nrows, dense,
+               dld, doff, ring, ih2, row_ptr, aff_node, gam, gsign, sine_table<T>(p.nx), out, stop, dfs, ofs);
+        return IIM_OK;
+    }));
+    IIM_LAUNCHED();
+    return IIM_OK;
+}
+
+// Row passes of the FP32 box solve for callers (iim_box_poisson with IIM_MIXED): the transforms of
+// dst.cuh, whose FP32 rounding is part of that call's result.
+static iim_status packed_rows_fwd(const Plan<float>& p, const double* dense, const double* ring, double ih2, float* out,
+                                  cudaStream_t s) {
+    const size_t sm = rows_smem<float>(p.nx);
+    auto go = [&](auto kern) -> iim_status {
+        IIM_CHECK(allow_smem(kern, sm));
+        launch("dst_rows_fwd_f32", (double)p.NY * p.NX * 12.0, (double)p.NY * dst_flops(p.nx), kern,
+               (p.NY + kRowWarps - 1) / kRowWarps, kRowWarps * 32, sm, s, p.NX, p.NY, p.nx, p.lognx, dense, ring, ih2,
+               twiddle_region<float>(p.nx, fft_path(p.nx)), out);
         return IIM_OK;
     };
-    const int fp = fft_path(p.nx, p.wide);
-    if (fp == 64) IIM_CHECK(go(k_rows_fwd<T, kRowWarps, 64>));
-    else if (fp == 16) IIM_CHECK(go(k_rows_fwd<T, kRowWarps, 16>));
-    else if (fp == 8) IIM_CHECK(go(k_rows_fwd<T, kRowWarps, 8>));
-    else IIM_CHECK(go(k_rows_fwd<T, kRowWarps, 0>));
+    const int fp = fft_path(p.nx);
+    if (fp == 16) IIM_CHECK(go(k_rows_fwd<float, kRowWarps, 16>));
+    else if (fp == 8) IIM_CHECK(go(k_rows_fwd<float, kRowWarps, 8>));
+    else IIM_CHECK(go(k_rows_fwd<float, kRowWarps, 0>));
+    IIM_LAUNCHED();
+    return IIM_OK;
+}
+static iim_status packed_rows_inv(const Plan<float>& p, const float* in, double* out, cudaStream_t s) {
+    const size_t sm = rows_smem<float>(p.nx);
+    auto go = [&](auto kern) -> iim_status {
+        IIM_CHECK(allow_smem(kern, sm));
+        launch("dst_rows_inv_f32", (double)p.NY * p.NX * 12.0, (double)p.NY * dst_flops(p.nx), kern,
+               (p.NY + kRowWarps - 1) / kRowWarps, kRowWarps * 32, sm, s, p.NX, p.NY, p.nx, p.lognx, in, out,
+               twiddle_region<float>(p.nx, fft_path(p.nx)));
+        return IIM_OK;
+    };
+    const int fp = fft_path(p.nx);
+    if (fp == 16) IIM_CHECK(go(k_rows_inv<float, kRowWarps, 16>));
+    else if (fp == 8) IIM_CHECK(go(k_rows_inv<float, kRowWarps, 8>));
+    else IIM_CHECK(go(k_rows_inv<float, kRowWarps, 0>));
     IIM_LAUNCHED();
     return IIM_OK;
 }
@@ -252,24 +325,18 @@ static iim_status rows_inv(const Plan<T>& p, int row0, int nrows, const T* in, T
                            int ooff, const uint8_t* cls, const int* stop, cudaStream_t s, int batch = 1,
                            long fstride = 0) {
     if (nrows <= 0) return IIM_OK;
-    const size_t sm = rows_smem<T>(p.nx);
-    auto go = [&](auto kern) -> iim_status {
+    const int lpb = sine_lines(p.nx, (long)nrows * batch);
+    const size_t sm = sine_smem<T>(p.nx, lpb);
+    IIM_CHECK(sine_dispatch(p.nx, lpb, [&](auto N, auto L) -> iim_status {
+        auto kern = k_sine_rows_inv<T, MODE, N.value, L.value>;
         IIM_CHECK(allow_smem(kern, sm));
         launch(sizeof(T) == 8 ? "dst_rows_inv_f64" : "dst_rows_inv_f32",
                (double)batch * nrows * p.NX *
                    (sizeof(T) + (MODE == INV_STORE_T ? sizeof(T) : MODE == INV_STORE_F64 ? 8.0 : 17.0)),
-               (double)batch * nrows * dst_flops(p.nx), kern,
-               dim3((nrows + rows_per_block(p.nx, p.wide) - 1) / rows_per_block(p.nx, p.wide), batch),
-               kRowWarps * 32, sm, s, p.NX, p.NY, p.nx, p.lognx, row0, nrows, in, outT, out64, old, ooff, cls,
-               twiddle_region<T>(p.nx, fft_path(p.nx, p.wide)),
-               stop, fstride);
+               (double)batch * nrows * dst_flops(p.nx), kern, dim3((nrows + lpb - 1) / lpb, batch), (Sine<N.value, L.value>::kBlock), sm,
+               s, p.NX, p.NY, p.nx, row0, nrows, in, outT, out64, old, ooff, cls, sine_table<T>(p.nx), stop, fstride);
         return IIM_OK;
-    };
-    const int fp = fft_path(p.nx, p.wide);
-    if (fp == 64) IIM_CHECK(go(k_rows_inv<T, kRowWarps, MODE, 64>));
-    else if (fp == 16) IIM_CHECK(go(k_rows_inv<T, kRowWarps, MODE, 16>));
-    else if (fp == 8) IIM_CHECK(go(k_rows_inv<T, kRowWarps, MODE, 8>));
-    else IIM_CHECK(go(k_rows_inv<T, kRowWarps, MODE, 0>));
+    }));
     IIM_LAUNCHED();
     return IIM_OK;
 }
@@ -2075,9 +2142,9 @@ extern "C" iim_status iim_box_poisson(const iim_grid* grid, const double* f, con
         IIM_TRY(cudaMemcpyAsync(lamf, fl.data(), sizeof(float) * (NX + NY), cudaMemcpyHostToDevice, s));
         Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(), (float)((2.0 / nx) * (2.0 / ny))};
         float* fb = (float*)buf;
-        IIM_CHECK(rows_fwd<float>(p, 0, NY, f, NX, 0, psi_box, ih2, nullptr, nullptr, kNoVec, 0.0, fb, nullptr, s));
+        IIM_CHECK(packed_rows_fwd(p, f, psi_box, ih2, fb, s));
         IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
-        IIM_CHECK((rows_inv<float, INV_STORE_F64>(p, 0, NY, fb, nullptr, u, NX, 0, nullptr, nullptr, s)));
+        IIM_CHECK(packed_rows_inv(p, fb, u, s));
     }
     // pageable-memory copies are staged before cudaMemcpyAsync returns, so the host vectors
     // may go out of scope here
@@ -2207,20 +2274,31 @@ __global__ void k_box_eigs(int NX, int NY, int nx, int ny, double h, int as_floa
     else lam[k] = v;
 }
 
-// Shared-memory limits of every transform kernel the allocation-free solve may launch (all
-// FFT paths), sized for the largest supported line.
-template <typename T>
+// Shared-memory limits of every transform kernel the allocation-free solve may launch, sized for
+// the largest supported line.
 static iim_status allow_noalloc_smem() {
-    const size_t rs = rows_smem<T>(kNoAllocMaxN), cs = cols_smem<T>(kNoAllocMaxN, 4);
-    IIM_CHECK(allow_smem(k_rows_fwd<T, kRowWarps, 0>, rs));
-    IIM_CHECK(allow_smem(k_rows_fwd<T, kRowWarps, 8>, rs));
-    IIM_CHECK(allow_smem(k_rows_fwd<T, kRowWarps, 16>, rs));
-    IIM_CHECK(allow_smem(k_cols<T, 4, 0>, cs));
-    IIM_CHECK(allow_smem(k_cols<T, 4, 8>, cs));
-    IIM_CHECK(allow_smem(k_cols<T, 4, 16>, cs));
-    IIM_CHECK(allow_smem(k_rows_inv<T, kRowWarps, INV_STORE_F64, 0>, rs));
-    IIM_CHECK(allow_smem(k_rows_inv<T, kRowWarps, INV_STORE_F64, 8>, rs));
-    IIM_CHECK(allow_smem(k_rows_inv<T, kRowWarps, INV_STORE_F64, 16>, rs));
+    const size_t rs = rows_smem<float>(kNoAllocMaxN);
+    IIM_CHECK(allow_smem(k_rows_fwd<float, kRowWarps, 0>, rs));
+    IIM_CHECK(allow_smem(k_rows_fwd<float, kRowWarps, 8>, rs));
+    IIM_CHECK(allow_smem(k_rows_fwd<float, kRowWarps, 16>, rs));
+    IIM_CHECK(allow_smem(k_rows_inv<float, kRowWarps, 0>, rs));
+    IIM_CHECK(allow_smem(k_rows_inv<float, kRowWarps, 8>, rs));
+    IIM_CHECK(allow_smem(k_rows_inv<float, kRowWarps, 16>, rs));
+    for (int n = 16; n <= kNoAllocMaxN; n *= 2)
+        for (int lines : {1, 4})
+            IIM_CHECK(sine_dispatch(n, n == 1024 ? std::min(lines, 2) : lines, [&](auto N, auto L) -> iim_status {
+                const size_t sm = sine_smem<double>(n, L.value);
+                IIM_CHECK(allow_smem(k_sine_rows_fwd<double, N.value, L.value>, sm));
+                IIM_CHECK((allow_smem(k_sine_rows_inv<double, INV_STORE_F64, N.value, L.value>, sm)));
+                return IIM_OK;
+            }));
+    const size_t c32 = cols_smem<float>(kNoAllocMaxN, 4), c64 = cols_smem<double>(kNoAllocMaxN, 4);
+    IIM_CHECK(allow_smem(k_cols<float, 4, 0>, c32));
+    IIM_CHECK(allow_smem(k_cols<float, 4, 8>, c32));
+    IIM_CHECK(allow_smem(k_cols<float, 4, 16>, c32));
+    IIM_CHECK(allow_smem(k_cols<double, 4, 0>, c64));
+    IIM_CHECK(allow_smem(k_cols<double, 4, 8>, c64));
+    IIM_CHECK(allow_smem(k_cols<double, 4, 16>, c64));
     return IIM_OK;
 }
 
@@ -2246,8 +2324,7 @@ static iim_status noalloc_setup(cudaStream_t s, double** out) {
         IIM_CHECK(ensure_twiddles());
         void* p = nullptr;
         IIM_TRY(cudaGetSymbolAddress(&p, g_noalloc_scratch));
-        IIM_CHECK(allow_noalloc_smem<double>());
-        IIM_CHECK(allow_noalloc_smem<float>());
+        IIM_CHECK(allow_noalloc_smem());
         g_noalloc_ptr[dev] = (double*)p;
     }
     *out = g_noalloc_ptr[dev];
@@ -2289,9 +2366,9 @@ extern "C" iim_status iim_box_poisson_noalloc(const iim_grid* grid, const double
         Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(),
                       (float)((2.0 / nx) * (2.0 / ny))};
         float* fb = reinterpret_cast<float*>(buf);
-        IIM_CHECK(rows_fwd<float>(p, 0, NY, f, NX, 0, psi_box, ih2, nullptr, nullptr, kNoVec, 0.0, fb, nullptr, s));
+        IIM_CHECK(packed_rows_fwd(p, f, psi_box, ih2, fb, s));
         IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
-        IIM_CHECK((rows_inv<float, INV_STORE_F64>(p, 0, NY, fb, nullptr, u, NX, 0, nullptr, nullptr, s)));
+        IIM_CHECK(packed_rows_inv(p, fb, u, s));
     }
     return IIM_OK;
 }
