@@ -80,7 +80,8 @@ typedef struct {
                           the c that minimises ||b - S x0||, so ||b - S x0|| <= ||b||; dropped
                           when c = 0 -- the learned-guess path */
     double inner_rtol; /* Krylov tolerance of each correction solve (<= 0: library default,
-                          rtol/20 in FP64 mode, 1e-4 in mixed mode) */
+                          rtol/20 in FP64 mode, 1e-4 in mixed mode; with precond 1 or 3 in mixed mode
+                          also no more than the un-reduced residual of the correction calls for) */
     int precond;       /* 0: plain GMRES; 1: right-precondition GMRES with the dense inverse of
                           the Schur matrix (built on first use, see iim_build_preconditioner);
                           2: each correction applies that inverse once, x = M b, with no Krylov

@@ -183,6 +183,7 @@ struct iim_geometry_s {
     double* small = nullptr;     // small per-solve vectors (see solve.cu)
     int krylov_m = 0;            // restart length the Krylov buffers were sized for
     double* V = nullptr;         // (m+1) * ns Krylov basis
+    double* Z = nullptr;         // (m+1) * ns: column j + 1 = M v_j of the preconditioned iteration (on first use)
     double* H = nullptr;         // small Hessenberg / Givens storage
     double* xsol = nullptr;      // ns
     double* bvec = nullptr;      // ns
@@ -195,7 +196,6 @@ struct iim_geometry_s {
     float* pc_S = nullptr;   // copy of S itself (ns x ns, FP32) kept before the inversion
     float* pc_f = nullptr;   // Gauss-Jordan scratch (gj_scratch_floats)
     int* pc_info = nullptr;
-    double* pc_z = nullptr;      // 2 ns
     int pc_ready = 0;
     float pc_setup_ms = 0.f;
     int cols_c = 4;              // column-pass tile width (autotuned per size bucket)
@@ -227,6 +227,7 @@ iim_status solve_enqueue(iim_geometry g, const double* omega, const double* psi_
                          const iim_opts* opts, iim_stats* stats, cudaStream_t s, int* enqueued);
 iim_status solve_finish(iim_geometry g, const iim_opts* opts, iim_stats* stats);
 void set_last_error(const char* msg);
+double inner_tolerance(const iim_opts& o, double* kappa, double* last);
 // lockstep batched solves (lockstep.cu): problems of one grid size advanced together, one launch
 // per step for all of them
 bool lockstep_eligible(iim_geometry g, const iim_opts& o);
@@ -256,11 +257,10 @@ iim_status launch_ring_residual(int nx, int ny, double h, const double* G, int l
 // [S | I] -> [I | S^-1] in place; scratch holds gj_scratch_floats(n) floats
 size_t gj_scratch_floats(int n);
 iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_t s);
+// out = M v, v = column *jidx of a basis when jidx is given, out = column *jidx + 1 when ostride > 0
 iim_status dense_matvec(int n, const float* M, long ldm, const double* v, const int* jidx, long vstride, double* out,
-                        int accumulate, const int* stop, cudaStream_t s);
+                        long ostride, const int* stop, cudaStream_t s);
 bool dense_matvec_fits(int n);
-iim_status dense_matvec_to(int n, const float* M, long ldm, const double* v, double* outb, const int* ojidx,
-                           long ostride, const int* stop, cudaStream_t s);
 __global__ void k_unit_vector(int n, int j, double* v);
 __global__ void k_store_column(int n, int j, const double* v, float* A);
 }

@@ -429,17 +429,27 @@ __device__ __forceinline__ void arnoldi_block_body(int* __restrict__ di, double*
     for (int e = tid; e < ns; e += BLOCK) w[e] *= inv;
 }
 
+// Krylov tolerance of a correction: rel ||b||, and with kappa > 0 at most max(kappa ||r||, last ||f||), r
+// and f the un-reduced residual of the correction and of psi = 0.  The Schur residual b - S x is what
+// the correction leaves at the affected nodes of the un-reduced residual, whose other rows keep FP32
+// noise of about kappa ||r||; ||b|| itself is larger than ||r|| by the 1/h^2 of the extrapolation (by 20
+// to 1000 on the grids here), so rel alone stops early: five bodies at 2048^2 then contract by 20 per
+// correction instead of several hundred.  last ||f|| = a tenth of the target: no more than the last correction needs.
+struct KTol {
+    double rel, kappa, last;
+};
+
 template <int BLOCK>
 __device__ __forceinline__ void start_block_body(int ns, const double* __restrict__ r, double* __restrict__ v0,
                                                  KLayout L, double* __restrict__ K, int* __restrict__ di,
-                                                 int init_maxit, double tol, double* __restrict__ norm2) {
+                                                 int init_maxit, KTol tol, double* __restrict__ small) {
     __shared__ double s_inv;
     double acc = 0.0;
     for (int e = threadIdx.x; e < ns; e += BLOCK) acc += r[e] * r[e];
     acc = block_sum<BLOCK>(acc);
     if (threadIdx.x == 0) {
         if (init_maxit >= 0) {
-            *norm2 = acc;
+            small[SM_NORM] = acc;
             di[DI_J] = 0;
             di[DI_STOP] = 0;
             di[DI_IT] = 0;
@@ -448,7 +458,10 @@ __device__ __forceinline__ void start_block_body(int ns, const double* __restric
             di[DI_TMPJ] = 0;
             di[DI_LOOP] = 0;
             di[DI_LOOPERR] = 0;
-            K[L.scal() + SC_TOL] = tol * sqrt(acc);
+            double t = tol.rel * sqrt(acc);
+            if (tol.kappa > 0.0)
+                t = fmin(t, fmax(tol.kappa * sqrt(small[SM_RES2]), tol.last * small[SM_FNORM]));
+            K[L.scal() + SC_TOL] = t;
         }
         const double beta = sqrt(acc);
         double* gv = K + L.gv();
@@ -468,8 +481,8 @@ __device__ __forceinline__ void start_block_body(int ns, const double* __restric
 
 template <int BLOCK>
 __device__ __forceinline__ void backsolve_update_body(const int* __restrict__ di, KLayout L, double* __restrict__ K,
-                                                      const double* __restrict__ V, long ld, int ns,
-                                                      double* __restrict__ out, int accumulate) {
+                                                      const double* __restrict__ Z, long ld, int ns,
+                                                      double* __restrict__ x) {
     const int k = di[DI_J];
     double* y = K + L.y();
     if (threadIdx.x < 32) {
@@ -491,8 +504,8 @@ __device__ __forceinline__ void backsolve_update_body(const int* __restrict__ di
     __syncthreads();
     for (int e = threadIdx.x; e < ns; e += BLOCK) {
         double s = 0.0;
-        for (int i = 0; i < k; ++i) s += y[i] * V[(long)i * ld + e];
-        out[e] = accumulate ? out[e] + s : 0.0 + s;
+        for (int i = 0; i < k; ++i) s += y[i] * Z[(long)i * ld + e];
+        x[e] += s;
     }
 }
 
@@ -525,10 +538,10 @@ __device__ __forceinline__ void final_rel_body(int* __restrict__ di, double* __r
 template <int WARPS>
 __device__ __forceinline__ void
 dense_matvec4_body(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
-                   const int* __restrict__ jidx, long vstride, double* __restrict__ out, int accumulate,
-                   const int* __restrict__ stop, const int* __restrict__ ojidx = nullptr, long ostride = 0) {
+                   const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
+                   const int* __restrict__ stop) {
     if (stop && *stop) return;
-    if (ojidx) out += (long)(*ojidx + 1) * ostride;   // out = column j + 1 of a Krylov basis
+    if (ostride) out += (long)(*jidx + 1) * ostride;   // out = column j + 1 of a basis
     extern __shared__ float4 s_v4[];
     float* s_v = reinterpret_cast<float*>(s_v4);
     const int stride = (n + 3) & ~3;
@@ -586,7 +599,7 @@ dense_matvec4_body(int n, const float* __restrict__ M, long ldm, const double* _
         }
         float acc = (a0 + a1) + (a2 + a3);
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) out[row] = accumulate ? out[row] + (double)acc : (double)acc;
+        if (lane == 0) out[row] = (double)acc;
     }
 }
 

@@ -22,6 +22,7 @@
 // which is how the per-kernel profiler times the batched kernels one launch at a time.
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 #include <cstring>
 #include <mutex>
 #include <vector>
@@ -51,7 +52,7 @@ struct LsProb {
     const iim_region* regions;
     const void* lam_x;
     const void* lam_y;
-    double *psi_ext, *res, *partial, *small, *V, *H, *xsol, *bvec, *pc_z;
+    double *psi_ext, *res, *partial, *small, *V, *Z, *H, *xsol, *bvec;
     void* tbuf;
     void* psiT;
     const float* pc_inv;   // right half of [S | S^-1], leading dimension 2 ns
@@ -67,7 +68,7 @@ struct LsProb {
 // Per-problem record gathered at the end of a solve (one device-to-host copy for the group).
 struct LsRec {
     int di[16];
-    double rel, circ_err, scal[4];
+    double rel, circ_err, scal[4], norm2;
 };
 
 __device__ __forceinline__ bool ls_off(const LsProb& p, int gate) {
@@ -84,10 +85,10 @@ __device__ __forceinline__ bool ls_off(const LsProb& p, int gate) {
 // Row / column pass modes: the right-hand side (dense residual in, rows the gather reads out),
 // the Schur operator on the preconditioned vector (iteration) or on V_1 (restart), and the
 // recovery of psi from the residual and the corrections.
-enum LsMode { M_RHS = 0, M_APPLY_PCZ = 1, M_APPLY_VTMP = 2, M_RECOVER = 3 };
+enum LsMode { M_RHS = 0, M_APPLY_Z = 1, M_APPLY_VTMP = 2, M_RECOVER = 3 };
 
 __device__ __forceinline__ VecArg ls_vec(const LsProb& p, int mode) {
-    if (mode == M_APPLY_PCZ) return VecArg{p.pc_z, nullptr, 0, 0};
+    if (mode == M_APPLY_Z) return VecArg{p.Z, p.di + DI_J, 1, (long)p.ns};
     if (mode == M_APPLY_VTMP) return VecArg{p.V, p.di + DI_TMPJ, 0, (long)p.ns};
     if (mode == M_RECOVER) return VecArg{p.na ? p.xsol : nullptr, nullptr, 0, 0};
     return VecArg{nullptr, nullptr, 0, 0};
@@ -112,7 +113,7 @@ kb_cols(const LsProb* __restrict__ P, int mode, int gate, T norm, const cpx<T>* 
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
-    if (mode == M_APPLY_PCZ || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
+    if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
     if (mode == M_RECOVER) { out0 = 0; out1 = p.NY - 1; }
     cols_body<T, C, FP>(p.NX, p.NY, p.NY + 1, __ffs(p.NY + 1) - 1, in0, in1, out0, out1, (T*)p.tbuf,
                         (const T*)p.lam_x, (const T*)p.lam_y, norm, tw);
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4) kb_cols_scan(const LsP
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
-    if (mode == M_APPLY_PCZ || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
+    if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
     if (mode == M_RECOVER) { out0 = 0; out1 = p.NY - 1; }
     cols_scan_body<T, CW, NT>(p.NX, p.NY, p.nx, in0, in1, out0, out1, (T*)p.tbuf, ls_scan<T>(p));
 }
@@ -160,28 +161,25 @@ __global__ void __launch_bounds__(BLOCK) kb_gather(const LsProb* __restrict__ P,
         return;
     }
     if ((int)blockIdx.x >= nga + p.ncirc) return;
-    const int* jidx = p.di + (mode == M_APPLY_PCZ ? DI_J : DI_TMPJ);
+    const int* jidx = p.di + (mode == M_APPLY_Z ? DI_J : DI_TMPJ);
     gather_body<T, BLOCK>(p.na, nga, p.gop_ptr, p.gop_idx, p.gop_w, (const T*)p.psiT, p.cp_body, p.body_circ,
                           p.aff_body, ls_vec(p, mode), 1, p.V, jidx, (long)p.ns, nullptr);
 }
 
-// Dense products: z = M V_j (iteration, skipped once the problem's GMRES stopped), x += M t
-// (cycle end), and with the dense inner operator V_{j+1} = S z (iteration) or V_2 = S V_1
-// (restart).
-enum { MV_PRECOND = 0, MV_XUPDATE = 1, MV_S_ITER = 2, MV_S_RESTART = 3 };
+// Dense products: z_j = M V_j (iteration, skipped once the problem's GMRES stopped), and with the
+// dense inner operator V_{j+1} = S z_j (iteration) or V_2 = S V_1 (restart).
+enum { MV_PRECOND = 0, MV_S_ITER = 1, MV_S_RESTART = 2 };
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32) kb_matvec(const LsProb* __restrict__ P, int op, int gate) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || p.ns == 0) return;
     const long ns = p.ns;
     if (op == MV_PRECOND)
-        dense_matvec4_body<WARPS>(p.ns, p.pc_inv, 2L * ns, p.V, p.di + DI_J, ns, p.pc_z, 0, p.di + DI_STOP);
-    else if (op == MV_XUPDATE)
-        dense_matvec4_body<WARPS>(p.ns, p.pc_inv, 2L * ns, p.pc_z + ns, nullptr, 0L, p.xsol, 1, nullptr);
+        dense_matvec4_body<WARPS>(p.ns, p.pc_inv, 2L * ns, p.V, p.di + DI_J, ns, p.Z, ns, p.di + DI_STOP);
     else if (op == MV_S_ITER)
-        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.pc_z, nullptr, 0L, p.V, 0, p.di + DI_STOP, p.di + DI_J, ns);
+        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.Z + ns, p.di + DI_J, ns, p.V, ns, p.di + DI_STOP);
     else
-        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.V + ns, nullptr, 0L, p.V, 0, nullptr, p.di + DI_TMPJ, ns);
+        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.V, p.di + DI_TMPJ, ns, p.V, ns, nullptr);
 }
 
 // ------------------------------------------------------------------------- Krylov kernels
@@ -197,17 +195,17 @@ __global__ void __launch_bounds__(BLOCK) kb_arnoldi(const LsProb* __restrict__ P
 // of a restart cycle (V_0 = (b - S x) / ||b - S x||).
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
-kb_start(const LsProb* __restrict__ P, KLayout L, int restart, int max_iter, double tol) {
+kb_start(const LsProb* __restrict__ P, KLayout L, int restart, int max_iter, KTol tol) {
     const LsProb& p = P[blockIdx.z];
     if (!restart) {
         if (!p.di[DI_RACT] || p.ns == 0) {
             if (threadIdx.x == 0) p.di[DI_STOP] = 1;
             return;
         }
-        start_block_body<BLOCK>(p.ns, p.bvec, p.V, L, p.H, p.di, max_iter, tol, p.small + SM_NORM);
+        start_block_body<BLOCK>(p.ns, p.bvec, p.V, L, p.H, p.di, max_iter, tol, p.small);
     } else {
         if (!p.di[DI_CACT]) return;
-        start_block_body<BLOCK>(p.ns, p.V + 2L * p.ns, p.V, L, p.H, p.di, -1, 0.0, nullptr);
+        start_block_body<BLOCK>(p.ns, p.V + 2L * p.ns, p.V, L, p.H, p.di, -1, KTol{}, nullptr);
     }
 }
 
@@ -215,7 +213,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) kb_backsolve(const LsProb* __restrict__ P, KLayout L) {
     const LsProb& p = P[blockIdx.z];
     if (!p.di[DI_CACT]) return;
-    backsolve_update_body<BLOCK>(p.di, L, p.H, p.V, (long)p.ns, p.ns, p.pc_z + p.ns, 0);
+    backsolve_update_body<BLOCK>(p.di, L, p.H, p.Z + p.ns, (long)p.ns, p.ns, p.xsol);
 }
 
 // Small vector steps: x = 0 at the start of a correction; V_1 = x and the scratch column index
@@ -321,6 +319,7 @@ __global__ void kb_records(const LsProb* __restrict__ P, int n, KLayout L, LsRec
     out[k].rel = p.small[SM_REL];
     out[k].circ_err = p.small[SM_CIRC_ERR];
     for (int i = 0; i < 4; ++i) out[k].scal[i] = p.H[L.scal() + i];
+    out[k].norm2 = p.small[SM_NORM];
 }
 
 // ------------------------------------------------------------------------- loop control
@@ -469,7 +468,7 @@ __global__ void kb_ref_ctl(const LsProb* __restrict__ P, int n, double rtol, int
 struct LsGroup {
     std::vector<iim_geometry> geos;
     int prec = 0, m = 0, max_refine = 0, max_iter = 0, cap = 0, dense = 0;
-    double rtol = 0.0, inner = 0.0;
+    double rtol = 0.0, inner = 0.0, kappa = 0.0, last = 0.0;
     int nx = 0, ny = 0, NX = 0, NY = 0, wide = 0, cols_c = 4, tri = 0;
     // launch extents: maxima over the group
     int max_na = 0, max_ns = 0, max_nminus = 0, max_ncirc = 0, max_ja_rows = 0, max_jo_rows = 0;
@@ -525,7 +524,7 @@ bool lockstep_eligible(iim_geometry g, const iim_opts& o) {
     const int ns = g->na + g->ncirc;
     return g_ls_group.load() >= 2 && g->host_solves > 0 && !g->solve_graph_failed && o.guess == 0 && !g->outer &&
            (o.precond == 1 || (o.precond == 3 && g->pc_S)) && ns > 0 && g->pc_ready &&
-           g->V && g->krylov_m >= o.restart && (g->ncirc == 0 || g->cap_ready) &&
+           g->V && g->Z && g->krylov_m >= o.restart && (g->ncirc == 0 || g->cap_ready) &&
            sizeof(float) * 4 * (size_t)((ns + 3) & ~3) <= 200 * 1024;
 }
 
@@ -544,7 +543,7 @@ static void fill_prob(LsProb& q, iim_geometry g, int prec, const double* omega, 
     q.lam_x = prec == IIM_FP64 ? (const void*)g->lam_x64 : (const void*)g->lam_x32;
     q.lam_y = prec == IIM_FP64 ? (const void*)g->lam_y64 : (const void*)g->lam_y32;
     q.psi_ext = g->psi_ext; q.res = g->res; q.partial = g->partial; q.small = g->small; q.V = g->V; q.H = g->H;
-    q.xsol = g->xsol; q.bvec = g->bvec; q.pc_z = g->pc_z; q.tbuf = g->tbuf; q.psiT = g->psiT;
+    q.xsol = g->xsol; q.bvec = g->bvec; q.Z = g->Z; q.tbuf = g->tbuf; q.psiT = g->psiT;
     q.pc_inv = g->pc_aug + (q.ns);
     q.pc_S = g->pc_S;
     if (g->col_solver == 1) {
@@ -602,7 +601,7 @@ struct LsEmit {
         double bytes = 0.0;
         for (iim_geometry g : G->geos) {
             int in = g->NY, out = g->jo1 - g->jo0 + 1;
-            if (mode == M_APPLY_PCZ || mode == M_APPLY_VTMP) in = g->ja1 - g->ja0 + 1;
+            if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) in = g->ja1 - g->ja0 + 1;
             if (mode == M_RECOVER) out = g->NY;
             bytes += (double)(in + out) * g->NX * sizeof(T);
         }
@@ -628,7 +627,7 @@ struct LsEmit {
             double bytes = 0.0;
             for (iim_geometry g : G->geos) {
                 int in = g->NY, out = g->jo1 - g->jo0 + 1;
-                if (mode == M_APPLY_PCZ || mode == M_APPLY_VTMP) in = g->ja1 - g->ja0 + 1;
+                if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) in = g->ja1 - g->ja0 + 1;
                 if (mode == M_RECOVER) out = g->NY;
                 bytes += (double)(in + out) * g->NX * sizeof(T);
             }
@@ -740,7 +739,7 @@ struct LsEmit {
         IIM_CHECK(gather<T>(M_RHS, G_REF));
         IIM_CHECK(vec(V_ZERO_X, G_REF));
         launch("ls_gmres_start", 0.0, 0.0, kb_start<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs, KLayout{G->m},
-               0, G->max_iter, G->inner);
+               0, G->max_iter, KTol{G->inner, G->kappa, G->last});
         launch("ls_cyc_begin", 0.0, 0.0, kb_cyc_begin, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(), G->max_iter,
                h_cyc, flag());
         IIM_LAUNCHED();
@@ -753,17 +752,17 @@ struct LsEmit {
         return IIM_OK;
     }
 
-    // one preconditioned GMRES iteration: z = M v_j, v_{j+1} = S z, Arnoldi step
+    // one preconditioned GMRES iteration: z_j = M v_j, v_{j+1} = S z_j, Arnoldi step
     template <typename T>
     iim_status iteration(cudaGraphConditionalHandle h_it) {
         IIM_CHECK(matvec(MV_PRECOND, G_IT));
         if (G->dense) {
             IIM_CHECK(matvec(MV_S_ITER, G_IT));
         } else {
-            IIM_CHECK(rows_fwd<T>(M_APPLY_PCZ, G_IT));
-            IIM_CHECK(cols<T>(M_APPLY_PCZ, G_IT));
+            IIM_CHECK(rows_fwd<T>(M_APPLY_Z, G_IT));
+            IIM_CHECK(cols<T>(M_APPLY_Z, G_IT));
             IIM_CHECK((rows_inv<T, INV_STORE_T>(G_IT)));
-            IIM_CHECK(gather<T>(M_APPLY_PCZ, G_IT));
+            IIM_CHECK(gather<T>(M_APPLY_Z, G_IT));
         }
         launch("ls_gmres_arnoldi", 0.0, 0.0, kb_arnoldi<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs,
                KLayout{G->m});
@@ -773,12 +772,10 @@ struct LsEmit {
         return IIM_OK;
     }
 
-    // x += M (V y), then another cycle (with the restart below) unless every problem is done
+    // x += sum y_j z_j, then another cycle (with the restart below) unless every problem is done
     iim_status cyc_post(cudaGraphConditionalHandle h_cyc, cudaGraphConditionalHandle h_rs) {
         launch("ls_gmres_backsolve", 0.0, 0.0, kb_backsolve<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs,
                KLayout{G->m});
-        IIM_LAUNCHED();
-        IIM_CHECK(matvec(MV_XUPDATE, G_CYC));
         launch("ls_cyc_ctl", 0.0, 0.0, kb_cyc_ctl, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(),
                G->max_iter / G->m + 2, h_cyc, h_rs, flag(), cnt());
         IIM_LAUNCHED();
@@ -799,7 +796,7 @@ struct LsEmit {
         }
         IIM_CHECK(vec(V_RESTART_RES, G_CYC));
         launch("ls_gmres_start", 0.0, 0.0, kb_start<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs, KLayout{G->m},
-               1, 0, 0.0);
+               1, 0, KTol{});
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -945,11 +942,12 @@ static iim_status build_group_graph(LsGroup* G) {
     return st;
 }
 
-static iim_status make_group(const std::vector<iim_geometry>& geos, const iim_opts& o, double inner, LsGroup** out) {
+static iim_status make_group(const std::vector<iim_geometry>& geos, const iim_opts& o, double inner, double kappa,
+                             double last, LsGroup** out) {
     LsGroup* G = new LsGroup();
     G->geos = geos;
     G->prec = o.prec; G->m = o.restart; G->max_refine = o.max_refine; G->max_iter = o.max_iter;
-    G->rtol = o.rtol; G->inner = inner; G->dense = o.precond == 3;
+    G->rtol = o.rtol; G->inner = inner; G->kappa = kappa; G->last = last; G->dense = o.precond == 3;
     iim_geometry g0 = geos[0];
     G->nx = g0->nx; G->ny = g0->ny; G->NX = g0->NX; G->NY = g0->NY; G->wide = g0->wide_lines; G->cols_c = g0->cols_c;
     G->tri = g0->col_solver == 1;
@@ -989,11 +987,11 @@ static iim_status make_group(const std::vector<iim_geometry>& geos, const iim_op
     return IIM_OK;
 }
 
-static LsGroup* find_group(const std::vector<iim_geometry>& geos, const iim_opts& o, double inner) {
+static LsGroup* find_group(const std::vector<iim_geometry>& geos, const iim_opts& o, double inner, double kappa) {
     for (LsGroup* G : g_ls_groups) {
         if (G->geos != geos || G->prec != o.prec || G->dense != (o.precond == 3) || G->m != o.restart ||
             G->max_refine != o.max_refine ||
-            G->max_iter != o.max_iter || G->rtol != o.rtol || G->inner != inner)
+            G->max_iter != o.max_iter || G->rtol != o.rtol || G->inner != inner || G->kappa != kappa)
             continue;
         bool same = true;
         for (iim_geometry g : geos)
@@ -1014,15 +1012,16 @@ iim_status lockstep_enqueue(const std::vector<int>& idx, iim_geometry const* geo
                             double* const* psibar, double* const* psi_out, double* const* ux_out,
                             double* const* uy_out, const iim_opts& o, cudaStream_t s, bool host_driven,
                             void** handle) {
-    const double inner = o.inner_rtol > 0.0 ? o.inner_rtol : (o.prec == IIM_FP64 ? o.rtol / 20.0 : 1e-4);
+    double kappa = 0.0, last = 0.0;
+    const double inner = inner_tolerance(o, &kappa, &last);
     std::vector<iim_geometry> geos;
     for (int k : idx) geos.push_back(geoms[k]);
     LsGroup* G = nullptr;
     {
         std::lock_guard<std::mutex> lock(g_ls_mutex);
-        G = find_group(geos, o, inner);
+        G = find_group(geos, o, inner, kappa);
         if (!G) {
-            IIM_CHECK(make_group(geos, o, inner, &G));
+            IIM_CHECK(make_group(geos, o, inner, kappa, last, &G));
             g_ls_groups.push_back(G);
         }
     }
@@ -1086,7 +1085,7 @@ void lockstep_finish(void* handle, const std::vector<int>& idx, const iim_opts& 
         S.refinements = r.di[DI_REF];
         S.status = st;
         S.rel_res = r.rel;
-        const double bn = r.scal[SC_TOL] / std::max(G->inner, 1e-300);
+        const double bn = std::sqrt(r.norm2);
         S.gmres_rel_res = (g->na + g->ncirc) > 0 && bn > 0.0 ? r.scal[SC_RESID] / bn : 0.0;
         S.circ_err_max = r.circ_err;
         S.seed_rel_res = 1.0;

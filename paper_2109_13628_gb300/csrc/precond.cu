@@ -209,16 +209,17 @@ __global__ void k_set_identity_aug(float* __restrict__ A, int n) {
     A[i * ld + n + j] = (i == j) ? 1.f : 0.f;
 }
 
-// out = M v (+ out when accumulate), M row-major n x n FP32 with leading dimension ldm (even);
+// out = M v, M row-major n x n FP32 with leading dimension ldm (even);
 // one warp per row.  v = vbase + (jidx ? *jidx : 0) * vstride is staged in shared memory as
 // FP32; each lane reads the row in 8-byte pairs (after one odd leading element when the row
 // starts 4 bytes off an 8-byte boundary) into four independent accumulators.
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 k_dense_matvec(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
-               const int* __restrict__ jidx, long vstride, double* __restrict__ out, int accumulate,
+               const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
                const int* __restrict__ stop) {
     if (stop && *stop) return;
+    if (ostride) out += (long)(*jidx + 1) * ostride;
     extern __shared__ float s_v[];
     const double* v = jidx ? vbase + (long)(*jidx) * vstride : vbase;
     for (int j = threadIdx.x; j < n; j += WARPS * 32) s_v[j] = (float)v[j];
@@ -247,7 +248,7 @@ k_dense_matvec(int n, const float* __restrict__ M, long ldm, const double* __res
         if (((n - head) & 1) && lane == 31) a1 = fmaf(r[n - 1], s_v[n - 1], a1);
         float acc = (a0 + a1) + (a2 + a3);
         for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) out[row] = accumulate ? out[row] + (double)acc : (double)acc;
+        if (lane == 0) out[row] = (double)acc;
     }
 }
 
@@ -258,9 +259,9 @@ k_dense_matvec(int n, const float* __restrict__ M, long ldm, const double* __res
 template <int WARPS>
 __global__ void __launch_bounds__(WARPS * 32)
 k_dense_matvec4(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
-                const int* __restrict__ jidx, long vstride, double* __restrict__ out, int accumulate,
+                const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
                 const int* __restrict__ stop) {
-    dense_matvec4_body<WARPS>(n, M, ldm, vbase, jidx, vstride, out, accumulate, stop);
+    dense_matvec4_body<WARPS>(n, M, ldm, vbase, jidx, vstride, out, ostride, stop);
 }
 
 iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_t s) {
@@ -299,33 +300,10 @@ iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_
     return IIM_OK;
 }
 
-// out_{j+1} = M v for the Krylov basis column after *ojidx (the dense Schur operator of the
-// inner iteration, iim_opts.precond == 3); M must fit the staged-vector kernel (4 n floats of
-// shared memory <= 200 KB).
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-k_dense_matvec4_to(int n, const float* __restrict__ M, long ldm, const double* __restrict__ v,
-                   double* __restrict__ outb, const int* __restrict__ ojidx, long ostride,
-                   const int* __restrict__ stop) {
-    dense_matvec4_body<WARPS>(n, M, ldm, v, nullptr, 0L, outb, 0, stop, ojidx, ostride);
-}
-
 bool dense_matvec_fits(int n) { return sizeof(float) * 4 * (size_t)((n + 3) & ~3) <= 200 * 1024; }
 
-iim_status dense_matvec_to(int n, const float* M, long ldm, const double* v, double* outb, const int* ojidx,
-                           long ostride, const int* stop, cudaStream_t s) {
-    constexpr int W = 8;
-    const size_t sm4 = sizeof(float) * 4 * (size_t)((n + 3) & ~3);
-    if (!dense_matvec_fits(n)) return IIM_ERR_INVALID_ARG;
-    IIM_CHECK(allow_smem(k_dense_matvec4_to<W>, sm4));
-    launch("dense_schur_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec4_to<W>, (n + W - 1) / W, W * 32,
-           sm4, s, n, M, ldm, v, outb, ojidx, ostride, stop);
-    IIM_LAUNCHED();
-    return IIM_OK;
-}
-
 iim_status dense_matvec(int n, const float* M, long ldm, const double* v, const int* jidx, long vstride, double* out,
-                        int accumulate, const int* stop, cudaStream_t s) {
+                        long ostride, const int* stop, cudaStream_t s) {
     constexpr int W = 8;
     const size_t sm4 = sizeof(float) * 4 * (size_t)((n + 3) & ~3);
     if (sm4 <= 200 * 1024) {
@@ -333,14 +311,14 @@ iim_status dense_matvec(int n, const float* M, long ldm, const double* v, const 
         // must not lower it under this launch
         IIM_CHECK(allow_smem(k_dense_matvec4<W>, sm4));
         launch("precond_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec4<W>, (n + W - 1) / W, W * 32, sm4, s,
-               n, M, ldm, v, jidx, vstride, out, accumulate, stop);
+               n, M, ldm, v, jidx, vstride, out, ostride, stop);
         IIM_LAUNCHED();
         return IIM_OK;
     }
     const size_t sm = sizeof(float) * (size_t)n;
     IIM_CHECK(allow_smem(k_dense_matvec<W>, sm));
     launch("precond_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec<W>, (n + W - 1) / W, W * 32, sm, s, n, M,
-           ldm, v, jidx, vstride, out, accumulate, stop);
+           ldm, v, jidx, vstride, out, ostride, stop);
     IIM_LAUNCHED();
     return IIM_OK;
 }

@@ -602,13 +602,13 @@ __global__ void k_start_cycle(int ns, const double* __restrict__ r, double* __re
 
 // One block: beta = ||r||, V_0 = r / beta and the GMRES start state (k_start_cycle's work,
 // with the norm reduced inside the block instead of by k_sumsq's blocks).  With init_maxit >= 0
-// it first does what the norm / k_gmres_init launches do at the start of a correction: *norm2 =
-// ||r||^2, the counters reset, the tolerance set to tol * ||r||.  Five launches become one.
+// it first does what the norm / k_gmres_init launches do at the start of a correction: ||r||^2
+// stored, the counters reset, the tolerance set (KTol).  Five launches become one.
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 k_start_block(int ns, const double* __restrict__ r, double* __restrict__ v0, KLayout L, double* __restrict__ K,
-              int* __restrict__ di, int init_maxit, double tol, double* __restrict__ norm2) {
-    start_block_body<BLOCK>(ns, r, v0, L, K, di, init_maxit, tol, norm2);
+              int* __restrict__ di, int init_maxit, KTol tol, double* __restrict__ small) {
+    start_block_body<BLOCK>(ns, r, v0, L, K, di, init_maxit, tol, small);
 }
 
 // y = H^{-1} g over the first k = j columns (one warp)
@@ -631,14 +631,12 @@ __global__ void k_backsolve(const int* __restrict__ di, KLayout L, double* __res
     }
 }
 
-// k_backsolve and the update in one block: warp 0 solves for y, then out = V y (accumulate 0)
-// or out += V y (accumulate 1) over the block -- the same operations in the same order as
-// k_backsolve followed by k_xupdate on a zeroed or the given out.
+// k_backsolve and the update in one block: warp 0 solves for y, then x += Z y over the block.
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
-k_backsolve_update(const int* __restrict__ di, KLayout L, double* __restrict__ K, const double* __restrict__ V,
-                   long ld, int ns, double* __restrict__ out, int accumulate) {
-    backsolve_update_body<BLOCK>(di, L, K, V, ld, ns, out, accumulate);
+k_backsolve_update(const int* __restrict__ di, KLayout L, double* __restrict__ K, const double* __restrict__ Z,
+                   long ld, int ns, double* __restrict__ x) {
+    backsolve_update_body<BLOCK>(di, L, K, Z, ld, ns, x);
 }
 
 __global__ void k_xupdate(const int* __restrict__ di, const double* __restrict__ V, long ld, const double* __restrict__ y,
@@ -848,7 +846,7 @@ struct SolveGraph {
     cudaGraphExec_t exec = nullptr;
     // key
     int prec = -1, m = 0, pc = 0, max_refine = 0, max_iter = 0, cap = 0;
-    double inner = 0.0, rtol = 0.0;
+    double inner = 0.0, kappa = 0.0, rtol = 0.0;
     const void* ptrs[9] = {};   // caller arrays and the Krylov basis
     // kernel nodes per execution of each level (launch accounting)
     long long k_top = 0, k_ref = 0, k_cyc = 0, k_it = 0, k_rs = 0;
@@ -991,7 +989,6 @@ struct Solver {
             IIM_TRY(cudaMalloc(&g->pc_aug, sizeof(float) * 2 * (size_t)n * n));
             IIM_TRY(cudaMalloc(&g->pc_f, sizeof(float) * gj_scratch_floats(n)));
             IIM_TRY(cudaMalloc(&g->pc_info, sizeof(int)));
-            IIM_TRY(cudaMalloc(&g->pc_z, sizeof(double) * 2 * (size_t)n));
         }
         IIM_TRY(cudaEventRecord(g->ev0, s));
         // gamma columns j < |A|, K at a time: unit row transforms, column pass, inverse rows of
@@ -1087,12 +1084,14 @@ struct Solver {
     template <typename T>
     iim_status iteration() {
         if (precond) {
-            // right preconditioning: z = M v_j, v_{j+1} = S z
-            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->V, di() + DI_J, (long)ns, g->pc_z, 0, di() + DI_STOP, s));
+            // flexible right preconditioning: z_j = M v_j kept, v_{j+1} = S z_j, so that x = sum y_j z_j
+            // satisfies S x = sum y_j S z_j as computed.  (x = M (V y) would round M's FP32 product anew, an
+            // error of cond(S) 2^-24 ||b|| that no further iteration removes.)
+            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->V, di() + DI_J, (long)ns, g->Z, (long)ns, di() + DI_STOP, s));
             if (dense_op)
-                IIM_CHECK(dense_matvec_to(ns, g->pc_S, (long)ns, g->pc_z, g->V, di() + DI_J, (long)ns, di() + DI_STOP, s));
+                IIM_CHECK(dense_matvec(ns, g->pc_S, (long)ns, g->Z + ns, di() + DI_J, (long)ns, g->V, (long)ns, di() + DI_STOP, s));
             else
-                IIM_CHECK(apply_vec<T>(VecArg{g->pc_z, nullptr, 0, 0}, di() + DI_J, di() + DI_STOP));
+                IIM_CHECK(apply_vec<T>(VecArg{g->Z, di() + DI_J, 1, (long)ns}, di() + DI_J, di() + DI_STOP));
         } else {
             IIM_CHECK(apply_at<T>(DI_J, di() + DI_STOP));
         }
@@ -1235,7 +1234,7 @@ struct Solver {
         if (!x0) {
             // ||b||, counters, tolerance and V_0 = b / ||b|| in one block
             launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns_, (const double*)g->bvec, V, L, K,
-                   di(), max_it, tol, g->small + SM_NORM);
+                   di(), max_it, KTol{tol, kappa, last}, g->small);
             started = true;
         } else {
             launch("gmres_sumsq", 0.0, 0.0, k_sumsq<256>, kNormBlocks, 256, 0, s, g->bvec, ns_, g->partial);
@@ -1299,11 +1298,9 @@ struct Solver {
                 }
             }
             if (precond) {
-                // x += M (V y)
-                double* t = g->pc_z + ns_;
+                // x += sum y_j z_j
                 launch("gmres_backsolve", 0.0, 0.0, k_backsolve_update<256>, 1, 256, 0, s, (const int*)di(), L, K,
-                       (const double*)V, ld, ns_, t, 0);
-                IIM_CHECK(dense_matvec(ns_, g->pc_aug + ns_, 2L * ns_, t, nullptr, 0, x, 1, nullptr, s));
+                       (const double*)(g->Z + ns_), ld, ns_, x);
             } else {
                 launch("gmres_backsolve", 0.0, 0.0, k_backsolve, 1, 32, 0, s, di(), L, K);
                 launch("gmres_xupdate", 0.0, 0.0, k_xupdate, eb, 256, 0, s, di(), V, ld, K + L.y(), ns_, x);
@@ -1316,9 +1313,10 @@ struct Solver {
             IIM_CHECK(read_state(st));
         }
         IIM_TRY(cudaMemcpyAsync(g->h_pinned + 12, K + L.scal(), 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        IIM_TRY(cudaMemcpyAsync(g->h_pinned + 25, g->small + SM_NORM, sizeof(double), cudaMemcpyDeviceToHost, s));
         IIM_TRY(cudaStreamSynchronize(s));
         iters += st[DI_IT];
-        const double bnorm = g->h_pinned[12 + SC_TOL] / std::max(tol, 1e-300);
+        const double bnorm = std::sqrt(g->h_pinned[25]);
         last_gmres_rel = bnorm > 0.0 ? g->h_pinned[12 + SC_RESID] / bnorm : 0.0;
         return IIM_OK;
     }
@@ -1333,7 +1331,7 @@ struct Solver {
         const int eb = (ns + 255) / 256;
         launch("set_tmpj", 0.0, 0.0, k_set_int, 1, 1, 0, s, di() + DI_TMPJ, 1);
         if (dense_op)
-            IIM_CHECK(dense_matvec_to(ns, g->pc_S, (long)ns, V + ld, V, di() + DI_TMPJ, ld, nullptr, s));
+            IIM_CHECK(dense_matvec(ns, g->pc_S, (long)ns, V, di() + DI_TMPJ, ld, V, ld, nullptr, s));
         else
             IIM_CHECK(apply_at<T>(DI_TMPJ, nullptr));
         if (seed)
@@ -1341,7 +1339,7 @@ struct Solver {
                    g->xsol, g->small + SM_SEED);
         launch("gmres_axpby", 0.0, 0.0, k_axpby, eb, 256, 0, s, ns, 1.0, g->bvec, -1.0, V + 2 * ld, V + 2 * ld);
         launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns, (const double*)(V + 2 * ld), V, L, K,
-               di(), -1, 0.0, (double*)nullptr);
+               di(), -1, KTol{}, (double*)nullptr);
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -1352,7 +1350,7 @@ struct Solver {
         IIM_CHECK(rhs<T>());
         if (direct) {
             // x = M b with the dense inverse of the Schur matrix: no Krylov iterations
-            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->bvec, nullptr, 0, g->xsol, 0, nullptr, s));
+            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->bvec, nullptr, 0, g->xsol, 0L, nullptr, s));
         } else {
             IIM_CHECK(gmres<T>(tol, max_it, x0));
         }
@@ -1364,6 +1362,7 @@ struct Solver {
     // (opts.precond == 3) instead of the transforms
     bool dense_op = false;
     int pc_mode() const { return precond ? (dense_op ? 2 : 1) : 0; }
+    double kappa = 0.0, last = 0.0;   // KTol of the corrections
 
     // ---- the whole solve as one graph (SolveGraph); built on the private capture stream
     template <typename T>
@@ -1420,7 +1419,7 @@ struct Solver {
                 IIM_CHECK(rhs<T>());
                 IIM_TRY(cudaMemsetAsync(x, 0, (size_t)ns_ * sizeof(double), s));
                 launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns_, (const double*)g->bvec, g->V, L,
-                       K, di(), o.max_iter, inner, g->small + SM_NORM);
+                       K, di(), o.max_iter, KTol{inner, kappa, last}, g->small);
                 launch("cyc_begin", 0.0, 0.0, k_cyc_begin, 1, 1, 0, s, h_cyc, di(), o.max_iter);
                 IIM_LAUNCHED();
                 return IIM_OK;
@@ -1444,10 +1443,8 @@ struct Solver {
             });
             piece(cyc_seg, [&]() -> iim_status {
                 if (precond) {
-                    double* t = g->pc_z + ns_;
                     launch("gmres_backsolve", 0.0, 0.0, k_backsolve_update<256>, 1, 256, 0, s, (const int*)di(), L, K,
-                           (const double*)g->V, ld, ns_, t, 0);
-                    IIM_CHECK(dense_matvec(ns_, g->pc_aug + ns_, 2L * ns_, t, nullptr, 0, x, 1, nullptr, s));
+                           (const double*)(g->Z + ns_), ld, ns_, x);
                 } else {
                     launch("gmres_backsolve", 0.0, 0.0, k_backsolve, 1, 32, 0, s, di(), L, K);
                     launch("gmres_xupdate", 0.0, 0.0, k_xupdate, eb, 256, 0, s, di(), g->V, ld, K + L.y(), ns_, x);
@@ -1547,9 +1544,16 @@ struct Solver {
     double seed_scale = 0.0, seed_reduction = 1.0;   // the seed's c and ||b - S c x0|| / ||b||
 };
 
-static iim_status ensure_krylov(iim_geometry g, int m) {
+// Krylov buffers for restart length m (with the z_j of the preconditioned iteration when pc).
+static iim_status ensure_krylov(iim_geometry g, int m, bool pc) {
     const int ns = g->na + g->ncirc;
-    if (g->V && g->krylov_m >= m) return IIM_OK;
+    if (g->V && g->krylov_m >= m) {
+        if (pc && !g->Z) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(g->krylov_m + 1) * std::max(ns, 1)));
+        return IIM_OK;
+    }
+    cudaFree(g->Z);
+    g->Z = nullptr;
+    if (pc) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(m + 1) * std::max(ns, 1)));
     cudaFree(g->V); cudaFree(g->H); cudaFree(g->xsol); cudaFree(g->bvec); cudaFree(g->x0g);
     g->V = g->H = g->xsol = g->bvec = g->x0g = nullptr;
     KLayout L{m};
@@ -1700,6 +1704,18 @@ static iim_status build_capacitance(iim_geometry g, const iim_opts& opts, cudaSt
 }
 
 namespace iim {
+// The Krylov tolerance of a correction relative to ||b||, and the bound by the un-reduced residual that
+// goes with the library's default in the preconditioned mixed forms (KTol; zeros otherwise).
+double inner_tolerance(const iim_opts& o, double* kappa, double* last) {
+    *kappa = *last = 0.0;
+    if (o.inner_rtol > 0.0) return o.inner_rtol;
+    if (o.prec == IIM_FP64) return o.rtol / 20.0;
+    if (o.precond == 1 || o.precond == 3) {
+        *kappa = 1e-5;
+        *last = 0.1 * o.rtol;
+    }
+    return 1e-4;
+}
 // For the batched solver: launch the whole-solve graph without waiting (see poisson_solve's
 // `enqueued`), and read its results once the stream has been synchronised.
 iim_status solve_enqueue(iim_geometry g, const double* omega, const double* psi_b, const double* psi_box,
@@ -1746,7 +1762,7 @@ static iim_status graph_finish(iim_geometry g, const iim_opts& opts, iim_stats* 
         stats->refinements = hi[DI_REF];
         stats->status = st;
         stats->rel_res = rel;
-        const double bn = g->h_pinned[44 + SC_TOL] / std::max(G->inner, 1e-300);
+        const double bn = std::sqrt(g->h_pinned[48]);
         stats->gmres_rel_res = (g->na + g->ncirc) > 0 && bn > 0.0 ? g->h_pinned[44 + SC_RESID] / bn : 0.0;
         stats->circ_err_max = g->h_pinned[41];
         stats->seed_rel_res = 1.0;
@@ -1785,7 +1801,7 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
     if (g->outer) psi_box = nullptr;                                  // the ring is part of the solution
     if (opts.guess < 0 || opts.guess > 2 || opts.precond < 0 || opts.precond > 3) return IIM_ERR_INVALID_ARG;
     IIM_CHECK(ensure_twiddles());
-    IIM_CHECK(ensure_krylov(g, opts.restart));
+    IIM_CHECK(ensure_krylov(g, opts.restart, opts.precond != 0));
     if (g->ncirc > 0)
         IIM_TRY(cudaMemcpyAsync(g->d_int + DI_CIRC, g->circ_ids.data(), g->ncirc * sizeof(int), cudaMemcpyHostToDevice, s));
 
@@ -1804,7 +1820,7 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
                                     cudaMemcpyHostToDevice, s));
     }
     const long npad = (long)g->nx * g->NY;
-    const double inner = opts.inner_rtol > 0.0 ? opts.inner_rtol : (opts.prec == IIM_FP64 ? opts.rtol / 20.0 : 1e-4);
+    const double inner = inner_tolerance(opts, &S.kappa, &S.last);
 
     // After one host-driven solve on the geometry, solves without a guess (and not profiled,
     // not in direct-correction mode) run as one device-driven graph: no host round trip per
@@ -1815,13 +1831,13 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
         SolveGraph* G = (SolveGraph*)g->solve_graph;
         const bool match = G && G->exec && G->prec == opts.prec && G->m == opts.restart && G->pc == S.pc_mode() &&
                            G->max_refine == opts.max_refine && G->max_iter == opts.max_iter &&
-                           G->cap == (int)use_cap && G->inner == inner && G->rtol == opts.rtol &&
+                           G->cap == (int)use_cap && G->inner == inner && G->kappa == S.kappa && G->rtol == opts.rtol &&
                            std::memcmp(G->ptrs, key, sizeof(key)) == 0;
         if (!match) {
             drop_solve_graph(g);
             G = new SolveGraph();
             G->prec = opts.prec; G->m = opts.restart; G->pc = S.pc_mode(); G->max_refine = opts.max_refine;
-            G->max_iter = opts.max_iter; G->cap = (int)use_cap; G->inner = inner; G->rtol = opts.rtol;
+            G->max_iter = opts.max_iter; G->cap = (int)use_cap; G->inner = inner; G->kappa = S.kappa; G->rtol = opts.rtol;
             std::memcpy(G->ptrs, key, sizeof(key));
             const iim_status bs =
                 opts.prec == IIM_FP64
@@ -1844,6 +1860,7 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
             IIM_TRY(cudaMemcpyAsync(g->h_pinned + 40, g->small + SM_REL, sizeof(double), cudaMemcpyDeviceToHost, s));
             IIM_TRY(cudaMemcpyAsync(g->h_pinned + 41, g->small + SM_CIRC_ERR, sizeof(double), cudaMemcpyDeviceToHost, s));
             IIM_TRY(cudaMemcpyAsync(g->h_pinned + 44, g->H + S.L.scal(), 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+            IIM_TRY(cudaMemcpyAsync(g->h_pinned + 48, g->small + SM_NORM, sizeof(double), cudaMemcpyDeviceToHost, s));
             if (enqueued) {
                 *enqueued = 1;
                 return IIM_OK;
@@ -1865,6 +1882,8 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
     IIM_CHECK(S.residual(&res2, &cerr));
     if (!std::isfinite(res2)) return IIM_ERR_NONFINITE;
     const double fnorm = std::sqrt(res2);
+    g->h_pinned[27] = fnorm;   // the corrections' tolerance reads it (KTol), as k_ref_init leaves it
+    IIM_TRY(cudaMemcpyAsync(g->small + SM_FNORM, g->h_pinned + 27, sizeof(double), cudaMemcpyHostToDevice, s));
     if (opts.guess == 1) {
         launch("init_psi", 0.0, 0.0, k_init_psi, (unsigned)((npad + 255) / 256), 256, 0, s, g->NX, g->NY, psi_guess,
                g->node_class, g->psi_ext);
@@ -2100,7 +2119,7 @@ extern "C" iim_status iim_build_preconditioner(iim_geometry g, float* setup_ms, 
     if (!g) return IIM_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     IIM_CHECK(ensure_twiddles());
-    IIM_CHECK(ensure_krylov(g, std::max(g->krylov_m, 2)));
+    IIM_CHECK(ensure_krylov(g, std::max(g->krylov_m, 2), true));
     if (g->ncirc > 0)
         IIM_TRY(cudaMemcpyAsync(g->d_int + DI_CIRC, g->circ_ids.data(), g->ncirc * sizeof(int), cudaMemcpyHostToDevice, s));
     Solver S;
