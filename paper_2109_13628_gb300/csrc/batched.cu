@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "krylov.cuh"
 
 using namespace iim;
 
@@ -25,16 +26,17 @@ iim_opts opts_or_default(const iim_opts* o) {
 }
 
 // Lockstep groups of a batched call: the problems that can take the lockstep path (see
-// lockstep.cu), bucketed by grid size and transform settings, largest grids first, each bucket
+// lockstep.cu), bucketed by grid size, transform settings and Krylov form, largest grids first, each bucket
 // split into groups of at most iim_set_lockstep's size (as even as possible; the groups run
 // concurrently on their own streams); groups of one problem stay on the per-problem path.
 std::vector<std::vector<int>> lockstep_groups(int n, iim_geometry const* geoms, const std::vector<int>& order,
                                               const iim_opts& o) {
-    std::map<std::tuple<long, int, int, int, int, int>, std::vector<int>> b;
+    std::map<std::tuple<long, int, int, int, int, int, int>, std::vector<int>> b;
     for (int k : order) {
         iim_geometry g = geoms[k];
         if (lockstep_eligible(g, o))
-            b[{-(long)g->nx * g->ny, g->nx, g->ny, g->wide_lines, g->cols_c, g->col_solver}].push_back(k);
+            b[{-(long)g->nx * g->ny, g->nx, g->ny, g->wide_lines, g->cols_c, g->col_solver, krylov_class(g->na + g->ncirc)}]
+                .push_back(k);
     }
     std::vector<std::vector<int>> out;
     const int gmax = std::max(lockstep_group_size(), 1);

@@ -191,10 +191,9 @@ struct iim_geometry_s {
     int* d_int = nullptr;        // device counters / flags
     double* h_pinned = nullptr;  // pinned host scalars
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
-    // dense Schur-complement preconditioner: [S | S^-1] row-major ns x 2ns (FP32), scratch
-    float* pc_aug = nullptr;
-    float* pc_S = nullptr;   // copy of S itself (ns x ns, FP32) kept before the inversion
-    float* pc_f = nullptr;   // Gauss-Jordan scratch (gj_scratch_floats)
+    // dense Schur-complement preconditioner
+    float* pc_M = nullptr;   // S^-1 and S (FP32, leading dimension dense_ld(ns), krylov.cuh)
+    float* pc_S = nullptr;
     int* pc_info = nullptr;
     int pc_ready = 0;
     float pc_setup_ms = 0.f;
@@ -258,7 +257,7 @@ iim_status launch_ring_residual(int nx, int ny, double h, const double* G, int l
 size_t gj_scratch_floats(int n);
 iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_t s);
 // out = M v, v = column *jidx of a basis when jidx is given, out = column *jidx + 1 when ostride > 0
-iim_status dense_matvec(int n, const float* M, long ldm, const double* v, const int* jidx, long vstride, double* out,
+iim_status dense_matvec(int n, const float* M, const double* v, const int* jidx, long vstride, double* out,
                         long ostride, const int* stop, cudaStream_t s);
 bool dense_matvec_fits(int n);
 __global__ void k_unit_vector(int n, int j, double* v);

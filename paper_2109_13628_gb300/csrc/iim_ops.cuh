@@ -89,6 +89,19 @@ inline iim_status allow_smem(KernelT k, size_t bytes) {
     return IIM_OK;
 }
 
+// The same for a kernel launched as clusters of up to 16 blocks.
+inline iim_status allow_cluster(const void* k, size_t bytes) {
+    int dev = 0;
+    IIM_TRY(cudaGetDevice(&dev));
+    std::lock_guard<std::mutex> lock(g_attr_mutex);
+    for (auto& e : g_attr_done)
+        if (e.first.first == dev && e.first.second == k && e.second >= bytes) return IIM_OK;
+    IIM_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    IIM_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    g_attr_done.push_back({{dev, k}, bytes});
+    return IIM_OK;
+}
+
 // ------------------------------------------------------------------------- reductions
 template <int BLOCK>
 __device__ __forceinline__ double block_sum(double v) {
@@ -140,44 +153,6 @@ struct KLayout {
     __host__ __device__ long total() const { return scal() + 8; }
 };
 enum { SC_INV = 0, SC_RESID = 1, SC_BETA = 2, SC_TOL = 3 };
-
-// Arnoldi step finish from the squared norm s of the orthogonalised vector: Hessenberg column
-// (the two Gram-Schmidt passes' coefficients summed), Givens rotations, residual estimate,
-// stop test.  One thread.
-__device__ inline void arnoldi_finish(int* __restrict__ di, KLayout L, double* __restrict__ K, double s) {
-    const int j = di[DI_J];
-    const double nrm = sqrt(s);
-    double* H = K + L.H();
-    const int ldh = L.m + 1;
-    double* col = H + (long)j * ldh;
-    for (int i = 0; i <= j; ++i) col[i] = K[L.hc1() + i] + K[L.hc2() + i];
-    col[j + 1] = nrm;
-    double* cs = K + L.cs();
-    double* sn = K + L.sn();
-    double* gv = K + L.gv();
-    for (int i = 0; i < j; ++i) {
-        const double t = cs[i] * col[i] + sn[i] * col[i + 1];
-        col[i + 1] = -sn[i] * col[i] + cs[i] * col[i + 1];
-        col[i] = t;
-    }
-    const double d = hypot(col[j], col[j + 1]);
-    const double c = d > 0.0 ? col[j] / d : 1.0, sg = d > 0.0 ? col[j + 1] / d : 0.0;
-    cs[j] = c;
-    sn[j] = sg;
-    col[j] = d;
-    col[j + 1] = 0.0;
-    gv[j + 1] = -sg * gv[j];
-    gv[j] = c * gv[j];
-    const double resid = fabs(gv[j + 1]);
-    K[L.scal() + SC_INV] = nrm > 0.0 ? 1.0 / nrm : 0.0;
-    K[L.scal() + SC_RESID] = resid;
-    const int jn = j + 1;
-    di[DI_J] = jn;
-    di[DI_IT] += 1;
-    const bool conv = !(resid > K[L.scal() + SC_TOL]);   // also stops on NaN
-    if (conv) di[DI_CONV] = 1;
-    if (conv || jn >= L.m || di[DI_IT] >= di[DI_MAXIT] || nrm == 0.0) di[DI_STOP] = 1;
-}
 
 template <typename T, int BLOCK>
 __device__ __forceinline__ void gather_body(int na, int nga, const int* __restrict__ ptr, const int* __restrict__ idx,
@@ -380,55 +355,6 @@ __device__ __forceinline__ void velocity_body(int NX, int NY, double inv2h, cons
     if (uy) uy[k] = vy;
 }
 
-template <int BLOCK>
-__device__ __forceinline__ void arnoldi_block_body(int* __restrict__ di, double* __restrict__ V, long ld, int ns,
-                                                   KLayout L, double* __restrict__ K) {
-    constexpr int NW = BLOCK / 32;
-    if (di[DI_STOP]) return;
-    const int j = di[DI_J];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    double* w = V + (long)(j + 1) * ld;
-    __shared__ double part[64][NW];
-    __shared__ double h[64];
-    for (int pass = 0; pass < 2; ++pass) {
-        for (int i = 0; i <= j; ++i) {
-            const double* vi = V + (long)i * ld;
-            double acc = 0.0;
-            for (int e = tid; e < ns; e += BLOCK) acc += vi[e] * w[e];
-            acc = warp_sum(acc);
-            if (lane == 0) part[i][warp] = acc;
-        }
-        __syncthreads();
-        if (tid <= j) {
-            double hi = 0.0;
-            for (int q = 0; q < NW; ++q) hi += part[tid][q];
-            h[tid] = hi;
-            K[(pass == 0 ? L.hc1() : L.hc2()) + tid] = hi;
-        }
-        __syncthreads();
-        for (int e = tid; e < ns; e += BLOCK) {
-            double sacc = 0.0;
-            for (int i = 0; i <= j; ++i) sacc += h[i] * V[(long)i * ld + e];
-            w[e] -= sacc;
-        }
-        __syncthreads();   // h and part are rewritten by the next pass
-    }
-    double sq = 0.0;
-    for (int e = tid; e < ns; e += BLOCK) sq += w[e] * w[e];
-    sq = warp_sum(sq);
-    if (lane == 0) part[0][warp] = sq;
-    __syncthreads();
-    if (tid == 0) {
-        double t = 0.0;
-        for (int q = 0; q < NW; ++q) t += part[0][q];
-        arnoldi_finish(di, L, K, t);
-    }
-    __syncthreads();
-    if (di[DI_STOP]) return;
-    const double inv = K[L.scal() + SC_INV];
-    for (int e = tid; e < ns; e += BLOCK) w[e] *= inv;
-}
-
 // Krylov tolerance of a correction: rel ||b||, and with kappa > 0 at most max(kappa ||r||, last ||f||), r
 // and f the un-reduced residual of the correction and of psi = 0.  The Schur residual b - S x is what
 // the correction leaves at the affected nodes of the un-reduced residual, whose other rows keep FP32
@@ -438,76 +364,6 @@ __device__ __forceinline__ void arnoldi_block_body(int* __restrict__ di, double*
 struct KTol {
     double rel, kappa, last;
 };
-
-template <int BLOCK>
-__device__ __forceinline__ void start_block_body(int ns, const double* __restrict__ r, double* __restrict__ v0,
-                                                 KLayout L, double* __restrict__ K, int* __restrict__ di,
-                                                 int init_maxit, KTol tol, double* __restrict__ small) {
-    __shared__ double s_inv;
-    double acc = 0.0;
-    for (int e = threadIdx.x; e < ns; e += BLOCK) acc += r[e] * r[e];
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) {
-        if (init_maxit >= 0) {
-            small[SM_NORM] = acc;
-            di[DI_J] = 0;
-            di[DI_STOP] = 0;
-            di[DI_IT] = 0;
-            di[DI_MAXIT] = init_maxit;
-            di[DI_CONV] = 0;
-            di[DI_TMPJ] = 0;
-            di[DI_LOOP] = 0;
-            di[DI_LOOPERR] = 0;
-            double t = tol.rel * sqrt(acc);
-            if (tol.kappa > 0.0)
-                t = fmin(t, fmax(tol.kappa * sqrt(small[SM_RES2]), tol.last * small[SM_FNORM]));
-            K[L.scal() + SC_TOL] = t;
-        }
-        const double beta = sqrt(acc);
-        double* gv = K + L.gv();
-        gv[0] = beta;
-        for (int i = 1; i <= L.m; ++i) gv[i] = 0.0;
-        K[L.scal() + SC_BETA] = beta;
-        K[L.scal() + SC_RESID] = beta;
-        di[DI_J] = 0;
-        di[DI_STOP] = (di[DI_IT] >= di[DI_MAXIT]) ? 1 : 0;
-        if (!(beta > K[L.scal() + SC_TOL])) { di[DI_CONV] = 1; di[DI_STOP] = 1; }
-        s_inv = beta > 0.0 ? 1.0 / beta : 0.0;
-    }
-    __syncthreads();
-    const double inv = s_inv;
-    for (int e = threadIdx.x; e < ns; e += BLOCK) v0[e] = r[e] * inv;
-}
-
-template <int BLOCK>
-__device__ __forceinline__ void backsolve_update_body(const int* __restrict__ di, KLayout L, double* __restrict__ K,
-                                                      const double* __restrict__ Z, long ld, int ns,
-                                                      double* __restrict__ x) {
-    const int k = di[DI_J];
-    double* y = K + L.y();
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        const double* H = K + L.H();
-        const int ldh = L.m + 1;
-        const double* gv = K + L.gv();
-        for (int i = k - 1; i >= 0; --i) {
-            double s = 0.0;
-            for (int l = i + 1 + lane; l < k; l += 32) s += H[(long)l * ldh + i] * y[l];
-            s = warp_sum(s);
-            if (lane == 0) {
-                const double d = H[(long)i * ldh + i];
-                y[i] = d != 0.0 ? (gv[i] - s) / d : 0.0;
-            }
-            __syncwarp();
-        }
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < ns; e += BLOCK) {
-        double s = 0.0;
-        for (int i = 0; i < k; ++i) s += y[i] * Z[(long)i * ld + e];
-        x[e] += s;
-    }
-}
 
 __device__ __forceinline__ void cap_coef_body(int nc, const double* __restrict__ rc, const double* __restrict__ cinv,
                                               const double* __restrict__ pb, double h2, double* __restrict__ coef,
@@ -532,75 +388,6 @@ __device__ __forceinline__ void final_rel_body(int* __restrict__ di, double* __r
     const double r2 = small[SM_RES2], fn = small[SM_FNORM];
     if (!isfinite(r2)) di[DI_NONFIN] = 1;
     small[SM_REL] = fn > 0.0 ? sqrt(r2) / fn : 0.0;
-}
-
-// z = M v for the dense FP32 preconditioner (one warp per row, v staged in shared memory).
-template <int WARPS>
-__device__ __forceinline__ void
-dense_matvec4_body(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
-                   const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
-                   const int* __restrict__ stop) {
-    if (stop && *stop) return;
-    if (ostride) out += (long)(*jidx + 1) * ostride;   // out = column j + 1 of a basis
-    extern __shared__ float4 s_v4[];
-    float* s_v = reinterpret_cast<float*>(s_v4);
-    const int stride = (n + 3) & ~3;
-    const double* v = jidx ? vbase + (long)(*jidx) * vstride : vbase;
-    for (int j = threadIdx.x; j < n; j += WARPS * 32) {
-        const float x = (float)v[j];
-#pragma unroll
-        for (int h = 0; h < 4; ++h)
-            if (j >= h) s_v[h * stride + j - h] = x;
-    }
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int row = blockIdx.x * WARPS + (threadIdx.x >> 5); row < n; row += gridDim.x * WARPS) {
-        const float* r = M + (long)row * ldm;
-        const int head = min((int)((4 - ((reinterpret_cast<uintptr_t>(r) >> 2) & 3)) & 3), n);
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        if (lane < head) a0 = r[lane] * s_v[lane];
-        const float4* r4 = reinterpret_cast<const float4*>(r + head);
-        const float4* v4 = reinterpret_cast<const float4*>(s_v + head * stride);
-        const int nq = (n - head) >> 2;
-        int q = lane;
-        // the at most seven vectors of the remainder loop are loaded first, so that they are in
-        // flight together with the main batches; the sums keep the order of the loops below
-        int qr = lane;
-        while (qr + 7 * 32 < nq) qr += 8 * 32;
-        float4 xr[7];
-#pragma unroll
-        for (int u = 0; u < 7; ++u) {
-            const int qq = qr + 32 * u;
-            xr[u] = qq < nq ? r4[qq] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        for (; q + 7 * 32 < nq; q += 8 * 32) {
-            float4 x[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) x[u] = r4[q + 32 * u];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                const float4 y = v4[q + 32 * u];
-                float& a = (u & 3) == 0 ? a0 : (u & 3) == 1 ? a1 : (u & 3) == 2 ? a2 : a3;
-                a = fmaf(x[u].x, y.x, fmaf(x[u].y, y.y, fmaf(x[u].z, y.z, fmaf(x[u].w, y.w, a))));
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 7; ++u) {
-            const int qq = qr + 32 * u;   // qr == q here
-            if (qq < nq) {
-                const float4 x = xr[u], y = v4[qq];
-                a1 = fmaf(x.x, y.x, fmaf(x.y, y.y, fmaf(x.z, y.z, fmaf(x.w, y.w, a1))));
-            }
-        }
-        const int rem = (n - head) & 3;
-        if (lane < rem) {
-            const int idx = head + 4 * nq + lane;
-            a2 = fmaf(r[idx], s_v[idx], a2);
-        }
-        float acc = (a0 + a1) + (a2 + a3);
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) out[row] = (double)acc;
-    }
 }
 
 // ------------------------------------------------------------------------- graph capture

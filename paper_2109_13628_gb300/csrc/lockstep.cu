@@ -30,6 +30,7 @@
 #include "common.cuh"
 #include "dst.cuh"
 #include "iim_ops.cuh"
+#include "krylov.cuh"
 #include "sine.cuh"
 
 namespace iim {
@@ -55,8 +56,7 @@ struct LsProb {
     double *psi_ext, *res, *partial, *small, *V, *Z, *H, *xsol, *bvec;
     void* tbuf;
     void* psiT;
-    const float* pc_inv;   // right half of [S | S^-1], leading dimension 2 ns
-    const float* pc_S;     // S itself (ns x ns), the inner operator of iim_opts.precond == 3
+    const float *pc_M, *pc_S;   // S^-1 and S (leading dimension dense_ld(ns))
     ScanTab<float> s32;    // factors of the tridiagonal column pass (used when the group's tri is set)
     ScanTab<double> s64;
     int* di;
@@ -169,51 +169,58 @@ __global__ void __launch_bounds__(BLOCK) kb_gather(const LsProb* __restrict__ P,
 // Dense products: z_j = M V_j (iteration, skipped once the problem's GMRES stopped), and with the
 // dense inner operator V_{j+1} = S z_j (iteration) or V_2 = S V_1 (restart).
 enum { MV_PRECOND = 0, MV_S_ITER = 1, MV_S_RESTART = 2 };
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32) kb_matvec(const LsProb* __restrict__ P, int op, int gate) {
+__global__ void __launch_bounds__(kDenseWarps * 32) kb_matvec(const LsProb* __restrict__ P, int op, int gate) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || p.ns == 0) return;
-    const long ns = p.ns;
+    const long ns = p.ns, ld = dense_ld(p.ns);
     if (op == MV_PRECOND)
-        dense_matvec4_body<WARPS>(p.ns, p.pc_inv, 2L * ns, p.V, p.di + DI_J, ns, p.Z, ns, p.di + DI_STOP);
+        dense_matvec_body(p.ns, p.pc_M, ld, p.V, p.di + DI_J, ns, p.Z, ns, p.di + DI_STOP);
     else if (op == MV_S_ITER)
-        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.Z + ns, p.di + DI_J, ns, p.V, ns, p.di + DI_STOP);
+        dense_matvec_body(p.ns, p.pc_S, ld, p.Z + ns, p.di + DI_J, ns, p.V, ns, p.di + DI_STOP);
     else
-        dense_matvec4_body<WARPS>(p.ns, p.pc_S, ns, p.V, p.di + DI_TMPJ, ns, p.V, ns, nullptr);
+        dense_matvec_body(p.ns, p.pc_S, ld, p.V, p.di + DI_TMPJ, ns, p.V, ns, nullptr);
 }
 
 // ------------------------------------------------------------------------- Krylov kernels
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) kb_arnoldi(const LsProb* __restrict__ P, KLayout L) {
+template <int CL>
+__global__ void __launch_bounds__(kKrylovThreads) kb_arnoldi(const LsProb* P, KLayout L) {
     const LsProb& p = P[blockIdx.z];
     if (p.ns == 0) return;
-    arnoldi_block_body<BLOCK>(p.di, p.V, (long)p.ns, p.ns, L, p.H);
+    arnoldi_cluster_body<CL>(p.di, p.V, p.ns, L, p.H);
+}
+
+// The whole correction solve with the dense operator of every refining problem, one cluster each.
+template <int CL>
+__global__ void __launch_bounds__(kKrylovThreads) kb_krylov(const LsProb* P, KLayout L, KTol tol, int max_iter) {
+    const LsProb& p = P[blockIdx.z];
+    if (!p.di[DI_RACT] || p.ns == 0) return;   // uniform over the cluster
+    krylov_body<CL>(KrylovArgs{p.ns, dense_ld(p.ns), p.pc_M, p.pc_S, p.bvec, p.V, p.Z, p.xsol, L, p.H, p.di,
+                               p.small, tol, max_iter, 1, max_iter / L.m + 2});
 }
 
 // GMRES start of a correction (restart = 0: ||b||, counters, tolerance, V_0 = b / ||b||; a
 // problem that is no longer refining, or has no Krylov unknowns, only gets its stop flag) or
 // of a restart cycle (V_0 = (b - S x) / ||b - S x||).
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-kb_start(const LsProb* __restrict__ P, KLayout L, int restart, int max_iter, KTol tol) {
+template <int CL>
+__global__ void __launch_bounds__(kKrylovThreads)
+kb_start(const LsProb* P, KLayout L, int restart, int max_iter, KTol tol) {
     const LsProb& p = P[blockIdx.z];
     if (!restart) {
         if (!p.di[DI_RACT] || p.ns == 0) {
-            if (threadIdx.x == 0) p.di[DI_STOP] = 1;
-            return;
+            if (threadIdx.x == 0 && Cluster<CL>::rank() == 0) p.di[DI_STOP] = 1;
+            return;   // uniform over the cluster
         }
-        start_block_body<BLOCK>(p.ns, p.bvec, p.V, L, p.H, p.di, max_iter, tol, p.small);
+        start_cluster_body<CL>(p.ns, p.bvec, p.V, L, p.H, p.di, max_iter, tol, p.small);
     } else {
         if (!p.di[DI_CACT]) return;
-        start_block_body<BLOCK>(p.ns, p.V + 2L * p.ns, p.V, L, p.H, p.di, -1, KTol{}, nullptr);
+        start_cluster_body<CL>(p.ns, p.V + 2L * p.ns, p.V, L, p.H, p.di, -1, KTol{}, nullptr);
     }
 }
 
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) kb_backsolve(const LsProb* __restrict__ P, KLayout L) {
+__global__ void __launch_bounds__(kUpdateRows) kb_update(const LsProb* __restrict__ P, KLayout L) {
     const LsProb& p = P[blockIdx.z];
-    if (!p.di[DI_CACT]) return;
-    backsolve_update_body<BLOCK>(p.di, L, p.H, p.Z + p.ns, (long)p.ns, p.ns, p.xsol);
+    if (!p.di[DI_CACT] || (int)blockIdx.x * kUpdateRows >= p.ns) return;
+    update_body(p.di, L, p.H, p.Z + p.ns, p.ns, p.xsol);
 }
 
 // Small vector steps: x = 0 at the start of a correction; V_1 = x and the scratch column index
@@ -483,6 +490,7 @@ struct LsGroup {
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     long long k_top = 0, k_ref = 0, k_cyc = 0, k_it = 0, k_rs = 0;
     int n() const { return (int)geos.size(); }
+    bool clustered() const { return dense && krylov_fits(max_ns); }   // the corrections' Krylov solves as clusters
 
     ~LsGroup() {
         if (exec) cudaGraphExecDestroy(exec);
@@ -544,7 +552,7 @@ static void fill_prob(LsProb& q, iim_geometry g, int prec, const double* omega, 
     q.lam_y = prec == IIM_FP64 ? (const void*)g->lam_y64 : (const void*)g->lam_y32;
     q.psi_ext = g->psi_ext; q.res = g->res; q.partial = g->partial; q.small = g->small; q.V = g->V; q.H = g->H;
     q.xsol = g->xsol; q.bvec = g->bvec; q.Z = g->Z; q.tbuf = g->tbuf; q.psiT = g->psiT;
-    q.pc_inv = g->pc_aug + (q.ns);
+    q.pc_M = g->pc_M;
     q.pc_S = g->pc_S;
     if (g->col_solver == 1) {
         q.s32 = ScanTab<float>{g->sc32_delta, g->sc32_rowoff, g->sc32_par, g->sc32_lim, g->sc32_dstar,
@@ -565,6 +573,9 @@ struct LsEmit {
     bool host;   // host-driven: control kernels write *flag, the host reads it
     int* flag() const { return host ? G->d_cnt + 8 : nullptr; }
     int* cnt() const { return host ? nullptr : G->d_cnt; }
+    // the corrections' Krylov solves as one kernel; host-driven runs take the same steps one launch at a
+    // time (the same arithmetic in the same order), so that the profiler sees them
+    bool fused() const { return G->clustered() && !host; }
     dim3 grid(long x) const { return dim3((unsigned)std::max<long>(x, 1), 1, (unsigned)G->n()); }
 
     // algorithmic bytes of a launch summed over the group (the per-kernel profiler's figure)
@@ -680,14 +691,21 @@ struct LsEmit {
         return IIM_OK;
     }
 
+    iim_status start(int restart, int max_iter, KTol tol) {
+        const int cl = krylov_cluster(G->max_ns);
+        const LsProb* P = G->d_probs;
+        const size_t sm = arnoldi_smem(G->max_ns, cl);
+        return cl == 8 ? launch_cluster("ls_gmres_start", 0.0, kb_start<8>, 8, G->n(), sm, s, P, KLayout{G->m}, restart, max_iter, tol)
+                       : launch_cluster("ls_gmres_start", 0.0, kb_start<16>, 16, G->n(), sm, s, P, KLayout{G->m}, restart, max_iter, tol);
+    }
+
     iim_status matvec(int op, int gate) {
-        constexpr int W = 8;
-        const size_t sm4 = sizeof(float) * 4 * (size_t)((G->max_ns + 3) & ~3);
-        IIM_CHECK(allow_smem(kb_matvec<W>, sm4));
+        const size_t sm = dense_smem(G->max_ns);
+        IIM_CHECK(allow_smem(kb_matvec, sm));
         double bytes = 0.0;
         for (iim_geometry g : G->geos) bytes += 4.0 * (double)(g->na + g->ncirc) * (g->na + g->ncirc);
-        launch(op >= MV_S_ITER ? "ls_dense_schur_matvec" : "ls_precond_matvec", bytes, 0.0, kb_matvec<W>,
-               grid((G->max_ns + W - 1) / W), W * 32, sm4, s, (const LsProb*)G->d_probs, op, gate);
+        launch(op >= MV_S_ITER ? "ls_dense_schur_matvec" : "ls_precond_matvec", bytes, 0.0, kb_matvec, grid(dense_blocks(G->max_ns)), kDenseWarps * 32, sm, s,
+               (const LsProb*)G->d_probs, op, gate);
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -737,9 +755,16 @@ struct LsEmit {
         IIM_CHECK(cols<T>(M_RHS, G_REF));
         IIM_CHECK((rows_inv<T, INV_STORE_T>(G_REF)));
         IIM_CHECK(gather<T>(M_RHS, G_REF));
+        if (fused()) {
+            const int cl = krylov_cluster(G->max_ns);
+            const LsProb* P = G->d_probs;
+            const KTol tol{G->inner, G->kappa, G->last};
+            const size_t sm = krylov_smem(G->max_ns, G->m, cl);
+            return cl == 8 ? launch_cluster("ls_gmres_krylov", 0.0, kb_krylov<8>, 8, G->n(), sm, s, P, KLayout{G->m}, tol, G->max_iter)
+                           : launch_cluster("ls_gmres_krylov", 0.0, kb_krylov<16>, 16, G->n(), sm, s, P, KLayout{G->m}, tol, G->max_iter);
+        }
         IIM_CHECK(vec(V_ZERO_X, G_REF));
-        launch("ls_gmres_start", 0.0, 0.0, kb_start<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs, KLayout{G->m},
-               0, G->max_iter, KTol{G->inner, G->kappa, G->last});
+        IIM_CHECK(start(0, G->max_iter, KTol{G->inner, G->kappa, G->last}));
         launch("ls_cyc_begin", 0.0, 0.0, kb_cyc_begin, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(), G->max_iter,
                h_cyc, flag());
         IIM_LAUNCHED();
@@ -764,8 +789,10 @@ struct LsEmit {
             IIM_CHECK((rows_inv<T, INV_STORE_T>(G_IT)));
             IIM_CHECK(gather<T>(M_APPLY_Z, G_IT));
         }
-        launch("ls_gmres_arnoldi", 0.0, 0.0, kb_arnoldi<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs,
-               KLayout{G->m});
+        const int cl = krylov_cluster(G->max_ns);
+        const LsProb* P = G->d_probs;
+        IIM_CHECK(cl == 8 ? launch_cluster("ls_gmres_arnoldi", 0.0, kb_arnoldi<8>, 8, G->n(), arnoldi_smem(G->max_ns, 8), s, P, KLayout{G->m})
+                          : launch_cluster("ls_gmres_arnoldi", 0.0, kb_arnoldi<16>, 16, G->n(), arnoldi_smem(G->max_ns, 16), s, P, KLayout{G->m}));
         launch("ls_loop_ctl", 0.0, 0.0, kb_loop_ctl, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(), G->m + 2, h_it,
                flag(), cnt());
         IIM_LAUNCHED();
@@ -774,8 +801,9 @@ struct LsEmit {
 
     // x += sum y_j z_j, then another cycle (with the restart below) unless every problem is done
     iim_status cyc_post(cudaGraphConditionalHandle h_cyc, cudaGraphConditionalHandle h_rs) {
-        launch("ls_gmres_backsolve", 0.0, 0.0, kb_backsolve<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs,
-               KLayout{G->m});
+        IIM_CHECK(allow_smem(kb_update, update_smem(G->m)));
+        launch("ls_gmres_update", 0.0, 0.0, kb_update, grid((G->max_ns + kUpdateRows - 1) / kUpdateRows), kUpdateRows,
+               update_smem(G->m), s, (const LsProb*)G->d_probs, KLayout{G->m});
         launch("ls_cyc_ctl", 0.0, 0.0, kb_cyc_ctl, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(),
                G->max_iter / G->m + 2, h_cyc, h_rs, flag(), cnt());
         IIM_LAUNCHED();
@@ -795,8 +823,7 @@ struct LsEmit {
             IIM_CHECK(gather<T>(M_APPLY_VTMP, G_CYC));
         }
         IIM_CHECK(vec(V_RESTART_RES, G_CYC));
-        launch("ls_gmres_start", 0.0, 0.0, kb_start<256>, grid(1), 256, 0, s, (const LsProb*)G->d_probs, KLayout{G->m},
-               1, 0, KTol{});
+        IIM_CHECK(start(1, 0, KTol{}));
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -903,29 +930,31 @@ static iim_status build_group_graph(LsGroup* G) {
     piece(top_seg, [&]() { return E.top_pre(h_ref); });
     cond(top_seg, h_ref, cudaGraphCondTypeWhile, &ref_body);
     CapSeg ref_seg{G->cap_stream, ref_body, {}};
-    handle(ref_body, &h_cyc);
+    if (!G->clustered()) handle(ref_body, &h_cyc);
     piece(ref_seg, [&]() { return E.ref_pre<T>(h_cyc); });
-    cond(ref_seg, h_cyc, cudaGraphCondTypeWhile, &cyc_body);
-    CapSeg cyc_seg{G->cap_stream, cyc_body, {}};
-    handle(cyc_body, &h_it);
-    handle(cyc_body, &h_rs);
-    piece(cyc_seg, [&]() { return E.cyc_pre(h_it); });
-    cond(cyc_seg, h_it, cudaGraphCondTypeWhile, &it_body);
-    CapSeg it_seg{G->cap_stream, it_body, {}};
-    piece(it_seg, [&]() { return E.iteration<T>(h_it); });
-    piece(cyc_seg, [&]() { return E.cyc_post(h_cyc, h_rs); });
-    cond(cyc_seg, h_rs, cudaGraphCondTypeIf, &rs_body);
-    CapSeg rs_seg{G->cap_stream, rs_body, {}};
-    piece(rs_seg, [&]() { return E.restart<T>(); });
+    if (!G->clustered()) {
+        cond(ref_seg, h_cyc, cudaGraphCondTypeWhile, &cyc_body);
+        CapSeg cyc_seg{G->cap_stream, cyc_body, {}};
+        handle(cyc_body, &h_it);
+        handle(cyc_body, &h_rs);
+        piece(cyc_seg, [&]() { return E.cyc_pre(h_it); });
+        cond(cyc_seg, h_it, cudaGraphCondTypeWhile, &it_body);
+        CapSeg it_seg{G->cap_stream, it_body, {}};
+        piece(it_seg, [&]() { return E.iteration<T>(h_it); });
+        piece(cyc_seg, [&]() { return E.cyc_post(h_cyc, h_rs); });
+        cond(cyc_seg, h_rs, cudaGraphCondTypeIf, &rs_body);
+        CapSeg rs_seg{G->cap_stream, rs_body, {}};
+        piece(rs_seg, [&]() { return E.restart<T>(); });
+    }
     piece(ref_seg, [&]() { return E.ref_post<T>(h_ref); });
     piece(top_seg, [&]() { return E.top_post(); });
     set_capture(false);
     if (st == IIM_OK && ce == cudaSuccess) {
         G->k_top = kernel_nodes(top);
         G->k_ref = kernel_nodes(ref_body);
-        G->k_cyc = kernel_nodes(cyc_body);
-        G->k_it = kernel_nodes(it_body);
-        G->k_rs = kernel_nodes(rs_body);
+        G->k_cyc = cyc_body ? kernel_nodes(cyc_body) : 0;
+        G->k_it = it_body ? kernel_nodes(it_body) : 0;
+        G->k_rs = rs_body ? kernel_nodes(rs_body) : 0;
         ce = cudaGraphInstantiate(&G->exec, top, 0);
     }
     cudaGraphDestroy(top);

@@ -12,6 +12,7 @@
 
 #include "common.cuh"
 #include "iim_ops.cuh"
+#include "krylov.cuh"
 
 namespace iim {
 
@@ -209,59 +210,11 @@ __global__ void k_set_identity_aug(float* __restrict__ A, int n) {
     A[i * ld + n + j] = (i == j) ? 1.f : 0.f;
 }
 
-// out = M v, M row-major n x n FP32 with leading dimension ldm (even);
-// one warp per row.  v = vbase + (jidx ? *jidx : 0) * vstride is staged in shared memory as
-// FP32; each lane reads the row in 8-byte pairs (after one odd leading element when the row
-// starts 4 bytes off an 8-byte boundary) into four independent accumulators.
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-k_dense_matvec(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
+__global__ void __launch_bounds__(kDenseWarps * 32)
+k_dense_matvec(int n, const float* __restrict__ M, long ld, const double* __restrict__ vbase,
                const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
                const int* __restrict__ stop) {
-    if (stop && *stop) return;
-    if (ostride) out += (long)(*jidx + 1) * ostride;
-    extern __shared__ float s_v[];
-    const double* v = jidx ? vbase + (long)(*jidx) * vstride : vbase;
-    for (int j = threadIdx.x; j < n; j += WARPS * 32) s_v[j] = (float)v[j];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    for (int row = blockIdx.x * WARPS + (threadIdx.x >> 5); row < n; row += gridDim.x * WARPS) {
-        const float* r = M + (long)row * ldm;
-        const int head = (reinterpret_cast<uintptr_t>(r) & 7) ? 1 : 0;
-        float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-        if (head && lane == 0) a0 = r[0] * s_v[0];
-        const float2* r2 = reinterpret_cast<const float2*>(r + head);
-        const float* sv = s_v + head;
-        const int np = (n - head) >> 1;
-        int q = lane;
-        for (; q + 96 < np; q += 128) {
-            const float2 x0 = r2[q], x1 = r2[q + 32], x2 = r2[q + 64], x3 = r2[q + 96];
-            a0 = fmaf(x0.x, sv[2 * q], fmaf(x0.y, sv[2 * q + 1], a0));
-            a1 = fmaf(x1.x, sv[2 * q + 64], fmaf(x1.y, sv[2 * q + 65], a1));
-            a2 = fmaf(x2.x, sv[2 * q + 128], fmaf(x2.y, sv[2 * q + 129], a2));
-            a3 = fmaf(x3.x, sv[2 * q + 192], fmaf(x3.y, sv[2 * q + 193], a3));
-        }
-        for (; q < np; q += 32) {
-            const float2 x0 = r2[q];
-            a0 = fmaf(x0.x, sv[2 * q], fmaf(x0.y, sv[2 * q + 1], a0));
-        }
-        if (((n - head) & 1) && lane == 31) a1 = fmaf(r[n - 1], s_v[n - 1], a1);
-        float acc = (a0 + a1) + (a2 + a3);
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0) out[row] = (double)acc;
-    }
-}
-
-// The same product with 16-byte row loads: a row starting h = 0..3 floats before a 16-byte
-// boundary is read as h leading floats, then float4s (eight in flight per lane), then the
-// remainder.  v is staged four times in shared memory, copy h shifted by h elements, so that
-// the float4 of the row always meets an aligned float4 of v.
-template <int WARPS>
-__global__ void __launch_bounds__(WARPS * 32)
-k_dense_matvec4(int n, const float* __restrict__ M, long ldm, const double* __restrict__ vbase,
-                const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
-                const int* __restrict__ stop) {
-    dense_matvec4_body<WARPS>(n, M, ldm, vbase, jidx, vstride, out, ostride, stop);
+    dense_matvec_body(n, M, ld, vbase, jidx, vstride, out, ostride, stop);
 }
 
 iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_t s) {
@@ -302,23 +255,11 @@ iim_status gj_invert_aug(float* A, int n, float* scratch, int* info, cudaStream_
 
 bool dense_matvec_fits(int n) { return sizeof(float) * 4 * (size_t)((n + 3) & ~3) <= 200 * 1024; }
 
-iim_status dense_matvec(int n, const float* M, long ldm, const double* v, const int* jidx, long vstride, double* out,
+iim_status dense_matvec(int n, const float* M, const double* v, const int* jidx, long vstride, double* out,
                         long ostride, const int* stop, cudaStream_t s) {
-    constexpr int W = 8;
-    const size_t sm4 = sizeof(float) * 4 * (size_t)((n + 3) & ~3);
-    if (sm4 <= 200 * 1024) {
-        // the limit only ever grows (allow_smem): solves of different sizes on other threads
-        // must not lower it under this launch
-        IIM_CHECK(allow_smem(k_dense_matvec4<W>, sm4));
-        launch("precond_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec4<W>, (n + W - 1) / W, W * 32, sm4, s,
-               n, M, ldm, v, jidx, vstride, out, ostride, stop);
-        IIM_LAUNCHED();
-        return IIM_OK;
-    }
-    const size_t sm = sizeof(float) * (size_t)n;
-    IIM_CHECK(allow_smem(k_dense_matvec<W>, sm));
-    launch("precond_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec<W>, (n + W - 1) / W, W * 32, sm, s, n, M,
-           ldm, v, jidx, vstride, out, ostride, stop);
+    IIM_CHECK(allow_smem(k_dense_matvec, dense_smem(n)));
+    launch("dense_matvec", (double)n * n * 4.0, 2.0 * n * n, k_dense_matvec, dense_blocks(n), kDenseWarps * 32,
+           dense_smem(n), s, n, M, dense_ld(n), v, jidx, vstride, out, ostride, stop);
     IIM_LAUNCHED();
     return IIM_OK;
 }

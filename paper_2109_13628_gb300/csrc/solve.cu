@@ -27,6 +27,7 @@
 #include "common.cuh"
 #include "dst.cuh"
 #include "iim_ops.cuh"
+#include "krylov.cuh"
 #include "sine.cuh"
 
 namespace iim {
@@ -505,42 +506,6 @@ __global__ void k_velocity(int NX, int NY, double inv2h, const double* __restric
 
 // ------------------------------------------------------------------------- GMRES kernels
 
-// h[i] = <V_i, V_{j+1}> for i <= j (one block per i)
-template <int BLOCK>
-__global__ void k_dots(const int* __restrict__ di, const double* __restrict__ V, long ld, int ns, double* __restrict__ out) {
-    if (di[DI_STOP]) return;
-    const int j = di[DI_J];
-    const int i = blockIdx.x;
-    if (i > j) return;
-    const double* vi = V + (long)i * ld;
-    const double* w = V + (long)(j + 1) * ld;
-    double acc = 0.0;
-    for (int e = threadIdx.x; e < ns; e += BLOCK) acc += vi[e] * w[e];
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) out[i] = acc;
-}
-
-// V_{j+1} -= sum_{i<=j} coef[i] V_i; with `partial`, per-block sums of squares of the result.
-template <int BLOCK>
-__global__ void k_update(const int* __restrict__ di, double* __restrict__ V, long ld, const double* __restrict__ coef,
-                         int ns, double* __restrict__ partial) {
-    if (di[DI_STOP]) return;
-    const int j = di[DI_J];
-    const int e = blockIdx.x * BLOCK + threadIdx.x;
-    double* w = V + (long)(j + 1) * ld;
-    double val = 0.0;
-    if (e < ns) {
-        double s = 0.0;
-        for (int i = 0; i <= j; ++i) s += coef[i] * V[(long)i * ld + e];
-        val = w[e] - s;
-        w[e] = val;
-    }
-    if (partial) {
-        const double sq = block_sum<BLOCK>(val * val);
-        if (threadIdx.x == 0) partial[blockIdx.x] = sq;
-    }
-}
-
 template <int BLOCK>
 __global__ void k_sumsq(const double* __restrict__ w, int ns, double* __restrict__ partial) {
     double acc = 0.0;
@@ -549,35 +514,6 @@ __global__ void k_sumsq(const double* __restrict__ w, int ns, double* __restrict
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
-
-// Arnoldi step finish after k_update: sums the per-block squares, then arnoldi_finish.
-__global__ void k_arnoldi_tail(int* __restrict__ di, KLayout L, int nparts, const double* __restrict__ partial,
-                               double* __restrict__ K) {
-    if (di[DI_STOP]) return;
-    const int lane = threadIdx.x;
-    double s = 0.0;
-    for (int b = lane; b < nparts; b += 32) s += partial[b];
-    s = warp_sum(s);
-    if (lane == 0) arnoldi_finish(di, L, K, s);
-}
-
-// The whole Arnoldi step in one block, for short Krylov bases (the preconditioned iteration
-// converges in a few steps): two classical Gram-Schmidt passes against V_0..V_j, the norm,
-// arnoldi_finish, and the scaling of V_{j+1} -- one launch instead of six.  Each thread owns
-// the same elements in every pass; the j+1 inner products of a pass are reduced together
-// (warp sums into part[i][warp], then one thread per i), so a pass synchronises twice.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_arnoldi_block(int* __restrict__ di, double* __restrict__ V, long ld, int ns, KLayout L, double* __restrict__ K) {
-    arnoldi_block_body<BLOCK>(di, V, ld, ns, L, K);
-}
-
-// V_j *= 1 / ||V_j|| (j already advanced by the tail)
-__global__ void k_scale(const int* __restrict__ di, double* __restrict__ V, long ld, int ns, const double* __restrict__ sc) {
-    if (di[DI_STOP]) return;
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e < ns) V[(long)di[DI_J] * ld + e] *= *sc;
-}
 
 // V_0 = r / ||r||, g = (beta, 0, ...), j = 0, stop unless there is work left
 __global__ void k_start_cycle(int ns, const double* __restrict__ r, double* __restrict__ v0, KLayout L, double* __restrict__ K,
@@ -600,53 +536,11 @@ __global__ void k_start_cycle(int ns, const double* __restrict__ r, double* __re
     }
 }
 
-// One block: beta = ||r||, V_0 = r / beta and the GMRES start state (k_start_cycle's work,
-// with the norm reduced inside the block instead of by k_sumsq's blocks).  With init_maxit >= 0
-// it first does what the norm / k_gmres_init launches do at the start of a correction: ||r||^2
-// stored, the counters reset, the tolerance set (KTol).  Five launches become one.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_start_block(int ns, const double* __restrict__ r, double* __restrict__ v0, KLayout L, double* __restrict__ K,
-              int* __restrict__ di, int init_maxit, KTol tol, double* __restrict__ small) {
-    start_block_body<BLOCK>(ns, r, v0, L, K, di, init_maxit, tol, small);
-}
-
-// y = H^{-1} g over the first k = j columns (one warp)
-__global__ void k_backsolve(const int* __restrict__ di, KLayout L, double* __restrict__ K) {
-    const int lane = threadIdx.x;
-    const int k = di[DI_J];
-    const double* H = K + L.H();
-    const int ldh = L.m + 1;
-    const double* gv = K + L.gv();
-    double* y = K + L.y();
-    for (int i = k - 1; i >= 0; --i) {
-        double s = 0.0;
-        for (int l = i + 1 + lane; l < k; l += 32) s += H[(long)l * ldh + i] * y[l];
-        s = warp_sum(s);
-        if (lane == 0) {
-            const double d = H[(long)i * ldh + i];
-            y[i] = d != 0.0 ? (gv[i] - s) / d : 0.0;
-        }
-        __syncwarp();
-    }
-}
-
-// k_backsolve and the update in one block: warp 0 solves for y, then x += Z y over the block.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_backsolve_update(const int* __restrict__ di, KLayout L, double* __restrict__ K, const double* __restrict__ Z,
-                   long ld, int ns, double* __restrict__ x) {
-    backsolve_update_body<BLOCK>(di, L, K, Z, ld, ns, x);
-}
-
-__global__ void k_xupdate(const int* __restrict__ di, const double* __restrict__ V, long ld, const double* __restrict__ y,
-                          int ns, double* __restrict__ x) {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e >= ns) return;
-    const int k = di[DI_J];
-    double s = 0.0;
-    for (int i = 0; i < k; ++i) s += y[i] * V[(long)i * ld + e];
-    x[e] += s;
+// End of a GMRES cycle (krylov.cuh).
+__global__ void __launch_bounds__(kUpdateRows)
+k_update(const int* __restrict__ di, KLayout L, const double* __restrict__ K, const double* __restrict__ B, int ns,
+         double* __restrict__ x) {
+    update_body(di, L, K, B, ns, x);
 }
 
 __global__ void k_axpby(int n, double a, const double* __restrict__ x, double b, const double* __restrict__ y,
@@ -985,11 +879,20 @@ struct Solver {
         if (g->pc_ready) return IIM_OK;
         const int n = ns;
         const long ld = ns;
-        if (!g->pc_aug) {
-            IIM_TRY(cudaMalloc(&g->pc_aug, sizeof(float) * 2 * (size_t)n * n));
-            IIM_TRY(cudaMalloc(&g->pc_f, sizeof(float) * gj_scratch_floats(n)));
+        const size_t mbytes = sizeof(float) * (size_t)dense_ld(n) * n;
+        if (!g->pc_M) {
+            IIM_TRY(cudaMalloc(&g->pc_M, mbytes));
+            IIM_TRY(cudaMalloc(&g->pc_S, mbytes));
             IIM_TRY(cudaMalloc(&g->pc_info, sizeof(int)));
         }
+        // [S | I] and the elimination's scratch, for the set-up only
+        struct Scratch {
+            float* p = nullptr;
+            ~Scratch() { cudaFree(p); }
+        } scratch;
+        const size_t aug_floats = (2 * (size_t)n * n + 63) & ~(size_t)63;   // the scratch is read in 16-byte vectors
+        IIM_TRY(cudaMalloc(&scratch.p, sizeof(float) * (aug_floats + gj_scratch_floats(n))));
+        float* aug = scratch.p;
         IIM_TRY(cudaEventRecord(g->ev0, s));
         // gamma columns j < |A|, K at a time: unit row transforms, column pass, inverse rows of
         // the gathered band, gather straight into the matrix (one launch each per batch); in free
@@ -1020,7 +923,7 @@ struct Solver {
                 if (bs == IIM_OK)
                     launch("pc_gather", 0.0, 0.0, k_gather_unit<float, 128>, dim3(nga + 1, kb), 128, 0, s, g->na, nga,
                            g->ncirc, (const int*)g->gop_ptr, (const int*)g->gop_idx, (const double*)g->gop_w,
-                           (const float*)pt, fstride, j0, (const int*)g->aff_body, (const int*)g->body_circ, g->pc_aug,
+                           (const float*)pt, fstride, j0, (const int*)g->aff_body, (const int*)g->body_circ, aug,
                            2L * n);
                 if (bs == IIM_OK && cudaGetLastError() != cudaSuccess) bs = IIM_ERR_CUDA;
             }
@@ -1035,14 +938,19 @@ struct Solver {
         for (int j = g->outer ? 0 : g->na; j < n; ++j) {
             launch("pc_unit", 0.0, 0.0, k_unit_vector, eb, 256, 0, s, n, j, g->V);
             IIM_CHECK(apply_at<float>(DI_TMPJ, nullptr));
-            launch("pc_column", 0.0, 0.0, k_store_column, eb, 256, 0, s, n, j, (const double*)(g->V + ld), g->pc_aug);
+            launch("pc_column", 0.0, 0.0, k_store_column, eb, 256, 0, s, n, j, (const double*)(g->V + ld), aug);
             IIM_LAUNCHED();
         }
-        // keep S (the left half) for the dense inner operator before it is reduced to I
-        if (!g->pc_S) IIM_TRY(cudaMalloc(&g->pc_S, sizeof(float) * (size_t)n * n));
-        IIM_TRY(cudaMemcpy2DAsync(g->pc_S, sizeof(float) * (size_t)n, g->pc_aug, sizeof(float) * 2 * (size_t)n,
-                                  sizeof(float) * (size_t)n, (size_t)n, cudaMemcpyDeviceToDevice, s));
-        IIM_CHECK(gj_invert_aug(g->pc_aug, n, g->pc_f, g->pc_info, s));
+        // S (the left half) is kept before it is reduced to I, then its inverse, both with padded rows
+        auto keep = [&](float* to, const float* from) -> iim_status {
+            IIM_TRY(cudaMemsetAsync(to, 0, mbytes, s));
+            IIM_TRY(cudaMemcpy2DAsync(to, sizeof(float) * (size_t)dense_ld(n), from, sizeof(float) * 2 * (size_t)n,
+                                      sizeof(float) * (size_t)n, (size_t)n, cudaMemcpyDeviceToDevice, s));
+            return IIM_OK;
+        };
+        IIM_CHECK(keep(g->pc_S, aug));
+        IIM_CHECK(gj_invert_aug(aug, n, aug + aug_floats, g->pc_info, s));
+        IIM_CHECK(keep(g->pc_M, aug + n));
         int info = 0;
         IIM_TRY(cudaMemcpyAsync(&info, g->pc_info, sizeof(int), cudaMemcpyDeviceToHost, s));
         IIM_TRY(cudaEventRecord(g->ev1, s));
@@ -1061,24 +969,40 @@ struct Solver {
         return IIM_OK;
     }
 
-    // ---- one Arnoldi step after the operator application
-    iim_status ortho_iter() {
-        const long ld = ns;
-        double* K = g->H;
-        if (precond) {
-            launch("gmres_arnoldi", 0.0, 0.0, k_arnoldi_block<256>, 1, 256, 0, s, di(), g->V, ld, ns, L, K);
-            IIM_LAUNCHED();
-            return IIM_OK;
-        }
-        const int eb = (ns + 255) / 256;
-        launch("gmres_dots", 0.0, 0.0, k_dots<256>, m, 256, 0, s, di(), g->V, ld, ns, K + L.hc1());
-        launch("gmres_update", 0.0, 0.0, k_update<256>, eb, 256, 0, s, di(), g->V, ld, K + L.hc1(), ns, nullptr);
-        launch("gmres_dots", 0.0, 0.0, k_dots<256>, m, 256, 0, s, di(), g->V, ld, ns, K + L.hc2());
-        launch("gmres_update", 0.0, 0.0, k_update<256>, eb, 256, 0, s, di(), g->V, ld, K + L.hc2(), ns, g->partial);
-        launch("gmres_tail", 0.0, 0.0, k_arnoldi_tail, 1, 32, 0, s, di(), L, eb, g->partial, K);
-        launch("gmres_scale", 0.0, 0.0, k_scale, eb, 256, 0, s, di(), g->V, ld, ns, K + L.scal() + SC_INV);
+    // ---- start of a correction (init_maxit >= 0) or a restart cycle from the residual r
+    iim_status start(const double* r, int init_maxit, KTol tol) {
+        const int cl = krylov_cluster(ns);
+        return cl == 8 ? launch_cluster("gmres_start", 0.0, k_start<8>, 8, 1, arnoldi_smem(ns, 8), s, ns, r, g->V, L, g->H, di(),
+                                        init_maxit, tol, g->small)
+                       : launch_cluster("gmres_start", 0.0, k_start<16>, 16, 1, arnoldi_smem(ns, 16), s, ns, r, g->V, L, g->H,
+                                        di(), init_maxit, tol, g->small);
+    }
+
+    // ---- end of a cycle: x += sum y_j z_j (V_j without preconditioner)
+    iim_status update() {
+        IIM_CHECK(allow_smem(k_update, update_smem(m)));
+        launch("gmres_update", 0.0, 0.0, k_update, (ns + kUpdateRows - 1) / kUpdateRows, kUpdateRows, update_smem(m), s,
+               (const int*)di(), L, (const double*)g->H, (const double*)(precond ? g->Z + ns : g->V), ns, g->xsol);
         IIM_LAUNCHED();
         return IIM_OK;
+    }
+
+    // ---- one Arnoldi step after the operator application
+    iim_status ortho_iter() {
+        const int cl = krylov_cluster(ns);
+        return cl == 8 ? launch_cluster("gmres_arnoldi", 0.0, k_arnoldi<8>, 8, 1, arnoldi_smem(ns, 8), s, di(), g->V, ns, L, g->H)
+                       : launch_cluster("gmres_arnoldi", 0.0, k_arnoldi<16>, 16, 1, arnoldi_smem(ns, 16), s, di(), g->V, ns, L, g->H);
+    }
+
+    // ---- the whole correction solve with the dense operator as one cluster (krylov.cuh); `its`: the
+    // iterations so far are in di[DI_ITS] (the whole-solve graph), else max_it is what is left
+    bool clustered() const { return dense_op && krylov_fits(ns); }
+    iim_status krylov(double tol, int max_it, bool its) {
+        const int cl = krylov_cluster(ns);
+        const KrylovArgs a{ns, dense_ld(ns), g->pc_M, g->pc_S, g->bvec, g->V, g->Z, g->xsol, L, g->H, di(), g->small,
+                           KTol{tol, kappa, last}, max_it, its ? 1 : 0, max_it / m + 2};
+        return cl == 8 ? launch_cluster("gmres_krylov", 0.0, k_krylov<8>, 8, 1, krylov_smem(ns, m, 8), s, a)
+                       : launch_cluster("gmres_krylov", 0.0, k_krylov<16>, 16, 1, krylov_smem(ns, m, 16), s, a);
     }
 
     template <typename T>
@@ -1087,9 +1011,9 @@ struct Solver {
             // flexible right preconditioning: z_j = M v_j kept, v_{j+1} = S z_j, so that x = sum y_j z_j
             // satisfies S x = sum y_j S z_j as computed.  (x = M (V y) would round M's FP32 product anew, an
             // error of cond(S) 2^-24 ||b|| that no further iteration removes.)
-            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->V, di() + DI_J, (long)ns, g->Z, (long)ns, di() + DI_STOP, s));
+            IIM_CHECK(dense_matvec(ns, g->pc_M, g->V, di() + DI_J, (long)ns, g->Z, (long)ns, di() + DI_STOP, s));
             if (dense_op)
-                IIM_CHECK(dense_matvec(ns, g->pc_S, (long)ns, g->Z + ns, di() + DI_J, (long)ns, g->V, (long)ns, di() + DI_STOP, s));
+                IIM_CHECK(dense_matvec(ns, g->pc_S, g->Z + ns, di() + DI_J, (long)ns, g->V, (long)ns, di() + DI_STOP, s));
             else
                 IIM_CHECK(apply_vec<T>(VecArg{g->Z, di() + DI_J, 1, (long)ns}, di() + DI_J, di() + DI_STOP));
         } else {
@@ -1229,12 +1153,17 @@ struct Solver {
         double* x = g->xsol;
         const long ld = ns_;
         const int eb = (ns_ + 255) / 256;
+        if (clustered() && !x0) {
+            IIM_CHECK(krylov(tol, max_it, false));
+            int st[8] = {0};
+            IIM_CHECK(read_state(st));
+            return gmres_done(st);
+        }
         IIM_TRY(cudaMemsetAsync(x, 0, (size_t)ns_ * sizeof(double), s));
         bool started = false;
         if (!x0) {
-            // ||b||, counters, tolerance and V_0 = b / ||b|| in one block
-            launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns_, (const double*)g->bvec, V, L, K,
-                   di(), max_it, KTol{tol, kappa, last}, g->small);
+            // ||b||, counters, tolerance and V_0 = b / ||b||
+            IIM_CHECK(start(g->bvec, max_it, KTol{tol, kappa, last}));
             started = true;
         } else {
             launch("gmres_sumsq", 0.0, 0.0, k_sumsq<256>, kNormBlocks, 256, 0, s, g->bvec, ns_, g->partial);
@@ -1297,22 +1226,19 @@ struct Solver {
                     IIM_CHECK(read_state(st));
                 }
             }
-            if (precond) {
-                // x += sum y_j z_j
-                launch("gmres_backsolve", 0.0, 0.0, k_backsolve_update<256>, 1, 256, 0, s, (const int*)di(), L, K,
-                       (const double*)(g->Z + ns_), ld, ns_, x);
-            } else {
-                launch("gmres_backsolve", 0.0, 0.0, k_backsolve, 1, 32, 0, s, di(), L, K);
-                launch("gmres_xupdate", 0.0, 0.0, k_xupdate, eb, 256, 0, s, di(), V, ld, K + L.y(), ns_, x);
-            }
-            IIM_LAUNCHED();
+            IIM_CHECK(update());
             if (st[DI_CONV] || st[DI_IT] >= max_it) break;
             // restart: V_1 = x, V_2 = S V_1, V_0 = (b - V_2) / ||b - V_2||
             IIM_TRY(cudaMemcpyAsync(V + ld, x, (size_t)ns_ * sizeof(double), cudaMemcpyDeviceToDevice, s));
             IIM_CHECK(restart_residual<T>());
             IIM_CHECK(read_state(st));
         }
-        IIM_TRY(cudaMemcpyAsync(g->h_pinned + 12, K + L.scal(), 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
+        return gmres_done(st);
+    }
+
+    // iterations and the relative residual of a finished Krylov solve
+    iim_status gmres_done(const int* st) {
+        IIM_TRY(cudaMemcpyAsync(g->h_pinned + 12, g->H + L.scal(), 4 * sizeof(double), cudaMemcpyDeviceToHost, s));
         IIM_TRY(cudaMemcpyAsync(g->h_pinned + 25, g->small + SM_NORM, sizeof(double), cudaMemcpyDeviceToHost, s));
         IIM_TRY(cudaStreamSynchronize(s));
         iters += st[DI_IT];
@@ -1331,15 +1257,14 @@ struct Solver {
         const int eb = (ns + 255) / 256;
         launch("set_tmpj", 0.0, 0.0, k_set_int, 1, 1, 0, s, di() + DI_TMPJ, 1);
         if (dense_op)
-            IIM_CHECK(dense_matvec(ns, g->pc_S, (long)ns, V, di() + DI_TMPJ, ld, V, ld, nullptr, s));
+            IIM_CHECK(dense_matvec(ns, g->pc_S, V, di() + DI_TMPJ, ld, V, ld, nullptr, s));
         else
             IIM_CHECK(apply_at<T>(DI_TMPJ, nullptr));
         if (seed)
             launch("seed_scale", 0.0, 0.0, k_seed_scale<1024>, 1, 1024, 0, s, ns, (const double*)g->bvec, V + 2 * ld,
                    g->xsol, g->small + SM_SEED);
         launch("gmres_axpby", 0.0, 0.0, k_axpby, eb, 256, 0, s, ns, 1.0, g->bvec, -1.0, V + 2 * ld, V + 2 * ld);
-        launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns, (const double*)(V + 2 * ld), V, L, K,
-               di(), -1, KTol{}, (double*)nullptr);
+        IIM_CHECK(start(V + 2 * ld, -1, KTol{}));
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -1350,7 +1275,7 @@ struct Solver {
         IIM_CHECK(rhs<T>());
         if (direct) {
             // x = M b with the dense inverse of the Schur matrix: no Krylov iterations
-            IIM_CHECK(dense_matvec(ns, g->pc_aug + ns, 2L * ns, g->bvec, nullptr, 0, g->xsol, 0L, nullptr, s));
+            IIM_CHECK(dense_matvec(ns, g->pc_M, g->bvec, nullptr, 0, g->xsol, 0L, nullptr, s));
         } else {
             IIM_CHECK(gmres<T>(tol, max_it, x0));
         }
@@ -1413,13 +1338,17 @@ struct Solver {
         });
         cond(top_seg, h_ref, cudaGraphCondTypeWhile, &ref_body);
         CapSeg ref_seg{s, ref_body, {}};
-        if (ns_ > 0) {
+        if (ns_ > 0 && clustered()) {
+            piece(ref_seg, [&]() -> iim_status {
+                IIM_CHECK(rhs<T>());
+                return krylov(inner, o.max_iter, true);
+            });
+        } else if (ns_ > 0) {
             handle(ref_body, &h_cyc);
             piece(ref_seg, [&]() -> iim_status {
                 IIM_CHECK(rhs<T>());
                 IIM_TRY(cudaMemsetAsync(x, 0, (size_t)ns_ * sizeof(double), s));
-                launch("gmres_start", 0.0, 0.0, k_start_block<256>, 1, 256, 0, s, ns_, (const double*)g->bvec, g->V, L,
-                       K, di(), o.max_iter, KTol{inner, kappa, last}, g->small);
+                IIM_CHECK(start(g->bvec, o.max_iter, KTol{inner, kappa, last}));
                 launch("cyc_begin", 0.0, 0.0, k_cyc_begin, 1, 1, 0, s, h_cyc, di(), o.max_iter);
                 IIM_LAUNCHED();
                 return IIM_OK;
@@ -1442,13 +1371,7 @@ struct Solver {
                 return IIM_OK;
             });
             piece(cyc_seg, [&]() -> iim_status {
-                if (precond) {
-                    launch("gmres_backsolve", 0.0, 0.0, k_backsolve_update<256>, 1, 256, 0, s, (const int*)di(), L, K,
-                           (const double*)(g->Z + ns_), ld, ns_, x);
-                } else {
-                    launch("gmres_backsolve", 0.0, 0.0, k_backsolve, 1, 32, 0, s, di(), L, K);
-                    launch("gmres_xupdate", 0.0, 0.0, k_xupdate, eb, 256, 0, s, di(), g->V, ld, K + L.y(), ns_, x);
-                }
+                IIM_CHECK(update());
                 launch("cyc_ctl", 0.0, 0.0, k_cyc_ctl, 1, 1, 0, s, h_cyc, h_rs, di(), o.max_iter / m + 2);
                 IIM_LAUNCHED();
                 return IIM_OK;
@@ -1548,24 +1471,25 @@ struct Solver {
 static iim_status ensure_krylov(iim_geometry g, int m, bool pc) {
     const int ns = g->na + g->ncirc;
     if (g->V && g->krylov_m >= m) {
-        if (pc && !g->Z) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(g->krylov_m + 1) * std::max(ns, 1)));
+        if (pc && !g->Z) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(std::max(g->krylov_m, 2) + 1) * std::max(ns, 1)));
         return IIM_OK;
     }
+    const int cols = std::max(m, 2) + 1;   // a restart uses columns 0 to 2
     cudaFree(g->Z);
     g->Z = nullptr;
-    if (pc) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(m + 1) * std::max(ns, 1)));
+    if (pc) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)cols * std::max(ns, 1)));
     cudaFree(g->V); cudaFree(g->H); cudaFree(g->xsol); cudaFree(g->bvec); cudaFree(g->x0g);
     g->V = g->H = g->xsol = g->bvec = g->x0g = nullptr;
     KLayout L{m};
     IIM_TRY(cudaMalloc(&g->x0g, sizeof(double) * (size_t)std::max(ns, 1)));
-    IIM_TRY(cudaMalloc(&g->V, sizeof(double) * (size_t)(m + 1) * std::max(ns, 1)));
+    IIM_TRY(cudaMalloc(&g->V, sizeof(double) * (size_t)cols * std::max(ns, 1)));
     IIM_TRY(cudaMalloc(&g->H, sizeof(double) * (size_t)L.total()));
     IIM_TRY(cudaMalloc(&g->xsol, sizeof(double) * (size_t)std::max(ns, 1)));
     IIM_TRY(cudaMalloc(&g->bvec, sizeof(double) * (size_t)std::max(ns, 1)));
     // zero-filled: the solve graph's control kernels read the scalar slots of H also in solves
     // that never run a Krylov iteration (no affected points), and must not see stale memory
     IIM_TRY(cudaMemset(g->x0g, 0, sizeof(double) * (size_t)std::max(ns, 1)));
-    IIM_TRY(cudaMemset(g->V, 0, sizeof(double) * (size_t)(m + 1) * std::max(ns, 1)));
+    IIM_TRY(cudaMemset(g->V, 0, sizeof(double) * (size_t)cols * std::max(ns, 1)));
     IIM_TRY(cudaMemset(g->H, 0, sizeof(double) * (size_t)L.total()));
     IIM_TRY(cudaMemset(g->xsol, 0, sizeof(double) * (size_t)std::max(ns, 1)));
     IIM_TRY(cudaMemset(g->bvec, 0, sizeof(double) * (size_t)std::max(ns, 1)));
