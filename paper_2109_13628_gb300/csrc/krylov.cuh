@@ -11,7 +11,8 @@
 //     ARNOLDI_TIME
 //   * k_krylov: the whole correction solve with the dense operator (iim_opts.precond 3): start, all
 //     iterations z_j = M v_j, v_{j+1} = S z_j, Arnoldi step, restarts, x = sum y_j z_j.  The matrices
-//     come from L2 at the rate of CL SMs, so it is used up to kKrylovRows unknowns; beyond, the products
+//     come from L2 at the rate of CL SMs, so it is used up to kKrylovRows unknowns; basis and z_j stay in
+//     shared memory (a global store before a cluster barrier would put its latency into it).  Beyond, the products
 //     take the whole GPU (k_dense_matvec) between k_arnoldi launches.  Both forms do the same arithmetic in
 //     the same order.
 //     KRYLOV_TIME
@@ -47,11 +48,12 @@ struct Cluster {
     static __device__ __forceinline__ P* at(P* p, int r) { return cooperative_groups::this_cluster().map_shared_rank(p, r); }
 };
 
-// Shared scratch of the steps: partial sums [3][CL][64], coefficients, rotations.
+// Shared scratch of the steps: partial sums of the two passes and of a norm, coefficients (entry j + 1 of
+// the second pass: the squared norm before it), rotations.
 template <int CL>
 struct KrylovShared {
-    double part[3][CL][64];
-    double h[64], hc[64], cs[64], sn[64];
+    double part[3][CL][65];
+    double h[65], hc[64], cs[64], sn[64];
     double sq, nrm, inv;     // the last squared norm, the norm and its reciprocal (0 for a zero norm)
     double resid;
 };
@@ -129,38 +131,52 @@ __device__ __forceinline__ void start_cluster_body(int ns, const double* __restr
     }
 }
 
-// Two classical Gram-Schmidt passes of w (this block's rows w[0..nr), global rows r0 ..) against V_0..V_j
-// and the norm of the result (s.nrm, s.inv); s.hc[i] = the two passes' coefficients summed.  Ends
-// synchronised.
+// Two classical Gram-Schmidt passes of w (this block's rows w[0..nr)) against V_0..V_j (this block's rows,
+// column i at V + i ldv) and the norm of the result (s.nrm, s.inv); s.hc[i] = the two passes'
+// coefficients summed.  The norm comes with the second pass's products, ||w||^2 less the squares of its
+// coefficients (V is orthonormal), which saves an exchange; where they are not small against ||w||^2 the
+// norm is taken of the result itself.  Ends synchronised.
 template <int CL, int NT>
-__device__ __forceinline__ void orthogonalise(const double* V, long ns, int j, int r0, int nr, double* w, KrylovShared<CL>& s) {
+__device__ __forceinline__ void orthogonalise(const double* V, long ldv, int j, int nr, double* w, KrylovShared<CL>& s) {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = Cluster<CL>::rank();
     for (int pass = 0; pass < 2; ++pass) {
-        for (int i = warp; i <= j; i += NW) {
-            const double* vi = V + (long)i * ns + r0;
+        for (int i = warp; i <= j + pass; i += NW) {
+            const double* vi = i <= j ? V + (long)i * ldv : w;
             double acc = 0.0;
             for (int e = lane; e < nr; e += 32) acc += vi[e] * w[e];
             acc = warp_sum(acc);
             if (lane < CL) *Cluster<CL>::at(&s.part[pass][rank][i], lane) = acc;
         }
         Cluster<CL>::sync();
-        if (tid <= j) {
+        if (tid <= j + pass) {
             double a = 0.0;
+#pragma unroll
             for (int c = 0; c < CL; ++c) a += s.part[pass][c][tid];
             s.h[tid] = a;
-            s.hc[tid] = pass ? s.hc[tid] + a : a;
+            if (tid <= j) s.hc[tid] = pass ? s.hc[tid] + a : a;
         }
         __syncthreads();
+        if (pass && warp == NW - 1) {   // the scalars beside the update below
+            double q = 0.0;
+            for (int i = lane; i <= j; i += 32) q += s.h[i] * s.h[i];
+            const double t = s.h[j + 1], n2 = t - warp_sum(q);
+            if (lane == 0) {
+                const double n = n2 > 0.0 ? sqrt(n2) : 0.0;
+                s.sq = n2 > 0.5 * t ? 1.0 : 0.0;   // whether the difference may stand for the norm
+                s.nrm = n;
+                s.inv = n > 0.0 ? 1.0 / n : 0.0;
+            }
+        }
         for (int e = tid; e < nr; e += NT) {
             double a = 0.0;
 #pragma unroll 4
-            for (int i = 0; i <= j; ++i) a += s.h[i] * V[(long)i * ns + r0 + e];
+            for (int i = 0; i <= j; ++i) a += s.h[i] * V[(long)i * ldv + e];
             w[e] -= a;
         }
         __syncthreads();
     }
-    norm_cluster<CL>(w, nr, s);
+    if (s.sq == 0.0) norm_cluster<CL>(w, nr, s);   // the same in every block (NaN and zero vectors too)
 }
 
 // Givens rotations of Hessenberg column j (in s.hc, the subdiagonal nrm) with the rotations s.cs, s.sn
@@ -201,7 +217,7 @@ __device__ __forceinline__ void arnoldi_cluster_body(int* __restrict__ di, doubl
         s.sn[tid] = K[L.sn() + tid];
     }
     Cluster<CL>::sync();   // every block runs before one writes to its shared memory
-    orthogonalise<CL, NT>(V, ns, j, r0, nr, s_w, s);
+    orthogonalise<CL, NT>(V + r0, ns, j, nr, s_w, s);
     for (int e = tid; e < nr; e += NT) wg[e] = s_w[e] * s.inv;
     if (rank == 0) {
         if (tid == 0) {
@@ -305,7 +321,7 @@ struct KrylovArgs {
     long ld;                 // dense_ld(ns)
     const float *M, *S;
     const double* b;
-    double *V, *Z, *x;       // Z: column j + 1 holds z_j
+    double* x;
     KLayout L;
     double* K;
     int* di;
@@ -315,9 +331,12 @@ struct KrylovArgs {
     int cap;                 // most restart cycles
 };
 
+// Shared memory: v_j and z_j (all rows, FP32), the rotated columns, gv, y; this block's rows of w, of the
+// basis (FP64) and of the z_j (FP32, as the product leaves them).
 inline size_t krylov_smem(int ns, int m, int cl) {
+    const size_t R = (ns + cl - 1) / cl;
     return 2 * dense_ld(ns) * sizeof(float) + ((size_t)(m + 1) * m + 2 * (m + 1)) * sizeof(double) +
-           (size_t)((ns + cl - 1) / cl) * (sizeof(double) + sizeof(float));
+           R * (m + 1) * sizeof(double) + R * m * sizeof(float);
 }
 inline size_t arnoldi_smem(int ns, int cl) { return (size_t)((ns + cl - 1) / cl) * sizeof(double); }
 
@@ -335,25 +354,27 @@ __device__ void krylov_body(const KrylovArgs& g) {
     double* H = reinterpret_cast<double*>(zf + g.ld);            // rotated columns, stride m + 1
     double* gv = H + (size_t)(m + 1) * m;
     double* y = gv + m + 1;
-    double* w = y + m + 1;                                       // this block's rows of the current vector
-    float* wf = reinterpret_cast<float*>(w + (ns + CL - 1) / CL);
     const int R = (ns + CL - 1) / CL, r0 = min(rank * R, ns), nr = min(R, ns - r0);
+    double* w = y + m + 1;                                       // this block's rows of the current vector,
+    double* V = w + R;                                           // of the basis (column i at i R)
+    float* Z = reinterpret_cast<float*>(V + (size_t)R * m);      // and of the z_i
     for (int e = tid; e < 2 * g.ld; e += NT) vf[e] = 0.f;        // the padding stays zero
     for (int e = tid; e < nr; e += NT) g.x[r0 + e] = 0.0;
     const int left = g.from_its ? g.max_iter - g.di[DI_ITS] : g.max_iter;
     const int maxit = max(left, 1);
 
-    // this block's rows of v (FP64) into every block's FP32 copy
+    // the next basis vector: this block's rows kept, and into every block's FP32 copy
     auto share = [&](int col) {
+        double* vc = V + (size_t)col * R;
         for (int e = tid; e < nr; e += NT) {
-            const double t = w[e] * s.inv;
-            g.V[(long)col * ns + r0 + e] = t;
-            wf[e] = (float)t;
+            vc[e] = w[e] * s.inv;
+            vf[r0 + e] = (float)vc[e];
         }
         __syncthreads();
-        for (int e = tid; e < nr * CL; e += NT) {
-            const int c = e / nr, q = e - c * nr;
-            *Cluster<CL>::at(vf + r0 + q, c) = wf[q];
+        for (int c = warp; c < CL; c += NW) {
+            if (c == rank) continue;
+            float* to = Cluster<CL>::at(vf + r0, c);
+            for (int e = lane; e < nr; e += 32) to[e] = vf[r0 + e];
         }
     };
     // rows r0 .. of A times the shared vector; put(row, value) in every lane of the row's warp
@@ -391,14 +412,14 @@ __device__ void krylov_body(const KrylovArgs& g) {
         for (j = 0; !stop;) {
             product(g.M, vf, [&](int q, float t) {
                 if (lane < CL) *Cluster<CL>::at(zf + r0 + q, lane) = t;
-                if (lane == 0) g.Z[(long)(j + 1) * ns + r0 + q] = (double)t;
+                if (lane == 0) Z[(size_t)j * R + q] = t;
             });
             Cluster<CL>::sync();
             product(g.S, zf, [&](int q, float t) {
                 if (lane == 0) w[q] = (double)t;
             });
             __syncthreads();
-            orthogonalise<CL, NT>(g.V, ns, j, r0, nr, w, s);
+            orthogonalise<CL, NT>(V, R, j, nr, w, s);
             // the next basis vector goes out while one thread rotates the Hessenberg column
             const bool more = j + 1 < m && it + 1 < maxit;
             const double nrm = s.nrm;
@@ -438,7 +459,7 @@ __device__ void krylov_body(const KrylovArgs& g) {
         __syncthreads();
         for (int e = tid; e < nr; e += NT) {
             double a = 0.0;
-            for (int i = 0; i < j; ++i) a += y[i] * g.Z[(long)(i + 1) * ns + r0 + e];
+            for (int i = 0; i < j; ++i) a += y[i] * (double)Z[(size_t)i * R + e];
             g.x[r0 + e] += a;
         }
         ++cyc;
@@ -449,9 +470,9 @@ __device__ void krylov_body(const KrylovArgs& g) {
         }
         // restart: w = b - S x
         __syncthreads();
-        for (int e = tid; e < nr * CL; e += NT) {
-            const int c = e / nr, q = e - c * nr;
-            *Cluster<CL>::at(zf + r0 + q, c) = (float)g.x[r0 + q];
+        for (int c = warp; c < CL; c += NW) {
+            float* to = Cluster<CL>::at(zf + r0, c);
+            for (int e = lane; e < nr; e += 32) to[e] = (float)g.x[r0 + e];
         }
         Cluster<CL>::sync();
         product(g.S, zf, [&](int q, float t) {

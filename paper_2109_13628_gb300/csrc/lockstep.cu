@@ -194,7 +194,7 @@ template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads) kb_krylov(const LsProb* P, KLayout L, KTol tol, int max_iter) {
     const LsProb& p = P[blockIdx.z];
     if (!p.di[DI_RACT] || p.ns == 0) return;   // uniform over the cluster
-    krylov_body<CL>(KrylovArgs{p.ns, dense_ld(p.ns), p.pc_M, p.pc_S, p.bvec, p.V, p.Z, p.xsol, L, p.H, p.di,
+    krylov_body<CL>(KrylovArgs{p.ns, dense_ld(p.ns), p.pc_M, p.pc_S, p.bvec, p.xsol, L, p.H, p.di,
                                p.small, tol, max_iter, 1, max_iter / L.m + 2});
 }
 

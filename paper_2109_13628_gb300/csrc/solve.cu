@@ -999,7 +999,7 @@ struct Solver {
     bool clustered() const { return dense_op && krylov_fits(ns); }
     iim_status krylov(double tol, int max_it, bool its) {
         const int cl = krylov_cluster(ns);
-        const KrylovArgs a{ns, dense_ld(ns), g->pc_M, g->pc_S, g->bvec, g->V, g->Z, g->xsol, L, g->H, di(), g->small,
+        const KrylovArgs a{ns, dense_ld(ns), g->pc_M, g->pc_S, g->bvec, g->xsol, L, g->H, di(), g->small,
                            KTol{tol, kappa, last}, max_it, its ? 1 : 0, max_it / m + 2};
         return cl == 8 ? launch_cluster("gmres_krylov", 0.0, k_krylov<8>, 8, 1, krylov_smem(ns, m, 8), s, a)
                        : launch_cluster("gmres_krylov", 0.0, k_krylov<16>, 16, 1, krylov_smem(ns, m, 16), s, a);
