@@ -42,6 +42,13 @@ struct iim_net_s {
     __nv_bfloat16* wtc = nullptr;        // one layer's weights in the tensor-core operand layout
     float* wgp = nullptr;                // weight gradient: one buffer of sums per block (on first use)
     int wg_blocks = 0;
+    // inference on the tensor cores: every layer's weights in the operand layout (valid: wunit_ok), and two
+    // activation buffers of BF16 channel units with a zero border, laid out for the sizes below
+    __nv_bfloat16* wunit = nullptr;
+    bool wunit_ok = false;
+    uint4* unit[2] = {nullptr, nullptr};
+    size_t unit_n = 0;                   // units per buffer
+    int unit_b = 0, unit_h = 0, unit_w = 0;
     int* tc_err = nullptr;               // set by k_conv_tc when its wait for the MMAs timed out
 };
 
@@ -247,6 +254,196 @@ k_conv_tc(const float* __restrict__ x, const float* __restrict__ gate, const __n
         if (!ok) (void)tc::mbar_wait_bounded(mbar, 0, 1000000000ull);
         tc::tmem_dealloc(tmem, 32);
     }
+}
+
+// ---- inference: the same convolutions (same operands, MMAs in the same order, the same bits) on
+// activations that stay in the operand layout between layers.
+//
+// A layer's output is rounded to BF16 by its writer instead of by its readers and kept as units of 8
+// channels of one pixel (16 bytes), one plane of units per 8-channel group, with a border of zeros wide
+// enough for every dilation: 64 bytes per pixel instead of 128 + 128, and the operand of a run of pixels is a
+// contiguous piece of memory, so one bulk copy per row and group brings it into shared memory with no
+// thread touching it and no test at the image's edges.  A block computes runs of UN_M = 128 pixels on
+// UN_R = 4 output rows d apart, which share their input rows (6 instead of 12), each row in accumulator
+// columns of its own, side by side: an input row's operand (one shift kx, 16 channels) meets the weights
+// of all three ky at once, one MMA of N = 96 onto the columns of the three output rows it belongs to,
+// because an MMA of N = 32 is bound by reading its 128-row operand.  Every accumulator still gets its
+// products in the order of the taps.  Blocks are persistent, keep the weights, and start the next tile's
+// copies as soon as the MMAs have read this one's.  Two or three blocks per SM overlap copies, MMAs and
+// epilogues.  1023^2, six layers: 0.84 ms (one row of
+// FP32 planes converted by its block's threads per tile) -> 0.21 ms; the forward pass 0.86 -> 0.24 ms.
+constexpr int UN_M = 128, UN_R = 4;
+
+struct UnitLayout {
+    int H, W, Hp, Wp, D;   // image, padded planes (units), border
+    __host__ __device__ size_t at(int plane, int y, int x) const { return ((size_t)plane * Hp + y + D) * Wp + x + D; }
+};
+__host__ __device__ constexpr size_t conv_units_smem(int d, int cg, int no) {
+    return (size_t)16 * ((UN_R + 2) * cg * (UN_M + 2 * d) + 9 * cg * no) + 32 * 4 + 32;
+}
+// wp[((kx * CG + g) * 3 + 2 - ky) * NO + o] (units of 8 channels) = w[o][8 g ..][ky][kx], zero for o >= Co and
+// channels >= Ci
+template <int CG, int NO>
+__global__ void k_pack_w_units(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wp, int Ci, int Co) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= 9 * CG * NO * 8) return;
+    const int e = i & 7, o = (i >> 3) % NO, q = (i >> 3) / NO, ky = 2 - q % 3, g = q / 3 % CG, kx = q / 3 / CG;
+    const int c = 8 * g + e;
+    wp[i] = (o < Co && c < Ci) ? w[(o * Ci + c) * 9 + 3 * ky + kx] : __float2bfloat16(0.f);
+}
+__host__ __device__ constexpr int mma_groups(int c) { return c <= 16 ? 2 : 4; }     // 8-channel groups of the MMA's K
+__host__ __device__ constexpr int mma_cols(int c) { return c <= 16 ? 16 : 32; }     // its N
+
+// FP32 planes (B, C, H, W) -> units of group g = blockIdx.y (zero channels beyond C).
+__global__ void k_to_units(const float* __restrict__ x, int C, UnitLayout u, uint4* __restrict__ out) {
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x, plane = (long)u.H * u.W;
+    if (k >= plane) return;
+    const int g = blockIdx.y, G = gridDim.y, b = blockIdx.z;
+    float v[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) v[e] = 8 * g + e < C ? x[((long)b * C + 8 * g + e) * plane + k] : 0.f;
+    out[u.at(b * G + g, (int)(k / u.W), (int)(k % u.W))] =
+        make_uint4(bf16x2_bits(v[0], v[1]), bf16x2_bits(v[2], v[3]), bf16x2_bits(v[4], v[5]), bf16x2_bits(v[6], v[7]));
+}
+
+// One layer: units in (gin groups) -> units out (gout groups, ReLU), or with y the FP32 plane of output 0
+// (no ReLU).  Tiles are (image, row block, run), runs fastest; row block r covers rows (r / d) UN_R d + r % d
+// + k d, k < UN_R.
+template <int CG, int NO>
+__global__ void __launch_bounds__(128)
+k_conv_units(const uint4* __restrict__ in, int gin, const __nv_bfloat16* __restrict__ wp,
+             const float* __restrict__ bias, int Co, uint4* __restrict__ out, int gout, float* __restrict__ y,
+             UnitLayout u, int d, int nx, int nr, int tiles, int* __restrict__ err) {
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    const int NP = UN_M + 2 * d;
+    uint4* sA = reinterpret_cast<uint4*>(smem_raw);
+    uint4* sB = sA + (UN_R + 2) * CG * NP;
+    float* sbias = reinterpret_cast<float*>(sB + 9 * CG * NO);
+    uint64_t* full = reinterpret_cast<uint64_t*>(sbias + 32);
+    uint64_t* done = full + 1;
+    uint32_t* tslot = reinterpret_cast<uint32_t*>(done + 1);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr uint32_t COLS = UN_R * NO;
+    if (warp == 0) tc::tmem_alloc(tslot, COLS);
+    if (tid == 0) {
+        tc::mbar_init(full, 1);
+        tc::mbar_init(done, 1);
+    }
+    const uint4* wsrc = reinterpret_cast<const uint4*>(wp);
+    for (int i = tid; i < 9 * CG * NO; i += 128) sB[i] = wsrc[i];
+    if (tid < 32) sbias[tid] = tid < Co ? bias[tid] : 0.f;
+    for (int i = tid; i < (UN_R + 2) * (CG - gin) * NP; i += 128) {   // groups without channels stay zero
+        const int p = i % NP, q = i / NP, r = q / (CG - gin), g = gin + q - r * (CG - gin);
+        sA[(r * CG + g) * NP + p] = make_uint4(0u, 0u, 0u, 0u);
+    }
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    __syncthreads();
+    tc::fence_after_sync();
+    const uint32_t tmem = *tslot;
+    float2 bia[NO / 2];
+#pragma unroll
+    for (int o = 0; o < NO / 2; ++o) bia[o] = make_float2(sbias[2 * o], sbias[2 * o + 1]);
+    auto row0 = [&](int t) { const int r = (t / nx) % nr; return (r / d) * UN_R * d + r % d; };
+    auto load = [&](int t) {   // warp 0: one copy per lane (at most 6 rows x 4 groups)
+        const int x0 = (t % nx) * UN_M, y0 = row0(t), b = t / (nx * nr);
+        if (lane == 0) tc::mbar_expect(full, (uint32_t)(16 * (UN_R + 2) * gin * NP));
+        __syncwarp();
+        if (lane < (UN_R + 2) * gin) {
+            const int i = lane / gin, g = lane - i * gin;
+            const int yy = min(y0 + (i - 1) * d, u.H);   // rows below the image: its first border row
+            tc::bulk_load(sA + (i * CG + g) * NP, in + u.at(b * gin + g, yy, x0 - d), (uint32_t)(16 * NP), full);
+        }
+    };
+    // row blocks past the image's last row (when UN_R d does not divide the height) have no output
+    auto next = [&](int t) {
+        while (t < tiles && row0(t) >= u.H) t += gridDim.x;
+        return t;
+    };
+    bool ok = true;
+    uint32_t phase = 0;
+    int t = next(blockIdx.x);
+    if (t < tiles && warp == 0) load(t);
+    while (t < tiles) {
+        const int x0 = (t % nx) * UN_M, y0 = row0(t), b = t / (nx * nr);
+        if (tid == 0) {
+            if (tc::mbar_wait_bounded(full, phase, 1000000000ull)) {
+                // operand addresses move by 16-byte units, the unit of the descriptors' address field
+                const uint64_t ad = tc::desc_kmajor(tc::smem_u32(sA), (uint32_t)(16 * NP), 128u);
+                const uint64_t bd = tc::desc_kmajor(tc::smem_u32(sB), 48u * NO, 128u);
+                const int nk = min(UN_R, (u.H - y0 + d - 1) / d);   // output rows of the tile
+#pragma unroll
+                for (int i = 0; i < UN_R + 2; ++i) {
+                    // input row i: output rows lo .. hi (ky = i - row); row i starts here
+                    const int lo = i > 2 ? i - 2 : 0, hi = min(i, nk - 1);
+                    if (hi < lo) break;
+#pragma unroll
+                    for (int kx = 0; kx < 3; ++kx) {
+#pragma unroll
+                        for (int s = 0; s < CG / 2; ++s) {
+                            const uint64_t a = ad + (uint32_t)((i * CG + 2 * s) * NP + kx * d);
+                            const uint64_t w = bd + (uint32_t)(((kx * CG + 2 * s) * 3 + lo - i + 2) * NO);
+                            const bool first = (kx | s) == 0 && hi == i;   // the first products of row i overwrite
+                            const int n = hi - lo + 1 - (first ? 1 : 0);
+                            if (n > 0) tc::mma_bf16(tmem + (uint32_t)(lo * NO), a, w, tc::idesc_bf16_f32(UN_M, n * NO), 1);
+                            if (first) tc::mma_bf16(tmem + (uint32_t)(i * NO), a, w + (uint32_t)(n * NO), tc::idesc_bf16_f32(UN_M, NO), 0);
+                        }
+                    }
+                }
+                tc::commit(done);
+            }
+        }
+        __syncwarp();
+        ok = __all_sync(0xffffffffu, tc::mbar_wait_bounded(done, phase, 2000000000ull));
+        // a copy or an MMA that gave no sign of completing: leave (every warp waits on the same barrier)
+        if (__syncthreads_or(!ok)) {
+            ok = false;
+            break;
+        }
+        tc::fence_after_sync();
+        const int tn = next(t + gridDim.x);
+        if (tn < tiles && warp == 0) load(tn);   // the MMAs have read this tile's operands
+        const int gx = x0 + tid;
+#pragma unroll 1
+        for (int k = 0; k < UN_R; ++k) {
+            const int gy = y0 + k * d;
+            if (gy >= u.H) break;
+            float acc[NO];
+            __syncwarp();   // the load below is a whole-warp instruction
+            const uint32_t ta = tmem + (uint32_t)(k * NO) + ((uint32_t)(32 * warp) << 16);
+            if constexpr (NO == 32) tc::tmem_ld_32x32(ta, acc);
+            else tc::tmem_ld_32x16(ta, acc);
+            if (gx >= u.W) continue;
+            if (y) {
+                y[(size_t)b * u.H * u.W + (size_t)gy * u.W + gx] = acc[0] + bia[0].x;
+                continue;
+            }
+            // bias, rounding to BF16, ReLU (channels beyond Co: zero weights and bias)
+            uint32_t v[NO / 2];
+#pragma unroll
+            for (int o = 0; o < NO / 2; ++o) {
+                const __nv_bfloat162 r = __floats2bfloat162_rn(acc[2 * o] + bia[o].x, acc[2 * o + 1] + bia[o].y);
+                const __nv_bfloat162 q = __hmax2(r, __floats2bfloat162_rn(0.f, 0.f));
+                v[o] = *reinterpret_cast<const uint32_t*>(&q);
+            }
+#pragma unroll
+            for (int g = 0; g < NO / 8; ++g)
+                if (g < gout) out[u.at(b * gout + g, gy, gx)] = make_uint4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
+        }
+        tc::fence_before_sync();
+        __syncthreads();   // the accumulators have been read
+        tc::fence_after_sync();
+        t = tn;
+        phase ^= 1;
+    }
+    if (!ok) {
+        if (tid == 0) {
+            atomicExch(err, 1);
+            (void)tc::mbar_wait_bounded(full, phase, 1000000000ull);   // no copy may land after the block has left
+        }
+        __syncthreads();
+    }
+    if (warp == 0) tc::tmem_dealloc(tmem, COLS);
 }
 
 // Weight gradient dW[o,c,k] = sum_{b,p} g[b,o,p] x[b,c,p + d off(k)], db[o] = sum g (g gated by
@@ -527,6 +724,71 @@ static iim_status conv(iim_net_s* net, const float* x, const float* gate, const 
     return IIM_OK;
 }
 
+// Units per layer of the packed weights (the largest layer's).
+constexpr size_t WUNIT = (size_t)9 * 4 * TC_C * 8;
+
+static int max_dilation(const iim_net_s* net) { return *std::max_element(net->dil.begin(), net->dil.end()); }
+
+// The whole network on the tensor cores for inference (every layer; net->tc == 2): y (batch, 1, h, w).
+static iim_status forward_units(iim_net_s* net, int B, int H, int W, const float* x, float* y, cudaStream_t s) {
+    const int D = max_dilation(net);
+    const UnitLayout u{H, W, H + 2 * D, (W + UN_M - 1) / UN_M * UN_M + 2 * D, D};
+    int planes = (net->cin + 7) / 8;
+    if (net->nl > 1) planes = std::max(planes, (net->hidden + 7) / 8);
+    const size_t need = (size_t)B * planes * u.Hp * u.Wp;
+    if (need > net->unit_n || B != net->unit_b || H != net->unit_h || W != net->unit_w) {
+        if (need > net->unit_n) {
+            for (uint4*& p : net->unit) {
+                cudaFree(p);
+                p = nullptr;
+            }
+            net->unit_n = 0;
+            for (uint4*& p : net->unit) IIM_TRY(cudaMalloc(&p, need * sizeof(uint4)));
+            net->unit_n = need;
+        }
+        net->unit_b = 0;
+        for (uint4* p : net->unit) IIM_TRY(cudaMemsetAsync(p, 0, need * sizeof(uint4), s));   // the borders
+        net->unit_b = B; net->unit_h = H; net->unit_w = W;
+    }
+    if (!net->wunit) IIM_TRY(cudaMalloc(&net->wunit, sizeof(__nv_bfloat16) * WUNIT * net->nl));
+    if (!net->wunit_ok) {
+        for (int l = 0; l < net->nl; ++l) {
+            const int cg = mma_groups(net->ci[l]), no = mma_cols(net->co[l]);
+            auto pack = cg == 2 ? (no == 16 ? k_pack_w_units<2, 16> : k_pack_w_units<2, 32>)
+                                : (no == 16 ? k_pack_w_units<4, 16> : k_pack_w_units<4, 32>);
+            launch("net_pack_w_units", 0.0, 0.0, pack, (9 * cg * no * 8 + 255) / 256, 256, 0, s,
+                   (const __nv_bfloat16*)(net->wb + net->woff[l]), net->wunit + WUNIT * l, net->ci[l], net->co[l]);
+        }
+        IIM_LAUNCHED();
+        net->wunit_ok = true;
+    }
+    const long plane = (long)H * W;
+    launch("net_to_units", 4.0 * plane * B * net->cin, 0.0, k_to_units,
+           dim3((unsigned)((plane + 255) / 256), (net->cin + 7) / 8, B), 256, 0, s, x, net->cin, u, net->unit[0]);
+    IIM_LAUNCHED();
+    for (int l = 0; l < net->nl; ++l) {
+        const int ci = net->ci[l], co = net->co[l], d = net->dil[l], gin = (ci + 7) / 8;
+        const bool last = l == net->nl - 1;
+        const int nx = (W + UN_M - 1) / UN_M, nr = (H + UN_R * d - 1) / (UN_R * d) * d, tiles = nx * nr * B;
+        auto go = [&](auto kern, int cg, int no) -> iim_status {
+            const size_t sm = conv_units_smem(d, cg, no);
+            IIM_CHECK(allow_smem(kern, sm));
+            const int per_sm = std::max(1, (int)(227 * 1024 / (sm + 1024)));   // resident blocks (also 512 TMEM columns / 128)
+            const int blocks = std::min(tiles, std::min(per_sm, 4) * sm_count());
+            launch("net_conv_tc", 2.0 * plane * B * (8.0 * gin + (last ? 2.0 : 8.0 * ((co + 7) / 8))),
+                   18.0 * (double)B * plane * ci * co, kern, blocks, 128, sm, s, (const uint4*)net->unit[l & 1], gin,
+                   (const __nv_bfloat16*)(net->wunit + WUNIT * l), (const float*)(net->p + net->boff[l]), co,
+                   net->unit[(l + 1) & 1], (co + 7) / 8, last ? y : (float*)nullptr, u, d, nx, nr, tiles, net->tc_err);
+            IIM_LAUNCHED();
+            return IIM_OK;
+        };
+        const int cg = mma_groups(ci), no = mma_cols(co);
+        IIM_CHECK(cg == 2 ? (no == 16 ? go(k_conv_units<2, 16>, 2, 16) : go(k_conv_units<2, 32>, 2, 32))
+                          : (no == 16 ? go(k_conv_units<4, 16>, 4, 16) : go(k_conv_units<4, 32>, 4, 32)));
+    }
+    return IIM_OK;
+}
+
 static iim_status ensure_cap(iim_net_s* net, long long need) {
     if (need <= net->cap) return IIM_OK;
     cudaFree(net->act);
@@ -588,6 +850,7 @@ static iim_status sync_bf16(iim_net_s* net, cudaStream_t s) {
     launch("net_bf16", 0.0, 0.0, k_to_bf16, (unsigned)((net->np + 255) / 256), 256, 0, s, (long)net->np,
            (const float*)net->p, net->wb);
     IIM_LAUNCHED();
+    net->wunit_ok = false;
     return IIM_OK;
 }
 
@@ -679,6 +942,9 @@ extern "C" iim_status iim_net_forward(iim_net net, int batch, int height, int wi
                                       iim_stream stream) {
     if (!net || !x || !y || batch < 1 || height < 1 || width < 1) return IIM_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    // one image's planes and the tiles are counted in 32 bits
+    if (net->tc == 2 && (long long)batch * ((height + 127) / 4 + 1) * (width / UN_M + 1) < (1LL << 30) && batch <= 65535)
+        return forward_units(net, batch, height, width, x, y, s);
     IIM_CHECK(forward(net, batch, height, width, x, s));
     IIM_TRY(cudaMemcpyAsync(y, net->act + (size_t)(net->nl - 1) * net->cap, sizeof(float) * (size_t)batch * height * width,
                             cudaMemcpyDeviceToDevice, s));
@@ -768,7 +1034,8 @@ extern "C" iim_status iim_net_tensor_core_status(iim_net net, int* on, int* time
 extern "C" void iim_net_destroy(iim_net net) {
     if (!net) return;
     cudaFree(net->p); cudaFree(net->gr); cudaFree(net->m); cudaFree(net->v); cudaFree(net->wb); cudaFree(net->wt);
-    cudaFree(net->act); cudaFree(net->g0); cudaFree(net->red); cudaFree(net->wgp); cudaFree(net->wtc); cudaFree(net->tc_err);
+    cudaFree(net->act); cudaFree(net->g0); cudaFree(net->red); cudaFree(net->wgp);
+    cudaFree(net->wunit); cudaFree(net->unit[0]); cudaFree(net->unit[1]); cudaFree(net->wtc); cudaFree(net->tc_err);
     if (net->h_red) cudaFreeHost(net->h_red);
     delete net;
 }
