@@ -127,7 +127,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // small[] layout
 enum { SM_RES2 = 0, SM_CIRC_ERR = 1, SM_CIRC = 8, SM_RC = 8 + 64, SM_REG = 8 + 128, SM_NORM = 2048, SM_SEED = 2049,
        SM_CAPC = 2112, SM_CAPP = 2176, SM_FNORM = 2240, SM_REL = 2241 };
-constexpr int kRegionParts = 16;
+// Blocks per region sum (small[] holds their partial sums).
+__host__ __device__ constexpr int region_parts(int ncirc) { return ncirc <= 8 ? 64 : 16; }
 
 // Device state (int): [0] j (column of the current cycle), [1] stop, [2] iterations of this
 // call, [3] max iterations of this call, [4] converged, [5] scratch column index,
@@ -136,7 +137,7 @@ enum { DI_J = 0, DI_STOP = 1, DI_IT = 2, DI_MAXIT = 3, DI_CONV = 4, DI_TMPJ = 5,
        // device-driven whole solve: refinements, Krylov iterations (all / first correction),
        // cycles of the current correction, cap hits, non-finite residual, cycles and restarts
        DI_REF = 8, DI_ITS = 9, DI_FIRST = 10, DI_CYC = 11, DI_CYCERR = 12, DI_NONFIN = 13, DI_CYCS = 14,
-       DI_RSS = 15, DI_CIRC = 32 };
+       DI_RSS = 15, DI_TICKET = 18, DI_CIRC = 32 };
 
 // Krylov small-storage layout inside g->H (m <= 64):
 //   H (m+1) x m column-major | cs[m] | sn[m] | gv[m+1] | hc1[m+1] | hc2[m+1] | y[m] | scal[8]
@@ -237,63 +238,82 @@ __device__ __forceinline__ void residual_body(int NX, int NY, double ih2, const 
     if (threadIdx.x == 0) partial[blockIdx.x] = acc;
 }
 
+// What follows the residual kernel: per circulation body the sum of the residual over R_k and the measured
+// circulation -h sum_{dR}(grad_h psi).n (Eq. discretecircconstraint), then small[SM_RES2] = sum partial
+// + sum rc^2 with rc_c = (Gamma_k - circ_k) / h^2, bcirc[c] = sum_{R_k} r - rc_c and max |Gamma_k - circ_k|.
+struct FinishArgs {
+    int nparts;
+    const double* partial;
+    int nx;
+    const double *psi, *res;
+    const iim_region* R;
+    int* di;                 // circulation body ids, ticket
+    int ncirc;
+    const double* gamma;
+    double ih2;
+    double *small, *bcirc;
+};
+__host__ __device__ constexpr int finish_blocks(int ncirc) { return ncirc > 0 ? ncirc * (region_parts(ncirc) + 1) : 1; }
+
+// One launch of finish_blocks(ncirc) blocks: region parts and circulations, and the block that ends last
+// adds everything up in a fixed order.  True in that block's thread 0.
 template <int BLOCK>
-__device__ __forceinline__ void region_sums_body(int nx, const double* __restrict__ f,
-                                                 const iim_region* __restrict__ R, const int* __restrict__ circ_ids,
-                                                 double* __restrict__ partial) {
-    const int c = blockIdx.x, part = blockIdx.y, S = gridDim.y;
-    const iim_region r = R[circ_ids[c]];
-    const int w = r.rx - r.lx + 1, hgt = r.ry - r.ly + 1;
-    const long n = (long)w * hgt;
-    double acc = 0.0;
-    for (long t = (long)part * BLOCK + threadIdx.x; t < n; t += (long)S * BLOCK) {
-        const int i = r.lx + (int)(t % w), j = r.ly + (int)(t / w);
-        acc += f[(long)(j - 1) * nx + i];
+__device__ __forceinline__ bool finish_body(const FinishArgs& a, int blk) {
+    const int P = region_parts(a.ncirc), nblk = finish_blocks(a.ncirc);
+    const int* ids = a.di + DI_CIRC;
+    if (a.ncirc > 0) {
+        const int c = blk / (P + 1), part = blk - c * (P + 1);
+        const iim_region r = a.R[ids[c]];
+        double acc = 0.0;
+        if (part < P) {
+            const int w = r.rx - r.lx + 1;
+            for (int j = r.ly + part; j <= r.ry; j += P)
+                for (int i = threadIdx.x; i < w; i += BLOCK) acc += a.res[(long)(j - 1) * a.nx + r.lx + i];
+            acc = block_sum<BLOCK>(acc);
+            if (threadIdx.x == 0) a.small[SM_REG + c * P + part] = acc;
+        } else {
+            auto at = [&](int i, int j) { return a.psi[(long)(j - 1) * a.nx + i]; };
+            for (int j = r.ly + threadIdx.x; j <= r.ry; j += BLOCK)
+                acc += (at(r.rx + 1, j) - at(r.rx, j)) - (at(r.lx, j) - at(r.lx - 1, j));
+            for (int i = r.lx + threadIdx.x; i <= r.rx; i += BLOCK)
+                acc += (at(i, r.ry + 1) - at(i, r.ry)) - (at(i, r.ly) - at(i, r.ly - 1));
+            acc = block_sum<BLOCK>(acc);
+            if (threadIdx.x == 0) a.small[SM_CIRC + c] = -acc;
+        }
+        __shared__ int last;
+        if (threadIdx.x == 0) {
+            __threadfence();
+            last = atomicAdd(a.di + DI_TICKET, 1) == nblk - 1;
+            if (last) a.di[DI_TICKET] = 0;
+        }
+        __syncthreads();
+        if (!last) return false;
+        __threadfence();
     }
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) partial[c * S + part] = acc;
-}
-
-template <int BLOCK>
-__device__ __forceinline__ void circ_measure_body(int nx, const double* __restrict__ psi,
-                                                  const iim_region* __restrict__ R, const int* __restrict__ circ_ids,
-                                                  double* __restrict__ out) {
-    const int c = blockIdx.x;
-    const iim_region r = R[circ_ids[c]];
-    auto P = [&](int i, int j) { return psi[(long)(j - 1) * nx + i]; };
-    double acc = 0.0;
-    for (int j = r.ly + threadIdx.x; j <= r.ry; j += BLOCK)
-        acc += (P(r.rx + 1, j) - P(r.rx, j)) - (P(r.lx, j) - P(r.lx - 1, j));
-    for (int i = r.lx + threadIdx.x; i <= r.rx; i += BLOCK)
-        acc += (P(i, r.ry + 1) - P(i, r.ry)) - (P(i, r.ly) - P(i, r.ly - 1));
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) out[c] = -acc;
-}
-
-template <int BLOCK>
-__device__ __forceinline__ void finish_residual_body(int nparts, const double* __restrict__ partial, int ncirc,
-                                                     const int* __restrict__ circ_ids,
-                                                     const double* __restrict__ gamma, double ih2,
-                                                     double* __restrict__ small, const double* __restrict__ regpart,
-                                                     double* __restrict__ bcirc, double* __restrict__ out_res2) {
+    __shared__ double reg[64];
+    const int lane = threadIdx.x & 31;
+    for (int c = threadIdx.x >> 5; c < a.ncirc; c += BLOCK / 32) {
+        double v = 0.0;
+        for (int p = lane; p < P; p += 32) v += __ldcg(a.small + SM_REG + c * P + p);
+        v = warp_sum(v);
+        if (lane == 0) reg[c] = v;
+    }
     double s = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += BLOCK) s += partial[b];
-    s = block_sum<BLOCK>(s);
-    if (threadIdx.x != 0) return;
+    for (int b = threadIdx.x; b < a.nparts; b += BLOCK) s += a.partial[b];
+    s = block_sum<BLOCK>(s);   // synchronises: reg is complete
+    if (threadIdx.x != 0) return false;
     double cerr = 0.0;
-    for (int c = 0; c < ncirc; ++c) {
-        const double gk = gamma ? gamma[circ_ids[c]] : 0.0;
-        const double diff = gk - small[SM_CIRC + c];
+    for (int c = 0; c < a.ncirc; ++c) {
+        const double diff = (a.gamma ? a.gamma[ids[c]] : 0.0) - __ldcg(a.small + SM_CIRC + c);
         cerr = fmax(cerr, fabs(diff));
-        const double rc = diff * ih2;
-        small[SM_RC + c] = rc;
+        const double rc = diff * a.ih2;
+        a.small[SM_RC + c] = rc;
         s += rc * rc;
-        double reg = 0.0;
-        for (int p = 0; p < kRegionParts; ++p) reg += regpart[c * kRegionParts + p];
-        if (bcirc) bcirc[c] = reg - rc;
+        if (a.bcirc) a.bcirc[c] = reg[c] - rc;
     }
-    out_res2[0] = s;
-    if (out_res2 == small + SM_RES2) small[SM_CIRC_ERR] = cerr;
+    a.small[SM_RES2] = s;
+    a.small[SM_CIRC_ERR] = cerr;
+    return true;
 }
 
 __device__ __forceinline__ void init_psi_body(int NX, int NY, const double* __restrict__ guess,
@@ -365,9 +385,10 @@ struct KTol {
     double rel, kappa, last;
 };
 
+// Capacitance coefficients coef = C^-1 (h^2 rc) and the body constants' step psibar += coef . Pb (one block).
 __device__ __forceinline__ void cap_coef_body(int nc, const double* __restrict__ rc, const double* __restrict__ cinv,
                                               const double* __restrict__ pb, double h2, double* __restrict__ coef,
-                                              double* __restrict__ dpb) {
+                                              const int* __restrict__ circ_ids, double* __restrict__ psibar) {
     __shared__ double c_sh[64];
     const int t = threadIdx.x;
     if (t < nc) {
@@ -380,7 +401,7 @@ __device__ __forceinline__ void cap_coef_body(int nc, const double* __restrict__
     if (t < nc) {
         double d = 0.0;
         for (int l = 0; l < nc; ++l) d += c_sh[l] * pb[l * nc + t];
-        dpb[t] = d;
+        psibar[circ_ids[t]] += d;
     }
 }
 

@@ -96,15 +96,17 @@ __device__ __forceinline__ VecArg ls_vec(const LsProb& p, int mode) {
 
 template <typename T, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
-kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, const cpx<T>* __restrict__ tab) {
+kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, int tri, const cpx<T>* __restrict__ tab) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     const bool dense = mode == M_RHS || mode == M_RECOVER;
-    const int row0 = dense ? 0 : p.ja0, nrows = dense ? p.NY : p.ja1 - p.ja0 + 1;
+    // the recovery redoes only the rows that gamma changes where tbuf still holds the others (tri)
+    const bool band = !dense || (mode == M_RECOVER && tri && p.na > 0);
+    const int row0 = band ? p.ja0 : 0, nrows = band ? p.ja1 - p.ja0 + 1 : p.NY;
     if ((int)blockIdx.x * L >= nrows) return;   // uniform over the block
     sine_rows_fwd_body<T, N, L>(p.NX, p.NY, p.nx, row0, nrows, dense ? p.res : nullptr, p.nx, 1, nullptr, 0.0,
                              mode == M_RHS ? nullptr : p.aff_row_ptr, mode == M_RHS ? nullptr : p.aff_node,
-                             ls_vec(p, mode), mode == M_RECOVER ? -1.0 : 1.0, tab, (T*)p.tbuf);
+                             ls_vec(p, mode), mode == M_RECOVER ? -1.0 : 1.0, tab, dense ? (T*)p.tbuf : (T*)p.psiT);
 }
 
 template <typename T, int C, int FP>
@@ -115,7 +117,8 @@ kb_cols(const LsProb* __restrict__ P, int mode, int gate, T norm, const cpx<T>* 
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
     if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
     if (mode == M_RECOVER) { out0 = 0; out1 = p.NY - 1; }
-    cols_body<T, C, FP>(p.NX, p.NY, p.NY + 1, __ffs(p.NY + 1) - 1, in0, in1, out0, out1, (T*)p.tbuf,
+    cols_body<T, C, FP>(p.NX, p.NY, p.NY + 1, __ffs(p.NY + 1) - 1, in0, in1, out0, out1,
+                        mode == M_RHS || mode == M_RECOVER ? (T*)p.tbuf : (T*)p.psiT,
                         (const T*)p.lam_x, (const T*)p.lam_y, norm, tw);
 }
 
@@ -132,17 +135,22 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4) kb_cols_scan(const LsP
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
     if (mode == M_APPLY_Z || mode == M_APPLY_VTMP) { in0 = p.ja0; in1 = p.ja1; }
     if (mode == M_RECOVER) { out0 = 0; out1 = p.NY - 1; }
-    cols_scan_body<T, CW, NT>(p.NX, p.NY, p.nx, in0, in1, out0, out1, (T*)p.tbuf, ls_scan<T>(p));
+    // as Solver: the right-hand side's band goes to psiT (tbuf keeps the row transforms), the operator
+    // works in psiT
+    const T* in = mode == M_RHS || mode == M_RECOVER ? (T*)p.tbuf : (T*)p.psiT;
+    cols_scan_body<T, CW, NT>(p.NX, p.NY, p.nx, in0, in1, out0, out1, in, mode == M_RECOVER ? (T*)p.tbuf : (T*)p.psiT,
+                              ls_scan<T>(p));
 }
 
 template <typename T, int MODE, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
-kb_rows_inv(const LsProb* __restrict__ P, int gate, const cpx<T>* __restrict__ tab) {
+kb_rows_inv(const LsProb* __restrict__ P, int from_psi, int gate, const cpx<T>* __restrict__ tab) {
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (MODE == INV_STORE_T && p.na == 0)) return;
     const int row0 = MODE == INV_STORE_T ? p.jo0 : 0, nrows = MODE == INV_STORE_T ? p.jo1 - p.jo0 + 1 : p.NY;
     if ((int)blockIdx.x * L >= nrows) return;
-    sine_rows_inv_body<T, MODE, N, L>(p.NX, p.NY, p.nx, row0, nrows, (const T*)p.tbuf,
+    if (MODE == INV_ACCUM_FLUID && blockIdx.x == 0) PsibarStep{p.ncirc, p.di + DI_CIRC, p.xsol + p.na, p.psibar}.apply();
+    sine_rows_inv_body<T, MODE, N, L>(p.NX, p.NY, p.nx, row0, nrows, (const T*)(from_psi ? p.psiT : p.tbuf),
                                    MODE == INV_STORE_T ? (T*)p.psiT : nullptr,
                                    MODE == INV_STORE_T ? nullptr : p.psi_ext, 0, 0, p.cls, tab);
 }
@@ -241,13 +249,9 @@ __global__ void kb_vec(const LsProb* __restrict__ P, int op, int gate) {
 // ------------------------------------------------------------------------- field kernels
 __global__ void kb_init(const LsProb* __restrict__ P) {
     const LsProb& p = P[blockIdx.z];
-    if ((long)blockIdx.x * blockDim.x >= (long)p.nx * p.NY) return;
-    init_psi_body(p.NX, p.NY, nullptr, p.cls, p.psi_ext);
-}
-
-__global__ void kb_init_psibar(const LsProb* __restrict__ P) {
-    const LsProb& p = P[blockIdx.z];
-    if (p.nb > 0) init_psibar_body(p.nb, p.body_circ, p.psibar, 0, p.psibar);
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < (long)p.nx * p.NY / 2) reinterpret_cast<double2*>(p.psi_ext)[k] = make_double2(0.0, 0.0);
+    if (blockIdx.x == 0 && p.nb > 0) init_psibar_body(p.nb, p.body_circ, p.psibar, 0, p.psibar);
 }
 
 __global__ void kb_ghost(const LsProb* __restrict__ P, int gate) {
@@ -264,32 +268,11 @@ __global__ void __launch_bounds__(BLOCK) kb_residual(const LsProb* __restrict__ 
 }
 
 template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) kb_circ_measure(const LsProb* __restrict__ P, int gate) {
-    const LsProb& p = P[blockIdx.z];
-    if (ls_off(p, gate) || (int)blockIdx.x >= p.ncirc) return;
-    circ_measure_body<BLOCK>(p.nx, p.psi_ext, p.regions, p.di + DI_CIRC, p.small + SM_CIRC);
-}
-
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK) kb_region_sums(const LsProb* __restrict__ P, int gate) {
-    const LsProb& p = P[blockIdx.z];
-    if (ls_off(p, gate) || (int)blockIdx.x >= p.ncirc) return;
-    region_sums_body<BLOCK>(p.nx, p.res, p.regions, p.di + DI_CIRC, p.small + SM_REG);
-}
-
-template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) kb_finish_residual(const LsProb* __restrict__ P, int gate, int nparts) {
     const LsProb& p = P[blockIdx.z];
-    if (ls_off(p, gate)) return;
-    finish_residual_body<BLOCK>(nparts, p.partial, p.ncirc, p.di + DI_CIRC, p.gamma, p.ih2, p.small, p.small + SM_REG,
-                                p.bvec ? p.bvec + p.na : nullptr, p.small + SM_RES2);
-}
-
-// psibar += the circulation part of the correction (from_cap = 0) or of the capacitance step
-__global__ void kb_add_psibar(const LsProb* __restrict__ P, int from_cap, int gate) {
-    const LsProb& p = P[blockIdx.z];
-    if (ls_off(p, gate) || p.ncirc == 0) return;
-    add_psibar_body(p.ncirc, p.di + DI_CIRC, from_cap ? p.small + SM_CAPP : p.xsol + p.na, p.psibar);
+    if (ls_off(p, gate) || (int)blockIdx.x >= finish_blocks(p.ncirc)) return;
+    finish_body<BLOCK>(FinishArgs{nparts, p.partial, p.nx, p.psi_ext, p.res, p.regions, p.di, p.ncirc, p.gamma, p.ih2, p.small,
+                                  p.bvec ? p.bvec + p.na : nullptr}, blockIdx.x);
 }
 
 __global__ void kb_cap_coef(const LsProb* __restrict__ P) {
@@ -297,7 +280,7 @@ __global__ void kb_cap_coef(const LsProb* __restrict__ P) {
     if (ls_off(p, G_CAP)) return;
     const int nc = p.ncirc;
     cap_coef_body(nc, p.small + SM_RC, p.cap_dev, p.cap_dev + (size_t)nc * nc, p.h * p.h, p.small + SM_CAPC,
-                  p.small + SM_CAPP);
+                  p.di + DI_CIRC, p.psibar);
 }
 
 __global__ void kb_cap_update(const LsProb* __restrict__ P) {
@@ -478,7 +461,7 @@ struct LsGroup {
     double rtol = 0.0, inner = 0.0, kappa = 0.0, last = 0.0;
     int nx = 0, ny = 0, NX = 0, NY = 0, wide = 0, cols_c = 4, tri = 0;
     // launch extents: maxima over the group
-    int max_na = 0, max_ns = 0, max_nminus = 0, max_ncirc = 0, max_ja_rows = 0, max_jo_rows = 0;
+    int max_na = 0, max_ns = 0, max_nminus = 0, max_ncirc = 0, max_finish = 1, min_na = 1, max_ja_rows = 0, max_jo_rows = 0;
     LsProb* d_probs = nullptr;
     LsProb* h_probs = nullptr;   // pinned
     LsRec* d_rec = nullptr;
@@ -589,8 +572,9 @@ struct LsEmit {
     template <typename T>
     iim_status rows_fwd(int mode, int gate) {
         const bool dense = mode == M_RHS || mode == M_RECOVER;
-        const int rows = dense ? G->NY : G->max_ja_rows;
-        const double bytes = sum_rows(dense ? 0 : 1, G->NX * ((dense ? 8.0 : 0.0) + sizeof(T)));
+        const bool full = mode == M_RHS || (mode == M_RECOVER && (!G->tri || G->min_na == 0));
+        const int rows = full ? G->NY : G->max_ja_rows;
+        const double bytes = sum_rows(full ? 0 : 1, G->NX * ((dense ? 8.0 : 0.0) + sizeof(T)));
         const int lpb = sine_lines(G->nx, (long)rows * G->n());
         IIM_CHECK(sine_dispatch(G->nx, lpb, [&](auto N, auto L) -> iim_status {
             auto kern = kb_rows_fwd<T, N.value, L.value>;
@@ -598,7 +582,7 @@ struct LsEmit {
             IIM_CHECK(allow_smem(kern, sm));
             launch(sizeof(T) == 8 ? "ls_rows_fwd_f64" : "ls_rows_fwd_f32", bytes, 0.0, kern,
                    grid((rows + lpb - 1) / lpb), (Sine<N.value, L.value>::kBlock), sm, s, (const LsProb*)G->d_probs, mode,
-                   gate, sine_table<T>(G->nx));
+                   gate, G->tri, sine_table<T>(G->nx));
             return IIM_OK;
         }));
         IIM_LAUNCHED();
@@ -665,7 +649,7 @@ struct LsEmit {
     }
 
     template <typename T, int MODE>
-    iim_status rows_inv(int gate) {
+    iim_status rows_inv(int gate, bool from_psi) {
         const int rows = MODE == INV_STORE_T ? G->max_jo_rows : G->NY;
         const double bytes = sum_rows(MODE == INV_STORE_T ? 2 : 0, G->NX * (sizeof(T) + (MODE == INV_STORE_T ? sizeof(T) : 17.0)));
         const int lpb = sine_lines(G->nx, (long)rows * G->n());
@@ -674,8 +658,8 @@ struct LsEmit {
             const size_t sm = sine_smem<T>(G->nx, lpb);
             IIM_CHECK(allow_smem(kern, sm));
             launch(sizeof(T) == 8 ? "ls_rows_inv_f64" : "ls_rows_inv_f32", bytes, 0.0, kern,
-                   grid((rows + lpb - 1) / lpb), (Sine<N.value, L.value>::kBlock), sm, s, (const LsProb*)G->d_probs, gate,
-                   sine_table<T>(G->nx));
+                   grid((rows + lpb - 1) / lpb), (Sine<N.value, L.value>::kBlock), sm, s, (const LsProb*)G->d_probs,
+                   from_psi ? 1 : 0, gate, sine_table<T>(G->nx));
             return IIM_OK;
         }));
         IIM_LAUNCHED();
@@ -726,12 +710,7 @@ struct LsEmit {
         double bytes = 0.0;
         for (iim_geometry g : G->geos) bytes += 25.0 * (double)g->NX * g->NY;
         launch("ls_residual_f64", bytes, 0.0, kb_residual<256>, grid(kResBlocks), 256, 0, s, P, gate);
-        if (G->max_ncirc > 0) {
-            launch("ls_circ_measure", 0.0, 0.0, kb_circ_measure<256>, grid(G->max_ncirc), 256, 0, s, P, gate);
-            launch("ls_region_sums", 0.0, 0.0, kb_region_sums<256>, dim3(G->max_ncirc, kRegionParts, G->n()), 256, 0,
-                   s, P, gate);
-        }
-        launch("ls_finish_residual", 0.0, 0.0, kb_finish_residual<256>, grid(1), 256, 0, s, P, gate, kResBlocks);
+        launch("ls_finish_residual", 0.0, 0.0, kb_finish_residual<256>, grid(G->max_finish), 256, 0, s, P, gate, kResBlocks);
         IIM_LAUNCHED();
         return IIM_OK;
     }
@@ -739,8 +718,7 @@ struct LsEmit {
     // --- the pieces between loop decisions
     iim_status top_pre(cudaGraphConditionalHandle h_ref) {
         const long npad = (long)G->nx * G->NY;
-        launch("ls_init_psi", 0.0, 0.0, kb_init, grid((npad + 255) / 256), 256, 0, s, (const LsProb*)G->d_probs);
-        launch("ls_init_psibar", 0.0, 0.0, kb_init_psibar, grid(1), 64, 0, s, (const LsProb*)G->d_probs);
+        launch("ls_init_solve", 0.0, 0.0, kb_init, grid((npad / 2 + 255) / 256), 256, 0, s, (const LsProb*)G->d_probs);
         IIM_LAUNCHED();
         IIM_CHECK(residual(G_ALL));
         launch("ls_ref_init", 0.0, 0.0, kb_ref_init, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(), G->rtol, h_ref,
@@ -753,7 +731,7 @@ struct LsEmit {
     iim_status ref_pre(cudaGraphConditionalHandle h_cyc) {
         IIM_CHECK(rows_fwd<T>(M_RHS, G_REF));
         IIM_CHECK(cols<T>(M_RHS, G_REF));
-        IIM_CHECK((rows_inv<T, INV_STORE_T>(G_REF)));
+        IIM_CHECK((rows_inv<T, INV_STORE_T>(G_REF, G->tri != 0)));
         IIM_CHECK(gather<T>(M_RHS, G_REF));
         if (fused()) {
             const int cl = krylov_cluster(G->max_ns);
@@ -786,7 +764,7 @@ struct LsEmit {
         } else {
             IIM_CHECK(rows_fwd<T>(M_APPLY_Z, G_IT));
             IIM_CHECK(cols<T>(M_APPLY_Z, G_IT));
-            IIM_CHECK((rows_inv<T, INV_STORE_T>(G_IT)));
+            IIM_CHECK((rows_inv<T, INV_STORE_T>(G_IT, true)));
             IIM_CHECK(gather<T>(M_APPLY_Z, G_IT));
         }
         const int cl = krylov_cluster(G->max_ns);
@@ -819,7 +797,7 @@ struct LsEmit {
         } else {
             IIM_CHECK(rows_fwd<T>(M_APPLY_VTMP, G_CYC));
             IIM_CHECK(cols<T>(M_APPLY_VTMP, G_CYC));
-            IIM_CHECK((rows_inv<T, INV_STORE_T>(G_CYC)));
+            IIM_CHECK((rows_inv<T, INV_STORE_T>(G_CYC, true)));
             IIM_CHECK(gather<T>(M_APPLY_VTMP, G_CYC));
         }
         IIM_CHECK(vec(V_RESTART_RES, G_CYC));
@@ -833,10 +811,7 @@ struct LsEmit {
     iim_status ref_post(cudaGraphConditionalHandle h_ref) {
         IIM_CHECK(rows_fwd<T>(M_RECOVER, G_REF));
         IIM_CHECK(cols<T>(M_RECOVER, G_REF));
-        IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(G_REF)));
-        if (G->max_ncirc > 0)
-            launch("ls_add_psibar", 0.0, 0.0, kb_add_psibar, grid(1), 64, 0, s, (const LsProb*)G->d_probs, 0, G_REF);
-        IIM_LAUNCHED();
+        IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(G_REF, false)));
         IIM_CHECK(residual(G_REF));
         launch("ls_ref_ctl", 0.0, 0.0, kb_ref_ctl, 1, 256, 0, s, (const LsProb*)G->d_probs, G->n(), G->rtol,
                std::min(G->max_refine, 1000), G->max_iter, h_ref, flag(), cnt());
@@ -852,7 +827,6 @@ struct LsEmit {
             const long npad = (long)G->nx * G->NY;
             launch("ls_cap_coef", 0.0, 0.0, kb_cap_coef, grid(1), 64, 0, s, P);
             launch("ls_cap_update", 0.0, 0.0, kb_cap_update, grid((npad + 255) / 256), 256, 0, s, P);
-            launch("ls_add_psibar", 0.0, 0.0, kb_add_psibar, grid(1), 64, 0, s, P, 1, G_CAP);
             IIM_LAUNCHED();
             IIM_CHECK(residual(G_CAP));
             launch("ls_final_rel", 0.0, 0.0, kb_final_rel, grid(1), 1, 0, s, P);
@@ -982,9 +956,11 @@ static iim_status make_group(const std::vector<iim_geometry>& geos, const iim_op
     G->tri = g0->col_solver == 1;
     for (iim_geometry g : geos) {
         G->max_na = std::max(G->max_na, g->na);
+        G->min_na = std::min(G->min_na, g->na);
         G->max_ns = std::max(G->max_ns, g->na + g->ncirc);
         G->max_nminus = std::max(G->max_nminus, g->nminus);
         G->max_ncirc = std::max(G->max_ncirc, g->ncirc);
+        G->max_finish = std::max(G->max_finish, finish_blocks(g->ncirc));
         G->max_ja_rows = std::max(G->max_ja_rows, g->ja1 - g->ja0 + 1);
         G->max_jo_rows = std::max(G->max_jo_rows, g->jo1 - g->jo0 + 1);
         G->cap |= (g->ncirc > 0 && g->cap_ready) ? 1 : 0;

@@ -372,10 +372,22 @@ k_sine_rows_fwd(int NX, int NY, int n, int row0, int nrows, const double* __rest
                              ih2, aff_row_ptr, aff_node, gam, gsign, tab, out + (long)blockIdx.y * ofs);
 }
 
-// Inverse row transforms of rows [row0, row0 + nrows) of a padded buffer, modes as RowsInvMode.
+// The body constants' step of a correction, psibar += x (circulation bodies), beside the recovery.
+struct PsibarStep {
+    int ncirc;
+    const int* ids;
+    const double* x;
+    double* psibar;
+    __device__ __forceinline__ void apply() const {
+        for (int c = threadIdx.x; c < ncirc; c += blockDim.x) psibar[ids[c]] += x[c];
+    }
+};
+
+// Inverse row transforms of rows [row0, row0 + nrows) of a padded buffer, modes as RowsInvMode (in and outT
+// may be the same rows: a block reads its lines before it writes them).
 template <typename T, int MODE, int N, int L>
 __device__ __forceinline__ void
-sine_rows_inv_body(int NX, int NY, int n_rt, int row0, int nrows, const T* __restrict__ in, T* __restrict__ outT,
+sine_rows_inv_body(int NX, int NY, int n_rt, int row0, int nrows, const T* in, T* outT,
                    double* __restrict__ out64, int old, int ooff, const uint8_t* __restrict__ cls,
                    const cpx<T>* __restrict__ tab) {
     using S = Sine<N, L>;
@@ -439,10 +451,11 @@ sine_rows_inv_body(int NX, int NY, int n_rt, int row0, int nrows, const T* __res
 
 template <typename T, int MODE, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
-k_sine_rows_inv(int NX, int NY, int n, int row0, int nrows, const T* __restrict__ in, T* __restrict__ outT,
+k_sine_rows_inv(int NX, int NY, int n, int row0, int nrows, const T* in, T* outT,
                 double* __restrict__ out64, int old, int ooff, const uint8_t* __restrict__ cls,
-                const cpx<T>* __restrict__ tab, const int* __restrict__ stop, long fstride) {
+                const cpx<T>* __restrict__ tab, const int* __restrict__ stop, long fstride, PsibarStep ps) {
     if (stop && *stop) return;
+    if (MODE == INV_ACCUM_FLUID && blockIdx.x == 0) ps.apply();
     sine_rows_inv_body<T, MODE, N, L>(NX, NY, n, row0, nrows, in + (long)blockIdx.y * fstride,
                                    outT ? outT + (long)blockIdx.y * fstride : nullptr, out64, old, ooff, cls, tab);
 }

@@ -254,44 +254,45 @@ static iim_status cols_tile(const Plan<T>& p, int in0, int in1, int out0, int ou
 // apart.
 template <typename T, int CW, int NT>
 __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4)
-k_cols_scan(int NX, int NY, int ld, int in0, int in1, int out0, int out1, T* __restrict__ buf, ScanTab<T> t,
+k_cols_scan(int NX, int NY, int ld, int in0, int in1, int out0, int out1, const T* buf, T* out, ScanTab<T> t,
             const int* __restrict__ stop, long fstride) {
     if (stop && *stop) return;
-    cols_scan_body<T, CW, NT>(NX, NY, ld, in0, in1, out0, out1, buf + (long)blockIdx.y * fstride, t);
+    cols_scan_body<T, CW, NT>(NX, NY, ld, in0, in1, out0, out1, buf + (long)blockIdx.y * fstride,
+                              out + (long)blockIdx.y * fstride, t);
 }
 
 // Launch: one block per 32-byte tile of padded columns (8 FP32 or 4 FP64 columns), batch
 // fields on grid y.
 template <typename T, int NT>
-static iim_status cols_scan_nt(const Plan<T>& p, int in0, int in1, int out0, int out1, T* buf, const int* stop,
-                               cudaStream_t s, int batch, long fstride) {
+static iim_status cols_scan_nt(const Plan<T>& p, int in0, int in1, int out0, int out1, const T* buf, T* out,
+                               const int* stop, cudaStream_t s, int batch, long fstride) {
     constexpr int CW = 32 / sizeof(T);
     const size_t sm = scan_smem<T, CW, NT>(p.NY);
     IIM_CHECK(allow_smem(k_cols_scan<T, CW, NT>, sm));
     launch(sizeof(T) == 8 ? "tri_cols_f64" : "tri_cols_f32",
            (double)batch * (in1 - in0 + 1 + out1 - out0 + 1) * p.NX * sizeof(T), (double)batch * p.NX * 14.0 * p.NY,
            k_cols_scan<T, CW, NT>, dim3(p.nx / CW, batch), NT, sm, s, p.NX, p.NY, p.nx, in0, in1, out0, out1, buf,
-           p.scan, stop, fstride);
+           out, p.scan, stop, fstride);
     IIM_LAUNCHED();
     return IIM_OK;
 }
 
 template <typename T>
-static iim_status cols_scan(const Plan<T>& p, int in0, int in1, int out0, int out1, T* buf, const int* stop,
+static iim_status cols_scan(const Plan<T>& p, int in0, int in1, int out0, int out1, const T* buf, T* out, const int* stop,
                             cudaStream_t s, int batch, long fstride) {
     constexpr int CW = 32 / sizeof(T);
     if constexpr (sizeof(T) == 4) {   // FP64 keeps 256 threads (it is bound by FP64 arithmetic)
         if (scan_threads(p.NY, (long)(p.nx / CW) * batch, sm_count()) == 1024)
-            return cols_scan_nt<T, 1024>(p, in0, in1, out0, out1, buf, stop, s, batch, fstride);
+            return cols_scan_nt<T, 1024>(p, in0, in1, out0, out1, buf, out, stop, s, batch, fstride);
     }
-    return cols_scan_nt<T, 256>(p, in0, in1, out0, out1, buf, stop, s, batch, fstride);
+    return cols_scan_nt<T, 256>(p, in0, in1, out0, out1, buf, out, stop, s, batch, fstride);
 }
 
 // batch > 1: as many fields, fstride elements apart, in one launch
 template <typename T>
 static iim_status cols(const Plan<T>& p, int in0, int in1, int out0, int out1, T* buf, const int* stop, cudaStream_t s,
                        int batch = 1, long fstride = 0) {
-    if (p.scan.lim) return cols_scan(p, in0, in1, out0, out1, buf, stop, s, batch, fstride);
+    if (p.scan.lim) return cols_scan<T>(p, in0, in1, out0, out1, buf, buf, stop, s, batch, fstride);
     const int C = tile_width<T>(p.cols_c);
     if (C == 8) return cols_tile<T, (sizeof(T) == 4 ? 8 : 4)>(p, in0, in1, out0, out1, buf, stop, s, batch, fstride);
     if (C == 2) return cols_tile<T, (sizeof(T) == 8 ? 2 : 4)>(p, in0, in1, out0, out1, buf, stop, s, batch, fstride);
@@ -324,7 +325,7 @@ static iim_status cols_tile(const Plan<T>& p, int in0, int in1, int out0, int ou
 template <typename T, int MODE>
 static iim_status rows_inv(const Plan<T>& p, int row0, int nrows, const T* in, T* outT, double* out64, int old,
                            int ooff, const uint8_t* cls, const int* stop, cudaStream_t s, int batch = 1,
-                           long fstride = 0) {
+                           long fstride = 0, PsibarStep ps = {}) {
     if (nrows <= 0) return IIM_OK;
     const int lpb = sine_lines(p.nx, (long)nrows * batch);
     const size_t sm = sine_smem<T>(p.nx, lpb);
@@ -335,7 +336,7 @@ static iim_status rows_inv(const Plan<T>& p, int row0, int nrows, const T* in, T
                (double)batch * nrows * p.NX *
                    (sizeof(T) + (MODE == INV_STORE_T ? sizeof(T) : MODE == INV_STORE_F64 ? 8.0 : 17.0)),
                (double)batch * nrows * dst_flops(p.nx), kern, dim3((nrows + lpb - 1) / lpb, batch), (Sine<N.value, L.value>::kBlock), sm,
-               s, p.NX, p.NY, p.nx, row0, nrows, in, outT, out64, old, ooff, cls, sine_table<T>(p.nx), stop, fstride);
+               s, p.NX, p.NY, p.nx, row0, nrows, in, outT, out64, old, ooff, cls, sine_table<T>(p.nx), stop, fstride, ps);
         return IIM_OK;
     }));
     IIM_LAUNCHED();
@@ -449,41 +450,42 @@ __global__ void k_residual(int NX, int NY, double ih2, const double* __restrict_
     residual_body<BLOCK>(NX, NY, ih2, psi, omega, cls, ring, res, partial);
 }
 
-// Sum of a padded field over region R_k of each circulation body; grid (ncirc, S).
+// The loop decision that follows a residual in the whole-solve graph: none, the start of the refinements,
+// the end of one, or the final residual after the capacitance step (below).
+enum { CTL_NONE = 0, CTL_INIT = 1, CTL_REFINE = 2, CTL_FINAL = 3 };
+struct RefCtl {
+    int mode;
+    cudaGraphConditionalHandle h;
+    double rtol;
+    int max_refine, max_iter;
+};
+__device__ void ref_control(const RefCtl& c, int* di, double* small);
+
 template <int BLOCK>
-__global__ void k_region_sums(int nx, const double* __restrict__ f, const iim_region* __restrict__ R,
-                              const int* __restrict__ circ_ids, double* __restrict__ partial) {
-    region_sums_body<BLOCK>(nx, f, R, circ_ids, partial);
+__global__ void __launch_bounds__(BLOCK) k_finish(FinishArgs a, RefCtl c) {
+    if (finish_body<BLOCK>(a, blockIdx.x) && c.mode != CTL_NONE) ref_control(c, a.di, a.small);
 }
 
-// Discrete circulation -h sum_{dR}(grad_h psi).n (Eq. discretecircconstraint) of each circulation
-// body, from the fluid values of psi on the faces of R_k.
+// out = sum of the partial sums (one block).
 template <int BLOCK>
-__global__ void k_circ_measure(int nx, const double* __restrict__ psi, const iim_region* __restrict__ R,
-                               const int* __restrict__ circ_ids, double* __restrict__ out) {
-    circ_measure_body<BLOCK>(nx, psi, R, circ_ids, out);
+__global__ void __launch_bounds__(BLOCK) k_sum_parts(int n, const double* __restrict__ partial, double* __restrict__ out) {
+    double s = 0.0;
+    for (int b = threadIdx.x; b < n; b += BLOCK) s += partial[b];
+    s = block_sum<BLOCK>(s);
+    if (threadIdx.x == 0) *out = s;
 }
 
-
-// Combines partial sums into *out_res2 = sum partial + sum rc^2 and, for circulation bodies,
-// bcirc[c] = sum_{R_k} r - rc_c with rc_c = (Gamma_k - circ_k) / h^2; max |Gamma_k - circ_k|
-// goes to small[SM_CIRC_ERR] when ncirc > 0 or out_res2 is small[SM_RES2].
-template <int BLOCK>
-__global__ void k_finish_residual(int nparts, const double* __restrict__ partial, int ncirc,
-                                  const int* __restrict__ circ_ids, const double* __restrict__ gamma, double ih2,
-                                  double* __restrict__ small, const double* __restrict__ regpart,
-                                  double* __restrict__ bcirc, double* __restrict__ out_res2) {
-    finish_residual_body<BLOCK>(nparts, partial, ncirc, circ_ids, gamma, ih2, small, regpart, bcirc, out_res2);
+// Start of a solve from psi = 0: the field zeroed, circulation bodies' constants zeroed.
+__global__ void k_init_solve(long n2, double2* __restrict__ psi, int nb, const int* __restrict__ body_circ,
+                             double* __restrict__ psibar) {
+    const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k < n2) psi[k] = make_double2(0.0, 0.0);
+    if (blockIdx.x == 0 && nb > 0) init_psibar_body(nb, body_circ, psibar, 0, psibar);
 }
 
 __global__ void k_init_psi(int NX, int NY, const double* __restrict__ guess, const uint8_t* __restrict__ cls,
                            double* __restrict__ psi) {
     init_psi_body(NX, NY, guess, cls, psi);
-}
-
-__global__ void k_init_psibar(int nb, const int* __restrict__ body_circ, const double* __restrict__ in, int keep_circ,
-                              double* __restrict__ out) {
-    init_psibar_body(nb, body_circ, in, keep_circ, out);
 }
 
 __global__ void k_add_psibar(int ncirc, const int* __restrict__ circ_ids, const double* __restrict__ x, double* __restrict__ psibar) {
@@ -648,19 +650,36 @@ __global__ void k_loop_ctl(cudaGraphConditionalHandle h, int* __restrict__ di, i
 }
 
 // ---- control kernels of the whole solve run as one graph (nested WHILE / IF nodes)
-// Before the refinement loop: ||f|| from the residual at psi = 0, counters reset, loop entered
-// unless there is nothing to solve.
-__global__ void k_ref_init(cudaGraphConditionalHandle h, int* __restrict__ di, double* __restrict__ small, double rtol) {
+// CTL_INIT, before the refinement loop: ||f|| from the residual at psi = 0, counters reset, loop entered
+// unless there is nothing to solve.  CTL_REFINE, end of a refinement: counters, the relative FP64
+// residual, and whether to go on (at most max_refine corrections and max_iter Krylov iterations).
+__device__ void ref_control(const RefCtl& c, int* di, double* small) {
     const double r2 = small[SM_RES2];
-    const double fn = sqrt(r2);
-    small[SM_FNORM] = fn;
-    small[SM_REL] = fn > 0.0 ? 1.0 : 0.0;
-    di[DI_REF] = 0; di[DI_ITS] = 0; di[DI_FIRST] = 0; di[DI_CYCERR] = 0; di[DI_CYCS] = 0; di[DI_RSS] = 0;
-    di[DI_LOOPERR] = 0;
     const bool fin = isfinite(r2);
-    di[DI_NONFIN] = fin ? 0 : 1;
-    cudaGraphSetConditional(h, (fin && fn > 0.0 && 1.0 > rtol) ? 1 : 0);
+    if (c.mode == CTL_INIT) {
+        const double fn = sqrt(r2);
+        small[SM_FNORM] = fn;
+        small[SM_REL] = fn > 0.0 ? 1.0 : 0.0;
+        di[DI_REF] = 0; di[DI_ITS] = 0; di[DI_FIRST] = 0; di[DI_CYCERR] = 0; di[DI_CYCS] = 0; di[DI_RSS] = 0;
+        di[DI_LOOPERR] = 0;
+        di[DI_NONFIN] = fin ? 0 : 1;
+        cudaGraphSetConditional(c.h, (fin && fn > 0.0 && 1.0 > c.rtol) ? 1 : 0);
+    } else if (c.mode == CTL_REFINE) {
+        if (di[DI_REF] == 0) di[DI_FIRST] = di[DI_IT];
+        di[DI_ITS] += di[DI_IT];
+        const int r = ++di[DI_REF];
+        const double fn = small[SM_FNORM];
+        if (!fin) di[DI_NONFIN] = 1;
+        const double rel = fn > 0.0 ? sqrt(r2) / fn : 0.0;
+        small[SM_REL] = rel;
+        const bool go = fin && rel > c.rtol && r < c.max_refine && di[DI_ITS] < c.max_iter && !di[DI_LOOPERR] && !di[DI_CYCERR];
+        cudaGraphSetConditional(c.h, go ? 1 : 0);
+    } else {
+        final_rel_body(di, small);
+    }
 }
+// The same after the ring rows of a free-space residual.
+__global__ void k_ref_control(RefCtl c, int* __restrict__ di, double* __restrict__ small) { ref_control(c, di, small); }
 
 // After gmres_init: the Krylov budget left for this correction; cycle counter reset; the cycle
 // loop entered unless the start already stopped (converged or no budget).
@@ -694,30 +713,10 @@ __global__ void k_cyc_ctl(cudaGraphConditionalHandle hc, cudaGraphConditionalHan
     cudaGraphSetConditional(hr, done ? 0 : 1);
 }
 
-// End of a refinement: counters, the relative FP64 residual, and whether to go on (at most
-// max_refine corrections and max_iter Krylov iterations).
-__global__ void k_ref_ctl(cudaGraphConditionalHandle h, int* __restrict__ di, double* __restrict__ small, double rtol,
-                          int max_refine, int max_iter) {
-    if (di[DI_REF] == 0) di[DI_FIRST] = di[DI_IT];
-    di[DI_ITS] += di[DI_IT];
-    const int r = ++di[DI_REF];
-    const double r2 = small[SM_RES2], fn = small[SM_FNORM];
-    const bool fin = isfinite(r2);
-    if (!fin) di[DI_NONFIN] = 1;
-    const double rel = fn > 0.0 ? sqrt(r2) / fn : 0.0;
-    small[SM_REL] = rel;
-    const bool go = fin && rel > rtol && r < max_refine && di[DI_ITS] < max_iter && !di[DI_LOOPERR] && !di[DI_CYCERR];
-    cudaGraphSetConditional(h, go ? 1 : 0);
-}
-
-// Capacitance coefficients on the device: coef = C^-1 (h^2 rc), dpb = coef . Pb (one block).
 __global__ void k_cap_coef(int nc, const double* __restrict__ rc, const double* __restrict__ cinv,
-                           const double* __restrict__ pb, double h2, double* __restrict__ coef, double* __restrict__ dpb) {
-    cap_coef_body(nc, rc, cinv, pb, h2, coef, dpb);
-}
-
-__global__ void k_final_rel(int* __restrict__ di, double* __restrict__ small) {
-    final_rel_body(di, small);
+                           const double* __restrict__ pb, double h2, double* __restrict__ coef,
+                           const int* __restrict__ circ_ids, double* __restrict__ psibar) {
+    cap_coef_body(nc, rc, cinv, pb, h2, coef, circ_ids, psibar);
 }
 
 // One GMRES cycle as a graph: a WHILE node whose body is one iteration (the captured kernel
@@ -777,9 +776,19 @@ struct Solver {
         return IIM_OK;
     }
 
-    // the kernels of residual(): ghosts, residual and partial norms, circulation measure,
-    // region sums, small[SM_RES2], small[SM_CIRC_ERR], small[SM_RC..], circulation rows of bvec
-    iim_status residual_launch() {
+    // psi = 0 and the circulation bodies' constants 0
+    iim_status init_solve() {
+        const long n2 = (long)g->nx * g->NY / 2;
+        launch("init_solve", 0.0, 0.0, k_init_solve, (unsigned)((n2 + 255) / 256), 256, 0, s, n2, (double2*)g->psi_ext, g->nb,
+               (const int*)g->body_circ, psibar);
+        IIM_LAUNCHED();
+        if (g->outer) IIM_TRY(cudaMemsetAsync(g->fs_ring, 0, sizeof(double) * 2 * (g->nx + g->ny), s));
+        return IIM_OK;
+    }
+
+    // the kernels of residual(): ghosts, residual and partial norms, then circulations and region sums with
+    // small[SM_RES2], small[SM_CIRC_ERR], small[SM_RC..] and the circulation rows of bvec
+    iim_status residual_launch(RefCtl ctl = {}) {
         const double ih2 = 1.0 / (g->h * g->h);
         if (g->nminus > 0) {
             launch("ghost_f64", 0.0, 0.0, k_ghost, (g->nminus + 255) / 256, 256, 0, s, g->nminus, g->minus_node, g->gh_ptr,
@@ -790,21 +799,19 @@ struct Solver {
                256, 0, s, g->NX, g->NY, ih2, g->psi_ext, omega, g->node_class, ring_now(), g->res, g->partial);
         IIM_LAUNCHED();
         double* small = g->small;
-        const int* circ_ids_d = g->d_int + DI_CIRC;
-        if (g->ncirc > 0) {
-            launch("circ_measure", 0.0, 0.0, k_circ_measure<256>, g->ncirc, 256, 0, s, g->nx, g->psi_ext, g->d_regions,
-                   circ_ids_d, small + SM_CIRC);
-            launch("region_sums", 0.0, 0.0, k_region_sums<256>, dim3(g->ncirc, kRegionParts), 256, 0, s, g->nx, g->res,
-                   g->d_regions, circ_ids_d, small + SM_REG);
-            IIM_LAUNCHED();
-        }
-        launch("finish_residual", 0.0, 0.0, k_finish_residual<256>, 1, 256, 0, s, kResBlocks, g->partial, g->ncirc,
-               circ_ids_d, gamma, ih2, small, small + SM_REG, g->bvec ? g->bvec + g->na : nullptr, small + SM_RES2);
+        const FinishArgs fa{kResBlocks, g->partial, g->nx, g->psi_ext, g->res, g->d_regions, di(), g->ncirc, gamma, ih2,
+                            small, g->bvec ? g->bvec + g->na : nullptr};
+        launch("finish_residual", 0.0, 0.0, k_finish<256>, finish_blocks(g->ncirc), 256, 0, s, fa,
+               g->outer ? RefCtl{} : ctl);
         IIM_LAUNCHED();
         if (g->outer)   // free space: the ring rows (freespace.cu), kept for the next recovery
             IIM_CHECK(launch_ring_residual(g->nx, g->ny, g->h, g->lgf, g->lgf_ld, g->outer == 2,
                                            g->outer == 2 && !g->plane_off ? g->fs_plane : nullptr, g->psi_ext,
                                            g->fs_ring, g->fs_rres, small + SM_RES2, s));
+        if (g->outer && ctl.mode != CTL_NONE) {
+            launch("ref_control", 0.0, 0.0, k_ref_control, 1, 1, 0, s, ctl, di(), small);
+            IIM_LAUNCHED();
+        }
         return IIM_OK;
     }
 
@@ -822,10 +829,11 @@ struct Solver {
         T* pt = (T*)g->psiT;
         const long ld = ns;
         if (g->na > 0 && !g->outer) {
+            // in psiT throughout: tbuf keeps the transformed residual of the correction
             IIM_CHECK(rows_fwd<T>(p, g->ja0, g->ja1 - g->ja0 + 1, nullptr, 0, 0, nullptr, 0.0, g->aff_row_ptr,
-                                  g->aff_node, vj, 1.0, tb, stop, s));
-            IIM_CHECK(cols<T>(p, g->ja0, g->ja1, g->jo0, g->jo1, tb, stop, s));
-            IIM_CHECK((rows_inv<T, INV_STORE_T>(p, g->jo0, g->jo1 - g->jo0 + 1, tb, pt, nullptr, 0, 0, nullptr, stop, s)));
+                                  g->aff_node, vj, 1.0, pt, stop, s));
+            IIM_CHECK(cols<T>(p, g->ja0, g->ja1, g->jo0, g->jo1, pt, stop, s));
+            IIM_CHECK((rows_inv<T, INV_STORE_T>(p, g->jo0, g->jo1 - g->jo0 + 1, pt, pt, nullptr, 0, 0, nullptr, stop, s)));
         } else if (g->na > 0) {
             // free space: psi_1 with every row of the column pass kept for the boundary values,
             // then the harmonic part with the ring data rho
@@ -1084,6 +1092,10 @@ struct Solver {
         return IIM_OK;
     }
 
+    // the column pass of the right-hand side writes its band to psiT, so that tbuf still holds the row
+    // transforms of r at the recovery, which then redoes only the rows that gamma changes
+    bool keep_rows() const { return g->col_solver == 1 && !g->outer && g->na > 0; }
+
     // ---- right-hand side b = [A P r ; sum_R r - rc] (circulation part filled by residual())
     template <typename T>
     iim_status rhs() {
@@ -1092,9 +1104,15 @@ struct Solver {
         T* pt = (T*)g->psiT;
         if (g->na == 0) return IIM_OK;
         IIM_CHECK(rows_fwd<T>(p, 0, g->NY, g->res, g->nx, 1, nullptr, 0.0, nullptr, nullptr, kNoVec, 0.0, tb, nullptr, s));
-        IIM_CHECK(cols<T>(p, 0, g->NY - 1, g->outer ? 0 : g->jo0, g->outer ? g->NY - 1 : g->jo1, tb, nullptr, s));
+        T* band = tb;
+        if (keep_rows()) {
+            band = pt;
+            IIM_CHECK(cols_scan<T>(p, 0, g->NY - 1, g->jo0, g->jo1, tb, pt, nullptr, s, 1, 0L));
+        } else {
+            IIM_CHECK(cols<T>(p, 0, g->NY - 1, g->outer ? 0 : g->jo0, g->outer ? g->NY - 1 : g->jo1, tb, nullptr, s));
+        }
         if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr));
-        IIM_CHECK((rows_inv<T, INV_STORE_T>(p, g->jo0, g->jo1 - g->jo0 + 1, tb, pt, nullptr, 0, 0, nullptr, nullptr, s)));
+        IIM_CHECK((rows_inv<T, INV_STORE_T>(p, g->jo0, g->jo1 - g->jo0 + 1, band, pt, nullptr, 0, 0, nullptr, nullptr, s)));
         if (g->outer) {
             // the harmonic part of the correction carries rho minus the ring rows of the residual,
             // as in the recovery below, so that the right-hand side sees the ring data and error
@@ -1115,11 +1133,13 @@ struct Solver {
         Plan<T> p = make_plan<T>(g);
         T* tb = (T*)g->tbuf;
         const VecArg xg{g->na ? x : nullptr, nullptr, 0, 0};
-        IIM_CHECK(rows_fwd<T>(p, 0, g->NY, g->res, g->nx, 1, nullptr, 0.0, g->aff_row_ptr, g->aff_node, xg, -1.0, tb,
+        const int r0 = keep_rows() ? g->ja0 : 0, nr = keep_rows() ? g->ja1 - g->ja0 + 1 : g->NY;
+        IIM_CHECK(rows_fwd<T>(p, r0, nr, g->res, g->nx, 1, nullptr, 0.0, g->aff_row_ptr, g->aff_node, xg, -1.0, tb,
                               nullptr, s));
         IIM_CHECK(cols<T>(p, 0, g->NY - 1, 0, g->NY - 1, tb, nullptr, s));
         if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr));
-        IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(p, 0, g->NY, tb, nullptr, g->psi_ext, 0, 0, g->node_class, nullptr, s)));
+        const PsibarStep ps{g->ncirc, di() + DI_CIRC, x + g->na, psibar};
+        IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(p, 0, g->NY, tb, nullptr, g->psi_ext, 0, 0, g->node_class, nullptr, s, 1, 0L, ps)));
         if (g->outer) {
             // the harmonic part carries rho minus the ring rows of the last residual: the field
             // harmonic inside the box that removes the ring error (the interior rows do not see
@@ -1129,10 +1149,6 @@ struct Solver {
             IIM_CHECK(free_harmonic<T>(p, 0, g->NY - 1, nullptr));
             IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(p, 0, g->NY, tb, nullptr, g->psi_ext, 0, 0, g->node_class, nullptr, s)));
             IIM_CHECK(launch_ring_add(nr, 1.0, g->fs_rho, g->fs_ring, nullptr, s));
-        }
-        if (g->ncirc > 0) {
-            launch("add_psibar", 0.0, 0.0, k_add_psibar, 1, 64, 0, s, g->ncirc, di() + DI_CIRC, x + g->na, psibar);
-            IIM_LAUNCHED();
         }
         return IIM_OK;
     }
@@ -1167,8 +1183,8 @@ struct Solver {
             started = true;
         } else {
             launch("gmres_sumsq", 0.0, 0.0, k_sumsq<256>, kNormBlocks, 256, 0, s, g->bvec, ns_, g->partial);
-            launch("finish_norm", 0.0, 0.0, k_finish_residual<256>, 1, 256, 0, s, kNormBlocks, g->partial, 0, nullptr,
-                   nullptr, 0.0, g->small, nullptr, nullptr, g->small + SM_NORM);
+            launch("finish_norm", 0.0, 0.0, k_sum_parts<256>, 1, 256, 0, s, kNormBlocks, (const double*)g->partial,
+                   g->small + SM_NORM);
             launch("gmres_init", 0.0, 0.0, k_gmres_init, 1, 1, 0, s, di(), max_it, K, L, g->small + SM_NORM, tol);
         }
         if (x0) {
@@ -1326,15 +1342,8 @@ struct Solver {
         cudaGraph_t ref_body = nullptr, cyc_body = nullptr, it_body = nullptr, rs_body = nullptr;
         handle(top, &h_ref);
         piece(top_seg, [&]() -> iim_status {
-            launch("init_psi", 0.0, 0.0, k_init_psi, (unsigned)((npad + 255) / 256), 256, 0, s, g->NX, g->NY, nullptr,
-                   g->node_class, g->psi_ext);
-            if (g->outer) IIM_TRY(cudaMemsetAsync(g->fs_ring, 0, sizeof(double) * 2 * (g->nx + g->ny), s));
-            if (g->nb > 0)
-                launch("init_psibar", 0.0, 0.0, k_init_psibar, 1, 64, 0, s, g->nb, g->body_circ, psibar, 0, psibar);
-            IIM_CHECK(residual_launch());
-            launch("ref_init", 0.0, 0.0, k_ref_init, 1, 1, 0, s, h_ref, di(), g->small, o.rtol);
-            IIM_LAUNCHED();
-            return IIM_OK;
+            IIM_CHECK(init_solve());
+            return residual_launch(RefCtl{CTL_INIT, h_ref, o.rtol, 0, 0});
         });
         cond(top_seg, h_ref, cudaGraphCondTypeWhile, &ref_body);
         CapSeg ref_seg{s, ref_body, {}};
@@ -1388,18 +1397,14 @@ struct Solver {
         }
         piece(ref_seg, [&]() -> iim_status {
             IIM_CHECK(recover<T>(x));
-            IIM_CHECK(residual_launch());
-            launch("ref_ctl", 0.0, 0.0, k_ref_ctl, 1, 1, 0, s, h_ref, di(), g->small, o.rtol,
-                   std::min(o.max_refine, 1000), o.max_iter);
-            IIM_LAUNCHED();
-            return IIM_OK;
+            return residual_launch(RefCtl{CTL_REFINE, h_ref, o.rtol, std::min(o.max_refine, 1000), o.max_iter});
         });
         piece(top_seg, [&]() -> iim_status {
             if (use_cap) {
                 const int nc = g->ncirc;
                 launch("cap_coef", 0.0, 0.0, k_cap_coef, 1, 64, 0, s, nc, (const double*)(g->small + SM_RC),
                        (const double*)g->cap_dev, (const double*)(g->cap_dev + (size_t)nc * nc), g->h * g->h,
-                       g->small + SM_CAPC, g->small + SM_CAPP);
+                       g->small + SM_CAPC, (const int*)(g->d_int + DI_CIRC), psibar);
                 launch("cap_update", 0.0, 0.0, k_cap_update, (unsigned)((npad + 255) / 256), 256, 0, s, npad, nc,
                        (const double*)g->cap_psi, (const double*)(g->small + SM_CAPC), g->psi_ext);
                 if (g->outer) {   // the responses' ring values move the free-space ring
@@ -1407,10 +1412,7 @@ struct Solver {
                     launch("cap_update", 0.0, 0.0, k_cap_update, (unsigned)((nr + 255) / 256), 256, 0, s, nr, nc,
                            (const double*)g->cap_ring, (const double*)(g->small + SM_CAPC), g->fs_ring);
                 }
-                launch("add_psibar", 0.0, 0.0, k_add_psibar, 1, 64, 0, s, nc, (const int*)(g->d_int + DI_CIRC),
-                       (const double*)(g->small + SM_CAPP), psibar);
-                IIM_CHECK(residual_launch());
-                launch("final_rel", 0.0, 0.0, k_final_rel, 1, 1, 0, s, di(), g->small);
+                IIM_CHECK(residual_launch(RefCtl{CTL_FINAL, 0, 0.0, 0, 0}));
             }
             const long n = (long)g->NX * g->NY;
             launch("velocity_f64", 0.0, 0.0, k_velocity, (unsigned)((n + 255) / 256), 256, 0, s, g->NX, g->NY,
@@ -1798,11 +1800,7 @@ static iim_status poisson_solve(iim_geometry g, const double* omega, const doubl
     // ||f||: residual at psi = 0 (ghosts from the boundary data only)
     double res2 = 0.0, cerr = 0.0;
     int fallback = 0;
-    launch("init_psi", 0.0, 0.0, k_init_psi, (unsigned)((npad + 255) / 256), 256, 0, s, g->NX, g->NY, nullptr,
-           g->node_class, g->psi_ext);
-    if (g->outer) IIM_TRY(cudaMemsetAsync(g->fs_ring, 0, sizeof(double) * 2 * (g->nx + g->ny), s));
-    if (g->nb > 0) launch("init_psibar", 0.0, 0.0, k_init_psibar, 1, 64, 0, s, g->nb, g->body_circ, psibar, 0, psibar);
-    IIM_LAUNCHED();
+    IIM_CHECK(S.init_solve());
     IIM_CHECK(S.residual(&res2, &cerr));
     if (!std::isfinite(res2)) return IIM_ERR_NONFINITE;
     const double fnorm = std::sqrt(res2);

@@ -126,12 +126,13 @@ __device__ __forceinline__ void scan_segment_maps(const T* sD, T* sB, bool rever
 
 // Tridiagonal column pass of one field in the padded layout (NY rows of ld = NX + 1 slots;
 // element (row j, data column c) at j * ld + c + 1; slot 0 of a row is a zero pad).  Rows
-// outside [in0, in1] are zero on input and not read; only rows [out0, out1] are written.  Block
+// outside [in0, in1] are zero on input and not read; only rows [out0, out1] are written, to `out` (which
+// may be buf).  Block
 // blockIdx.x: padded columns [CW blockIdx.x, CW blockIdx.x + CW); NT threads; dynamic shared
 // memory scan_smem<T, CW, NT>(NY).
 template <typename T, int CW, int NT>
 __device__ __forceinline__ void cols_scan_body(int NX, int NY, int ld, int in0, int in1, int out0, int out1,
-                                               T* __restrict__ buf, ScanTab<T> t) {
+                                               const T* buf, T* out, ScanTab<T> t) {
     constexpr int S = NT / CW;
     constexpr int V = 16 / (int)sizeof(T), PPR = CW / V;   // elements per 16-byte piece, pieces per row
     using VT = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
@@ -271,7 +272,7 @@ __device__ __forceinline__ void cols_scan_body(int NX, int NY, int ld, int in0, 
     const int nst = (out1 - out0 + 1) * PPR;
     for (int e = threadIdx.x; e < nst; e += NT) {
         const int j = out0 + e / PPR, q = e % PPR;
-        *reinterpret_cast<VT*>(buf + (size_t)j * ld + P0 + q * V) = *reinterpret_cast<const VT*>(tile + j * CW + q * V);
+        *reinterpret_cast<VT*>(out + (size_t)j * ld + P0 + q * V) = *reinterpret_cast<const VT*>(tile + j * CW + q * V);
     }
 }
 
