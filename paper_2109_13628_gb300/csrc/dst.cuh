@@ -662,6 +662,7 @@ template <typename T, int WARPS, int FP>
 __global__ void __launch_bounds__(WARPS * 32)
 k_rows_fwd(int NX, int NY, int n, int logn, const double* __restrict__ dense, const double* __restrict__ ring,
            double ih2, const cpx<T>* __restrict__ g_tw, T* __restrict__ out) {
+    pdl_wait();
     constexpr bool PADL = padded_lines(FP);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const cpx<T>* s_tw = block_twiddles<FP, T>(smem_raw, g_tw, n);
@@ -790,6 +791,7 @@ __global__ void __launch_bounds__(C * line_threads(FP), sizeof(T) == 4 ? 2 : 1)
 k_cols(int NX, int NY, int n, int logn, int in0, int in1, int out0, int out1, T* __restrict__ buf,
        const T* __restrict__ lam_x, const T* __restrict__ lam_y, T norm, const cpx<T>* __restrict__ g_tw,
        const int* __restrict__ stop, long fstride) {
+    pdl_wait();
     if (stop && *stop) return;
     cols_body<T, C, FP>(NX, NY, n, logn, in0, in1, out0, out1, buf + (long)blockIdx.y * fstride, lam_x, lam_y, norm,
                         g_tw);
@@ -800,6 +802,7 @@ template <typename T, int WARPS, int FP>
 __global__ void __launch_bounds__(WARPS * 32)
 k_rows_inv(int NX, int NY, int n, int logn, const T* __restrict__ in, double* __restrict__ out,
            const cpx<T>* __restrict__ g_tw) {
+    pdl_wait();
     constexpr bool PADL = padded_lines(FP);
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const cpx<T>* s_tw = block_twiddles<FP, T>(smem_raw, g_tw, n);

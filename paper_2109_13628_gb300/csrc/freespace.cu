@@ -112,6 +112,7 @@ __device__ double lgf_far(int m, int n) {
 
 // G[n * (M + 1) + m] for 0 <= m <= M, 0 <= n <= N
 __global__ void k_lgf_table(int M, int N, GaussRule R, double* __restrict__ G) {
+    pdl_wait();
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= (long)(M + 1) * (N + 1)) return;
     const int m = (int)(k % (M + 1)), n = (int)(k / (M + 1));
@@ -162,6 +163,7 @@ iim_status lgf_table(int nx, int ny, const double** out) {
 template <typename T>
 __global__ void k_bnd_cols(int NX, int NY, int nx, const T* __restrict__ buf, double* __restrict__ vl,
                            double* __restrict__ vr, const int* __restrict__ stop) {
+    pdl_wait();
     if (stop && *stop) return;
     const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= NY) return;
@@ -190,6 +192,7 @@ __global__ void __launch_bounds__(BLOCK)
 k_ring_conv(int nx, int ny, const double* __restrict__ G, int ld, int sym, const double* __restrict__ bnd,
             const double* __restrict__ vl, const double* __restrict__ vr, double* __restrict__ rho,
             const int* __restrict__ stop) {
+    pdl_wait();
     if (stop && *stop) return;
     const int t = blockIdx.x;
     int xi, xj;
@@ -219,6 +222,7 @@ k_ring_conv(int nx, int ny, const double* __restrict__ G, int ld, int sym, const
 // y += a x over n values (ring updates)
 __global__ void k_ring_add(int n, double a, const double* __restrict__ x, double* __restrict__ y,
                            const int* __restrict__ stop) {
+    pdl_wait();
     if (stop && *stop) return;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) y[k] += a * x[k];
@@ -240,6 +244,7 @@ __global__ void __launch_bounds__(BLOCK)
 k_ring_residual(int nx, int ny, double h2, const double* __restrict__ G, int ld, int sym,
                 const double* __restrict__ plane, const double* __restrict__ psi, const double* __restrict__ ring,
                 double* __restrict__ rres) {
+    pdl_wait();
     const int t = blockIdx.x;
     int xi, xj;
     if (t <= nx) { xi = t; xj = 0; }
@@ -276,6 +281,7 @@ k_ring_residual(int nx, int ny, double h2, const double* __restrict__ G, int ld,
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 k_ring_res_norm(int n, const double* __restrict__ rres, double scale2, double* __restrict__ res2) {
+    pdl_wait();
     double acc = 0.0;
     for (int t = threadIdx.x; t < n; t += BLOCK) acc += rres[t] * rres[t];
     acc = block_sum<BLOCK>(acc);

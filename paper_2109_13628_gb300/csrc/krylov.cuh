@@ -505,15 +505,18 @@ template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads)
 k_start(int ns, const double* __restrict__ r, double* __restrict__ v0, KLayout L, double* __restrict__ K,
         int* __restrict__ di, int init_maxit, KTol tol, double* __restrict__ small) {
+    pdl_wait();
     start_cluster_body<CL>(ns, r, v0, L, K, di, init_maxit, tol, small);
 }
 template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads)
 k_arnoldi(int* __restrict__ di, double* __restrict__ V, int ns, KLayout L, double* __restrict__ K) {
+    pdl_wait();
     arnoldi_cluster_body<CL>(di, V, ns, L, K);
 }
 template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads) k_krylov(KrylovArgs g) {
+    pdl_wait();
     krylov_body<CL>(g);
 }
 
@@ -562,13 +565,15 @@ inline iim_status launch_cluster(const char* name, double bytes, void (*k)(KArgs
     cfg.blockDim = dim3(kKrylovThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
-    cudaLaunchAttribute at = {};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = cl;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = chain_launch(s) ? 2 : 1;
     IIM_TRY(cudaLaunchKernelEx(&cfg, k, args...));
     return IIM_OK;
 }

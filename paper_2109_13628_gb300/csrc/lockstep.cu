@@ -97,6 +97,7 @@ __device__ __forceinline__ VecArg ls_vec(const LsProb& p, int mode) {
 template <typename T, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
 kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, int tri, const cpx<T>* __restrict__ tab) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     const bool dense = mode == M_RHS || mode == M_RECOVER;
@@ -112,6 +113,7 @@ kb_rows_fwd(const LsProb* __restrict__ P, int mode, int gate, int tri, const cpx
 template <typename T, int C, int FP>
 __global__ void __launch_bounds__(C * line_threads(FP), sizeof(T) == 4 ? 2 : 1)
 kb_cols(const LsProb* __restrict__ P, int mode, int gate, T norm, const cpx<T>* __restrict__ tw) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
@@ -130,6 +132,7 @@ __device__ __forceinline__ const ScanTab<T>& ls_scan(const LsProb& p) {
 
 template <typename T, int CW, int NT>
 __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4) kb_cols_scan(const LsProb* __restrict__ P, int mode, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (mode != M_RECOVER && p.na == 0)) return;
     int in0 = 0, in1 = p.NY - 1, out0 = p.jo0, out1 = p.jo1;
@@ -145,6 +148,7 @@ __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4) kb_cols_scan(const LsP
 template <typename T, int MODE, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
 kb_rows_inv(const LsProb* __restrict__ P, int from_psi, int gate, const cpx<T>* __restrict__ tab) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (MODE == INV_STORE_T && p.na == 0)) return;
     const int row0 = MODE == INV_STORE_T ? p.jo0 : 0, nrows = MODE == INV_STORE_T ? p.jo1 - p.jo0 + 1 : p.NY;
@@ -159,6 +163,7 @@ kb_rows_inv(const LsProb* __restrict__ P, int from_psi, int gate, const cpx<T>* 
 // the Schur operator's output column (+ circulation rows) of the iteration / restart.
 template <typename T, int BLOCK>
 __global__ void __launch_bounds__(BLOCK) kb_gather(const LsProb* __restrict__ P, int mode, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate)) return;
     const int nga = (p.na + BLOCK / 32 - 1) / (BLOCK / 32);
@@ -178,6 +183,7 @@ __global__ void __launch_bounds__(BLOCK) kb_gather(const LsProb* __restrict__ P,
 // dense inner operator V_{j+1} = S z_j (iteration) or V_2 = S V_1 (restart).
 enum { MV_PRECOND = 0, MV_S_ITER = 1, MV_S_RESTART = 2 };
 __global__ void __launch_bounds__(kDenseWarps * 32) kb_matvec(const LsProb* __restrict__ P, int op, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || p.ns == 0) return;
     const long ns = p.ns, ld = dense_ld(p.ns);
@@ -192,6 +198,7 @@ __global__ void __launch_bounds__(kDenseWarps * 32) kb_matvec(const LsProb* __re
 // ------------------------------------------------------------------------- Krylov kernels
 template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads) kb_arnoldi(const LsProb* P, KLayout L) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (p.ns == 0) return;
     arnoldi_cluster_body<CL>(p.di, p.V, p.ns, L, p.H);
@@ -200,6 +207,7 @@ __global__ void __launch_bounds__(kKrylovThreads) kb_arnoldi(const LsProb* P, KL
 // The whole correction solve with the dense operator of every refining problem, one cluster each.
 template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads) kb_krylov(const LsProb* P, KLayout L, KTol tol, int max_iter) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (!p.di[DI_RACT] || p.ns == 0) return;   // uniform over the cluster
     krylov_body<CL>(KrylovArgs{p.ns, dense_ld(p.ns), p.pc_M, p.pc_S, p.bvec, p.xsol, L, p.H, p.di,
@@ -212,6 +220,7 @@ __global__ void __launch_bounds__(kKrylovThreads) kb_krylov(const LsProb* P, KLa
 template <int CL>
 __global__ void __launch_bounds__(kKrylovThreads)
 kb_start(const LsProb* P, KLayout L, int restart, int max_iter, KTol tol) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (!restart) {
         if (!p.di[DI_RACT] || p.ns == 0) {
@@ -226,6 +235,7 @@ kb_start(const LsProb* P, KLayout L, int restart, int max_iter, KTol tol) {
 }
 
 __global__ void __launch_bounds__(kUpdateRows) kb_update(const LsProb* __restrict__ P, KLayout L) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (!p.di[DI_CACT] || (int)blockIdx.x * kUpdateRows >= p.ns) return;
     update_body(p.di, L, p.H, p.Z + p.ns, p.ns, p.xsol);
@@ -235,6 +245,7 @@ __global__ void __launch_bounds__(kUpdateRows) kb_update(const LsProb* __restric
 // before the restart's operator application; V_2 = b - V_2 after it.
 enum { V_ZERO_X = 0, V_RESTART_PREP = 1, V_RESTART_RES = 2 };
 __global__ void kb_vec(const LsProb* __restrict__ P, int op, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate)) return;
     const long ns = p.ns;
@@ -248,6 +259,7 @@ __global__ void kb_vec(const LsProb* __restrict__ P, int op, int gate) {
 
 // ------------------------------------------------------------------------- field kernels
 __global__ void kb_init(const LsProb* __restrict__ P) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < (long)p.nx * p.NY / 2) reinterpret_cast<double2*>(p.psi_ext)[k] = make_double2(0.0, 0.0);
@@ -255,6 +267,7 @@ __global__ void kb_init(const LsProb* __restrict__ P) {
 }
 
 __global__ void kb_ghost(const LsProb* __restrict__ P, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || p.nminus == 0) return;
     ghost_body(p.nminus, p.minus_node, p.gh_ptr, p.gh_idx, p.gh_w, p.psi_b, p.psibar, p.cp_body, p.psi_ext);
@@ -262,6 +275,7 @@ __global__ void kb_ghost(const LsProb* __restrict__ P, int gate) {
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) kb_residual(const LsProb* __restrict__ P, int gate) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate)) return;
     residual_body<BLOCK>(p.NX, p.NY, p.ih2, p.psi_ext, p.omega, p.cls, p.ring, p.res, p.partial);
@@ -269,6 +283,7 @@ __global__ void __launch_bounds__(BLOCK) kb_residual(const LsProb* __restrict__ 
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) kb_finish_residual(const LsProb* __restrict__ P, int gate, int nparts) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, gate) || (int)blockIdx.x >= finish_blocks(p.ncirc)) return;
     finish_body<BLOCK>(FinishArgs{nparts, p.partial, p.nx, p.psi_ext, p.res, p.regions, p.di, p.ncirc, p.gamma, p.ih2, p.small,
@@ -276,6 +291,7 @@ __global__ void __launch_bounds__(BLOCK) kb_finish_residual(const LsProb* __rest
 }
 
 __global__ void kb_cap_coef(const LsProb* __restrict__ P) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, G_CAP)) return;
     const int nc = p.ncirc;
@@ -284,24 +300,28 @@ __global__ void kb_cap_coef(const LsProb* __restrict__ P) {
 }
 
 __global__ void kb_cap_update(const LsProb* __restrict__ P) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, G_CAP)) return;
     cap_update_body((long)p.nx * p.NY, p.ncirc, p.cap_psi, p.small + SM_CAPC, p.psi_ext);
 }
 
 __global__ void kb_final_rel(const LsProb* __restrict__ P) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if (ls_off(p, G_CAP)) return;
     final_rel_body(p.di, p.small);
 }
 
 __global__ void kb_velocity(const LsProb* __restrict__ P) {
+    pdl_wait();
     const LsProb& p = P[blockIdx.z];
     if ((long)blockIdx.x * blockDim.x >= (long)p.NX * p.NY) return;
     velocity_body(p.NX, p.NY, 0.5 / p.h, p.psi_ext, p.cls, p.ring, p.psi_out, p.ux_out, p.uy_out);
 }
 
 __global__ void kb_records(const LsProb* __restrict__ P, int n, KLayout L, LsRec* __restrict__ out) {
+    pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const LsProb& p = P[k];
@@ -326,6 +346,7 @@ __device__ __forceinline__ void ls_decide(int any, cudaGraphConditionalHandle h,
 
 __global__ void kb_ref_init(const LsProb* __restrict__ P, int n, double rtol, cudaGraphConditionalHandle h, int* flag,
                             int* cnt) {
+    pdl_wait();
     int go_any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;
@@ -350,6 +371,7 @@ __global__ void kb_ref_init(const LsProb* __restrict__ P, int n, double rtol, cu
 
 __global__ void kb_cyc_begin(const LsProb* __restrict__ P, int n, int max_iter, cudaGraphConditionalHandle h,
                              int* flag) {
+    pdl_wait();
     int any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;
@@ -370,6 +392,7 @@ __global__ void kb_cyc_begin(const LsProb* __restrict__ P, int n, int max_iter, 
 }
 
 __global__ void kb_it_begin(const LsProb* __restrict__ P, int n, cudaGraphConditionalHandle h, int* flag) {
+    pdl_wait();
     int any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;
@@ -383,6 +406,7 @@ __global__ void kb_it_begin(const LsProb* __restrict__ P, int n, cudaGraphCondit
 
 __global__ void kb_loop_ctl(const LsProb* __restrict__ P, int n, int cap, cudaGraphConditionalHandle h, int* flag,
                             int* cnt) {
+    pdl_wait();
     int any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;
@@ -401,6 +425,7 @@ __global__ void kb_loop_ctl(const LsProb* __restrict__ P, int n, int cap, cudaGr
 
 __global__ void kb_cyc_ctl(const LsProb* __restrict__ P, int n, int cap, cudaGraphConditionalHandle hc,
                            cudaGraphConditionalHandle hr, int* flag, int* cnt) {
+    pdl_wait();
     int any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;
@@ -432,6 +457,7 @@ __global__ void kb_cyc_ctl(const LsProb* __restrict__ P, int n, int cap, cudaGra
 
 __global__ void kb_ref_ctl(const LsProb* __restrict__ P, int n, double rtol, int max_refine, int max_iter,
                            cudaGraphConditionalHandle h, int* flag, int* cnt) {
+    pdl_wait();
     int any = 0;
     for (int k = threadIdx.x; k < n; k += blockDim.x) {
         int* di = P[k].di;

@@ -32,6 +32,7 @@ size_t gj_scratch_floats(int n) { return 2 * (size_t)GJ_LDW * n + (size_t)GJ_B *
 
 __global__ void k_gj_panel_init(const float* __restrict__ A, long lda, int n, int k0, int bb, float* __restrict__ W,
                                 const int* __restrict__ info) {
+    pdl_wait();
     if (*info) return;
     const long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (e >= (long)n * GJ_LDW) return;
@@ -55,6 +56,7 @@ template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK)
 k_gj_panel_step(const float* __restrict__ Win, float* __restrict__ Wout, int n, int k0, int j, int* __restrict__ perm,
                 int* __restrict__ info) {
+    pdl_wait();
     if (*info) return;
     const int r0 = k0 + j;
     __shared__ float sv[BLOCK];
@@ -113,6 +115,7 @@ k_gj_panel_step(const float* __restrict__ Win, float* __restrict__ Wout, int n, 
 // thread per column.
 __global__ void k_gj_swap_rows(float* __restrict__ A, long lda, int k0, int bb, int c0, int m,
                                const int* __restrict__ perm, float* __restrict__ T, long ldt, const int* __restrict__ info) {
+    pdl_wait();
     if (*info) return;
     __shared__ int sp[GJ_B];
     if (threadIdx.x < bb) sp[threadIdx.x] = perm[threadIdx.x];
@@ -141,6 +144,7 @@ constexpr int GJ_TILE = 128;
 __global__ void __launch_bounds__(256, 2)
 k_gj_update(float* __restrict__ A, long lda, int n, int c0, int m, const float* __restrict__ W, int k0, int bb,
             const float* __restrict__ T, long ldt, const int* __restrict__ info) {
+    pdl_wait();
     if (*info) return;
     extern __shared__ float4 gj_smem4[];
     float* Gs = reinterpret_cast<float*>(gj_smem4);   // [GJ_B][GJ_TILE]: Gs[t][r]
@@ -203,6 +207,7 @@ k_gj_update(float* __restrict__ A, long lda, int n, int c0, int m, const float* 
 }
 
 __global__ void k_set_identity_aug(float* __restrict__ A, int n) {
+    pdl_wait();
     const long ld = 2L * n;
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= (long)n * n) return;
@@ -214,6 +219,7 @@ __global__ void __launch_bounds__(kDenseWarps * 32)
 k_dense_matvec(int n, const float* __restrict__ M, long ld, const double* __restrict__ vbase,
                const int* __restrict__ jidx, long vstride, double* __restrict__ out, long ostride,
                const int* __restrict__ stop) {
+    pdl_wait();
     dense_matvec_body(n, M, ld, vbase, jidx, vstride, out, ostride, stop);
 }
 
@@ -265,12 +271,14 @@ iim_status dense_matvec(int n, const float* M, const double* v, const int* jidx,
 }
 
 __global__ void k_unit_vector(int n, int j, double* __restrict__ v) {
+    pdl_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < n) v[e] = (e == j) ? 1.0 : 0.0;
 }
 
 // column j of the left half of the augmented array from an FP64 vector
 __global__ void k_store_column(int n, int j, const double* __restrict__ v, float* __restrict__ A) {
+    pdl_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < n) A[(long)e * 2 * n + j] = (float)v[e];
 }

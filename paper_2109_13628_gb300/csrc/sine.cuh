@@ -95,6 +95,7 @@ __device__ __forceinline__ cpx<T> sine_root(const cpx<T>* __restrict__ g_tw, int
 
 template <typename T>
 __global__ void k_sine_region(const cpx<T>* __restrict__ g_tw, int n, int logn, cpx<T>* __restrict__ out) {
+    pdl_wait();
     const int M = n / 4, shift = kTwLog - logn;
     const T hf = T(0.5);
     for (int e = threadIdx.x; e < 5 * M; e += blockDim.x) {
@@ -367,6 +368,7 @@ k_sine_rows_fwd(int NX, int NY, int n, int row0, int nrows, const double* __rest
                 const double* __restrict__ ring, double ih2, const int* __restrict__ aff_row_ptr,
                 const int* __restrict__ aff_node, VecArg gam, double gsign, const cpx<T>* __restrict__ tab,
                 T* __restrict__ out, const int* __restrict__ stop, long dfs, long ofs) {
+    pdl_wait();
     if (stop && *stop) return;
     sine_rows_fwd_body<T, N, L>(NX, NY, n, row0, nrows, dense ? dense + (long)blockIdx.y * dfs : nullptr, dld, doff, ring,
                              ih2, aff_row_ptr, aff_node, gam, gsign, tab, out + (long)blockIdx.y * ofs);
@@ -454,6 +456,7 @@ __global__ void __launch_bounds__((Sine<N, L>::kBlock))
 k_sine_rows_inv(int NX, int NY, int n, int row0, int nrows, const T* in, T* outT,
                 double* __restrict__ out64, int old, int ooff, const uint8_t* __restrict__ cls,
                 const cpx<T>* __restrict__ tab, const int* __restrict__ stop, long fstride, PsibarStep ps) {
+    pdl_wait();
     if (stop && *stop) return;
     if (MODE == INV_ACCUM_FLUID && blockIdx.x == 0) ps.apply();
     sine_rows_inv_body<T, MODE, N, L>(NX, NY, n, row0, nrows, in + (long)blockIdx.y * fstride,

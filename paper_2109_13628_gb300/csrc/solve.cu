@@ -69,6 +69,7 @@ __device__ cpx<float> g_sine32[sine_total()];
 
 template <typename T, int FP>
 __global__ void k_twiddle_region(const cpx<T>* __restrict__ g_tw, int n, int logn, cpx<T>* __restrict__ out) {
+    pdl_wait();
     load_twiddles<FP>(out, g_tw, n, logn);
 }
 
@@ -256,6 +257,7 @@ template <typename T, int CW, int NT>
 __global__ void __launch_bounds__(NT, NT == 1024 ? 2 : 4)
 k_cols_scan(int NX, int NY, int ld, int in0, int in1, int out0, int out1, const T* buf, T* out, ScanTab<T> t,
             const int* __restrict__ stop, long fstride) {
+    pdl_wait();
     if (stop && *stop) return;
     cols_scan_body<T, CW, NT>(NX, NY, ld, in0, in1, out0, out1, buf + (long)blockIdx.y * fstride,
                               out + (long)blockIdx.y * fstride, t);
@@ -376,6 +378,7 @@ k_gather(int na, int nga, const int* __restrict__ ptr, const int* __restrict__ i
          const T* __restrict__ psi, const int* __restrict__ cp_body, const int* __restrict__ body_circ,
          const int* __restrict__ aff_body, VecArg vin, int use_xc, double* __restrict__ outb, const int* __restrict__ jidx,
          long stride, const int* __restrict__ stop) {
+    pdl_wait();
     gather_body<T, BLOCK>(na, nga, ptr, idx, w, psi, cp_body, body_circ, aff_body, vin, use_xc, outb, jidx, stride, stop);
 }
 
@@ -386,6 +389,7 @@ k_gather(int na, int nga, const int* __restrict__ ptr, const int* __restrict__ i
 template <typename T>
 __global__ void k_unit_rows(int nx, int logn, int rmin, int rmax, int j0, int na, const int* __restrict__ aff_node,
                             const cpx<T>* __restrict__ g_tw, T* __restrict__ out, long fstride) {
+    pdl_wait();
     const int f = blockIdx.y, a = j0 + f;
     T* o = out + (long)f * fstride;
     int prow = -1, slot = 0;
@@ -416,6 +420,7 @@ __global__ void __launch_bounds__(BLOCK)
 k_gather_unit(int na, int nga, int ncirc, const int* __restrict__ ptr, const int* __restrict__ idx,
               const double* __restrict__ w, const T* __restrict__ psi, long fstride, int j0,
               const int* __restrict__ aff_body, const int* __restrict__ body_circ, float* __restrict__ A, long lda) {
+    pdl_wait();
     const int f = blockIdx.y, j = j0 + f;
     if (j >= na) return;
     if ((int)blockIdx.x < nga) {
@@ -438,6 +443,7 @@ k_gather_unit(int na, int nga, int ncirc, const int* __restrict__ ptr, const int
 __global__ void k_ghost(int nm, const int* __restrict__ minus_node, const int* __restrict__ ptr, const int* __restrict__ idx,
                         const double* __restrict__ w, const double* __restrict__ psi_b, const double* __restrict__ psibar,
                         const int* __restrict__ cp_body, double* __restrict__ psi) {
+    pdl_wait();
     ghost_body(nm, minus_node, ptr, idx, w, psi_b, psibar, cp_body, psi);
 }
 
@@ -447,6 +453,7 @@ template <int BLOCK>
 __global__ void k_residual(int NX, int NY, double ih2, const double* __restrict__ psi, const double* __restrict__ omega,
                            const uint8_t* __restrict__ cls, const double* __restrict__ ring, double* __restrict__ res,
                            double* __restrict__ partial) {
+    pdl_wait();
     residual_body<BLOCK>(NX, NY, ih2, psi, omega, cls, ring, res, partial);
 }
 
@@ -463,12 +470,14 @@ __device__ void ref_control(const RefCtl& c, int* di, double* small);
 
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_finish(FinishArgs a, RefCtl c) {
+    pdl_wait();
     if (finish_body<BLOCK>(a, blockIdx.x) && c.mode != CTL_NONE) ref_control(c, a.di, a.small);
 }
 
 // out = sum of the partial sums (one block).
 template <int BLOCK>
 __global__ void __launch_bounds__(BLOCK) k_sum_parts(int n, const double* __restrict__ partial, double* __restrict__ out) {
+    pdl_wait();
     double s = 0.0;
     for (int b = threadIdx.x; b < n; b += BLOCK) s += partial[b];
     s = block_sum<BLOCK>(s);
@@ -478,6 +487,7 @@ __global__ void __launch_bounds__(BLOCK) k_sum_parts(int n, const double* __rest
 // Start of a solve from psi = 0: the field zeroed, circulation bodies' constants zeroed.
 __global__ void k_init_solve(long n2, double2* __restrict__ psi, int nb, const int* __restrict__ body_circ,
                              double* __restrict__ psibar) {
+    pdl_wait();
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n2) psi[k] = make_double2(0.0, 0.0);
     if (blockIdx.x == 0 && nb > 0) init_psibar_body(nb, body_circ, psibar, 0, psibar);
@@ -485,16 +495,19 @@ __global__ void k_init_solve(long n2, double2* __restrict__ psi, int nb, const i
 
 __global__ void k_init_psi(int NX, int NY, const double* __restrict__ guess, const uint8_t* __restrict__ cls,
                            double* __restrict__ psi) {
+    pdl_wait();
     init_psi_body(NX, NY, guess, cls, psi);
 }
 
 __global__ void k_add_psibar(int ncirc, const int* __restrict__ circ_ids, const double* __restrict__ x, double* __restrict__ psibar) {
+    pdl_wait();
     add_psibar_body(ncirc, circ_ids, x, psibar);
 }
 
 // psi_ext += sum_l coef[l] resp_l (padded fields, npad values each): the capacitance correction.
 __global__ void k_cap_update(long npad, int ncirc, const double* __restrict__ resp, const double* __restrict__ coef,
                              double* __restrict__ psi) {
+    pdl_wait();
     cap_update_body(npad, ncirc, resp, coef, psi);
 }
 
@@ -503,6 +516,7 @@ __global__ void k_cap_update(long npad, int ncirc, const double* __restrict__ re
 __global__ void k_velocity(int NX, int NY, double inv2h, const double* __restrict__ psi, const uint8_t* __restrict__ cls,
                            const double* __restrict__ ring, double* __restrict__ psi_out, double* __restrict__ ux,
                            double* __restrict__ uy) {
+    pdl_wait();
     velocity_body(NX, NY, inv2h, psi, cls, ring, psi_out, ux, uy);
 }
 
@@ -510,6 +524,7 @@ __global__ void k_velocity(int NX, int NY, double inv2h, const double* __restric
 
 template <int BLOCK>
 __global__ void k_sumsq(const double* __restrict__ w, int ns, double* __restrict__ partial) {
+    pdl_wait();
     double acc = 0.0;
     for (int e = blockIdx.x * BLOCK + threadIdx.x; e < ns; e += gridDim.x * BLOCK) acc += w[e] * w[e];
     acc = block_sum<BLOCK>(acc);
@@ -520,6 +535,7 @@ __global__ void k_sumsq(const double* __restrict__ w, int ns, double* __restrict
 // V_0 = r / ||r||, g = (beta, 0, ...), j = 0, stop unless there is work left
 __global__ void k_start_cycle(int ns, const double* __restrict__ r, double* __restrict__ v0, KLayout L, double* __restrict__ K,
                               int nparts, const double* __restrict__ partial, int* __restrict__ di) {
+    pdl_wait();
     double s = 0.0;
     for (int b = 0; b < nparts; ++b) s += partial[b];
     const double beta = sqrt(s);
@@ -542,18 +558,21 @@ __global__ void k_start_cycle(int ns, const double* __restrict__ r, double* __re
 __global__ void __launch_bounds__(kUpdateRows)
 k_update(const int* __restrict__ di, KLayout L, const double* __restrict__ K, const double* __restrict__ B, int ns,
          double* __restrict__ x) {
+    pdl_wait();
     update_body(di, L, K, B, ns, x);
 }
 
 __global__ void k_axpby(int n, double a, const double* __restrict__ x, double b, const double* __restrict__ y,
                         double* __restrict__ out) {
+    pdl_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < n) out[e] = a * x[e] + b * y[e];
 }
 
-__global__ void k_set_int(int* __restrict__ p, int v) { *p = v; }
+__global__ void k_set_int(int* __restrict__ p, int v) { pdl_wait(); *p = v; }
 
 __global__ void k_negate(int n, double* __restrict__ v) {
+    pdl_wait();
     const int i = threadIdx.x;
     if (i < n) v[i] = -v[i];
 }
@@ -564,6 +583,7 @@ __global__ void k_negate(int n, double* __restrict__ v) {
 template <int BLOCK>
 __global__ void k_seed_scale(int ns, const double* __restrict__ b, double* __restrict__ sx, double* __restrict__ x,
                              double* __restrict__ out) {
+    pdl_wait();
     __shared__ double c_sh;
     double d = 0.0, q = 0.0;
     for (int e = threadIdx.x; e < ns; e += BLOCK) {
@@ -594,6 +614,7 @@ __global__ void k_psibar_estimate(int ncp, int nx, int ny, const int* __restrict
                                   const int* __restrict__ cp_body, const int* __restrict__ body_circ,
                                   const uint8_t* __restrict__ cls, const double* __restrict__ psi,
                                   const double* __restrict__ psi_b, double* __restrict__ out, double sgn) {
+    pdl_wait();
     const int c = blockIdx.x;
     double s = 0.0, cnt = 0.0;
     for (int k = threadIdx.x; k < ncp; k += BLOCK) {
@@ -624,6 +645,7 @@ __global__ void k_psibar_estimate(int ncp, int nx, int ny, const int* __restrict
 
 __global__ void k_gmres_init(int* __restrict__ di, int maxit, double* __restrict__ K, KLayout L, const double* __restrict__ b2,
                              double tol) {
+    pdl_wait();
     di[DI_J] = 0;
     di[DI_STOP] = 0;
     di[DI_IT] = 0;
@@ -641,6 +663,7 @@ __global__ void k_gmres_init(int* __restrict__ di, int maxit, double* __restrict
 // cap (restart length + 2, never reached while the kernels follow their stopping rule) makes
 // the loop finite in any case; hitting it sets the stop flag and an error flag for the host.
 __global__ void k_loop_ctl(cudaGraphConditionalHandle h, int* __restrict__ di, int cap) {
+    pdl_wait();
     const int c = ++di[DI_LOOP];
     if (!di[DI_STOP] && c >= cap) {
         di[DI_STOP] = 1;
@@ -679,11 +702,12 @@ __device__ void ref_control(const RefCtl& c, int* di, double* small) {
     }
 }
 // The same after the ring rows of a free-space residual.
-__global__ void k_ref_control(RefCtl c, int* __restrict__ di, double* __restrict__ small) { ref_control(c, di, small); }
+__global__ void k_ref_control(RefCtl c, int* __restrict__ di, double* __restrict__ small) { pdl_wait(); ref_control(c, di, small); }
 
 // After gmres_init: the Krylov budget left for this correction; cycle counter reset; the cycle
 // loop entered unless the start already stopped (converged or no budget).
 __global__ void k_cyc_begin(cudaGraphConditionalHandle h, int* __restrict__ di, int max_iter) {
+    pdl_wait();
     const int left = max_iter - di[DI_ITS];
     di[DI_MAXIT] = left > 1 ? left : 1;
     di[DI_CYC] = 0;
@@ -693,6 +717,7 @@ __global__ void k_cyc_begin(cudaGraphConditionalHandle h, int* __restrict__ di, 
 
 // Start of a cycle: the iteration loop is entered unless the stop flag is set.
 __global__ void k_it_begin(cudaGraphConditionalHandle h, int* __restrict__ di) {
+    pdl_wait();
     di[DI_LOOP] = 0;
     cudaGraphSetConditional(h, di[DI_STOP] ? 0 : 1);
 }
@@ -701,6 +726,7 @@ __global__ void k_it_begin(cudaGraphConditionalHandle h, int* __restrict__ di) {
 // converged, out of budget, or capped (cap: max_iter / restart + 2 cycles; reaching it without
 // one of the others sets an error flag).
 __global__ void k_cyc_ctl(cudaGraphConditionalHandle hc, cudaGraphConditionalHandle hr, int* __restrict__ di, int cap) {
+    pdl_wait();
     const int c = ++di[DI_CYC];
     ++di[DI_CYCS];
     bool done = di[DI_CONV] || di[DI_IT] >= di[DI_MAXIT] || di[DI_LOOPERR];
@@ -716,6 +742,7 @@ __global__ void k_cyc_ctl(cudaGraphConditionalHandle hc, cudaGraphConditionalHan
 __global__ void k_cap_coef(int nc, const double* __restrict__ rc, const double* __restrict__ cinv,
                            const double* __restrict__ pb, double h2, double* __restrict__ coef,
                            const int* __restrict__ circ_ids, double* __restrict__ psibar) {
+    pdl_wait();
     cap_coef_body(nc, rc, cinv, pb, h2, coef, circ_ids, psibar);
 }
 
@@ -2207,6 +2234,7 @@ static double* g_noalloc_ptr[64];
 
 // Eigenvalues of the 1D three-point operators (x modes, then y modes), in FP64 or FP32.
 __global__ void k_box_eigs(int NX, int NY, int nx, int ny, double h, int as_float, double* lam) {
+    pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= NX + NY) return;
     const double v = k < NX ? (2.0 - 2.0 * cospi((double)(k + 1) / nx)) / (h * h)

@@ -31,6 +31,19 @@ static cudaEvent_t pool_event() {
 }
 
 void set_capture(bool on) { t_capture = on; }
+bool chain_launch(cudaStream_t s) {
+    if (!t_capture) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t n = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, nullptr, nullptr, &deps, nullptr, &n) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    cudaGraphNodeType type = cudaGraphNodeTypeEmpty;
+    return st == cudaStreamCaptureStatusActive && n == 1 && cudaGraphNodeGetType(deps[0], &type) == cudaSuccess &&
+           type == cudaGraphNodeTypeKernel;
+}
 bool profiling_active() { return t_prof; }
 void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 
