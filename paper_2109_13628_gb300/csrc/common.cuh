@@ -275,10 +275,10 @@ template <typename T>
 iim_status launch_bnd_cols(int NX, int NY, int nx, const T* buf, double* vl, double* vr, const int* stop,
                            cudaStream_t s);
 iim_status launch_ring_conv(int nx, int ny, const double* G, int ld, int sym, const double* bnd, const double* vl,
-                            const double* vr, double* rho, const int* stop, cudaStream_t s);
-iim_status launch_ring_add(int n, double a, const double* x, double* y, const int* stop, cudaStream_t s);
+                            const double* vr, const double* sub, double* rho, double* ring, const int* stop,
+                            cudaStream_t s);
 iim_status launch_ring_residual(int nx, int ny, double h, const double* G, int ld, int sym, const double* plane,
-                                const double* psi, const double* ring, double* rres, double* res2, cudaStream_t s);
+                                const double* psi, const double* ring, double* rres, cudaStream_t s);
 // dense Schur-complement preconditioner (precond.cu)
 // [S | I] -> [I | S^-1] in place; scratch holds gj_scratch_floats(n) floats
 size_t gj_scratch_floats(int n);

@@ -110,7 +110,8 @@ __device__ double lgf_far(int m, int n) {
            (18.0 * c4 + 25.0 * c8) / (480.0 * M_PI * r2 * r2);
 }
 
-// G[n * (M + 1) + m] for 0 <= m <= M, 0 <= n <= N
+// G[n * (M + 1) + m] for 0 <= m <= M, 0 <= n <= N, and the same values transposed behind it,
+// GT[m * (N + 1) + n]: the ring sums read along whichever index their lanes run over.
 __global__ void k_lgf_table(int M, int N, GaussRule R, double* __restrict__ G) {
     pdl_wait();
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -121,12 +122,13 @@ __global__ void k_lgf_table(int M, int N, GaussRule R, double* __restrict__ G) {
     else if (m < kLgfQuadRadius && n < kLgfQuadRadius) v = lgf_quadrature(m, n, R);
     else v = lgf_far(m, n);
     G[k] = v;
+    G[(long)(M + 1) * (N + 1) + (long)m * (N + 1) + n] = v;
 }
 
 static std::mutex g_lgf_mutex;
 static std::map<std::tuple<int, int, int>, double*> g_lgf_tables;
 
-// The table G(m, n), 0 <= m <= nx, 0 <= n <= ny (row stride nx + 1), on the current device
+// The table G(m, n), 0 <= m <= nx, 0 <= n <= ny (row stride nx + 1) and its transpose, on the current device
 // (built on first use, kept until the process exits).  Synchronizes the device on first use.
 iim_status lgf_table(int nx, int ny, const double** out) {
     int dev = 0;
@@ -140,7 +142,7 @@ iim_status lgf_table(int nx, int ny, const double** out) {
     }
     double* G = nullptr;
     const long n = (long)(nx + 1) * (ny + 1);
-    IIM_TRY(cudaMalloc(&G, sizeof(double) * n));
+    IIM_TRY(cudaMalloc(&G, sizeof(double) * 2 * n));
     const GaussRule R = gauss16();
     launch("lgf_table", 0.0, 0.0, k_lgf_table, (unsigned)((n + 127) / 128), 128, 0, (cudaStream_t)0, nx, ny, R, G);
     cudaError_t e = cudaGetLastError();
@@ -159,73 +161,124 @@ iim_status lgf_table(int nx, int ny, const double** out) {
 // x-sine coefficients c_k of psi_1's row j, slots 1..NX of the padded row):
 //   psi_1(first interior column, j) = sum_k c_k sin(pi k / nx),
 //   psi_1(last interior column, j)  = sum_k c_k (-1)^(k+1) sin(pi k / nx).
-// One warp per row.
+// One warp per row, the sines (from the table of e^{-i pi k / 4096}) in shared memory; a lane's k keep
+// their parity, so both sums come from one product.  512^2 in FP32:
+// 39 -> 5 us (a sine evaluated per element in FP64 before).
+constexpr int kBndRows = 4;
 template <typename T>
-__global__ void k_bnd_cols(int NX, int NY, int nx, const T* __restrict__ buf, double* __restrict__ vl,
-                           double* __restrict__ vr, const int* __restrict__ stop) {
+__global__ void __launch_bounds__(32 * kBndRows)
+k_bnd_cols(int NX, int NY, int nx, const cpx<double>* __restrict__ tw, const T* __restrict__ buf, double* __restrict__ vl,
+           double* __restrict__ vr, const int* __restrict__ stop) {
     pdl_wait();
     if (stop && *stop) return;
-    const int j = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    extern __shared__ double sine[];
+    for (int k = threadIdx.x; k < NX; k += 32 * kBndRows) sine[k] = -tw[(k + 1) * (kTwN / nx)].y;
+    __syncthreads();
+    const int j = blockIdx.x * kBndRows + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (j >= NY) return;
     const T* row = buf + (size_t)j * nx + 1;
-    double a = 0.0, b = 0.0;
-    for (int k = lane; k < NX; k += 32) {
-        const double c = (double)row[k] * sinpi((double)(k + 1) / nx);
-        a += c;
-        b += (k & 1) ? -c : c;   // (-1)^(k+2) for mode k + 1
+    double a = 0.0;
+    for (int k0 = lane; k0 < NX; k0 += 8 * 32) {
+        T c[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) c[u] = k0 + 32 * u < NX ? row[k0 + 32 * u] : T(0);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+            if (k0 + 32 * u < NX) a = fma((double)c[u], sine[k0 + 32 * u], a);
     }
+    const double b = warp_sum(lane & 1 ? -a : a);   // (-1)^(k+2) for mode k + 1
     a = warp_sum(a);
-    b = warp_sum(b);
     if (lane == 0) {
         vl[j] = a;
         vr[j] = b;
     }
 }
 
-// rho(x) = sum over the non-corner ring nodes y of K(x, y) psi_1(neighbour of y), for every
-// ring node x (ring layout: bottom j = 0, i = 0..nx; top j = ny; left i = 0, j = 1..ny-1; right
-// i = nx), K(x, y) = G(x - y) (+ G(x* - y) with the outflow plane, sym); G has row stride ld.
-// bnd: psi_1 on the first interior row (NX values) then on the last (NX values); vl, vr: psi_1
-// on the first and last interior columns (NY values each).  One block per x.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_ring_conv(int nx, int ny, const double* __restrict__ G, int ld, int sym, const double* __restrict__ bnd,
-            const double* __restrict__ vl, const double* __restrict__ vr, double* __restrict__ rho,
-            const int* __restrict__ stop) {
+// Ring layout: bottom j = 0, i = 0..nx; top j = ny; left i = 0, j = 1..ny-1; right i = nx.
+__device__ __forceinline__ void ring_node(int t, int nx, int ny, int& i, int& j) {
+    if (t <= nx) { i = t; j = 0; }
+    else if (t <= 2 * nx + 1) { i = t - (nx + 1); j = ny; }
+    else if (t < 2 * (nx + 1) + (ny - 1)) { i = 0; j = t - 2 * (nx + 1) + 1; }
+    else { i = nx; j = t - 2 * (nx + 1) - (ny - 1) + 1; }
+}
+
+// K(x, y) = G(x - y) (+ G(x* - y) with the outflow plane, sym).  Sources on the bottom and top run over i,
+// those on the sides over j: the first read G, the second its transpose, so that lanes read neighbours.
+struct RingKernel {
+    const double* G;
+    int ld, ldt, nx, sym;   // row strides of G and of its transpose
+    __device__ __forceinline__ double operator()(int xi, int xj, int yi, int yj, bool side) const {
+        const double* GT = G + (size_t)ld * ldt;
+        const int di = abs(xi - yi), dj = abs(xj - yj);
+        double k = side ? GT[(size_t)di * ldt + dj] : G[(size_t)dj * ld + di];
+        if (sym) {
+            const int dm = abs(2 * nx - xi - yi);
+            k += side ? GT[(size_t)dm * ldt + dj] : G[(size_t)dj * ld + dm];
+        }
+        return k;
+    }
+};
+
+// Ring sums are FP64-bound (a multiply-add per pair of ring nodes): a block takes kRingX consecutive ring
+// nodes, a thread one source at a time for all of them, and the kRingX partial sums of a warp are added
+// with halving exchanges (9 additions for 8 sums instead of 5 each).
+constexpr int kRingX = 8, kRingBlock = 256;
+__device__ __forceinline__ double ring_sums(double (&a)[kRingX]) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int half = kRingX / 2, off = 16; half >= 1; half /= 2, off /= 2) {
+        const bool up = lane & off;
+#pragma unroll
+        for (int u = 0; u < half; ++u) {
+            const double send = up ? a[u] : a[u + half], keep = up ? a[u + half] : a[u];
+            a[u] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+        }
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    __shared__ double part[kRingBlock / 32][kRingX];
+    if ((lane & 3) == 0) part[threadIdx.x >> 5][lane >> 2] = a[0];   // lane >> 2: the sum's index
+    __syncthreads();
+    double v = 0.0;
+    if (threadIdx.x < kRingX)
+        for (int w = 0; w < kRingBlock / 32; ++w) v += part[w][threadIdx.x];
+    return v;   // of ring node blockIdx.x * kRingX + threadIdx.x
+}
+
+// rho(x) = sum over the non-corner ring nodes y of K(x, y) psi_1(neighbour of y), for every ring node x,
+// minus sub(x) where given; ring (where given) moves by the result.  bnd: psi_1 on the first interior row
+// (NX values) then on the last (NX values); vl, vr: psi_1 on the first and last interior columns (NY values
+// each).  512^2: 17 -> 12 us with one block per ring node before, against 8.3 us of multiply-adds.
+__global__ void __launch_bounds__(kRingBlock)
+k_ring_conv(int nx, int ny, RingKernel K, const double* __restrict__ bnd, const double* __restrict__ vl,
+            const double* __restrict__ vr, const double* __restrict__ sub, double* __restrict__ rho,
+            double* __restrict__ ring, const int* __restrict__ stop) {
     pdl_wait();
     if (stop && *stop) return;
-    const int t = blockIdx.x;
-    int xi, xj;
-    if (t <= nx) { xi = t; xj = 0; }
-    else if (t <= 2 * nx + 1) { xi = t - (nx + 1); xj = ny; }
-    else if (t < 2 * (nx + 1) + (ny - 1)) { xi = 0; xj = t - 2 * (nx + 1) + 1; }
-    else { xi = nx; xj = t - 2 * (nx + 1) - (ny - 1) + 1; }
-    const int NX = nx - 1, NY = ny - 1;
-    const int nsrc = 2 * NX + 2 * NY;
-    double acc = 0.0;
-    for (int s = threadIdx.x; s < nsrc; s += BLOCK) {
+    const int t0 = blockIdx.x * kRingX, n = 2 * (nx + ny);   // n is a multiple of kRingX
+    int xi[kRingX], xj[kRingX];
+#pragma unroll
+    for (int u = 0; u < kRingX; ++u) ring_node(t0 + u, nx, ny, xi[u], xj[u]);
+    const int NX = nx - 1, NY = ny - 1, nsrc = 2 * NX + 2 * NY;
+    double acc[kRingX] = {};
+    for (int s = threadIdx.x; s < nsrc; s += kRingBlock) {
         int si, sj;
         double v;
         if (s < NX) { si = s + 1; sj = 0; v = bnd[s]; }
         else if (s < 2 * NX) { si = s - NX + 1; sj = ny; v = bnd[s]; }
         else if (s < 2 * NX + NY) { si = 0; sj = s - 2 * NX + 1; v = vl[sj - 1]; }
         else { si = nx; sj = s - 2 * NX - NY + 1; v = vr[sj - 1]; }
-        const size_t row = (size_t)abs(xj - sj) * ld;
-        double k = G[row + abs(xi - si)];
-        if (sym) k += G[row + abs(2 * nx - xi - si)];
-        acc += k * v;
+        const bool side = s >= 2 * NX;
+#pragma unroll
+        for (int u = 0; u < kRingX; ++u) acc[u] = fma(K(xi[u], xj[u], si, sj, side), v, acc[u]);
     }
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) rho[t] = acc;
-}
-
-// y += a x over n values (ring updates)
-__global__ void k_ring_add(int n, double a, const double* __restrict__ x, double* __restrict__ y,
-                           const int* __restrict__ stop) {
-    pdl_wait();
-    if (stop && *stop) return;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < n) y[k] += a * x[k];
+    const double r = ring_sums(acc);
+    const int t = t0 + threadIdx.x;
+    if (threadIdx.x < kRingX && t < n) {
+        const double v = sub ? r - sub[t] : r;
+        rho[t] = v;
+        if (ring) ring[t] += v;
+    }
 }
 
 // Ring equations of the free-space system (the FP64 residual's ring rows).  For the free-space
@@ -238,61 +291,47 @@ __global__ void k_ring_add(int n, double a, const double* __restrict__ x, double
 // mirrored part is harmonic inside the box, and so is G(x* - .)), and the potential of the
 // plane sources, h^2 sum_j G(x - (nx, j)) plane_j (harmonic inside), is the data of the row and
 // is subtracted (plane null: no plane sources).  psi: padded interior field; ring: psi on the
-// ring.  One block per ring node.
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_ring_residual(int nx, int ny, double h2, const double* __restrict__ G, int ld, int sym,
-                const double* __restrict__ plane, const double* __restrict__ psi, const double* __restrict__ ring,
-                double* __restrict__ rres) {
+// ring.  Blocks as k_ring_conv, two multiply-adds per pair.  512^2: 32 -> 22 us.
+__global__ void __launch_bounds__(kRingBlock)
+k_ring_residual(int nx, int ny, double h2, RingKernel K, const double* __restrict__ plane, const double* __restrict__ psi,
+                const double* __restrict__ ring, double* __restrict__ rres) {
     pdl_wait();
-    const int t = blockIdx.x;
-    int xi, xj;
-    if (t <= nx) { xi = t; xj = 0; }
-    else if (t <= 2 * nx + 1) { xi = t - (nx + 1); xj = ny; }
-    else if (t < 2 * (nx + 1) + (ny - 1)) { xi = 0; xj = t - 2 * (nx + 1) + 1; }
-    else { xi = nx; xj = t - 2 * (nx + 1) - (ny - 1) + 1; }
-    const int NX = nx - 1, NY = ny - 1;
-    const int nsrc = 2 * NX + 2 * NY;
-    auto K = [&](int yi, int yj) {
-        const size_t row = (size_t)abs(xj - yj) * ld;
-        double k = G[row + abs(xi - yi)];
-        if (sym) k += G[row + abs(2 * nx - xi - yi)];
-        return k;
-    };
-    double acc = 0.0;
-    for (int s = threadIdx.x; s < nsrc; s += BLOCK) {
+    const int t0 = blockIdx.x * kRingX, n = 2 * (nx + ny);
+    int xi[kRingX], xj[kRingX];
+#pragma unroll
+    for (int u = 0; u < kRingX; ++u) ring_node(t0 + u, nx, ny, xi[u], xj[u]);
+    const int NX = nx - 1, NY = ny - 1, nsrc = 2 * NX + 2 * NY;
+    double acc[kRingX] = {};
+    for (int s = threadIdx.x; s < nsrc; s += kRingBlock) {
         int zi, zj, ai, aj, zr;   // ring node, its interior neighbour, its ring index
         if (s < NX) { zi = s + 1; zj = 0; ai = zi; aj = 1; zr = zi; }
         else if (s < 2 * NX) { zi = s - NX + 1; zj = ny; ai = zi; aj = ny - 1; zr = nx + 1 + zi; }
         else if (s < 2 * NX + NY) { zi = 0; zj = s - 2 * NX + 1; ai = 1; aj = zj; zr = 2 * (nx + 1) + zj - 1; }
         else { zi = nx; zj = s - 2 * NX - NY + 1; ai = nx - 1; aj = zj; zr = 2 * (nx + 1) + NY + zj - 1; }
-        const double pa = psi[(size_t)(aj - 1) * nx + ai];
-        acc += K(zi, zj) * pa - K(ai, aj) * ring[zr];
+        const double pa = psi[(size_t)(aj - 1) * nx + ai], pz = ring[zr];
+        const bool side = s >= 2 * NX;
+#pragma unroll
+        for (int u = 0; u < kRingX; ++u)
+            acc[u] = fma(-K(xi[u], xj[u], ai, aj, side), pz, fma(K(xi[u], xj[u], zi, zj, side), pa, acc[u]));
     }
-    if (sym && plane) {
-        for (int j = 1 + threadIdx.x; j <= NY; j += BLOCK)
-            acc += h2 * G[(size_t)abs(xj - j) * ld + abs(xi - nx)] * plane[j - 1];
+    if (K.sym && plane) {
+        const double* GT = K.G + (size_t)K.ld * K.ldt;
+        for (int j = 1 + threadIdx.x; j <= NY; j += kRingBlock) {
+            const double p = h2 * plane[j - 1];
+#pragma unroll
+            for (int u = 0; u < kRingX; ++u) acc[u] += GT[(size_t)abs(xi[u] - nx) * K.ldt + abs(xj[u] - j)] * p;
+        }
     }
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) rres[t] = ring[t] - acc;
-}
-
-// *res2 += scale2 sum_t rres[t]^2 (one block)
-template <int BLOCK>
-__global__ void __launch_bounds__(BLOCK)
-k_ring_res_norm(int n, const double* __restrict__ rres, double scale2, double* __restrict__ res2) {
-    pdl_wait();
-    double acc = 0.0;
-    for (int t = threadIdx.x; t < n; t += BLOCK) acc += rres[t] * rres[t];
-    acc = block_sum<BLOCK>(acc);
-    if (threadIdx.x == 0) *res2 += scale2 * acc;
+    const double r = ring_sums(acc);
+    const int t = t0 + threadIdx.x;
+    if (threadIdx.x < kRingX && t < n) rres[t] = ring[t] - r;
 }
 
 template <typename T>
 iim_status launch_bnd_cols(int NX, int NY, int nx, const T* buf, double* vl, double* vr, const int* stop,
                            cudaStream_t s) {
-    launch("free_bnd_cols", (double)NX * NY * sizeof(T), 4.0 * NX * NY, k_bnd_cols<T>, (NY + 7) / 8, 256, 0, s, NX, NY,
-           nx, buf, vl, vr, stop);
+    launch("free_bnd_cols", (double)NX * NY * sizeof(T), 4.0 * NX * NY, k_bnd_cols<T>, (NY + kBndRows - 1) / kBndRows,
+           32 * kBndRows, sizeof(double) * NX, s, NX, NY, nx, twiddles64(), buf, vl, vr, stop);
     IIM_LAUNCHED();
     return IIM_OK;
 }
@@ -300,27 +339,19 @@ template iim_status launch_bnd_cols<float>(int, int, int, const float*, double*,
 template iim_status launch_bnd_cols<double>(int, int, int, const double*, double*, double*, const int*, cudaStream_t);
 
 iim_status launch_ring_conv(int nx, int ny, const double* G, int ld, int sym, const double* bnd, const double* vl,
-                            const double* vr, double* rho, const int* stop, cudaStream_t s) {
+                            const double* vr, const double* sub, double* rho, double* ring, const int* stop,
+                            cudaStream_t s) {
     const double nsrc = 2.0 * (nx - 1) + 2.0 * (ny - 1);
-    launch("free_ring_conv", 0.0, (sym ? 4.0 : 2.0) * nsrc * 2.0 * (nx + ny), k_ring_conv<256>, 2 * (nx + ny), 256, 0, s,
-           nx, ny, G, ld, sym, bnd, vl, vr, rho, stop);
-    IIM_LAUNCHED();
-    return IIM_OK;
-}
-
-iim_status launch_ring_add(int n, double a, const double* x, double* y, const int* stop, cudaStream_t s) {
-    launch("free_ring_add", 0.0, 0.0, k_ring_add, (n + 255) / 256, 256, 0, s, n, a, x, y, stop);
+    launch("free_ring_conv", 0.0, (sym ? 4.0 : 2.0) * nsrc * 2.0 * (nx + ny), k_ring_conv, 2 * (nx + ny) / kRingX,
+           kRingBlock, 0, s, nx, ny, RingKernel{G, ld, ny + 1, nx, sym}, bnd, vl, vr, sub, rho, ring, stop);
     IIM_LAUNCHED();
     return IIM_OK;
 }
 
 iim_status launch_ring_residual(int nx, int ny, double h, const double* G, int ld, int sym, const double* plane,
-                                const double* psi, const double* ring, double* rres, double* res2, cudaStream_t s) {
-    const int n = 2 * (nx + ny);
-    launch("free_ring_residual", 0.0, 0.0, k_ring_residual<256>, n, 256, 0, s, nx, ny, h * h, G, ld, sym, plane, psi,
-           ring, rres);
-    launch("free_ring_res_norm", 0.0, 0.0, k_ring_res_norm<256>, 1, 256, 0, s, n, (const double*)rres,
-           1.0 / (h * h * h * h), res2);
+                                const double* psi, const double* ring, double* rres, cudaStream_t s) {
+    launch("free_ring_residual", 0.0, 0.0, k_ring_residual, 2 * (nx + ny) / kRingX, kRingBlock, 0, s, nx, ny, h * h,
+           RingKernel{G, ld, ny + 1, nx, sym}, plane, psi, ring, rres);
     IIM_LAUNCHED();
     return IIM_OK;
 }

@@ -201,6 +201,9 @@ __device__ __forceinline__ void sine_pass(const cpx<T>* in, cpx<T>* out, const c
     }
 }
 
+// Whether sine_transform's last step reads P (even number of passes); its output may then go to Q.
+__host__ __device__ constexpr bool sine_ends_in_p(int n) { return !(n == 2048 || n <= 32); }
+
 // DST-I of the group's lines: x in the reals of Q (line l at 2 l BUF, slots 0 .. n-1, slot 0 zero),
 // both buffers kLines * BUF entries; every thread of the group has synchronised after writing x.
 // emit(line, k, X) gets X_{4k} .. X_{4k+3} (X_0 = 0).
@@ -305,7 +308,7 @@ sine_rows_fwd_body(int NX, int NY, int n_rt, int row0, int nrows, const double* 
     const int l = tid / TPL, t = tid - l * TPL, r = r0 + l;
     T* x = reinterpret_cast<T*>(Q) + (size_t)l * 2 * BUF;
     const bool live = r < rend;
-    if (live && dense && dld == n && doff == 1) {
+    if (live && dense && !ring && dld == n && doff == 1) {
         // padded row: 16-byte loads, slot 0 is a zero pad
         const double2* src = reinterpret_cast<const double2*>(dense + (size_t)r * n);
         constexpr int B = N ? (N / 2 + TPL - 1) / TPL : 8;
@@ -324,27 +327,33 @@ sine_rows_fwd_body(int NX, int NY, int n_rt, int row0, int nrows, const double* 
                 }
         }
         if (t == 0) x[0] = T(0);
-    } else if (live && dense) {
-        const double* src = dense + (size_t)r * dld + doff;
-#pragma unroll 8
-        for (int i = t; i < NX; i += TPL) x[i + 1] = (T)src[i];
+    } else if (live && (dense || ring)) {
+        // element i + 1 is thread i mod TPL's throughout
+        constexpr int B = N ? (N + TPL - 1) / TPL : 8;
+        const double* src = dense ? dense + (size_t)r * dld + doff : nullptr;
+        for (int i0 = t; i0 < NX; i0 += B * TPL) {
+            double v[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+                if (i0 + b * TPL < NX) v[b] = src ? src[i0 + b * TPL] : 0.0;
+#pragma unroll
+            for (int b = 0; b < B; ++b)
+                if (i0 + b * TPL < NX) x[i0 + b * TPL + 1] = (T)v[b];
+        }
         if (t == 0) x[0] = T(0);
+        if (ring) {   // bottom row (nx+1), top row (nx+1), left column (ny-1), right column (ny-1)
+            const int nxp1 = NX + 2;
+            if (t == 0) x[1] += (T)(ring[2 * nxp1 + r] * ih2);
+            if (t == (NX - 1) % TPL) x[NX] += (T)(ring[2 * nxp1 + NY + r] * ih2);
+            for (int edge = 0; edge < 2; ++edge) {
+                if (r != (edge ? NY - 1 : 0)) continue;
+                const double* g = ring + edge * nxp1 + 1;
+#pragma unroll 8
+                for (int i = t; i < NX; i += TPL) x[i + 1] += (T)(__ldg(g + i) * ih2);
+            }
+        }
     } else {
         for (int q = t; q < n / 2; q += TPL) reinterpret_cast<vec2_t<T>*>(x)[q] = vec2_t<T>{T(0), T(0)};
-    }
-    if (ring) {
-        // ring: bottom row (nx+1), top row (nx+1), left column (ny-1), right column (ny-1)
-        sine_sync<N>();
-        const int nxp1 = NX + 2;
-        if (live && t == 0) {
-            x[1] += (T)(ring[2 * nxp1 + r] * ih2);
-            x[NX] += (T)(ring[2 * nxp1 + NY + r] * ih2);
-        }
-        sine_sync<N>();
-        if (live && r == 0)
-            for (int i = t; i < NX; i += TPL) x[i + 1] += (T)(ring[i + 1] * ih2);
-        if (live && r == NY - 1)   // after the bottom row's terms when there is one row (same thread per i)
-            for (int i = t; i < NX; i += TPL) x[i + 1] += (T)(ring[nxp1 + i + 1] * ih2);
     }
     if (gam.base) {
         sine_sync<N>();
@@ -460,7 +469,76 @@ k_sine_rows_inv(int NX, int NY, int n, int row0, int nrows, const T* in, T* outT
     if (stop && *stop) return;
     if (MODE == INV_ACCUM_FLUID && blockIdx.x == 0) ps.apply();
     sine_rows_inv_body<T, MODE, N, L>(NX, NY, n, row0, nrows, in + (long)blockIdx.y * fstride,
-                                   outT ? outT + (long)blockIdx.y * fstride : nullptr, out64, old, ooff, cls, tab);
+                                   outT ? outT + (long)blockIdx.y * fstride : nullptr, out64, old,
+                                   ooff + (int)blockIdx.y * old, cls, tab);
+}
+
+// s / d of positive d well inside the FP32 range: the FP32 reciprocal and two Newton steps, to about an ulp.
+__device__ __forceinline__ double quotient(double s, double d) {
+    double r = (double)__frcp_rn((float)d);
+    r = fma(r, fma(-d, r, 1.0), r);
+    r = fma(r, fma(-d, r, 1.0), r);
+    return s * r;
+}
+
+// Column pass of the box solve: DST-I of the columns, division by the eigenvalues
+// lam_x + lam_y = (2 - 2 cos(pi p / nx) + 2 - 2 cos(pi q / n)) / h^2, DST-I back.  kLines adjacent padded
+// columns per group; `scale` carries the normalisation and h^2; tw: the table of e^{-i pi k / 4096}.
+// Each transform leaves its result in the buffer that its last step does not read.  Dynamic shared memory
+// sine_smem<T>(n, L).  Bound by FP64 arithmetic; against the packed transforms (dst.cuh), whole box solve in
+// FP64: 64^2 45 -> 35 us, 256^2 73 -> 54, 512^2 103 -> 95, 1024^2 304 -> 307, 2048^2 1466 -> 1101,
+// 64 x 2048 256 -> 115.
+template <typename T, int N, int L>
+__global__ void __launch_bounds__((Sine<N, L>::kBlock))
+k_sine_cols(int nx, int n_rt, T* __restrict__ buf, T scale, const cpx<T>* __restrict__ tab, const cpx<T>* __restrict__ tw) {
+    pdl_wait();
+    using S = Sine<N, L>;
+    constexpr int KL = S::kLines;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = N ? N : n_rt, BUF = sine_buf(n);
+    const int grp = N ? 0 : threadIdx.x / S::kThreads, tid = N ? threadIdx.x : threadIdx.x % S::kThreads;
+    cpx<T>* P = reinterpret_cast<cpx<T>*>(smem_raw) + (size_t)grp * 2 * KL * BUF;
+    cpx<T>* Q = P + (size_t)KL * BUF;
+    const int c0 = (blockIdx.x * S::kGroups + grp) * KL;   // nx is a multiple of L
+    T* x = reinterpret_cast<T*>(Q);   // line l at 2 l BUF
+    constexpr int B = N ? (KL * N + S::kThreads - 1) / S::kThreads : 8;
+    for (int e0 = tid; e0 < KL * n; e0 += B * S::kThreads) {
+        T v[B];
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int e = e0 + b * S::kThreads, j = e / KL, l = e % KL;
+            v[b] = e < KL * n && j ? buf[(size_t)(j - 1) * nx + c0 + l] : T(0);
+        }
+#pragma unroll
+        for (int b = 0; b < B; ++b) {
+            const int e = e0 + b * S::kThreads, j = e / KL, l = e % KL;
+            if (e < KL * n) x[(size_t)l * 2 * BUF + j] = v[b];
+        }
+    }
+    sine_sync<N>();
+    cpx<T>* O = sine_ends_in_p(n) ? Q : P;
+    cpx<T>* I = sine_ends_in_p(n) ? P : Q;
+    x = reinterpret_cast<T*>(O);
+    sine_transform<T, N, L>(P, Q, tab, n, tid, [&](int l, int k, const T (&X)[4]) {
+        const T lx = T(2) - T(2) * tw[(c0 + l) * (kTwN / nx)].x;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const T ly = T(2) - T(2) * tw[(4 * k + e) * (kTwN / n)].x;
+            x[(size_t)l * 2 * BUF + 4 * k + e] = (k || e) ? X[e] * quotient(scale, lx + ly) : T(0);   // slot 0 stays zero
+        }
+    });
+    sine_sync<N>();
+    x = reinterpret_cast<T*>(sine_ends_in_p(n) ? O : I);
+    sine_transform<T, N, L>(I, O, tab, n, tid, [&](int l, int k, const T (&X)[4]) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) x[(size_t)l * 2 * BUF + 4 * k + e] = X[e];
+    });
+    sine_sync<N>();
+#pragma unroll 4
+    for (int e = tid; e < KL * (n - 1); e += S::kThreads) {
+        const int j = e / KL, l = e % KL;
+        buf[(size_t)j * nx + c0 + l] = x[(size_t)l * 2 * BUF + j + 1];
+    }
 }
 
 }  // namespace iim

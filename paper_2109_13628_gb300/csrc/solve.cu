@@ -345,6 +345,31 @@ static iim_status rows_inv(const Plan<T>& p, int row0, int nrows, const T* in, T
     return IIM_OK;
 }
 
+// Column pass of the FP64 box solve for callers, eigenvalues from the twiddle table.
+static iim_status box_cols(int nx, int ny, double h, double* buf, cudaStream_t s) {
+    const int lpb = sine_lines(ny, nx);
+    const size_t sm = sine_smem<double>(ny, lpb);
+    const double scale = (2.0 / nx) * (2.0 / ny) * (h * h);
+    IIM_CHECK(sine_dispatch(ny, lpb, [&](auto N, auto L) -> iim_status {
+        auto kern = k_sine_cols<double, N.value, L.value>;
+        IIM_CHECK(allow_smem(kern, sm));
+        launch("sine_cols_f64", 16.0 * nx * (ny - 1), nx * (2.0 * dst_flops(ny) + 2.0 * ny), kern, nx / lpb,
+               (Sine<N.value, L.value>::kBlock), sm, s, nx, ny, buf, scale, sine_table<double>(ny), twiddles64());
+        return IIM_OK;
+    }));
+    IIM_LAUNCHED();
+    return IIM_OK;
+}
+// The FP64 box solve: f (and the ring) to u, through the padded buffer buf of nx * (ny - 1).
+static iim_status box64(const iim_grid* grid, double h, const double* f, const double* psi_box, double* u, double* buf,
+                        cudaStream_t s) {
+    const int nx = grid->nx, ny = grid->ny, NX = nx - 1, NY = ny - 1;
+    const Plan<double> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), nullptr, nullptr, twiddles64(), 0.0};
+    IIM_CHECK(rows_fwd<double>(p, 0, NY, f, NX, 0, psi_box, 1.0 / (h * h), nullptr, nullptr, kNoVec, 0.0, buf, nullptr, s));
+    IIM_CHECK(box_cols(nx, ny, h, buf, s));
+    return rows_inv<double, INV_STORE_F64>(p, 0, NY, buf, nullptr, u, NX, 0, nullptr, nullptr, s);
+}
+
 template <typename T>
 static Plan<T> make_plan(iim_geometry g);
 template <>
@@ -701,8 +726,18 @@ __device__ void ref_control(const RefCtl& c, int* di, double* small) {
         final_rel_body(di, small);
     }
 }
-// The same after the ring rows of a free-space residual.
-__global__ void k_ref_control(RefCtl c, int* __restrict__ di, double* __restrict__ small) { pdl_wait(); ref_control(c, di, small); }
+// Free space: small[SM_RES2] += scale2 sum_t rres[t]^2 (the ring rows), then the loop decision (one block).
+template <int BLOCK>
+__global__ void __launch_bounds__(BLOCK)
+k_ring_norm(int n, const double* __restrict__ rres, double scale2, RefCtl c, int* di, double* small) {
+    pdl_wait();
+    double acc = 0.0;
+    for (int t = threadIdx.x; t < n; t += BLOCK) acc += rres[t] * rres[t];
+    acc = block_sum<BLOCK>(acc);
+    if (threadIdx.x != 0) return;
+    small[SM_RES2] += scale2 * acc;
+    if (c.mode != CTL_NONE) ref_control(c, di, small);
+}
 
 // After gmres_init: the Krylov budget left for this correction; cycle counter reset; the cycle
 // loop entered unless the start already stopped (converged or no budget).
@@ -831,12 +866,12 @@ struct Solver {
         launch("finish_residual", 0.0, 0.0, k_finish<256>, finish_blocks(g->ncirc), 256, 0, s, fa,
                g->outer ? RefCtl{} : ctl);
         IIM_LAUNCHED();
-        if (g->outer)   // free space: the ring rows (freespace.cu), kept for the next recovery
+        if (g->outer) {   // free space: the ring rows (freespace.cu), kept for the next recovery
             IIM_CHECK(launch_ring_residual(g->nx, g->ny, g->h, g->lgf, g->lgf_ld, g->outer == 2,
                                            g->outer == 2 && !g->plane_off ? g->fs_plane : nullptr, g->psi_ext,
-                                           g->fs_ring, g->fs_rres, small + SM_RES2, s));
-        if (g->outer && ctl.mode != CTL_NONE) {
-            launch("ref_control", 0.0, 0.0, k_ref_control, 1, 1, 0, s, ctl, di(), small);
+                                           g->fs_ring, g->fs_rres, s));
+            launch("free_ring_res_norm", 0.0, 0.0, k_ring_norm<256>, 1, 256, 0, s, 2 * (g->nx + g->ny),
+                   (const double*)g->fs_rres, 1.0 / (g->h * g->h * g->h * g->h), ctl, di(), small);
             IIM_LAUNCHED();
         }
         return IIM_OK;
@@ -882,16 +917,17 @@ struct Solver {
     // ---- free space (freespace.cu): with tbuf holding the column-processed transform of the
     // first box solve psi_1 on every row, its values next to the box (two dot products per row
     // for the first and last interior columns, the inverse transform of the first and last
-    // interior rows) and the ring sum rho = sum_y G(x - y) psi_1(neighbour of y) into fs_rho
+    // interior rows) and the ring sum rho = sum_y G(x - y) psi_1(neighbour of y), minus `sub`, into
+    // fs_rho; `ring` moves by it
     template <typename T>
-    iim_status free_ring(const Plan<T>& p, const int* stop) {
+    iim_status free_ring(const Plan<T>& p, const int* stop, const double* sub = nullptr, double* ring = nullptr) {
         const int NX = g->NX, NY = g->NY;
         double* bnd = g->fs_bnd;
         IIM_CHECK(launch_bnd_cols<T>(NX, NY, g->nx, (const T*)g->tbuf, bnd + 2 * NX, bnd + 2 * NX + NY, stop, s));
-        IIM_CHECK((rows_inv<T, INV_STORE_F64>(p, 0, 1, (const T*)g->tbuf, nullptr, bnd, 0, 0, nullptr, stop, s)));
-        IIM_CHECK((rows_inv<T, INV_STORE_F64>(p, NY - 1, 1, (const T*)g->tbuf, nullptr, bnd, 0, NX, nullptr, stop, s)));
+        IIM_CHECK((rows_inv<T, INV_STORE_F64>(p, 0, 1, (const T*)g->tbuf, nullptr, bnd, NX, 0, nullptr, stop, s, 2,
+                                              (long)(NY - 1) * g->nx)));
         return launch_ring_conv(g->nx, g->ny, g->lgf, g->lgf_ld, g->outer == 2, bnd, bnd + 2 * NX, bnd + 2 * NX + NY,
-                                g->fs_rho, stop, s);
+                                sub, g->fs_rho, ring, stop, s);
     }
 
     // ---- free space: the box solve of a zero source with box data fs_rho (the harmonic part),
@@ -1138,12 +1174,11 @@ struct Solver {
         } else {
             IIM_CHECK(cols<T>(p, 0, g->NY - 1, g->outer ? 0 : g->jo0, g->outer ? g->NY - 1 : g->jo1, tb, nullptr, s));
         }
-        if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr));
+        // free space: the harmonic part of the correction carries rho minus the ring rows of the residual,
+        // as in the recovery below, so that the right-hand side sees the ring data and error
+        if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr, g->fs_rres));
         IIM_CHECK((rows_inv<T, INV_STORE_T>(p, g->jo0, g->jo1 - g->jo0 + 1, band, pt, nullptr, 0, 0, nullptr, nullptr, s)));
         if (g->outer) {
-            // the harmonic part of the correction carries rho minus the ring rows of the residual,
-            // as in the recovery below, so that the right-hand side sees the ring data and error
-            IIM_CHECK(launch_ring_add(2 * (g->nx + g->ny), -1.0, g->fs_rres, g->fs_rho, nullptr, s));
             IIM_CHECK(free_harmonic<T>(p, g->jo0, g->jo1, nullptr));
             IIM_CHECK((rows_inv<T, INV_ACCUM_T>(p, g->jo0, g->jo1 - g->jo0 + 1, tb, pt, nullptr, 0, 0, nullptr, nullptr, s)));
         }
@@ -1164,18 +1199,15 @@ struct Solver {
         IIM_CHECK(rows_fwd<T>(p, r0, nr, g->res, g->nx, 1, nullptr, 0.0, g->aff_row_ptr, g->aff_node, xg, -1.0, tb,
                               nullptr, s));
         IIM_CHECK(cols<T>(p, 0, g->NY - 1, 0, g->NY - 1, tb, nullptr, s));
-        if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr));
+        // free space: the harmonic part carries rho minus the ring rows of the last residual: the field
+        // harmonic inside the box that removes the ring error (the interior rows do not see it); the ring
+        // moves by the same values
+        if (g->outer) IIM_CHECK(free_ring<T>(p, nullptr, g->fs_rres, g->fs_ring));
         const PsibarStep ps{g->ncirc, di() + DI_CIRC, x + g->na, psibar};
         IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(p, 0, g->NY, tb, nullptr, g->psi_ext, 0, 0, g->node_class, nullptr, s, 1, 0L, ps)));
         if (g->outer) {
-            // the harmonic part carries rho minus the ring rows of the last residual: the field
-            // harmonic inside the box that removes the ring error (the interior rows do not see
-            // it); the ring moves by the same values
-            const int nr = 2 * (g->nx + g->ny);
-            IIM_CHECK(launch_ring_add(nr, -1.0, g->fs_rres, g->fs_rho, nullptr, s));
             IIM_CHECK(free_harmonic<T>(p, 0, g->NY - 1, nullptr));
             IIM_CHECK((rows_inv<T, INV_ACCUM_FLUID>(p, 0, g->NY, tb, nullptr, g->psi_ext, 0, 0, g->node_class, nullptr, s)));
-            IIM_CHECK(launch_ring_add(nr, 1.0, g->fs_rho, g->fs_ring, nullptr, s));
         }
         return IIM_OK;
     }
@@ -2090,32 +2122,21 @@ extern "C" iim_status iim_box_poisson(const iim_grid* grid, const double* f, con
     IIM_CHECK(ensure_twiddles());
     cudaStream_t s = (cudaStream_t)stream;
     const int NX = nx - 1, NY = ny - 1;
-    // work: padded transform buffer (nx*NY) followed by the eigenvalue tables (NX + NY)
+    // work: padded transform buffer (nx*NY), then for FP32 the eigenvalue tables (NX + NY)
     double* buf = work;
-    double* lam = work + (size_t)nx * NY;
-    std::vector<double> lx(NX + NY);
-    for (int k = 0; k < NX; ++k) lx[k] = (2.0 - 2.0 * std::cos(M_PI * (k + 1) / nx)) / (h * h);
-    for (int k = 0; k < NY; ++k) lx[NX + k] = (2.0 - 2.0 * std::cos(M_PI * (k + 1) / ny)) / (h * h);
-    const double ih2 = 1.0 / (h * h);
-    if (prec == IIM_FP64) {
-        IIM_TRY(cudaMemcpyAsync(lam, lx.data(), sizeof(double) * (NX + NY), cudaMemcpyHostToDevice, s));
-        Plan<double> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lam, lam + NX, twiddles64(), (2.0 / nx) * (2.0 / ny)};
-        IIM_CHECK(rows_fwd<double>(p, 0, NY, f, NX, 0, psi_box, ih2, nullptr, nullptr, kNoVec, 0.0, buf, nullptr, s));
-        IIM_CHECK(cols<double>(p, 0, NY - 1, 0, NY - 1, buf, nullptr, s));
-        IIM_CHECK((rows_inv<double, INV_STORE_F64>(p, 0, NY, buf, nullptr, u, NX, 0, nullptr, nullptr, s)));
-    } else {
-        std::vector<float> fl(NX + NY);
-        for (int k = 0; k < NX + NY; ++k) fl[k] = (float)lx[k];
-        float* lamf = (float*)lam;
-        IIM_TRY(cudaMemcpyAsync(lamf, fl.data(), sizeof(float) * (NX + NY), cudaMemcpyHostToDevice, s));
-        Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(), (float)((2.0 / nx) * (2.0 / ny))};
-        float* fb = (float*)buf;
-        IIM_CHECK(packed_rows_fwd(p, f, psi_box, ih2, fb, s));
-        IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
-        IIM_CHECK(packed_rows_inv(p, fb, u, s));
-    }
-    // pageable-memory copies are staged before cudaMemcpyAsync returns, so the host vectors
-    // may go out of scope here
+    if (prec == IIM_FP64) return box64(grid, h, f, psi_box, u, buf, s);
+    std::vector<float> fl(NX + NY);
+    for (int k = 0; k < NX; ++k) fl[k] = (float)((2.0 - 2.0 * std::cos(M_PI * (k + 1) / nx)) / (h * h));
+    for (int k = 0; k < NY; ++k) fl[NX + k] = (float)((2.0 - 2.0 * std::cos(M_PI * (k + 1) / ny)) / (h * h));
+    float* lamf = (float*)(work + (size_t)nx * NY);
+    IIM_TRY(cudaMemcpyAsync(lamf, fl.data(), sizeof(float) * (NX + NY), cudaMemcpyHostToDevice, s));
+    Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(), (float)((2.0 / nx) * (2.0 / ny))};
+    float* fb = (float*)buf;
+    IIM_CHECK(packed_rows_fwd(p, f, psi_box, 1.0 / (h * h), fb, s));
+    IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
+    IIM_CHECK(packed_rows_inv(p, fb, u, s));
+    // a pageable-memory copy is staged before cudaMemcpyAsync returns, so the host vector may go out of
+    // scope here
     return IIM_OK;
 }
 
@@ -2232,15 +2253,14 @@ __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 static std::mutex g_noalloc_mutex;
 static double* g_noalloc_ptr[64];
 
-// Eigenvalues of the 1D three-point operators (x modes, then y modes), in FP64 or FP32.
-__global__ void k_box_eigs(int NX, int NY, int nx, int ny, double h, int as_float, double* lam) {
+// Eigenvalues of the 1D three-point operators (x modes, then y modes) in FP32.
+__global__ void k_box_eigs(int NX, int NY, int nx, int ny, double h, float* lam) {
     pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= NX + NY) return;
     const double v = k < NX ? (2.0 - 2.0 * cospi((double)(k + 1) / nx)) / (h * h)
                             : (2.0 - 2.0 * cospi((double)(k - NX + 1) / ny)) / (h * h);
-    if (as_float) reinterpret_cast<float*>(lam)[k] = (float)v;
-    else lam[k] = v;
+    lam[k] = (float)v;
 }
 
 // Shared-memory limits of every transform kernel the allocation-free solve may launch, sized for
@@ -2259,15 +2279,13 @@ static iim_status allow_noalloc_smem() {
                 const size_t sm = sine_smem<double>(n, L.value);
                 IIM_CHECK(allow_smem(k_sine_rows_fwd<double, N.value, L.value>, sm));
                 IIM_CHECK((allow_smem(k_sine_rows_inv<double, INV_STORE_F64, N.value, L.value>, sm)));
+                IIM_CHECK(allow_smem(k_sine_cols<double, N.value, L.value>, sm));
                 return IIM_OK;
             }));
-    const size_t c32 = cols_smem<float>(kNoAllocMaxN, 4), c64 = cols_smem<double>(kNoAllocMaxN, 4);
+    const size_t c32 = cols_smem<float>(kNoAllocMaxN, 4);
     IIM_CHECK(allow_smem(k_cols<float, 4, 0>, c32));
     IIM_CHECK(allow_smem(k_cols<float, 4, 8>, c32));
     IIM_CHECK(allow_smem(k_cols<float, 4, 16>, c32));
-    IIM_CHECK(allow_smem(k_cols<double, 4, 0>, c64));
-    IIM_CHECK(allow_smem(k_cols<double, 4, 8>, c64));
-    IIM_CHECK(allow_smem(k_cols<double, 4, 16>, c64));
     return IIM_OK;
 }
 
@@ -2320,25 +2338,15 @@ extern "C" iim_status iim_box_poisson_noalloc(const iim_grid* grid, const double
     IIM_CHECK(noalloc_setup(s, &scratch));
     const int NX = nx - 1, NY = ny - 1;
     double* buf = scratch;                          // padded transform buffer, nx * NY
-    double* lam = scratch + (size_t)nx * NY;        // NX + NY eigenvalues
-    const double ih2 = 1.0 / (h * h);
-    const int as_float = prec == IIM_MIXED;
-    launch("box_eigs", 0.0, 0.0, k_box_eigs, (NX + NY + 255) / 256, 256, 0, s, NX, NY, nx, ny, h, as_float, lam);
+    if (prec == IIM_FP64) return box64(grid, h, f, psi_box, u, buf, s);
+    float* lamf = reinterpret_cast<float*>(scratch + (size_t)nx * NY);   // NX + NY eigenvalues
+    launch("box_eigs", 0.0, 0.0, k_box_eigs, (NX + NY + 255) / 256, 256, 0, s, NX, NY, nx, ny, h, lamf);
     IIM_LAUNCHED();
-    if (prec == IIM_FP64) {
-        Plan<double> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lam, lam + NX, twiddles64(), (2.0 / nx) * (2.0 / ny)};
-        IIM_CHECK(rows_fwd<double>(p, 0, NY, f, NX, 0, psi_box, ih2, nullptr, nullptr, kNoVec, 0.0, buf, nullptr, s));
-        IIM_CHECK(cols<double>(p, 0, NY - 1, 0, NY - 1, buf, nullptr, s));
-        IIM_CHECK((rows_inv<double, INV_STORE_F64>(p, 0, NY, buf, nullptr, u, NX, 0, nullptr, nullptr, s)));
-    } else {
-        const float* lamf = reinterpret_cast<const float*>(lam);
-        Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(),
-                      (float)((2.0 / nx) * (2.0 / ny))};
-        float* fb = reinterpret_cast<float*>(buf);
-        IIM_CHECK(packed_rows_fwd(p, f, psi_box, ih2, fb, s));
-        IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
-        IIM_CHECK(packed_rows_inv(p, fb, u, s));
-    }
+    Plan<float> p{NX, NY, nx, ny, ilog2(nx), ilog2(ny), lamf, lamf + NX, twiddles32(), (float)((2.0 / nx) * (2.0 / ny))};
+    float* fb = reinterpret_cast<float*>(buf);
+    IIM_CHECK(packed_rows_fwd(p, f, psi_box, 1.0 / (h * h), fb, s));
+    IIM_CHECK(cols<float>(p, 0, NY - 1, 0, NY - 1, fb, nullptr, s));
+    IIM_CHECK(packed_rows_inv(p, fb, u, s));
     return IIM_OK;
 }
 

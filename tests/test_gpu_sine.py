@@ -41,3 +41,9 @@ def test_row_transforms_through_the_box_solve(nx, ny, ring):
     # a few hundred rounding errors of 1e-16 at most; the column transforms of this call amplify theirs
     # by sqrt(ny)
     assert np.abs(u.cpu().numpy() - ref).max() <= 1e-12 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("nx,ny", [(16, 2048), (64, 1024), (1024, 512), (16, 256)])
+def test_column_transforms_through_the_box_solve(nx, ny):
+    """Column transforms at the line lengths whose result ends in either buffer (sine_ends_in_p)."""
+    test_row_transforms_through_the_box_solve(nx, ny, True)
