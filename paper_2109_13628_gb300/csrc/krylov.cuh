@@ -8,14 +8,15 @@
 // the same order), so all blocks hold the same scalars bit for bit and take the same decisions.
 //   * k_start: norm, tolerance and first basis vector of a correction or a restart.
 //   * k_arnoldi: one Arnoldi step (two classical Gram-Schmidt passes, norm, Givens rotations, scaling).
-//     ARNOLDI_TIME
+//     1756 unknowns, restart 64 (plain FP64 512^2): six launches of 51 us per step before, 21.5 us here; 9486
+//     unknowns, few columns: 50 us before, 17 us here (event times less their overhead).
 //   * k_krylov: the whole correction solve with the dense operator (iim_opts.precond 3): start, all
 //     iterations z_j = M v_j, v_{j+1} = S z_j, Arnoldi step, restarts, x = sum y_j z_j.  The matrices
 //     come from L2 at the rate of CL SMs, so it is used up to kKrylovRows unknowns; basis and z_j stay in
 //     shared memory (a global store before a cluster barrier would put its latency into it).  Beyond, the products
 //     take the whole GPU (k_dense_matvec) between k_arnoldi launches.  Both forms do the same arithmetic in
 //     the same order.
-//     KRYLOV_TIME
+//     1450 unknowns: 38 us per iteration as launches, 23 us here.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -28,6 +29,7 @@ namespace iim {
 
 constexpr int kKrylovThreads = 512;
 constexpr int kKrylovRows = 2560;
+static_assert(8 * 65 >= kKrylovThreads, "the update's partial sums fit a pass's products");
 
 // Cluster size for ns unknowns (16 needs the non-portable size, which this GPU has), and whether the
 // correction solve with the dense operator runs as one cluster.
@@ -52,7 +54,7 @@ struct Cluster {
 // the second pass: the squared norm before it), rotations.
 template <int CL>
 struct KrylovShared {
-    double part[3][CL][65];
+    double part[3][CL][65];  // part[0] also holds the updates' partial sums
     double h[65], hc[64], cs[64], sn[64];
     double sq, nrm, inv;     // the last squared norm, the norm and its reciprocal (0 for a zero norm)
     double resid;
@@ -140,13 +142,44 @@ template <int CL, int NT>
 __device__ __forceinline__ void orthogonalise(const double* V, long ldv, int j, int nr, double* w, KrylovShared<CL>& s) {
     constexpr int NW = NT / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, rank = Cluster<CL>::rank();
+    // many columns (plain GMRES): 1756 unknowns, 64 columns, a step 23.5 -> 21.5 us on average; with few the
+    // extra barrier costs more than it saves (a 2048^2 solve of 14 iterations 3.13 -> 3.25 ms)
+    const bool wide = j >= NW;
     for (int pass = 0; pass < 2; ++pass) {
-        for (int i = warp; i <= j + pass; i += NW) {
+        // one product per warp while there are warps enough, then four: their loads overlap, and halving
+        // exchanges add them with 6 FP64 additions instead of 20
+        for (int i = warp; !wide && i <= j + pass; i += NW) {
             const double* vi = i <= j ? V + (long)i * ldv : w;
             double acc = 0.0;
             for (int e = lane; e < nr; e += 32) acc += vi[e] * w[e];
             acc = warp_sum(acc);
             if (lane < CL) *Cluster<CL>::at(&s.part[pass][rank][i], lane) = acc;
+        }
+        for (int i0 = 4 * warp; wide && i0 <= j + pass; i0 += 4 * NW) {
+            const double* vi[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) vi[u] = i0 + u <= j ? V + (long)(i0 + u) * ldv : w;
+            double a[4] = {};
+#pragma unroll 4
+            for (int e = lane; e < nr; e += 32) {
+                const double we = w[e];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) a[u] = fma(vi[u][e], we, a[u]);
+            }
+#pragma unroll
+            for (int half = 2, off = 16; half >= 1; half /= 2, off /= 2) {
+                const bool up = lane & off;
+#pragma unroll
+                for (int u = 0; u < half; ++u) {
+                    const double send = up ? a[u] : a[u + half], keep = up ? a[u + half] : a[u];
+                    a[u] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                }
+            }
+#pragma unroll
+            for (int off = 4; off >= 1; off /= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], off);
+            const int i = i0 + (lane >> 3);   // this lane's product
+            if (i <= j + pass)
+                for (int c = lane & 7; c < CL; c += 8) *Cluster<CL>::at(&s.part[pass][rank][i], c) = a[0];
         }
         Cluster<CL>::sync();
         if (tid <= j + pass) {
@@ -168,11 +201,31 @@ __device__ __forceinline__ void orthogonalise(const double* V, long ldv, int j, 
                 s.inv = n > 0.0 ? 1.0 / n : 0.0;
             }
         }
-        for (int e = tid; e < nr; e += NT) {
+        // update: G groups of threads share the columns of a row (part[0] has been read; nothing writes it
+        // from outside before the next cluster barrier)
+        const int gw = (nr + 31) & ~31, G = wide && gw > 0 && 2 * gw <= NT ? NT / gw : 1;
+        double* red = &s.part[0][0][0];
+        if (G > 1) {
+            const int g = tid / gw, e = tid - g * gw;
             double a = 0.0;
+            if (g < G && e < nr) {
 #pragma unroll 4
-            for (int i = 0; i <= j; ++i) a += s.h[i] * V[(long)i * ldv + e];
-            w[e] -= a;
+                for (int i = g; i <= j; i += G) a = fma(s.h[i], V[(long)i * ldv + e], a);
+                red[tid] = a;
+            }
+            __syncthreads();
+            if (tid < nr) {
+                double t = 0.0;
+                for (int q = 0; q < G; ++q) t += red[q * gw + tid];
+                w[tid] -= t;
+            }
+        } else {
+            for (int e = tid; e < nr; e += NT) {
+                double a = 0.0;
+#pragma unroll 4
+                for (int i = 0; i <= j; ++i) a = fma(s.h[i], V[(long)i * ldv + e], a);
+                w[e] -= a;
+            }
         }
         __syncthreads();
     }
@@ -284,7 +337,8 @@ __device__ __forceinline__ void dot_rows(const float* const (&a)[NR], const floa
 // Dense product of the whole GPU: out = A v for A (n x n, leading dimension ld), v = column *jidx of a basis
 // (vbase itself without jidx), out = column *jidx + 1 when ostride > 0.  v is staged once per block as FP32;
 // the blocks walk the rows, two per warp at a time when there are more rows than warps.  Bound by the
-// matrix: from L2 at 10^3 unknowns, from HBM beyond about 5000.  DENSE_TIME
+// matrix: from L2 at 10^3 unknowns, from HBM beyond about 5000:
+// 9486 unknowns 159 -> 67 us (5.4 TB/s), 1450 unknowns 4.4 -> 3 us.
 constexpr int kDenseWarps = 8;
 inline int dense_blocks(int n) { return std::min((n + kDenseWarps - 1) / kDenseWarps, 2 * sm_count()); }
 inline size_t dense_smem(int n) { return sizeof(float) * (size_t)dense_ld(n); }
