@@ -293,7 +293,7 @@ iim_status iim_geometry_set_column_solver(iim_geometry g, int mode);
  * Errors: IIM_ERR_INVALID_ARG (kind not 0 or 1, or kind 1 with a circulation body), IIM_ERR_CUDA. */
 iim_status iim_geometry_set_wall_condition(iim_geometry g, int kind, iim_stream stream);
 
-/* Threads per transformed line for 1024-point lines: 32 (default: one warp, fewest
+/* Threads per line of the column DSTs (iim_geometry_set_column_solver 0) for 1024-point lines: 32 (default: one warp, fewest
  * instructions, best when many solves share the GPU) or 64 (two warps per line: lower latency
  * of one solve, about 6 % more instructions).  Other line lengths use one warp.  Errors:
  * IIM_ERR_INVALID_ARG. */
@@ -302,7 +302,8 @@ iim_status iim_geometry_set_lines(iim_geometry g, int threads_per_line);
 /* Builds the dense Schur-complement preconditioner of a geometry: the matrix S of the augmented
  * system of Sec. 4.2 (gamma plus circulation unknowns), one column per FP32 operator
  * application, and its inverse by Gauss-Jordan elimination with partial pivoting in FP32,
- * kept as an (ns x 2ns) FP32 array on the device (ns = |A| + circulation bodies).  The paper
+ * kept in FP32 on the device (S^-1 and S, ns rows each padded to a multiple of 32, ns = |A| +
+ * circulation bodies).  The paper
  * solves with plain GMRes; this is a one-time cost per geometry that pays when many solves
  * share the geometry (time stepping).  Its milliseconds go to *setup_ms (host, may be NULL).
  * Errors: IIM_ERR_NOT_CONVERGED (singular pivot), IIM_ERR_CUDA.  Synchronizes `stream`. */

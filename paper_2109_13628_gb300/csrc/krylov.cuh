@@ -13,9 +13,9 @@
 //   * k_krylov: the whole correction solve with the dense operator (iim_opts.precond 3): start, all
 //     iterations z_j = M v_j, v_{j+1} = S z_j, Arnoldi step, restarts, x = sum y_j z_j.  The matrices
 //     come from L2 at the rate of CL SMs, so it is used up to kKrylovRows unknowns; basis and z_j stay in
-//     shared memory (a global store before a cluster barrier would put its latency into it).  Beyond, the products
-//     take the whole GPU (k_dense_matvec) between k_arnoldi launches.  Both forms do the same arithmetic in
-//     the same order.
+//     shared memory (a global store before a cluster barrier would put its latency into it).  Beyond, the
+//     products take the whole GPU (k_dense_matvec) between k_arnoldi launches.  Both forms do the same
+//     arithmetic in the same order.
 //     1450 unknowns: 38 us per iteration as launches, 23 us here.
 #pragma once
 

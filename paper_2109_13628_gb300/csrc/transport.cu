@@ -410,9 +410,8 @@ __device__ __forceinline__ void kelvin_body(const TrView& v, double c, int k, co
 // differences them -- about 20 FP64 instructions per node instead of 88 (four faces per node with a
 // division each).  Faces whose stencil meets a solid node (found per block, then per face) take the
 // general form, from the tile and the extensions, so a face has one value whichever block evaluates
-// it.  The first nk blocks integrate
-// one body's Kelvin ODE each (a chain of latencies: started first).  1024 x 512, one cylinder:
-// 98 -> 30 us (the whole right-hand side 177 -> 65 us).
+// it.  The first nk blocks integrate one body's Kelvin ODE each (a chain of latencies: started first).
+// 1024 x 512, one cylinder: 98 -> 30 us (the whole right-hand side 177 -> 65 us).
 constexpr int TR_X = 32, TR_Y = 16, TR_THREADS = 256, TR_W = TR_X + 4, TR_H = TR_Y + 4;
 __global__ void __launch_bounds__(TR_THREADS)
 k_transport_rhs(TrView v, double c, int mode, double a, double dt, double* __restrict__ out, int tx, int nk,

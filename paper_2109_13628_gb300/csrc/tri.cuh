@@ -127,8 +127,7 @@ __device__ __forceinline__ void scan_segment_maps(const T* sD, T* sB, bool rever
 // Tridiagonal column pass of one field in the padded layout (NY rows of ld = NX + 1 slots;
 // element (row j, data column c) at j * ld + c + 1; slot 0 of a row is a zero pad).  Rows
 // outside [in0, in1] are zero on input and not read; only rows [out0, out1] are written, to `out` (which
-// may be buf).  Block
-// blockIdx.x: padded columns [CW blockIdx.x, CW blockIdx.x + CW); NT threads; dynamic shared
+// may be buf).  Block blockIdx.x: padded columns [CW blockIdx.x, CW blockIdx.x + CW); NT threads; dynamic shared
 // memory scan_smem<T, CW, NT>(NY).
 template <typename T, int CW, int NT>
 __device__ __forceinline__ void cols_scan_body(int NX, int NY, int ld, int in0, int in1, int out0, int out1,
