@@ -61,6 +61,7 @@ template <int CO_T>
 __global__ void __launch_bounds__(TX * TY)
 k_conv(const float* __restrict__ x, const float* __restrict__ gate, const __nv_bfloat16* __restrict__ w,
        const float* __restrict__ bias, float* __restrict__ y, int Ci, int Co, int H, int W, int d, int relu) {
+    pdl_wait();
     extern __shared__ float sm[];
     const int tw = TX + 2 * d, th = TY + 2 * d;
     float* tile = sm;
@@ -138,6 +139,7 @@ __host__ __device__ constexpr size_t conv_tc_smem(int d, int cg, int no) {
 // 8 g + e >= Ci
 template <int CG, int NO>
 __global__ void k_pack_w_tc(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wp, int Ci, int Co) {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 9 * CG * NO * 8) return;
     const int e = i & 7, o = (i >> 3) % NO, g = ((i >> 3) / NO) % CG, t = (i >> 3) / (NO * CG);
@@ -155,6 +157,7 @@ __global__ void __launch_bounds__(128)
 k_conv_tc(const float* __restrict__ x, const float* __restrict__ gate, const __nv_bfloat16* __restrict__ wp,
           const float* __restrict__ bias, float* __restrict__ y, int Ci, int Co, int H, int W, int d, int relu,
           int* __restrict__ err) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int NP = TC_M + 2 * d;
     uint4* sA = reinterpret_cast<uint4*>(smem_raw);
@@ -285,6 +288,7 @@ __host__ __device__ constexpr size_t conv_units_smem(int d, int cg, int no) {
 // channels >= Ci
 template <int CG, int NO>
 __global__ void k_pack_w_units(const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wp, int Ci, int Co) {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 9 * CG * NO * 8) return;
     const int e = i & 7, o = (i >> 3) % NO, q = (i >> 3) / NO, ky = 2 - q % 3, g = q / 3 % CG, kx = q / 3 / CG;
@@ -296,6 +300,7 @@ __host__ __device__ constexpr int mma_cols(int c) { return c <= 16 ? 16 : 32; } 
 
 // FP32 planes (B, C, H, W) -> units of group g = blockIdx.y (zero channels beyond C).
 __global__ void k_to_units(const float* __restrict__ x, int C, UnitLayout u, uint4* __restrict__ out) {
+    pdl_wait();
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x, plane = (long)u.H * u.W;
     if (k >= plane) return;
     const int g = blockIdx.y, G = gridDim.y, b = blockIdx.z;
@@ -314,6 +319,7 @@ __global__ void __launch_bounds__(128)
 k_conv_units(const uint4* __restrict__ in, int gin, const __nv_bfloat16* __restrict__ wp,
              const float* __restrict__ bias, int Co, uint4* __restrict__ out, int gout, float* __restrict__ y,
              UnitLayout u, int d, int nx, int nr, int tiles, int* __restrict__ err) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int NP = UN_M + 2 * d;
     uint4* sA = reinterpret_cast<uint4*>(smem_raw);
@@ -460,7 +466,7 @@ k_conv_units(const uint4* __restrict__ in, int gin, const __nv_bfloat16* __restr
 // first, then over strips, then over blocks.  8 x 127^2, 32 channels (backward's six launches):
 // 17.96 ms for one thread per (output, tap) with two shared loads per FMA; now
 // 0.59 ms (8.1 TMAC/s, about a quarter of the FP32 rate, the staging of the strips between the
-// products; a training step 18.6 -> 1.24 ms).
+// products; a training step 18.6 -> 1.13 ms).
 constexpr int WG_PX = 64, WG_THREADS = 288, WG_PART = 32 * 32 * 9 + 32;
 
 __host__ __device__ constexpr int wg_groups(int ch, int per) {   // tiles of `per` channels, a power of two
@@ -474,6 +480,7 @@ inline size_t wgrad_smem(int nog, int ncg, int d) {
 __global__ void __launch_bounds__(WG_THREADS, 2)
 k_conv_wgrad(const float* __restrict__ x, const float* __restrict__ g, const float* __restrict__ gate,
              float* __restrict__ part, int Ci, int Co, int H, int W, int d, int strips) {
+    pdl_wait();
     extern __shared__ __align__(128) unsigned char smem_raw[];
     const int nog = wg_groups(Co, 8), ncg = wg_groups(Ci, 4);
     const int GP = wg_stride(8 * nog), XP = wg_stride(4 * ncg);
@@ -587,6 +594,7 @@ k_conv_wgrad(const float* __restrict__ x, const float* __restrict__ g, const flo
 // buffers per block.
 __global__ void __launch_bounds__(256)
 k_wgrad_sum(int nblk, int n, const float* __restrict__ part, float* __restrict__ dst) {
+    pdl_wait();
     __shared__ float red[8][33];
     const int e = blockIdx.x * 32 + (threadIdx.x & 31), sl = threadIdx.x >> 5;
     float s = 0.f;
@@ -605,6 +613,7 @@ k_wgrad_sum(int nblk, int n, const float* __restrict__ part, float* __restrict__
 // diff = (pred - target) mask; partial sums of diff^2 and mask
 __global__ void k_mse_partial(long n, const float* __restrict__ pred, const float* __restrict__ target,
                               const float* __restrict__ mask, float* __restrict__ diff, float* __restrict__ part) {
+    pdl_wait();
     float s2 = 0.f, sm_ = 0.f;
     for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
         const float m = mask ? mask[i] : 1.f;
@@ -629,6 +638,7 @@ __global__ void k_mse_partial(long n, const float* __restrict__ pred, const floa
 }
 
 __global__ void k_mse_finish(int nb, float* __restrict__ part, float* __restrict__ out) {
+    pdl_wait();
     if (threadIdx.x != 0) return;
     float x2 = 0.f, xm = 0.f;
     for (int b = 0; b < nb; ++b) { x2 += part[2 * b]; xm += part[2 * b + 1]; }
@@ -637,12 +647,14 @@ __global__ void k_mse_finish(int nb, float* __restrict__ part, float* __restrict
 }
 
 __global__ void k_scale_vec(long n, float* __restrict__ v, const float* __restrict__ s) {
+    pdl_wait();
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) v[i] *= *s;
 }
 
 __global__ void k_adam(long n, float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m, float* __restrict__ v,
                        float lr, float b1, float b2, float eps, float c1, float c2) {
+    pdl_wait();
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const float gi = g[i];
@@ -654,12 +666,14 @@ __global__ void k_adam(long n, float* __restrict__ p, const float* __restrict__ 
 }
 
 __global__ void k_to_bf16(long n, const float* __restrict__ p, __nv_bfloat16* __restrict__ out) {
+    pdl_wait();
     const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) out[i] = __float2bfloat16(p[i]);
 }
 
 // wt[c][o][k] = W[o][c][8 - k]
 __global__ void k_flip(int Ci, int Co, const __nv_bfloat16* __restrict__ w, __nv_bfloat16* __restrict__ wt) {
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= Ci * Co * 9) return;
     const int k = t % 9, o = (t / 9) % Co, c = t / (9 * Co);
@@ -669,6 +683,7 @@ __global__ void k_flip(int Ci, int Co, const __nv_bfloat16* __restrict__ w, __nv
 // x[b] = (omega s0, phi s1, ub s2) on the interior grid, channel planes of NX x NY
 __global__ void k_net_input(int NX, int NY, const double* __restrict__ omega, const double* __restrict__ phi,
                             const double* __restrict__ ub, float s0, float s1, float s2, float* __restrict__ x) {
+    pdl_wait();
     const long n = (long)NX * NY;
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -682,6 +697,7 @@ __global__ void k_net_input(int NX, int NY, const double* __restrict__ omega, co
 // psi = ub + y / s
 __global__ void k_net_guess(long n, const double* __restrict__ ub, const float* __restrict__ y, float inv_s,
                             double* __restrict__ psi) {
+    pdl_wait();
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) psi[k] = ub[k] + (double)(y[k] * inv_s);
 }
@@ -694,11 +710,11 @@ static iim_status conv(iim_net_s* net, const float* x, const float* gate, const 
     // tensor cores: mode 1 the 32 -> 32 layers, mode 2 every layer (K and N padded to 16 / 32)
     if ((net->tc == 1 && Ci == TC_C && Co == TC_C) || (net->tc == 2 && Ci <= TC_C && Co <= TC_C)) {
         auto go = [&](auto pack, auto kern, int cg, int no) -> iim_status {
-            launch("net_pack_w_tc", 0.0, 0.0, pack, (9 * cg * no * 8 + 255) / 256, 256, 0, s, w, net->wtc, Ci, Co);
+            launch_next("net_pack_w_tc", 0.0, 0.0, pack, (9 * cg * no * 8 + 255) / 256, 256, 0, s, w, net->wtc, Ci, Co);
             IIM_LAUNCHED();
             const size_t sm = conv_tc_smem(d, cg, no);
             IIM_CHECK(allow_smem(kern, sm));
-            launch("net_conv_tc", 4.0 * (double)B * H * W * (Ci * (gate ? 2 : 1) + Co),
+            launch_next("net_conv_tc", 4.0 * (double)B * H * W * (Ci * (gate ? 2 : 1) + Co),
                    18.0 * (double)B * H * W * Ci * Co, kern, dim3((W + TC_M - 1) / TC_M, H, B), 128, sm, s, x, gate,
                    (const __nv_bfloat16*)net->wtc, bias, y, Ci, Co, H, W, d, relu, net->tc_err);
             IIM_LAUNCHED();
@@ -713,11 +729,11 @@ static iim_status conv(iim_net_s* net, const float* x, const float* gate, const 
         const int ncot = (Co + 31) / 32;
         const size_t sm = conv_smem(d, 32);
         IIM_CHECK(allow_smem(k_conv<32>, sm));
-        launch("net_conv", 4.0 * (double)B * H * W * (Ci + Co), 18.0 * (double)B * H * W * Ci * Co, k_conv<32>,
+        launch_next("net_conv", 4.0 * (double)B * H * W * (Ci + Co), 18.0 * (double)B * H * W * Ci * Co, k_conv<32>,
                dim3((W + TX - 1) / TX, (H + TY - 1) / TY, B * ncot), blk, sm, s, x, gate, w, bias, y, Ci, Co, H, W, d, relu);
     } else {
         const size_t sm = conv_smem(d, 1);
-        launch("net_conv", 4.0 * (double)B * H * W * (Ci + Co), 18.0 * (double)B * H * W * Ci * Co, k_conv<1>,
+        launch_next("net_conv", 4.0 * (double)B * H * W * (Ci + Co), 18.0 * (double)B * H * W * Ci * Co, k_conv<1>,
                dim3((W + TX - 1) / TX, (H + TY - 1) / TY, B), blk, sm, s, x, gate, w, bias, y, Ci, Co, H, W, d, relu);
     }
     IIM_LAUNCHED();
@@ -756,14 +772,14 @@ static iim_status forward_units(iim_net_s* net, int B, int H, int W, const float
             const int cg = mma_groups(net->ci[l]), no = mma_cols(net->co[l]);
             auto pack = cg == 2 ? (no == 16 ? k_pack_w_units<2, 16> : k_pack_w_units<2, 32>)
                                 : (no == 16 ? k_pack_w_units<4, 16> : k_pack_w_units<4, 32>);
-            launch("net_pack_w_units", 0.0, 0.0, pack, (9 * cg * no * 8 + 255) / 256, 256, 0, s,
+            launch_next("net_pack_w_units", 0.0, 0.0, pack, (9 * cg * no * 8 + 255) / 256, 256, 0, s,
                    (const __nv_bfloat16*)(net->wb + net->woff[l]), net->wunit + WUNIT * l, net->ci[l], net->co[l]);
         }
         IIM_LAUNCHED();
         net->wunit_ok = true;
     }
     const long plane = (long)H * W;
-    launch("net_to_units", 4.0 * plane * B * net->cin, 0.0, k_to_units,
+    launch_next("net_to_units", 4.0 * plane * B * net->cin, 0.0, k_to_units,
            dim3((unsigned)((plane + 255) / 256), (net->cin + 7) / 8, B), 256, 0, s, x, net->cin, u, net->unit[0]);
     IIM_LAUNCHED();
     for (int l = 0; l < net->nl; ++l) {
@@ -775,7 +791,7 @@ static iim_status forward_units(iim_net_s* net, int B, int H, int W, const float
             IIM_CHECK(allow_smem(kern, sm));
             const int per_sm = std::max(1, (int)(227 * 1024 / (sm + 1024)));   // resident blocks (also 512 TMEM columns / 128)
             const int blocks = std::min(tiles, std::min(per_sm, 4) * sm_count());
-            launch("net_conv_tc", 2.0 * plane * B * (8.0 * gin + (last ? 2.0 : 8.0 * ((co + 7) / 8))),
+            launch_next("net_conv_tc", 2.0 * plane * B * (8.0 * gin + (last ? 2.0 : 8.0 * ((co + 7) / 8))),
                    18.0 * (double)B * plane * ci * co, kern, blocks, 128, sm, s, (const uint4*)net->unit[l & 1], gin,
                    (const __nv_bfloat16*)(net->wunit + WUNIT * l), (const float*)(net->p + net->boff[l]), co,
                    net->unit[(l + 1) & 1], (co + 7) / 8, last ? y : (float*)nullptr, u, d, nx, nr, tiles, net->tc_err);
@@ -828,15 +844,15 @@ static iim_status backward(iim_net_s* net, int B, int H, int W, const float* x, 
         const int strips = B * H * ((W + WG_PX - 1) / WG_PX), nblk = std::min(strips, net->wg_blocks);
         const int nw = net->ci[l] * net->co[l] * 9 + net->co[l];   // the layer's weights, then its biases
         IIM_CHECK(allow_smem(k_conv_wgrad, sm));
-        launch("net_wgrad", 4.0 * (double)B * H * W * (net->ci[l] + net->co[l]), 2.0 * B * H * W * 9.0 * net->ci[l] * net->co[l],
+        launch_next("net_wgrad", 4.0 * (double)B * H * W * (net->ci[l] + net->co[l]), 2.0 * B * H * W * 9.0 * net->ci[l] * net->co[l],
                k_conv_wgrad, nblk, WG_THREADS, sm, s, xin, (const float*)g, gate, net->wgp, net->ci[l], net->co[l], H, W, d,
                strips);
-        launch("net_wgrad_sum", 4.0 * nblk * (double)nw, 0.0, k_wgrad_sum, (nw + 31) / 32, 256, 0, s, nblk, nw,
+        launch_next("net_wgrad_sum", 4.0 * nblk * (double)nw, 0.0, k_wgrad_sum, (nw + 31) / 32, 256, 0, s, nblk, nw,
                (const float*)net->wgp, net->gr + net->woff[l]);
         IIM_LAUNCHED();
         if (l > 0) {
             const int n = net->ci[l] * net->co[l] * 9;
-            launch("net_flip", 0.0, 0.0, k_flip, (n + 255) / 256, 256, 0, s, net->ci[l], net->co[l],
+            launch_next("net_flip", 0.0, 0.0, k_flip, (n + 255) / 256, 256, 0, s, net->ci[l], net->co[l],
                    (const __nv_bfloat16*)(net->wb + net->woff[l]), net->wt);
             float* gprev = net->g0 + (size_t)((net->nl - 1 - l) & 1) * net->cap;
             IIM_CHECK(conv(net, g, gate, net->wt, nullptr, gprev, B, net->co[l], net->ci[l], H, W, d, 0, s));
@@ -847,7 +863,7 @@ static iim_status backward(iim_net_s* net, int B, int H, int W, const float* x, 
 }
 
 static iim_status sync_bf16(iim_net_s* net, cudaStream_t s) {
-    launch("net_bf16", 0.0, 0.0, k_to_bf16, (unsigned)((net->np + 255) / 256), 256, 0, s, (long)net->np,
+    launch_next("net_bf16", 0.0, 0.0, k_to_bf16, (unsigned)((net->np + 255) / 256), 256, 0, s, (long)net->np,
            (const float*)net->p, net->wb);
     IIM_LAUNCHED();
     net->wunit_ok = false;
@@ -977,15 +993,15 @@ extern "C" iim_status iim_net_train_step(iim_net net, int batch, int height, int
     const float* pred = net->act + (size_t)(net->nl - 1) * net->cap;
     float* diff = net->g0 + net->cap;
     const int nb = 256;
-    launch("net_mse", 12.0 * n, 0.0, k_mse_partial, nb, 256, 0, s, n, pred, target, mask, diff, net->red);
-    launch("net_mse_finish", 0.0, 0.0, k_mse_finish, 1, 32, 0, s, nb, net->red, net->red + 1024);
-    launch("net_scale", 0.0, 0.0, k_scale_vec, (unsigned)((n + 255) / 256), 256, 0, s, n, diff, (const float*)(net->red + 1025));
+    launch_next("net_mse", 12.0 * n, 0.0, k_mse_partial, nb, 256, 0, s, n, pred, target, mask, diff, net->red);
+    launch_next("net_mse_finish", 0.0, 0.0, k_mse_finish, 1, 32, 0, s, nb, net->red, net->red + 1024);
+    launch_next("net_scale", 0.0, 0.0, k_scale_vec, (unsigned)((n + 255) / 256), 256, 0, s, n, diff, (const float*)(net->red + 1025));
     IIM_LAUNCHED();
     IIM_CHECK(backward(net, batch, height, width, x, diff, s));
     net->t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.f - std::pow(b1, (float)net->t), c2 = 1.f - std::pow(b2, (float)net->t);
-    launch("net_adam", 0.0, 0.0, k_adam, (unsigned)((net->np + 255) / 256), 256, 0, s, (long)net->np, net->p,
+    launch_next("net_adam", 0.0, 0.0, k_adam, (unsigned)((net->np + 255) / 256), 256, 0, s, (long)net->np, net->p,
            (const float*)net->gr, net->m, net->v, lr, b1, b2, 1e-8f, c1, c2);
     IIM_LAUNCHED();
     IIM_CHECK(sync_bf16(net, s));
@@ -1002,7 +1018,7 @@ extern "C" iim_status iim_net_prepare_input(int nx, int ny, const double* omega,
                                             iim_stream stream) {
     if (nx < 3 || ny < 3 || !omega || !phi_nodes || !u_box || !x) return IIM_ERR_INVALID_ARG;
     const long n = (long)(nx - 1) * (ny - 1);
-    launch("net_input", 0.0, 0.0, k_net_input, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, nx - 1, ny - 1,
+    launch_next("net_input", 0.0, 0.0, k_net_input, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, nx - 1, ny - 1,
            omega, phi_nodes, u_box, s_omega, s_phi, s_box, x);
     IIM_LAUNCHED();
     return IIM_OK;
@@ -1011,7 +1027,7 @@ extern "C" iim_status iim_net_prepare_input(int nx, int ny, const double* omega,
 extern "C" iim_status iim_net_compose_guess(long long n, const double* u_box, const float* y, float s_out,
                                             double* psi_guess, iim_stream stream) {
     if (n < 0 || !u_box || !y || !psi_guess || !(s_out != 0.f)) return IIM_ERR_INVALID_ARG;
-    launch("net_guess", 0.0, 0.0, k_net_guess, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, (long)n, u_box, y,
+    launch_next("net_guess", 0.0, 0.0, k_net_guess, (unsigned)((n + 255) / 256), 256, 0, (cudaStream_t)stream, (long)n, u_box, y,
            1.f / s_out, psi_guess);
     IIM_LAUNCHED();
     return IIM_OK;

@@ -486,7 +486,7 @@ __device__ __forceinline__ double quotient(double s, double d) {
 // columns per group; `scale` carries the normalisation and h^2; tw: the table of e^{-i pi k / 4096}.
 // Each transform leaves its result in the buffer that its last step does not read.  Dynamic shared memory
 // sine_smem<T>(n, L).  Bound by FP64 arithmetic; against the packed transforms (dst.cuh), whole box solve in
-// FP64: 64^2 45 -> 35 us, 256^2 73 -> 54, 512^2 103 -> 95, 1024^2 304 -> 307, 2048^2 1466 -> 1101,
+// FP64: 64^2 45 -> 28 us, 256^2 73 -> 54, 512^2 103 -> 95, 1024^2 304 -> 307, 2048^2 1466 -> 1101,
 // 64 x 2048 256 -> 115.
 template <typename T, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))

@@ -201,7 +201,7 @@ static iim_status rows_fwd(const Plan<T>& p, int row0, int nrows, const double* 
     IIM_CHECK(sine_dispatch(p.nx, lpb, [&](auto N, auto L) -> iim_status {
         auto kern = k_sine_rows_fwd<T, N.value, L.value>;
         IIM_CHECK(allow_smem(kern, sm));
-        launch(sizeof(T) == 8 ? "dst_rows_fwd_f64" : "dst_rows_fwd_f32",
+        launch_next(sizeof(T) == 8 ? "dst_rows_fwd_f64" : "dst_rows_fwd_f32",
                (double)batch * nrows * p.NX * ((dense ? 8.0 : 0.0) + sizeof(T)), (double)batch * nrows * dst_flops(p.nx),
                kern, dim3((nrows + lpb - 1) / lpb, batch), (Sine<N.value, L.value>::kBlock), sm, s, p.NX, p.NY, p.nx, row0, nrows, dense,
                dld, doff, ring, ih2, row_ptr, aff_node, gam, gsign, sine_table<T>(p.nx), out, stop, dfs, ofs);
@@ -334,7 +334,7 @@ static iim_status rows_inv(const Plan<T>& p, int row0, int nrows, const T* in, T
     IIM_CHECK(sine_dispatch(p.nx, lpb, [&](auto N, auto L) -> iim_status {
         auto kern = k_sine_rows_inv<T, MODE, N.value, L.value>;
         IIM_CHECK(allow_smem(kern, sm));
-        launch(sizeof(T) == 8 ? "dst_rows_inv_f64" : "dst_rows_inv_f32",
+        launch_next(sizeof(T) == 8 ? "dst_rows_inv_f64" : "dst_rows_inv_f32",
                (double)batch * nrows * p.NX *
                    (sizeof(T) + (MODE == INV_STORE_T ? sizeof(T) : MODE == INV_STORE_F64 ? 8.0 : 17.0)),
                (double)batch * nrows * dst_flops(p.nx), kern, dim3((nrows + lpb - 1) / lpb, batch), (Sine<N.value, L.value>::kBlock), sm,
@@ -353,7 +353,7 @@ static iim_status box_cols(int nx, int ny, double h, double* buf, cudaStream_t s
     IIM_CHECK(sine_dispatch(ny, lpb, [&](auto N, auto L) -> iim_status {
         auto kern = k_sine_cols<double, N.value, L.value>;
         IIM_CHECK(allow_smem(kern, sm));
-        launch("sine_cols_f64", 16.0 * nx * (ny - 1), nx * (2.0 * dst_flops(ny) + 2.0 * ny), kern, nx / lpb,
+        launch_next("sine_cols_f64", 16.0 * nx * (ny - 1), nx * (2.0 * dst_flops(ny) + 2.0 * ny), kern, nx / lpb,
                (Sine<N.value, L.value>::kBlock), sm, s, nx, ny, buf, scale, sine_table<double>(ny), twiddles64());
         return IIM_OK;
     }));

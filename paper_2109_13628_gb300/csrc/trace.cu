@@ -44,6 +44,16 @@ bool chain_launch(cudaStream_t s) {
     return st == cudaStreamCaptureStatusActive && n == 1 && cudaGraphNodeGetType(deps[0], &type) == cudaSuccess &&
            type == cudaGraphNodeTypeKernel;
 }
+bool chain_stream(cudaStream_t s) {
+    if (t_capture) return chain_launch(s);
+    if (t_prof) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st == cudaStreamCaptureStatusNone;
+}
 bool profiling_active() { return t_prof; }
 void count_launches(long long n) { g_launches.fetch_add(n, std::memory_order_relaxed); }
 

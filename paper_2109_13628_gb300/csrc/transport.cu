@@ -134,6 +134,7 @@ __global__ void k_ext_velocity(int nm, TrView v, const int* __restrict__ minus_n
                                const uint8_t* __restrict__ minus_mask, const double* __restrict__ cp_t,
                                const double* __restrict__ ubx, const double* __restrict__ uby, double* __restrict__ gux,
                                double* __restrict__ guy) {
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3;
     const int m = min(t >> 2, nm - 1);   // the last warp stays whole for the shuffles
     const int mask = minus_mask[m] >> 4;
@@ -164,6 +165,7 @@ __global__ void k_ext_vorticity(int nm, TrView v, const int* __restrict__ minus_
                                 const uint8_t* __restrict__ minus_mask, const double* __restrict__ cp_t,
                                 const double* __restrict__ wb, double* __restrict__ g4, double* __restrict__ g3,
                                 double* __restrict__ g3n) {
+    pdl_wait();
     const int t = blockIdx.x * blockDim.x + threadIdx.x, d = t & 3;
     const int m = min(t >> 2, nm - 1);
     int mask = minus_mask[m];
@@ -208,6 +210,7 @@ __global__ void k_ext_vorticity(int nm, TrView v, const int* __restrict__ minus_
 __global__ void k_vorticity_bc(int ncp, TrView v, int nx_cells, int ny_cells, const int* __restrict__ cp_axis,
                                const int* __restrict__ cp_ei, const int* __restrict__ cp_ej, const double* __restrict__ cp_t,
                                const double* __restrict__ ubx, const double* __restrict__ uby, double* __restrict__ wb) {
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncp) return;
     const bool along_x = cp_axis[c] == 0;
@@ -268,6 +271,7 @@ __global__ void k_vorticity_bc(int ncp, TrView v, int nx_cells, int ny_cells, co
 // differences of the products, the third-order extensions (velocity with u_b, vorticity with
 // omega_b) at A- nodes and the box values beyond (caller layout, 0 in the solid).
 __global__ void k_pressure_rhs(TrView v, double* __restrict__ f) {
+    pdl_wait();
     const long n = (long)v.NX * v.NY;
     const long k = (long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -292,6 +296,7 @@ __global__ void k_pressure_wall_data(int ncp, TrView v, int nx_cells, int ny_cel
                                      const int* __restrict__ cp_ei, const int* __restrict__ cp_ej,
                                      const double* __restrict__ cp_t, const double* __restrict__ wb, double nu,
                                      double* __restrict__ out) {
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncp) return;
     const bool along_x = cp_axis[c] == 0;
@@ -340,6 +345,7 @@ __global__ void k_pressure_wall_data(int ncp, TrView v, int nx_cells, int ny_cel
 __global__ void k_wall_values(int ncp, TrView v, const int* __restrict__ cp_axis, const int* __restrict__ cp_ei,
                               const int* __restrict__ cp_ej, const double* __restrict__ cp_t,
                               const double* __restrict__ field, double* __restrict__ out) {
+    pdl_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= ncp) return;
     const bool along_x = cp_axis[c] == 0;
@@ -411,11 +417,12 @@ __device__ __forceinline__ void kelvin_body(const TrView& v, double c, int k, co
 // division each).  Faces whose stencil meets a solid node (found per block, then per face) take the
 // general form, from the tile and the extensions, so a face has one value whichever block evaluates
 // it.  The first nk blocks integrate one body's Kelvin ODE each (a chain of latencies: started first).
-// 1024 x 512, one cylinder: 98 -> 30 us (the whole right-hand side 177 -> 65 us).
+// 1024 x 512, one cylinder: 98 -> 30 us (the whole right-hand side 177 -> 55 us).
 constexpr int TR_X = 32, TR_Y = 16, TR_THREADS = 256, TR_W = TR_X + 4, TR_H = TR_Y + 4;
 __global__ void __launch_bounds__(TR_THREADS)
 k_transport_rhs(TrView v, double c, int mode, double a, double dt, double* __restrict__ out, int tx, int nk,
                 KelvinArgs kv) {
+    pdl_wait();
     if ((int)blockIdx.x < nk) {
         kelvin_body<TR_THREADS>(v, c, blockIdx.x, kv, a, dt);
         return;
@@ -556,6 +563,7 @@ k_transport_rhs(TrView v, double c, int mode, double a, double dt, double* __res
 
 __global__ void k_rk_omega(int NX, int NY, double b, const double* __restrict__ dw, const uint8_t* __restrict__ cls,
                            double* __restrict__ omega) {
+    pdl_wait();
     const int n = NX * NY;
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
@@ -566,6 +574,7 @@ __global__ void k_rk_omega(int NX, int NY, double b, const double* __restrict__ 
 
 template <int BLOCK>
 __global__ void k_speed_max(long n, const double* __restrict__ ux, const double* __restrict__ uy, double* __restrict__ part) {
+    pdl_wait();
     double m = 0.0;
     for (long k = (long)blockIdx.x * BLOCK + threadIdx.x; k < n; k += (long)gridDim.x * BLOCK)
         m = fmax(m, fabs(ux[k]) + fabs(uy[k]));
@@ -632,15 +641,15 @@ static iim_status prepare_stage(iim_geometry g, const TrWork& W, const TrView& v
     const double* uby = u_b ? u_b + g->ncp : W.zeros;
     const unsigned eb = (unsigned)((4 * g->nminus + 127) / 128);   // four lanes per A- node
     if (g->nminus > 0)
-        launch("tr_ext_velocity", 0.0, 0.0, k_ext_velocity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
+        launch_next("tr_ext_velocity", 0.0, 0.0, k_ext_velocity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
                g->minus_mask, g->cp_t, ubx, uby, W.gux, W.guy);
     if (g->ncp > 0 && wb_in) {
         IIM_TRY(cudaMemcpyAsync(W.wb, wb_in, g->ncp * sizeof(double), cudaMemcpyDeviceToDevice, s));
     } else if (g->ncp > 0)
-        launch("tr_vorticity_bc", 0.0, 0.0, k_vorticity_bc, (g->ncp + 63) / 64, 64, 0, s, g->ncp, v, g->nx, g->ny,
+        launch_next("tr_vorticity_bc", 0.0, 0.0, k_vorticity_bc, (g->ncp + 63) / 64, 64, 0, s, g->ncp, v, g->nx, g->ny,
                g->cp_axis, g->cp_ei, g->cp_ej, g->cp_t, ubx, uby, W.wb);
     if (g->nminus > 0)
-        launch("tr_ext_vorticity", 0.0, 0.0, k_ext_vorticity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
+        launch_next("tr_ext_vorticity", 0.0, 0.0, k_ext_vorticity, eb, 128, 0, s, g->nminus, v, g->minus_node, g->minus_cp,
                g->minus_mask, g->cp_t, W.wb, W.g4, W.g3, W.g3n);
     IIM_LAUNCHED();
     if (wb_out && g->ncp > 0)
@@ -654,7 +663,7 @@ static iim_status transport_rhs(iim_geometry g, const TrView& v, double nu, int 
                                 const KelvinArgs& kv, cudaStream_t s) {
     const int tx = (g->NX + TR_X - 1) / TR_X, ty = (g->NY + TR_Y - 1) / TR_Y;
     const int nk = kv.R ? g->nb : 0;
-    launch("tr_rhs", 40.0 * (double)g->NX * g->NY, 0.0, k_transport_rhs, tx * ty + nk, TR_THREADS, 0, s, v, nu / g->h, mode,
+    launch_next("tr_rhs", 40.0 * (double)g->NX * g->NY, 0.0, k_transport_rhs, tx * ty + nk, TR_THREADS, 0, s, v, nu / g->h, mode,
            a, dt, out, tx, nk, kv);
     IIM_LAUNCHED();
     return IIM_OK;
@@ -688,9 +697,9 @@ extern "C" iim_status iim_total_pressure_problem(iim_geometry g, const double* o
     const TrView v = make_view(g, W, Uinf, omega, ux, uy);
     IIM_CHECK(prepare_stage(g, W, v, u_b, omega_b_in, omega_b_out, s));
     const long n = (long)g->NX * g->NY;
-    launch("pressure_rhs", 48.0 * (double)n, 0.0, k_pressure_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, f_out);
+    launch_next("pressure_rhs", 48.0 * (double)n, 0.0, k_pressure_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, f_out);
     if (g->ncp > 0)
-        launch("pressure_wall_data", 0.0, 0.0, k_pressure_wall_data, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->nx,
+        launch_next("pressure_wall_data", 0.0, 0.0, k_pressure_wall_data, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->nx,
                g->ny, g->cp_axis, g->cp_ei, g->cp_ej, g->cp_t, (const double*)W.wb, nu, data_out);
     IIM_LAUNCHED();
     return IIM_OK;
@@ -703,7 +712,7 @@ extern "C" iim_status iim_wall_values(iim_geometry g, const double* field, doubl
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
     const TrView v = make_view(g, W, nullptr, nullptr, nullptr, nullptr);
-    launch("wall_values", 0.0, 0.0, k_wall_values, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->cp_axis, g->cp_ei,
+    launch_next("wall_values", 0.0, 0.0, k_wall_values, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->cp_axis, g->cp_ei,
            g->cp_ej, g->cp_t, field, out);
     IIM_LAUNCHED();
     return IIM_OK;
@@ -734,6 +743,7 @@ static constexpr double kRK3C[3] = {0.0, 1.0 / 3.0, 3.0 / 4.0};
 // u_b at a stage time: u_b + c dt du_b/dt (u_b NULL = 0)
 __global__ void k_ub_stage(int m, const double* __restrict__ ub, const double* __restrict__ rate, double cdt,
                            double* __restrict__ out) {
+    pdl_wait();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e < m) out[e] = (ub ? ub[e] : 0.0) + cdt * rate[e];
 }
@@ -758,7 +768,7 @@ static iim_status rk3_step(iim_geometry g, double* omega, double* gamma, double*
         if (per_stage) per_stage[st] = stats;
         if (ps != IIM_OK) return ps;
         if (st == 0 && dt <= 0.0) {
-            launch("tr_speed_max", 0.0, 0.0, k_speed_max<256>, 256, 256, 0, s, n, (const double*)W.vx, (const double*)W.vy,
+            launch_next("tr_speed_max", 0.0, 0.0, k_speed_max<256>, 256, 256, 0, s, n, (const double*)W.vx, (const double*)W.vy,
                    W.part);
             IIM_LAUNCHED();
             std::vector<double> part(256);
@@ -773,14 +783,14 @@ static iim_status rk3_step(iim_geometry g, double* omega, double* gamma, double*
         if (u_b_rate) {
             const int m = 2 * g->ncp;
             if (m > 0)
-                launch("tr_ub_stage", 0.0, 0.0, k_ub_stage, (unsigned)((m + 255) / 256), 256, 0, s, m, u_b, u_b_rate,
+                launch_next("tr_ub_stage", 0.0, 0.0, k_ub_stage, (unsigned)((m + 255) / 256), 256, 0, s, m, u_b, u_b_rate,
                        kRK3C[st] * dt, W.ub_stage);
             ub = W.ub_stage;
         }
         IIM_CHECK(prepare_stage(g, W, v, ub, nullptr, nullptr, s));
         const KelvinArgs kv{g->d_regions, nullptr, 1, kRK3B[st], W.dG, gamma};
         IIM_CHECK(transport_rhs(g, v, nu, 1, kRK3A[st], dt, W.dw, kv, s));
-        launch("tr_rk_omega", 24.0 * (double)n, 0.0, k_rk_omega, (unsigned)((n + 255) / 256), 256, 0, s, g->NX, g->NY,
+        launch_next("tr_rk_omega", 24.0 * (double)n, 0.0, k_rk_omega, (unsigned)((n + 255) / 256), 256, 0, s, g->NX, g->NY,
                kRK3B[st], (const double*)W.dw, g->node_class, omega);
         IIM_LAUNCHED();
     }

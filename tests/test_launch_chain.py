@@ -20,7 +20,7 @@ def kernels(text):
 
 
 @pytest.mark.parametrize("name", ["solve.cu", "lockstep.cu", "krylov.cuh", "sine.cuh", "dst.cuh", "freespace.cu",
-                                  "precond.cu"])
+                                  "precond.cu", "net.cu", "transport.cu"])
 def test_every_kernel_waits_first(name):
     with open(os.path.join(CSRC, name)) as f:
         found = list(kernels(f.read()))
