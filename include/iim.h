@@ -387,6 +387,7 @@ iim_status iim_cv_terms(iim_geometry g, const double* psi, const double* ux, con
  *   omega_b_out    |C| values or NULL (the omega_b used)
  *   rhs_out        interior array: d omega / dt (0 in the solid)
  *   dgamma_out     n_bodies values: -h sum_{dR_k}(f + q).n, or NULL
+ * The outputs may overlap omega, ux and uy (each is then read from a copy).
  * Box: vorticity 0 at and beyond the box except the right edge (outflow), which copies the
  * last interior column.  Errors: IIM_ERR_INVALID_ARG, IIM_ERR_CUDA.  Asynchronous. */
 iim_status iim_transport_rhs(iim_geometry g, const double* omega, const double* ux, const double* uy,
@@ -409,7 +410,7 @@ iim_status iim_transport_rhs(iim_geometry g, const double* omega, const double* 
  *              crossing: the cross-line stencil of the vorticity boundary condition (Sec. 5.3, as
  *              in iim_transport_rhs) on the vorticity extended at third order with omega_b.
  *   other arguments as in iim_transport_rhs (u_b only extends the velocity: the wall relation
- *              above assumes a stationary wall).
+ *              above assumes a stationary wall).  The outputs may overlap omega, ux and uy.
  * Errors: IIM_ERR_INVALID_ARG, IIM_ERR_CUDA.  Asynchronous. */
 iim_status iim_total_pressure_problem(iim_geometry g, const double* omega, const double* ux, const double* uy,
                                       const double* u_b, const double Uinf[2], double nu, const double* omega_b_in,

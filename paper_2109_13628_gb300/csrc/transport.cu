@@ -21,7 +21,10 @@
 // edge, where the last interior column is copied (zero gradient).
 #include <algorithm>
 #include <cmath>
+#include <cstdint>
 #include <cstring>
+#include <initializer_list>
+#include <utility>
 
 #include "common.cuh"
 
@@ -634,6 +637,30 @@ static TrView make_view(iim_geometry g, const TrWork& W, const double Uinf[2], c
     return v;
 }
 
+// The kernels read the caller's fields, neighbours included, while others write results: a field that an
+// output overlaps is read from a copy (outputs in place of inputs are allowed, as with separate arrays).
+struct Span {
+    const double* p;
+    size_t n;
+};
+static iim_status detach_fields(iim_geometry g, const TrWork& W, std::initializer_list<Span> outs, const double** omega,
+                                const double** ux, const double** uy, cudaStream_t s) {
+    const size_t n = (size_t)g->NX * g->NY;
+    const std::pair<const double**, double*> fields[3] = {{omega, W.psi}, {ux, W.vx}, {uy, W.vy}};
+    for (const auto& f : fields) {
+        const uintptr_t a = (uintptr_t)*f.first;
+        bool hit = false;
+        for (const Span& o : outs) {
+            const uintptr_t b = (uintptr_t)o.p;
+            hit = hit || (o.p && a < b + o.n * sizeof(double) && b < a + n * sizeof(double));
+        }
+        if (!hit) continue;
+        IIM_TRY(cudaMemcpyAsync(f.second, *f.first, n * sizeof(double), cudaMemcpyDefault, s));
+        *f.first = f.second;
+    }
+    return IIM_OK;
+}
+
 // Velocity extension; vorticity BC; vorticity extensions (v holds the fields).
 static iim_status prepare_stage(iim_geometry g, const TrWork& W, const TrView& v, const double* u_b,
                                 const double* wb_in, double* wb_out, cudaStream_t s) {
@@ -680,6 +707,8 @@ extern "C" iim_status iim_transport_rhs(iim_geometry g, const double* omega, con
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
+    const size_t n = (size_t)g->NX * g->NY, ncp = (size_t)g->ncp;
+    IIM_CHECK(detach_fields(g, W, {{rhs_out, n}, {omega_b_out, ncp}, {dgamma_out, (size_t)g->nb}}, &omega, &ux, &uy, s));
     const TrView v = make_view(g, W, Uinf, omega, ux, uy);
     IIM_CHECK(prepare_stage(g, W, v, u_b, omega_b_in, omega_b_out, s));
     const KelvinArgs kv{dgamma_out ? g->d_regions : nullptr, dgamma_out, 0, 0.0, nullptr, nullptr};
@@ -694,9 +723,11 @@ extern "C" iim_status iim_total_pressure_problem(iim_geometry g, const double* o
     cudaStream_t s = (cudaStream_t)stream;
     TrWork W;
     IIM_CHECK(tr_work(g, &W));
+    const long n = (long)g->NX * g->NY;
+    const size_t ncp = (size_t)g->ncp;
+    IIM_CHECK(detach_fields(g, W, {{f_out, (size_t)n}, {data_out, ncp}, {omega_b_out, ncp}}, &omega, &ux, &uy, s));
     const TrView v = make_view(g, W, Uinf, omega, ux, uy);
     IIM_CHECK(prepare_stage(g, W, v, u_b, omega_b_in, omega_b_out, s));
-    const long n = (long)g->NX * g->NY;
     launch_next("pressure_rhs", 48.0 * (double)n, 0.0, k_pressure_rhs, (unsigned)((n + 255) / 256), 256, 0, s, v, f_out);
     if (g->ncp > 0)
         launch_next("pressure_wall_data", 0.0, 0.0, k_pressure_wall_data, (g->ncp + 127) / 128, 128, 0, s, g->ncp, v, g->nx,
