@@ -1528,6 +1528,8 @@ struct Solver {
     double seed_scale = 0.0, seed_reduction = 1.0;   // the seed's c and ||b - S c x0|| / ||b||
 };
 
+static void drop_solve_graph(iim_geometry g);
+
 // Krylov buffers for restart length m (with the z_j of the preconditioned iteration when pc).
 static iim_status ensure_krylov(iim_geometry g, int m, bool pc) {
     const int ns = g->na + g->ncirc;
@@ -1535,6 +1537,13 @@ static iim_status ensure_krylov(iim_geometry g, int m, bool pc) {
         if (pc && !g->Z) IIM_TRY(cudaMalloc(&g->Z, sizeof(double) * (size_t)(std::max(g->krylov_m, 2) + 1) * std::max(ns, 1)));
         return IIM_OK;
     }
+    // every captured graph holds the buffers freed here, and the new ones may come back at an old address
+    drop_solve_graph(g);
+    for (void** gp : {&g->graph64, &g->graph32}) {
+        IterGraph* G = (IterGraph*)*gp;
+        if (G && G->exec) { cudaGraphExecDestroy(G->exec); G->exec = nullptr; }
+    }
+    g->krylov_m = 0;                       // until all of them are there
     const int cols = std::max(m, 2) + 1;   // a restart uses columns 0 to 2
     cudaFree(g->Z);
     g->Z = nullptr;
@@ -1555,11 +1564,6 @@ static iim_status ensure_krylov(iim_geometry g, int m, bool pc) {
     IIM_TRY(cudaMemset(g->xsol, 0, sizeof(double) * (size_t)std::max(ns, 1)));
     IIM_TRY(cudaMemset(g->bvec, 0, sizeof(double) * (size_t)std::max(ns, 1)));
     g->krylov_m = m;
-    // the captured iteration graphs refer to the old buffers
-    for (void** gp : {&g->graph64, &g->graph32}) {
-        IterGraph* G = (IterGraph*)*gp;
-        if (G && G->exec) { cudaGraphExecDestroy(G->exec); G->exec = nullptr; }
-    }
     return IIM_OK;
 }
 
