@@ -13,12 +13,19 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <initializer_list>
 #include <random>
 #include <vector>
 
 #include "common.cuh"
 #include "iim_ops.cuh"
 #include "tcgen05.cuh"
+
+// Buffers that grow with the sizes of the calls (grow() below).
+struct NetBuffers {
+    size_t n = 0;             // items they hold
+    std::vector<void*> old;   // outgrown
+};
 
 struct iim_net_s {
     int device = 0;
@@ -36,20 +43,20 @@ struct iim_net_s {
     float* act = nullptr;                // layer outputs, nl x cap floats
     float* g0 = nullptr;                 // gradient ping-pong, 2 x cap floats
     float* red = nullptr;                // reductions
-    long long cap = 0;                   // floats per activation buffer
+    NetBuffers acts;                     // act and g0; items: floats per layer (cap())
+    size_t act_try = 0;                  // largest size inference has asked them for
+    size_t cap() const { return acts.n; }
     float* h_red = nullptr;              // pinned
     int tc = 0;                          // tensor cores (k_conv_tc): 0 off, 1 the 32 -> 32 layers, 2 every layer
     __nv_bfloat16* wtc = nullptr;        // one layer's weights in the tensor-core operand layout
-    float* wgp = nullptr;                // weight gradient: one buffer of sums per block (on first use)
+    float* wgp = nullptr;                // weight gradient: one buffer of sums per block
     int wg_blocks = 0;
     // inference on the tensor cores: every layer's weights in the operand layout, and two activation
     // buffers of BF16 channel units with a zero border.  Every call writes what it reads of them (a captured
-    // call replays between others); buffers outgrown by a larger call stay until the net is destroyed, since
-    // a caller's graph may hold them.
+    // call replays between others).
     __nv_bfloat16* wunit = nullptr;
     uint4* unit[2] = {nullptr, nullptr};
-    size_t unit_n = 0;                   // units per buffer
-    std::vector<uint4*> unit_old;
+    NetBuffers units;                    // both; items: units of one
     int* tc_err = nullptr;               // set by k_conv_tc when its wait for the MMAs timed out
 };
 
@@ -801,39 +808,63 @@ static iim_status conv(iim_net_s* net, const float* x, const float* gate, const 
 
 static int max_dilation(const iim_net_s* net) { return *std::max_element(net->dil.begin(), net->dil.end()); }
 
-// Both activation buffers grown to hold `need` units.  They grow by doubling, so that the outgrown ones that
-// are kept add up to less than the last; only where the device has no room beside those are they given up.
-static iim_status grow_units(iim_net_s* net, size_t need) {
-    auto alloc = [&](size_t n, uint4* (&p)[2]) {
-        cudaError_t e = cudaMalloc(&p[0], n * sizeof(uint4));
-        if (e == cudaSuccess && (e = cudaMalloc(&p[1], n * sizeof(uint4))) != cudaSuccess) cudaFree(p[0]);
-        return e;
-    };
-    size_t n = std::max(need, 2 * net->unit_n);
-    uint4* p[2] = {nullptr, nullptr};
-    cudaError_t e = alloc(n, p);
-    if (e == cudaErrorMemoryAllocation) {
-        cudaGetLastError();
-        for (uint4* q : net->unit_old) cudaFree(q);
-        net->unit_old.clear();
-        for (uint4*& q : net->unit) {
-            cudaFree(q);
-            q = nullptr;
+// The buffers at `parts` (bytes per item each) grown to hold `need` items.  Outgrown ones are kept until the
+// net is destroyed, since a caller's graph may hold them; they grow by doubling, so that those add up to
+// less than the last.  Only where the device has no room beside them are they given up (`optional`: left as
+// they are, with an error).
+struct NetPart {
+    void** p;
+    size_t bytes;
+};
+static iim_status grow(NetBuffers& b, size_t need, std::initializer_list<NetPart> parts, bool optional = false) {
+    if (need <= b.n) return IIM_OK;
+    std::vector<void*> got;
+    auto alloc = [&](size_t n) {
+        for (const NetPart& part : parts) {
+            void* q = nullptr;
+            const cudaError_t e = cudaMalloc(&q, n * part.bytes);
+            if (e != cudaSuccess) {
+                cudaGetLastError();
+                for (void* r : got) cudaFree(r);
+                got.clear();
+                return e;
+            }
+            got.push_back(q);
         }
-        net->unit_n = 0;
+        return cudaSuccess;
+    };
+    size_t n = std::max(need, 2 * b.n);
+    cudaError_t e = alloc(n);
+    if (e == cudaErrorMemoryAllocation && !optional) {
+        for (void* q : b.old) cudaFree(q);
+        b.old.clear();
+        for (const NetPart& part : parts) {
+            cudaFree(*part.p);
+            *part.p = nullptr;
+        }
+        b.n = 0;
         n = need;
-        e = alloc(n, p);
+        e = alloc(n);
     }
     if (e != cudaSuccess) {
-        record_cuda_error(e, "cudaMalloc", __FILE__, __LINE__);
+        if (!optional) record_cuda_error(e, "cudaMalloc", __FILE__, __LINE__);
         return IIM_ERR_CUDA;
     }
-    for (int k = 0; k < 2; ++k) {
-        if (net->unit[k]) net->unit_old.push_back(net->unit[k]);
-        net->unit[k] = p[k];
+    size_t k = 0;
+    for (const NetPart& part : parts) {
+        if (*part.p) b.old.push_back(*part.p);
+        *part.p = got[k++];
     }
-    net->unit_n = n;
+    b.n = n;
     return IIM_OK;
+}
+// Activations and gradients of training (and of inference off the tensor cores) for B images.
+static size_t act_floats(const iim_net_s* net, int B, int H, int W) {
+    return (size_t)B * H * W * std::max(net->hidden, 1);
+}
+static iim_status ensure_acts(iim_net_s* net, size_t need, bool optional = false) {
+    return grow(net->acts, need, {{(void**)&net->act, sizeof(float) * net->nl}, {(void**)&net->g0, sizeof(float) * 2}},
+                optional);
 }
 
 // The whole network on the tensor cores for inference (every layer; net->tc == 2): y (batch, 1, h, w).
@@ -843,7 +874,7 @@ static iim_status forward_units(iim_net_s* net, int B, int H, int W, const float
     int planes = (net->cin + 7) / 8;
     if (net->nl > 1) planes = std::max(planes, (net->hidden + 7) / 8);
     const size_t need = (size_t)B * planes * u.Hp * u.Wp;
-    if (need > net->unit_n) IIM_CHECK(grow_units(net, need));
+    IIM_CHECK(grow(net->units, need, {{(void**)&net->unit[0], sizeof(uint4)}, {(void**)&net->unit[1], sizeof(uint4)}}));
     if (!net->wunit) IIM_TRY(cudaMalloc(&net->wunit, sizeof(uint4) * WUNIT * net->nl));
     UnitLayers L{net->nl};
     for (int l = 0; l < net->nl; ++l) {
@@ -881,23 +912,11 @@ static iim_status forward_units(iim_net_s* net, int B, int H, int W, const float
     return IIM_OK;
 }
 
-static iim_status ensure_cap(iim_net_s* net, long long need) {
-    if (need <= net->cap) return IIM_OK;
-    cudaFree(net->act);
-    cudaFree(net->g0);
-    net->act = net->g0 = nullptr;
-    IIM_TRY(cudaMalloc(&net->act, sizeof(float) * (size_t)need * net->nl));
-    IIM_TRY(cudaMalloc(&net->g0, sizeof(float) * (size_t)need * 2));
-    net->cap = need;
-    return IIM_OK;
-}
-
 static iim_status forward(iim_net_s* net, int B, int H, int W, const float* x, cudaStream_t s) {
-    const long long cap = (long long)B * H * W * std::max(net->hidden, 1);
-    IIM_CHECK(ensure_cap(net, cap));
+    IIM_CHECK(ensure_acts(net, act_floats(net, B, H, W)));
     const float* in = x;
     for (int l = 0; l < net->nl; ++l) {
-        float* out = net->act + (size_t)l * net->cap;
+        float* out = net->act + (size_t)l * net->cap();
         IIM_CHECK(conv(net, in, nullptr, net->wb + net->woff[l], net->p + net->boff[l], out, B, net->ci[l], net->co[l], H, W,
                        net->dil[l], l < net->nl - 1, s));
         in = out;
@@ -907,14 +926,10 @@ static iim_status forward(iim_net_s* net, int B, int H, int W, const float* x, c
 
 // gradients of sum(dy * pred) w.r.t. the parameters (into net->gr); dy is overwritten
 static iim_status backward(iim_net_s* net, int B, int H, int W, const float* x, float* dy, cudaStream_t s) {
-    if (!net->wgp) {
-        net->wg_blocks = 2 * sm_count();   // two resident blocks per SM
-        IIM_TRY(cudaMalloc(&net->wgp, sizeof(float) * (size_t)net->wg_blocks * WG_PART));
-    }
     float* g = dy;
     for (int l = net->nl - 1; l >= 0; --l) {
-        const float* xin = l == 0 ? x : net->act + (size_t)(l - 1) * net->cap;
-        const float* gate = l == net->nl - 1 ? nullptr : net->act + (size_t)l * net->cap;
+        const float* xin = l == 0 ? x : net->act + (size_t)(l - 1) * net->cap();
+        const float* gate = l == net->nl - 1 ? nullptr : net->act + (size_t)l * net->cap();
         const int d = net->dil[l];
         const size_t sm = wgrad_smem(wg_groups(net->co[l], 8), wg_groups(net->ci[l], 4), d);
         const int strips = B * H * ((W + WG_PX - 1) / WG_PX), nblk = std::min(strips, net->wg_blocks);
@@ -930,7 +945,7 @@ static iim_status backward(iim_net_s* net, int B, int H, int W, const float* x, 
             const int n = net->ci[l] * net->co[l] * 9;
             launch_next("net_flip", 0.0, 0.0, k_flip, (n + 255) / 256, 256, 0, s, net->ci[l], net->co[l],
                    (const __nv_bfloat16*)(net->wb + net->woff[l]), net->wt);
-            float* gprev = net->g0 + (size_t)((net->nl - 1 - l) & 1) * net->cap;
+            float* gprev = net->g0 + (size_t)((net->nl - 1 - l) & 1) * net->cap();
             IIM_CHECK(conv(net, g, gate, net->wt, nullptr, gprev, B, net->co[l], net->ci[l], H, W, d, 0, s));
             g = gprev;
         }
@@ -984,7 +999,7 @@ extern "C" iim_status iim_net_create(int in_channels, int hidden, int n_layers, 
     auto fail = [&](cudaError_t e) {
         record_cuda_error(e, "iim_net_create", __FILE__, __LINE__);
         cudaFree(net->p); cudaFree(net->gr); cudaFree(net->m); cudaFree(net->v); cudaFree(net->wb); cudaFree(net->wt);
-        cudaFree(net->red); cudaFree(net->wtc); cudaFree(net->tc_err);
+        cudaFree(net->red); cudaFree(net->wtc); cudaFree(net->tc_err); cudaFree(net->wgp);
         delete net;
         return IIM_ERR_CUDA;
     };
@@ -998,6 +1013,8 @@ extern "C" iim_status iim_net_create(int in_channels, int hidden, int n_layers, 
     if ((e = cudaMalloc(&net->red, sizeof(float) * 4096)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc(&net->wtc, sizeof(__nv_bfloat16) * 9 * 4 * TC_C * 8)) != cudaSuccess) return fail(e);
     if ((e = cudaMalloc(&net->tc_err, sizeof(int))) != cudaSuccess) return fail(e);
+    net->wg_blocks = 2 * sm_count();   // two resident blocks per SM
+    if ((e = cudaMalloc(&net->wgp, sizeof(float) * (size_t)net->wg_blocks * WG_PART)) != cudaSuccess) return fail(e);
     cudaMemset(net->tc_err, 0, sizeof(int));
     net->tc = 2;
     if ((e = cudaMemcpy(net->p, h.data(), sizeof(float) * off, cudaMemcpyHostToDevice)) != cudaSuccess) return fail(e);
@@ -1034,10 +1051,22 @@ extern "C" iim_status iim_net_forward(iim_net net, int batch, int height, int wi
     if (!net || !x || !y || batch < 1 || height < 1 || width < 1) return IIM_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     // one image's planes and the tiles are counted in 32 bits
-    if (net->tc == 2 && (long long)batch * ((height + 127) / 4 + 1) * (width / UN_M + 1) < (1LL << 30) && batch <= 65535)
+    if (net->tc == 2 && (long long)batch * ((height + 127) / 4 + 1) * (width / UN_M + 1) < (1LL << 30) && batch <= 65535) {
+        // the buffers of a training step of this size, which a stream capture could not allocate after this
+        // call; inference itself does without them
+        const size_t need = act_floats(net, batch, height, width);
+        if (need > net->act_try) {
+            cudaStreamCaptureStatus st = cudaStreamCaptureStatusActive;
+            if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+            if (st == cudaStreamCaptureStatusNone) {
+                net->act_try = need;
+                (void)ensure_acts(net, need, true);
+            }
+        }
         return forward_units(net, batch, height, width, x, y, s);
+    }
     IIM_CHECK(forward(net, batch, height, width, x, s));
-    IIM_TRY(cudaMemcpyAsync(y, net->act + (size_t)(net->nl - 1) * net->cap, sizeof(float) * (size_t)batch * height * width,
+    IIM_TRY(cudaMemcpyAsync(y, net->act + (size_t)(net->nl - 1) * net->cap(), sizeof(float) * (size_t)batch * height * width,
                             cudaMemcpyDeviceToDevice, s));
     return IIM_OK;
 }
@@ -1048,7 +1077,7 @@ extern "C" iim_status iim_net_backward(iim_net net, int batch, int height, int w
     cudaStream_t s = (cudaStream_t)stream;
     IIM_CHECK(forward(net, batch, height, width, x, s));
     const size_t n = (size_t)batch * height * width;
-    float* g = net->g0 + net->cap;   // scratch copy of dy (the backward pass overwrites its input)
+    float* g = net->g0 + net->cap();   // scratch copy of dy (the backward pass overwrites its input)
     IIM_TRY(cudaMemcpyAsync(g, dy, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
     IIM_CHECK(backward(net, batch, height, width, x, g, s));
     if (grad_host) {
@@ -1065,8 +1094,8 @@ extern "C" iim_status iim_net_train_step(iim_net net, int batch, int height, int
     cudaStream_t s = (cudaStream_t)stream;
     IIM_CHECK(forward(net, batch, height, width, x, s));
     const long n = (long)batch * height * width;
-    const float* pred = net->act + (size_t)(net->nl - 1) * net->cap;
-    float* diff = net->g0 + net->cap;
+    const float* pred = net->act + (size_t)(net->nl - 1) * net->cap();
+    float* diff = net->g0 + net->cap();
     const int nb = 256;
     launch_next("net_mse", 12.0 * n, 0.0, k_mse_partial, nb, 256, 0, s, n, pred, target, mask, diff, net->red);
     launch_next("net_mse_finish", 0.0, 0.0, k_mse_finish, 1, 32, 0, s, nb, net->red, net->red + 1024);
@@ -1126,7 +1155,8 @@ extern "C" void iim_net_destroy(iim_net net) {
     if (!net) return;
     cudaFree(net->p); cudaFree(net->gr); cudaFree(net->m); cudaFree(net->v); cudaFree(net->wb); cudaFree(net->wt);
     cudaFree(net->act); cudaFree(net->g0); cudaFree(net->red); cudaFree(net->wgp);
-    for (uint4* p : net->unit_old) cudaFree(p);
+    for (const NetBuffers* b : {&net->acts, &net->units})
+        for (void* p : b->old) cudaFree(p);
     cudaFree(net->wunit); cudaFree(net->unit[0]); cudaFree(net->unit[1]); cudaFree(net->wtc); cudaFree(net->tc_err);
     if (net->h_red) cudaFreeHost(net->h_red);
     delete net;

@@ -103,3 +103,26 @@ def test_replay_between_calls_of_another_size(other):
         g.replay()
         assert torch.equal(y, direct(p, x))
     n.close()
+
+
+@pytest.mark.parametrize("shape", [(2, 37, 150), (1, 64, 64)])
+def test_training_step_captured_after_inference_only(shape):
+    """The buffers of a training step exist once a direct call of the size has run, whichever it was."""
+    p = weights(7)
+    x = image(shape, 8)
+    t = torch.zeros(shape[0], 1, *shape[1:], device="cuda")
+    m = torch.ones_like(t)
+    n, ref = net_with(p), net_with(p)
+    forward(n, x)
+    ref.train_step(x, t, m, 0.01)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        n.train_step(x, t, m, 0.01, want_loss=False)
+    x2 = image((3, 90, 90), 9)
+    assert torch.equal(forward(n, x2), direct(p, x2))      # larger buffers; the graph keeps its own
+    g.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(n.get(), ref.get()) and not np.array_equal(n.get(), p)
+    n.close()
+    ref.close()
