@@ -114,10 +114,12 @@ __device__ __noinline__ double t_face_flux(const TrView& v, double c, int axis, 
     return t_flux(pos, p[0], p[1], p[2], t_omega(v, 0, ai, aj), t_omega(v, 0, bi, bj), c);
 }
 
-// a / h: a product when 1 / h is exact, else the product corrected by one residual step (Markstein).
+// a / h: a product when 1 / h is exact, else the product corrected by one residual step (Markstein), which
+// an infinite product does not take (its residual is inf - inf).
 __device__ __forceinline__ double t_div_h(const TrView& v, double a) {
     const double q = a * v.rh;
-    return v.h_pow2 ? q : fma(fma(-q, v.h, a), v.rh, q);
+    const bool finite = (__double2hiint(q) & 0x7ff00000) != 0x7ff00000;
+    return v.h_pow2 || !finite ? q : fma(fma(-q, v.h, a), v.rh, q);
 }
 
 // Sums over the four lanes of one A- node in direction order (the lanes of a warp are nodes x
