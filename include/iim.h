@@ -81,7 +81,10 @@ typedef struct {
                           when c = 0 -- the learned-guess path */
     double inner_rtol; /* Krylov tolerance of each correction solve (<= 0: library default,
                           rtol/20 in FP64 mode, 1e-4 in mixed mode; with precond 1 or 3 in mixed mode
-                          also no more than the un-reduced residual of the correction calls for) */
+                          also at most max(1e-5 of the un-reduced residual, rtol/100 of ||f||),
+                          except in a correction that starts from a seed, guess = 2).  Corrections
+                          are then strong and few, and the last one ends anywhere below rtol: a
+                          caller that needs a margin under rtol asks for a smaller rtol */
     int precond;       /* 0: plain GMRES; 1: right-precondition GMRES with the dense inverse of
                           the Schur matrix (built on first use, see iim_build_preconditioner);
                           2: each correction applies that inverse once, x = M b, with no Krylov

@@ -1701,7 +1701,7 @@ double inner_tolerance(const iim_opts& o, double* kappa, double* last) {
     if (o.prec == IIM_FP64) return o.rtol / 20.0;
     if (o.precond == 1 || o.precond == 3) {
         *kappa = 1e-5;
-        *last = 0.1 * o.rtol;
+        *last = 0.01 * o.rtol;
     }
     return 1e-4;
 }
