@@ -140,17 +140,14 @@ enum { DI_J = 0, DI_STOP = 1, DI_IT = 2, DI_MAXIT = 3, DI_CONV = 4, DI_TMPJ = 5,
        DI_RSS = 15, DI_TICKET = 18, DI_CIRC = 32 };
 
 // Krylov small-storage layout inside g->H (m <= 64):
-//   H (m+1) x m column-major | cs[m] | sn[m] | gv[m+1] | hc1[m+1] | hc2[m+1] | y[m] | scal[8]
+//   H (m+1) x m column-major | cs[m] | sn[m] | gv[m+1] | scal[8]
 struct KLayout {
     int m;
     __host__ __device__ long H() const { return 0; }
     __host__ __device__ long cs() const { return (long)(m + 1) * m; }
     __host__ __device__ long sn() const { return cs() + m; }
     __host__ __device__ long gv() const { return sn() + m; }
-    __host__ __device__ long hc1() const { return gv() + m + 1; }
-    __host__ __device__ long hc2() const { return hc1() + m + 1; }
-    __host__ __device__ long y() const { return hc2() + m + 1; }
-    __host__ __device__ long scal() const { return y() + m; }
+    __host__ __device__ long scal() const { return gv() + m + 1; }
     __host__ __device__ long total() const { return scal() + 8; }
 };
 enum { SC_INV = 0, SC_RESID = 1, SC_BETA = 2, SC_TOL = 3 };

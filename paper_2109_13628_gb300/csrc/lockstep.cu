@@ -542,7 +542,7 @@ bool lockstep_eligible(iim_geometry g, const iim_opts& o) {
     return g_ls_group.load() >= 2 && g->host_solves > 0 && !g->solve_graph_failed && o.guess == 0 && !g->outer &&
            (o.precond == 1 || (o.precond == 3 && g->pc_S)) && ns > 0 && g->pc_ready &&
            g->V && g->Z && g->krylov_m >= o.restart && (g->ncirc == 0 || g->cap_ready) &&
-           sizeof(float) * 4 * (size_t)((ns + 3) & ~3) <= 200 * 1024;
+           dense_matvec_fits(ns);
 }
 
 static void fill_prob(LsProb& q, iim_geometry g, int prec, const double* omega, const double* psi_b,
