@@ -70,7 +70,7 @@ def kernel_source_hash():
     """Hash of the files holding the transform kernels' code (the launch shape of a capture is
     recorded beside it: tile width, fields per launch)."""
     h = hashlib.sha256()
-    for f in ("dst.cuh", "tri.cuh"):
+    for f in ("dst.cuh", "sine.cuh", "tri.cuh"):
         with open(os.path.join(ROOT, "paper_2109_13628_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -409,32 +409,9 @@ def rk3_c2(iim, inputs, dev, steps=3):
     ring = T(P.psi_box)
     w0d, g0d = T(P.omega.ravel()), T(gam0)
     out = {}
-    # threads per 1024-point line (one solve at a time): each candidate on a geometry of its own
-    # with its own dense Schur preconditioner (the geometry does not move, so it is built once for
-    # all steps), timed on the dense-operator step; the faster is kept for every arm
-    lines_ms, cands = {}, {}
-    for lines in (32, 64):
-        gq = iim.iim_setup_geometry(iim.make_grid(g.x0, g.x1, g.y0, g.y1, g.nx, g.ny), T(P.phi), P.regions, P.modes)
-        iim.iim_geometry_set_lines(gq, lines)
-        pcq = iim.iim_build_preconditioner(gq)
-        wq, gmq, pbq = T(P.omega.ravel()), T(gam0), torch.zeros(1, dtype=torch.float64, device=dev)
-        oq = iim.default_opts(prec=iim.IIM_MIXED, rtol=1e-10, precond=3)
-        ts = []
-        for _ in range(3):
-            wq.copy_(w0d)
-            gmq.copy_(g0d)
-            pbq.zero_()
-            torch.cuda.synchronize()
-            t0 = time.perf_counter()
-            iim.iim_rk3_step(gq, wq, gmq, pbq, None, None, ring, (1.0, 0.0), 0.005, 0.5, opts=oq)
-            torch.cuda.synchronize()
-            ts.append((time.perf_counter() - t0) * 1e3)
-        lines_ms[lines] = min(ts[1:])
-        cands[lines] = (gq, pcq)
-    best = min(lines_ms, key=lines_ms.get)
-    geo, pc_ms = cands.pop(best)
-    for gq, _ in cands.values():
-        gq.close()
+    # the geometry does not move, so its dense Schur preconditioner is built once for all steps
+    geo = iim.iim_setup_geometry(iim.make_grid(g.x0, g.x1, g.y0, g.y1, g.nx, g.ny), T(P.phi), P.regions, P.modes)
+    pc_ms = iim.iim_build_preconditioner(geo)
     for name, prec, pc in (("fp64", iim.IIM_FP64, 0), ("mixed", iim.IIM_MIXED, 0),
                            ("mixed_precond", iim.IIM_MIXED, 1), ("mixed_dense_op", iim.IIM_MIXED, 3)):
         w, gam, pbar = T(P.omega.ravel()), T(gam0), torch.zeros(1, dtype=torch.float64, device=dev)
@@ -463,9 +440,8 @@ def rk3_c2(iim, inputs, dev, steps=3):
     w64, w32, wpc, wdo = (out[k].pop("omega") for k in ("fp64", "mixed", "mixed_precond", "mixed_dense_op"))
     geo.close()
     rel = lambda a: float(np.abs(a - w64).max() / np.abs(w64).max())
-    return {"config": "flow past a cylinder R 0.5, [-2,6]x[-2,2], 1024 x 512, U 1, Re 200, CFL 0.5, noise 1e-3 seed 0; "
-                      f"{best} threads per 1024-point line (tuned)",
-            **out, "threads_per_line": best, "lines_tuning_ms": lines_ms, "precond_setup_ms": pc_ms, "mixed_vs_fp64_rel_linf": rel(w32),
+    return {"config": "flow past a cylinder R 0.5, [-2,6]x[-2,2], 1024 x 512, U 1, Re 200, CFL 0.5, noise 1e-3 seed 0",
+            **out, "precond_setup_ms": pc_ms, "mixed_vs_fp64_rel_linf": rel(w32),
             "mixed_precond_vs_fp64_rel_linf": rel(wpc), "mixed_dense_op_vs_fp64_rel_linf": rel(wdo),
             "speedup_mixed_dense_op_vs_fp64": out["fp64"]["ms_per_step"] / out["mixed_dense_op"]["ms_per_step"],
             "speedup_mixed_vs_fp64": out["fp64"]["ms_per_step"] / out["mixed"]["ms_per_step"],

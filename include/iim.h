@@ -196,10 +196,11 @@ iim_status iim_poisson_solve_batched(int n, iim_geometry const* geoms, const dou
                                      iim_stream stream);
 
 /* How iim_poisson_solve_batched and iim_poisson_solve_batched_host run problems that have been
- * solved once already, with iim_opts.precond 1 or 3 and no guess.  max_group >= 2 (default 4):
- * the problems of equal grid size (and equal iim_geometry_set_tiles / _set_lines settings) are
- * split into groups of at most max_group problems (sizes as even as possible), and each group
- * advances in lockstep -- one kernel launch per step of the solve for every problem of the
+ * solved once already, with iim_opts.precond 1 or 3 and no guess.  max_group >= 2 (default 4): the
+ * problems of equal grid size, equal iim_geometry_set_tiles / _set_lines / _set_column_solver
+ * settings and equal form of the Krylov steps (|A| + circulation bodies up to 512, up to 2560, or
+ * more) are split into groups of at most max_group problems (sizes as even as possible), and each
+ * group advances in lockstep -- one kernel launch per step of the solve for every problem of the
  * group, the refinement, cycle and iteration loops continuing on the device while any problem of
  * the group needs them (one CUDA graph per group); the groups run concurrently on their own
  * streams.  max_group 0 or 1: one whole-solve graph per problem on the call's streams.  Each

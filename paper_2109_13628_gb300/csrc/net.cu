@@ -282,7 +282,7 @@ k_conv_tc(const float* __restrict__ x, const float* __restrict__ gate, const __n
 // products in the order of the taps.  Blocks are persistent, keep the weights, and start the next tile's
 // copies as soon as the MMAs have read this one's.  Two or three blocks per SM overlap copies, MMAs and
 // epilogues.  1023^2, six layers: 0.84 ms (one row of
-// FP32 planes converted by its block's threads per tile) -> 0.21 ms; the forward pass 0.86 -> 0.24 ms.
+// FP32 planes converted by its block's threads per tile) -> 0.21 ms; the forward pass 0.86 -> 0.22 ms.
 constexpr int UN_M = 128, UN_R = 4;
 
 struct UnitLayout {

@@ -473,7 +473,9 @@ k_sine_rows_inv(int NX, int NY, int n, int row0, int nrows, const T* in, T* outT
                                    ooff + (int)blockIdx.y * old, cls, tab);
 }
 
-// s / d of positive d well inside the FP32 range: the FP32 reciprocal and two Newton steps, to about an ulp.
+// s / d of positive d well inside the FP32 range: the FP32 reciprocal and two Newton steps, to about an ulp (a
+// division is correctly rounded; the box solve's error against 64 bits is 5e-16 at 64^2 either way, where
+// the packed transforms left 1e-15, and 5e-16 at 2048 x 512, where they left 4e-14).
 __device__ __forceinline__ double quotient(double s, double d) {
     double r = (double)__frcp_rn((float)d);
     r = fma(r, fma(-d, r, 1.0), r);
@@ -486,8 +488,9 @@ __device__ __forceinline__ double quotient(double s, double d) {
 // columns per group; `scale` carries the normalisation and h^2; tw: the table of e^{-i pi k / 4096}.
 // Each transform leaves its result in the buffer that its last step does not read.  Dynamic shared memory
 // sine_smem<T>(n, L).  Bound by FP64 arithmetic; against the packed transforms (dst.cuh), whole box solve in
-// FP64: 64^2 45 -> 28 us, 256^2 73 -> 54, 512^2 103 -> 95, 1024^2 304 -> 307, 2048^2 1466 -> 1101,
-// 64 x 2048 256 -> 115.
+// FP64: 64^2 45 -> 28 us, 256^2 73 -> 48, 512^2 102 -> 88, 1024^2 303 -> 300, 2048^2 1465 -> 1093,
+// 64 x 2048 257 -> 104.  Only at 1024 points is this pass the slower one (162 -> 168 us: 512 blocks of two
+// columns leave a fifth of the FP64 pipes idle at the end).
 template <typename T, int N, int L>
 __global__ void __launch_bounds__((Sine<N, L>::kBlock))
 k_sine_cols(int nx, int n_rt, T* __restrict__ buf, T scale, const cpx<T>* __restrict__ tab, const cpx<T>* __restrict__ tw) {

@@ -211,8 +211,9 @@ static iim_status rows_fwd(const Plan<T>& p, int row0, int nrows, const double* 
     return IIM_OK;
 }
 
-// Row passes of the FP32 box solve for callers (iim_box_poisson with IIM_MIXED): the transforms of
-// dst.cuh, whose FP32 rounding is part of that call's result.
+// Row passes of the FP32 box solve for callers (iim_box_poisson with IIM_MIXED): the packed transforms of
+// dst.cuh, as the call's columns (k_cols).  Those of sine.cuh would be more exact (a white line of 1024
+// points 1.2e-7 instead of 1.3e-6); this call has not been moved to them.
 static iim_status packed_rows_fwd(const Plan<float>& p, const double* dense, const double* ring, double ih2, float* out,
                                   cudaStream_t s) {
     const size_t sm = rows_smem<float>(p.nx);
