@@ -33,31 +33,36 @@ RTOL = 1e-10
 WORKLOAD = ("c1_cylinder_1024: [-2,2]^2, 1024x1024 cells (1023^2 unknowns), one cylinder R=0.5 at the origin, "
             "manufactured psi = sin(pi x/2) sin(pi y/2) + 0.1 log r, Dirichlet box and body data from psi, "
             "fixed-psibar body, solve to un-reduced FP64 relative residual 1e-10")
-# DRAM traffic per launch of the dominant kernel from the committed ncu capture, valid for
-# the kernel source hash below (null otherwise).
+# DRAM traffic per launch of the dominant kernel from the committed ncu captures, valid for the hash of the
+# kernel's source files (null otherwise).
 NCU_TRAFFIC = {
-    # python -m paper_2109_13628_gb300.passes --n 1024 --col 0 --batch 40 under ncu --metrics (DRAM
-    # and L2 sector counters, -k regex:k_cols -c 1): 40 fields in one launch, DRAM 167.7 MB read +
-    # 111.7 MB written, L2 (requests from the SMs) 12.92 M read + 5.24 M write sectors; scaled by
-    # the fields to the roofline's launch of 95 fields
-    "dst_cols_f32": {"bytes_per_launch": 279431424 / 40 * 95, "l2_bytes_per_launch": 18158481 * 32 / 40 * 95,
-                     "launches": 1, "tile_width": 8, "source_hash": "9d871bd9078dccd9",
+    # python -m paper_2109_13628_gb300.passes --n 1024 --col 0 (column DSTs) or 1 --batch 40 under ncu --metrics
+    # (DRAM and L2 sector counters, -k regex:<kernel> -c 1): 40 fields in one launch; scaled by the fields to
+    # the roofline's launch of 95 fields
+    # k_cols: DRAM 167.7 MB read + 112.3 MB written, L2 12.92 M + 5.24 M sectors
+    "dst_cols_f32": {"bytes_per_launch": 280002816 / 40 * 95, "l2_bytes_per_launch": 18161676 * 32 / 40 * 95,
+                     "launches": 1, "tile_width": 8, "source_hash": "fb6051612007d295",
                      "note": "one launch over 40 fields of 1023^2 (cold caches under ncu), scaled to 95 fields"},
-    # the same with --col 1 (-k regex:k_cols_scan): DRAM 167.7 MB + 112.1 MB, L2 11.08 M + 5.24 M
-    "tri_cols_f32": {"bytes_per_launch": 279818240 / 40 * 95, "l2_bytes_per_launch": 16315596 * 32 / 40 * 95,
-                     "launches": 1, "tile_width": 8, "source_hash": "9d871bd9078dccd9",
+    # k_cols_scan: DRAM 167.7 MB read + 111.7 MB written, L2 10.99 M + 5.24 M sectors
+    "tri_cols_f32": {"bytes_per_launch": 279393024 / 40 * 95, "l2_bytes_per_launch": 16229570 * 32 / 40 * 95,
+                     "launches": 1, "tile_width": 8, "source_hash": "fb6051612007d295",
                      "note": "one launch over 40 fields of 1023^2 (cold caches under ncu), scaled to 95 fields"},
-    # the same with --col 1, -k regex:k_rows_inv (FP32-store mode, the form iim_time_box_passes
-    # times): DRAM 167.7 MB read + 117.8 MB written, L2 9.12 M + 5.24 M sectors
-    # the same, -k regex:k_rows_fwd (dense FP64 input rows, FP32 output): DRAM 335.4 MB read +
-    # 132.3 MB written (algorithmic 40 x 1023^2 x 12 B = 502.3 MB), L2 15.22 M + 5.24 M sectors
-    "dst_rows_fwd_f32": {"bytes_per_launch": 467641088 / 40 * 95, "l2_bytes_per_launch": 20460365 * 32 / 40 * 95,
-                         "launches": 1, "tile_width": None, "source_hash": "9d871bd9078dccd9",
+    # k_sine_rows_fwd (FP64 rows in, FP32 out): DRAM 335.3 MB read + 134.8 MB written, L2 15.07 M + 5.24 M sectors
+    "dst_rows_fwd_f32": {"bytes_per_launch": 470086656 / 40 * 95, "l2_bytes_per_launch": 20304869 * 32 / 40 * 95,
+                         "launches": 1, "tile_width": None, "source_hash": "fb6051612007d295",
                          "note": "one launch over 40 fields of 1023^2 (cold caches under ncu), scaled to 95 fields"},
-    "dst_rows_inv_f32": {"bytes_per_launch": 285513728 / 40 * 95, "l2_bytes_per_launch": 14361815 * 32 / 40 * 95,
-                         "launches": 1, "tile_width": None, "source_hash": "9d871bd9078dccd9",
+    # k_sine_rows_inv (FP32 store, the form iim_time_box_passes times): DRAM 167.7 MB read + 120.5 MB written,
+    # L2 8.71 M + 5.24 M sectors
+    "dst_rows_inv_f32": {"bytes_per_launch": 288142080 / 40 * 95, "l2_bytes_per_launch": 13950553 * 32 / 40 * 95,
+                         "launches": 1, "tile_width": None, "source_hash": "fb6051612007d295",
                          "note": "one launch over 40 fields of 1023^2 (cold caches under ncu), scaled to 95 fields"},
+    # k_residual of a 1024^2 solve with one cylinder: DRAM 17.1 MB read (17 B per node), the 8 B per node it writes
+    # still in L2; L2 0.93 M + 0.26 M sectors
+    "residual_f64": {"bytes_per_launch": 17050624, "l2_bytes_per_launch": 1191620 * 32, "launches": 1,
+                     "tile_width": None, "sources": ("iim_ops.cuh",), "source_hash": "e035dce4d191b813",
+                     "note": "one launch on 1023^2 (cold caches under ncu)"},
 }
+TRANSFORM_SOURCES = ("dst.cuh", "sine.cuh", "tri.cuh")
 
 
 L2_BYTES = 126 * 1024 * 1024
@@ -66,11 +71,11 @@ PASS_NAMES = {0: ("dst_rows_fwd_f32", "dst_cols_f32", "dst_rows_inv_f32"),
               1: ("dst_rows_fwd_f32", "tri_cols_f32", "dst_rows_inv_f32")}
 
 
-def kernel_source_hash():
-    """Hash of the files holding the transform kernels' code (the launch shape of a capture is
-    recorded beside it: tile width, fields per launch)."""
+def kernel_source_hash(files=TRANSFORM_SOURCES):
+    """Hash of the files holding a captured kernel's code (the launch shape of a capture is recorded
+    beside it: tile width, fields per launch)."""
     h = hashlib.sha256()
-    for f in ("dst.cuh", "sine.cuh", "tri.cuh"):
+    for f in files:
         with open(os.path.join(ROOT, "paper_2109_13628_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -958,7 +963,7 @@ def main():
         per_launch_s = dom["ms"] * 1e-3 / dom["launches"]
         ev_achieved = dom["bytes"] / dom["launches"] / per_launch_s / 1e9
         tr = NCU_TRAFFIC.get(dom["name"])
-        valid = (bool(tr) and tr.get("source_hash") == kernel_source_hash()
+        valid = (bool(tr) and tr["source_hash"] == kernel_source_hash(tr.get("sources", TRANSFORM_SOURCES))
                  and tr.get("tile_width") in (None, tile_w))   # the tile width matters for the column pass only
         traffic = tr["bytes_per_launch"] if valid else None
         l2_traffic = tr.get("l2_bytes_per_launch") if valid else None
